@@ -628,7 +628,7 @@ def sample_xi(tab, qs, chi, u):
     m = torch.clamp(lo, max=n - 2)
     p0, dp = row(m), dt[i, m] + w * (dt[i + 1, m] - dt[i, m])  # (differences first: neighbours are close)
     x0, dx = (math.log(1e-12), -math.log(1e-12) / (n - 1)) if qs else (0.0, 0.5 / (n - 1))
-    x = x0 + dx * m + torch.where(dp > 0, (r - p0) * dx / torch.where(dp > 0, dp, 1.0), 0.0)
+    x = x0 + dx * m.double() + torch.where(dp > 0, (r - p0) * dx / torch.where(dp > 0, dp, 1.0), 0.0)
     return (torch.exp(torch.clamp(x, max=0.0)) if qs else torch.clamp(x, 0.0, 0.5)), electron
 
 

@@ -8,18 +8,27 @@
 //   which converges exponentially for this analytic, even integrand (Trefethen &
 //   Weideman, SIAM Review 56 (2014) 385).  Step h = min(1/4, 0.6/sqrt(x)) keeps
 //   the discretisation error near exp(-40); both integrals share one pass.
-//   Outer integrals over xi: tanh-sinh (double-exponential) quadrature on every
-//   table interval (Takahasi & Mori 1974; Bailey, Jeyabalan & Li, Exp. Math. 14
-//   (2005) 317), which absorbs the steep endpoint behaviour at xi -> 0 and 1.
+//   The tables need them at millions of arguments but only as functions of one
+//   variable, so the trapezoid rule runs at the Chebyshev nodes of 160 pieces of
+//   that variable (bessel_pieces_kernel) and the integrands evaluate the pieces'
+//   polynomials: 26 FMAs instead of ~25 steps of an exponential, a hyperbolic
+//   sine and divisions each.
+//   Outer integrals over xi: 16-point Gauss-Legendre on the table intervals
+//   where the integrand is smooth (gl_interval), at nodes that all rows share;
+//   tanh-sinh (double-exponential) quadrature (Takahasi & Mori 1974; Bailey,
+//   Jeyabalan & Li, Exp. Math. 14 (2005) 317) on the others, which absorbs the
+//   steep endpoint behaviour at xi -> 0 and 1.
 //   QS (Eq. (qs_g_func)) integrates S(chi, xi) d(ln xi); BW (Eq. (t_func_0))
 //   integrates the bracket in xi = chi_- / chi_gamma over [0, 1/2].
 //
-// One CTA per table row; one warp per xi interval; the interval sums are
-// reduced by shuffles in a fixed order, so the tables are bit-reproducible.
+// One CTA per table row; one thread per Gauss-Legendre interval, one warp per
+// tanh-sinh interval, whose sums are reduced by shuffles in a fixed order, so the
+// tables are bit-reproducible.
 #include <cmath>
 #include <vector>
 
 #include "common.cuh"
+#include "fp64_math.cuh"
 
 namespace qed {
 
@@ -59,19 +68,6 @@ __device__ void bessel_scaled(double x, double nu_a, double nu_b, double &ia, do
     kb = h * sb;
 }
 
-// QS integrand in u = ln xi: S(chi, xi) = sqrt(3)/(2 pi) xi [int_Y K_{5/3} + xi^2/(1-xi) K_{2/3}(Y)]
-__device__ double qs_integrand(double chi, double u)
-{
-    const double xi = exp(u);
-    const double om = -expm1(u);  // 1 - xi
-    if (!(om > 0.0)) return 0.0;
-    const double Y = (2.0 / 3.0) * xi / (chi * om);
-    if (Y > 745.0) return 0.0;
-    double ia, kb;
-    bessel_scaled(Y, 5.0 / 3.0, 2.0 / 3.0, ia, kb);
-    return (0.27566444771089600 /* sqrt(3) / (2 pi) */) * xi * exp(-Y) * (ia + xi * xi / om * kb);
-}
-
 // BW bracket in xi: int_z K_{1/3} + (xi/(1-xi) + (1-xi)/xi) K_{2/3}(z), z = 2/(3 chi xi (1-xi))
 __device__ double bw_integrand(double chi, double xi)
 {
@@ -84,98 +80,292 @@ __device__ double bw_integrand(double chi, double xi)
     return exp(-z) * (ia + (xi / om + om / xi) * kb);
 }
 
-// node k of tanh-sinh on [a, b]: abscissa (taken as an offset from the nearer
-// end so that it stays exact near the ends) and weight
-__device__ __forceinline__ void ts_node(double a, double b, int k, double &x, double &w)
+// ---------------------------------------------------------------------------
+// The two scaled functions of a process, e^x int_x^inf K_a and e^x K_b, as
+// piecewise polynomials: four pieces per octave of x from 2^-30 to 2^10 (the
+// integrands end at x = 745), degree 13.  Both functions are analytic in x but
+// for x <= 0; a piece's centre lies at least 9 of its half-widths from 0, so its
+// Chebyshev coefficients fall by a factor of 9 + sqrt(80) = 17.9 each and the
+// truncation after 14 is below 3e-18.  The piece comes from the bits of x: no
+// logarithm.  Below 2^-30 the two leading terms of the power series, whose
+// relative remainder is of order x^2 < 2^-60.
+// ---------------------------------------------------------------------------
+constexpr int kPieceOct = -30, kPieceOcts = 40, kPieces = 4 * kPieceOcts, kPieceCoef = 14;
+constexpr int kPieceRow = 2 * kPieceCoef;  // both functions of a piece
+
+// one warp per piece of one process; blockIdx.y: QS (nu 5/3, 2/3) or BW (1/3, 2/3)
+__global__ void __launch_bounds__(32) bessel_pieces_kernel(double *out)
 {
-    const double r = 0.5 * (b - a);
-    const double tk = k * kTsStep;
-    const double s = 0.5 * kPi * sinh(tk);
-    const double e = exp(2.0 * fabs(s));
-    const double d = 2.0 * r / (1.0 + e);  // distance to the nearer end
-    x = (k < 0) ? a + d : (k > 0 ? b - d : 0.5 * (a + b));
-    const double ch = cosh(s);
-    w = r * kTsStep * 0.5 * kPi * cosh(tk) / (ch * ch);
+    const int piece = blockIdx.x, lane = threadIdx.x;
+    const double scale = ldexp(1.0, kPieceOct + piece / 4);
+    double f[2] = {0.0, 0.0};
+    if (lane < kPieceCoef) {
+        const double x = cospi((lane + 0.5) / kPieceCoef);  // Chebyshev node in [-1, 1]
+        bessel_scaled(scale * (1.0 + (2 * (piece % 4) + 1 + x) / 8.0), (blockIdx.y ? 1.0 : 5.0) / 3.0, 2.0 / 3.0, f[0],
+                      f[1]);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        // lane i: Chebyshev coefficient i, then the coefficient of x^i by the
+        // recurrence T_k = 2 x T_{k-1} - T_{k-2}
+        double c = 0.0;
+        for (int i = 0; i < kPieceCoef; ++i) {
+            const int turn = (2 * i + 1) * lane % (4 * kPieceCoef);  // the angle in units of pi / (2 kPieceCoef)
+            c += __shfl_sync(0xffffffffu, f[k], i) * cospi((double)turn / (2 * kPieceCoef));
+        }
+        c *= (lane ? 2.0 : 1.0) / kPieceCoef;
+        double t0 = lane == 0 ? 1.0 : 0.0, t1 = lane == 1 ? 1.0 : 0.0;  // T_0, T_1
+        double p = __shfl_sync(0xffffffffu, c, 0) * t0 + __shfl_sync(0xffffffffu, c, 1) * t1;
+        for (int n = 2; n < kPieceCoef; ++n) {
+            const double up = __shfl_up_sync(0xffffffffu, t1, 1);
+            const double t2 = 2.0 * (lane ? up : 0.0) - t0;
+            p += __shfl_sync(0xffffffffu, c, n) * t2;
+            t0 = t1, t1 = t2;
+        }
+        if (lane < kPieceCoef) out[((size_t)blockIdx.y * kPieces + piece) * kPieceRow + k * kPieceCoef + lane] = p;
+    }
+}
+
+constexpr double kGamma13 = 2.6789385347077476, kGamma23 = 1.3541179394264004;  // Gamma(1/3), Gamma(2/3)
+constexpr double kTwo13 = 1.2599210498948732, kTwo23 = 1.5874010519681994;      // 2^(1/3), 2^(2/3)
+constexpr double kPiSqrt3 = 1.8137993642342178;                                  // pi / sqrt(3)
+
+// e^x int_x^inf K_{5/3 or 1/3} and e^x K_{2/3} for 0 < x < 2^10 from the pieces `c` of the process
+__device__ __forceinline__ void bessel_at(const double *c, bool qs, double x, double &ia, double &kb)
+{
+    const int hi = __double2hiint(x);
+    const int i = ((hi >> 20) - 1023 - kPieceOct) * 4 + ((hi >> 18) & 3);
+    if (i < 0) {
+        const double r = cbrt(x), r2 = r * r;
+        kb = (1.0 + x) * (0.5 * kGamma23 * kTwo23 / r2 - 0.75 * kGamma13 / kTwo23 * r2);
+        ia = (1.0 + x) * (qs ? kGamma23 * kTwo23 / r2 - kPiSqrt3
+                             : kPiSqrt3 - 0.75 * kGamma13 * kTwo13 * r2 + 1.125 * kGamma23 / kTwo13 * r2 * r2);
+        return;
+    }
+    const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));  // x / 2^e in [1, 2)
+    const double t = fma(m, 8.0, -(9.0 + 2 * ((hi >> 18) & 3)));                           // the piece's [-1, 1]
+    const double *p = c + min(i, kPieces - 1) * kPieceRow;
+    double a = p[kPieceCoef - 1], b = p[2 * kPieceCoef - 1];
+#pragma unroll
+    for (int k = kPieceCoef - 2; k >= 0; --k) {
+        a = fma(a, t, p[k]);
+        b = fma(b, t, p[kPieceCoef + k]);
+    }
+    ia = a, kb = b;
+}
+
+// QS integrand in u = ln xi: S(chi, xi) = sqrt(3)/(2 pi) xi [int_Y K_{5/3} + xi^2/(1-xi) K_{2/3}(Y)],
+// Y = (2/3) xi / (chi (1 - xi)); BW the bracket in xi.  The integrand is
+// e^(-q/chi) [va int(q/chi) + vb K_{2/3}(q/chi)] with q, va, vb functions of xi alone.
+constexpr double kQsFactor = 0.27566444771089600;  // sqrt(3) / (2 pi)
+
+__device__ __forceinline__ void node_terms(bool qs, double x, double &q, double &va, double &vb)
+{
+    if (qs) {
+        const double xi = exp(x), om = -expm1(x);  // 1 - xi
+        q = (2.0 / 3.0) * xi / om;
+        va = kQsFactor * xi;
+        vb = va * (xi * xi / om);
+    } else {
+        const double om = 1.0 - x;
+        q = (2.0 / 3.0) / (x * om);
+        va = 1.0;
+        vb = x / om + om / x;
+    }
+}
+
+__device__ __forceinline__ double row_integrand(const double *c, bool qs, double inv_chi, double q, double va,
+                                                double vb)
+{
+    const double y = q * inv_chi;
+    if (!(y <= 745.0)) return 0.0;  // (also 1 - xi = 0, where q is infinite)
+    double ia, kb;
+    bessel_at(c, qs, y, ia, kb);
+    return exp_tang(-y) * fma(vb, kb, va * ia);
 }
 
 struct GenArgs {
     double *qs_lnG, *qs_lnP, *bw_lnT, *bw_P;
     double qs_l0, qs_l1, qs_xi_min, bw_l0, bw_l1;
     int qs_n_chi, qs_n_xi, bw_n_chi, bw_n_xi;
+    double *pieces;  // [2][kPieces][kPieceRow]: the Bessel functions
+    double *nodes;   // [2][3][kGl][QED_MAX_TABLE_N]: q, w va, w vb at the Gauss-Legendre nodes of every interval
 };
 
+// interval j of a row: QS j = 0 is [xi_min e^-100, xi_min] in ln xi, j >= 1 is
+// [xi_{j-1}, xi_j]; BW j >= 1 is [xi_{j-1}, xi_j] on the linear grid, j = 0 empty
+__device__ __forceinline__ void row_interval(bool qs, double ln_xi_min, int M, int j, double &lo, double &hi)
+{
+    if (qs) {
+        lo = j == 0 ? ln_xi_min - kQsBelow : ln_xi_min + (j - 1) * (-ln_xi_min) / (M - 1);
+        hi = (j == M - 1) ? 0.0 : ln_xi_min + j * (-ln_xi_min) / (M - 1);
+    } else {
+        lo = 0.5 * (j - 1) / (M - 1);
+        hi = (j == M - 1) ? 0.5 : 0.5 * j / (M - 1);
+    }
+}
+
+// Gauss-Legendre (16 points, weights and nodes of the reference interval by
+// value): where the integrand's singularity (QS: ln xi = 0, where 1 - xi
+// vanishes; BW: xi = 0) lies at least twice the interval's half-width from its
+// centre (the error falls like (2 + sqrt 3)^-32 = 5e-19), the interval is not
+// wide against the integrand's own scale in ln xi, and e^-Y falls by at most
+// e^-12 across it (the error of e^-6t on [-1, 1] is 2e-20).
+constexpr int kGl = 16;
+struct GaussLegendre16 {
+    double x[kGl], w[kGl];
+};
+
+__device__ __forceinline__ bool gl_smooth(bool qs, double lo, double hi)
+{
+    const double c = 0.5 * (lo + hi), h = 0.5 * (hi - lo);
+    return qs ? (-c >= 2.0 * h && h <= 0.5) : (c >= 2.0 * h);
+}
+
+// the nodes that every row of a process shares: thread = interval, blockIdx.y = process
+__global__ void __launch_bounds__(128) row_nodes_kernel(const __grid_constant__ GenArgs a,
+                                                         const __grid_constant__ GaussLegendre16 g)
+{
+    const bool qs = blockIdx.y == 0;
+    const int M = qs ? a.qs_n_xi : a.bw_n_xi;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < 1 || j >= M) return;
+    double lo, hi;
+    row_interval(qs, log(a.qs_xi_min), M, j, lo, hi);
+    double *out = a.nodes + (size_t)blockIdx.y * 3 * kGl * QED_MAX_TABLE_N;
+    const double c = 0.5 * (lo + hi), h = 0.5 * (hi - lo);
+    for (int k = 0; k < kGl; ++k) {
+        double q, va, vb;
+        node_terms(qs, fma(h, g.x[k], c), q, va, vb);
+        out[(size_t)k * QED_MAX_TABLE_N + j] = q;
+        out[(size_t)(kGl + k) * QED_MAX_TABLE_N + j] = g.w[k] * h * va;
+        out[(size_t)(2 * kGl + k) * QED_MAX_TABLE_N + j] = g.w[k] * h * vb;
+    }
+}
+
+// One CTA per row.  Bound by the FP64 pipe: ~60 FP64 instructions per
+// Gauss-Legendre node, 256 x 16 nodes in a row of the 256 x 256 tables, and the
+// tanh-sinh intervals (two at the ends, and the few per row across which e^-Y
+// falls steeply), whose nodes and weights on [-1, 1] are shared too.
 __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__ GenArgs a)
 {
-    __shared__ double acc[QED_MAX_TABLE_N];
+    __shared__ double acc[QED_MAX_TABLE_N], tail[QED_MAX_TABLE_N];
+    extern __shared__ double s_c[];  // [kPieces][kPieceRow]
+    __shared__ double s_ts[2][kTsHalf + 1];  // tanh-sinh: distance of node k from the nearer end, weight (half-widths)
+    __shared__ short s_hard[QED_MAX_TABLE_N];
+    __shared__ int s_n_hard;
+    __shared__ double s_tot;
     const bool qs = blockIdx.x < (unsigned)a.qs_n_chi;
     const int row = qs ? blockIdx.x : blockIdx.x - a.qs_n_chi;
     const int N = qs ? a.qs_n_chi : a.bw_n_chi;
     const int M = qs ? a.qs_n_xi : a.bw_n_xi;
     const double l0 = qs ? a.qs_l0 : a.bw_l0, l1 = qs ? a.qs_l1 : a.bw_l1;
     const double chi = exp(row == N - 1 ? l1 : l0 + row * (l1 - l0) / (N - 1));
+    const double inv_chi = 1.0 / chi;
     const double lxm = log(a.qs_xi_min);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
 
-    // interval j of the row: QS j = 0 is [xi_min e^-100, xi_min] in ln xi, j >= 1 is
-    // [xi_{j-1}, xi_j]; BW j >= 1 is [xi_{j-1}, xi_j] on the linear grid, j = 0 empty
-    for (int j = warp; j < M; j += nw) {
+    const double *pieces = a.pieces + (qs ? 0 : (size_t)kPieces * kPieceRow);
+    for (int i = threadIdx.x; i < kPieces * kPieceRow; i += blockDim.x) s_c[i] = pieces[i];
+    if (threadIdx.x <= kTsHalf) {
+        const double tk = threadIdx.x * kTsStep;
+        const double s = 0.5 * kPi * sinh(tk), ch = cosh(s);
+        s_ts[0][threadIdx.x] = 2.0 / (1.0 + exp(2.0 * s));
+        s_ts[1][threadIdx.x] = kTsStep * 0.5 * kPi * cosh(tk) / (ch * ch);
+    }
+    if (threadIdx.x == 0) s_n_hard = 0;
+    __syncthreads();
+
+    const double *nodes = a.nodes + (qs ? 0 : (size_t)3 * kGl * QED_MAX_TABLE_N);
+    for (int j = threadIdx.x; j < M; j += blockDim.x) {
         double lo, hi;
-        if (qs) {
-            if (j == 0) {
-                lo = lxm - kQsBelow, hi = lxm;
-            } else {
-                lo = lxm + (j - 1) * (-lxm) / (M - 1);
-                hi = (j == M - 1) ? 0.0 : lxm + j * (-lxm) / (M - 1);
-            }
-        } else {
-            lo = 0.5 * (j - 1) / (M - 1);
-            hi = (j == M - 1) ? 0.5 : 0.5 * j / (M - 1);
+        row_interval(qs, lxm, M, j, lo, hi);
+        if (!qs && j == 0) {
+            acc[0] = 0.0;
+            continue;
         }
-        double part = 0.0;
-        if (qs || j > 0) {
-            for (int k = lane - kTsHalf; k <= kTsHalf; k += 32) {
-                double x, w;
-                ts_node(lo, hi, k, x, w);
-                part += w * (qs ? qs_integrand(chi, x) : bw_integrand(chi, x));
+        bool smooth = j > 0 && gl_smooth(qs, lo, hi);
+        if (smooth) {
+            // the outermost nodes lie within 1 % of the ends: Y's fall between them
+            const double q0 = nodes[j], q1 = nodes[(size_t)(kGl - 1) * QED_MAX_TABLE_N + j];
+            if (fmin(q0, q1) * inv_chi > 800.0) {  // e^-Y is zero on all of it
+                acc[j] = 0.0;
+                continue;
             }
+            smooth = fabs(q1 - q0) * inv_chi <= 11.5;
+        }
+        if (smooth) {
+            double part = 0.0;
+            for (int k = 0; k < kGl; ++k) {
+                const double *p = nodes + (size_t)k * QED_MAX_TABLE_N + j;
+                part += row_integrand(s_c, qs, inv_chi, p[0], p[(size_t)kGl * QED_MAX_TABLE_N],
+                                      p[(size_t)2 * kGl * QED_MAX_TABLE_N]);
+            }
+            acc[j] = part;
+        } else {
+            s_hard[atomicAdd(&s_n_hard, 1)] = (short)j;
+        }
+    }
+    __syncthreads();
+    for (int i = warp; i < s_n_hard; i += nw) {
+        const int j = s_hard[i];
+        double lo, hi;
+        row_interval(qs, lxm, M, j, lo, hi);
+        const double r = 0.5 * (hi - lo);
+        double part = 0.0;
+        for (int k = lane - kTsHalf; k <= kTsHalf; k += 32) {
+            const double d = r * s_ts[0][abs(k)];  // offset from the nearer end, exact near the ends
+            const double x = k < 0 ? lo + d : (k > 0 ? hi - d : 0.5 * (lo + hi));
+            if (!qs && !(x > 0.0)) continue;
+            double q, va, vb;
+            node_terms(qs, x, q, va, vb);
+            part += s_ts[1][abs(k)] * row_integrand(s_c, qs, inv_chi, q, va, vb);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-        if (lane == 0) acc[j] = part;
+        if (lane == 0) acc[j] = r * part;
+    }
+    __syncthreads();
+    // running sums from both ends, in order (one thread each)
+    if (threadIdx.x == 0) {
+        double c = 0.0;
+        for (int m = M - 1; m >= 0; --m) {
+            tail[m] = c;  // the sum right of m
+            c += acc[m];
+        }
+    } else if (threadIdx.x == 32) {
+        double c = 0.0;
+        for (int m = 0; m < M; ++m) c += acc[m];
+        s_tot = c;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int j = 0; j < M; ++j) tot += acc[j];
-        if (qs) {
-            double *out = a.qs_lnP + (size_t)row * M;
-            double C = 0.0;
-            for (int m = 0; m < M; ++m) {
-                C += acc[m];
-                out[m] = C / tot;  // P_m
-            }
-            // ln P = ln(C/G), except near P = 1 where log1p(-tail/G) keeps the
-            // relative accuracy; tail = sum of the intervals right of m
-            double tr = 0.0;
-            for (int m = M - 1; m >= 0; --m) {
-                const double q = tr / tot;
-                out[m] = (q < 0.5) ? log1p(-q) : log(out[m]);
-                tr += acc[m];
-            }
-            out[M - 1] = 0.0;
-            a.qs_lnG[row] = log(tot);
-        } else {
-            double *out = a.bw_P + (size_t)row * M;
-            double C = 0.0;
-            for (int m = 0; m < M; ++m) {
-                C += acc[m];
-                out[m] = tot > 0.0 ? C / (2.0 * tot) : 0.0;
-            }
-            out[0] = 0.0;
-            if (tot > 0.0) out[M - 1] = 0.5;
-            // T = int_0^1 bracket / (pi sqrt(3) chi) = 2 tot / (pi sqrt(3) chi)
-            a.bw_lnT[row] = log(2.0 * tot / (kPi * 1.7320508075688772 * chi));
+        double c = 0.0;
+        for (int m = 0; m < M; ++m) {
+            c += acc[m];
+            acc[m] = c;
         }
+    }
+    __syncthreads();
+    const double tot = s_tot;
+    if (qs) {
+        // ln P = ln(C/G), except near P = 1 where log1p(-tail/G) keeps the relative accuracy
+        double *out = a.qs_lnP + (size_t)row * M;
+        for (int m = threadIdx.x; m < M; m += blockDim.x) {
+            const double t = tail[m] / tot;
+            out[m] = m == M - 1 ? 0.0 : (t < 0.5 ? log1p(-t) : log(acc[m] / tot));
+        }
+        if (threadIdx.x == 0) a.qs_lnG[row] = log(tot);
+    } else {
+        double *out = a.bw_P + (size_t)row * M;
+        for (int m = threadIdx.x; m < M; m += blockDim.x) {
+            double v = tot > 0.0 ? acc[m] / (2.0 * tot) : 0.0;
+            if (m == 0) v = 0.0;
+            if (m == M - 1 && tot > 0.0) v = 0.5;
+            out[m] = v;
+        }
+        // T = int_0^1 bracket / (pi sqrt(3) chi) = 2 tot / (pi sqrt(3) chi)
+        if (threadIdx.x == 0) a.bw_lnT[row] = log(2.0 * tot / (kPi * 1.7320508075688772 * chi));
     }
 }
 
@@ -383,11 +573,11 @@ __global__ void __launch_bounds__(128) exact_draw_kernel(int qs, const double *_
     }
 }
 
-// Gauss-Legendre nodes and weights (Newton's method on the three-term recurrence)
-static GaussLegendre8 gauss_legendre8()
+// Gauss-Legendre nodes and weights, n points (Newton's method on the three-term recurrence)
+template <typename G, int n>
+static G gauss_legendre()
 {
-    GaussLegendre8 g;
-    const int n = 8;
+    G g;
     for (int i = 0; i < n; ++i) {
         double x = std::cos(kPi * (i + 0.75) / (n + 0.5));
         double dp = 1.0;
@@ -425,7 +615,7 @@ extern "C" qed_status qed_exact_sample(qed_process proc, const double *d_chi, in
         QED_FAIL(QED_ERR_INVALID_ARG, "d_work holds %lld doubles, %lld needed", (long long)work_capacity,
                  (long long)QED_EXACT_WORK(m));
     static_assert(QED_EXACT_WORK(1) == kExactRowStride, "work layout");
-    static const GaussLegendre8 gl = gauss_legendre8();
+    static const GaussLegendre8 gl = gauss_legendre<GaussLegendre8, 8>();
     cudaStream_t st = as_stream(stream);
     const int qs = proc == QED_PROC_QS;
     exact_rows_kernel<<<(unsigned)m, 256, 0, st>>>(qs, d_chi, d_work, gl);
@@ -457,9 +647,25 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
     a.bw_l0 = std::log(params->bw.chi_min), a.bw_l1 = std::log(params->bw.chi_max);
     a.qs_n_chi = params->qs.n_chi, a.qs_n_xi = params->qs.n_xi;
     a.bw_n_chi = params->bw.n_chi, a.bw_n_xi = params->bw.n_xi;
-    table_rows_kernel<<<params->qs.n_chi + params->bw.n_chi, 256, 0, st>>>(a);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    // scratch of this call: the pieces and the shared nodes
+    constexpr size_t n_pieces = (size_t)2 * kPieces * kPieceRow, n_nodes = (size_t)2 * 3 * kGl * QED_MAX_TABLE_N;
+    double *work = nullptr;
+    cudaError_t e = cudaMalloc((void **)&work, (n_pieces + n_nodes) * sizeof(double));
+    if (e == cudaSuccess) {
+        a.pieces = work, a.nodes = work + n_pieces;
+        static const GaussLegendre16 gl = gauss_legendre<GaussLegendre16, kGl>();
+        const int m = params->qs.n_xi > params->bw.n_xi ? params->qs.n_xi : params->bw.n_xi;
+        bessel_pieces_kernel<<<dim3(kPieces, 2), 32, 0, st>>>(work);
+        row_nodes_kernel<<<dim3((m + 127) / 128, 2), 128, 0, st>>>(a, gl);
+        constexpr int dyn = kPieces * kPieceRow * (int)sizeof(double);
+        e = cudaFuncSetAttribute(table_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+        if (e == cudaSuccess) {
+            table_rows_kernel<<<params->qs.n_chi + params->bw.n_chi, 256, dyn, st>>>(a);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        cudaFree(work);
+    }
     if (e != cudaSuccess) {
         qed_tables_destroy(t);
         QED_FAIL(QED_ERR_CUDA, "table generation failed: %s", cudaGetErrorString(e));

@@ -84,3 +84,24 @@ def test_generation_rejects_underflowing_range(api):
     with pytest.raises(api.QedError) as e:
         api.qed_tables_generate(p)
     assert "QED_ERR_NUMERIC" in str(e.value)
+
+
+@pytest.mark.parametrize("n_chi,n_xi,xi_min,chi,tol", [
+    (5, 3, 0.3, (0.5, 20.0), 1e-10),       # intervals next to the singular end
+    (6, 64, 1e-6, (0.02, 1e3), 1e-10),     # e^-Y falls steeply: Gauss-Legendre and tanh-sinh side by side in a row
+    (4, 300, 1e-12, (0.02, 0.1), 1e-10),
+    (2, 1024, 1e-15, (0.1, 1e4), 1e-10),   # the largest row
+    (3, 2, 1e-12, (0.05, 1e3), 5e-9),      # one interval over the whole range: tanh-sinh only
+    (3, 40, 1e-3, (1e8, 1e10), 5e-9),      # arguments below the pieces' lower end (power series) in both processes
+])
+def test_generated_rows_over_the_axes_range(api, n_chi, n_xi, xi_min, chi, tol):
+    """Every kind of row interval (Gauss-Legendre, tanh-sinh) and of Bessel argument (pieces, power series) against the
+    oracle's adaptive quadrature, to the tolerance of the paper-size tables; where one interval spans many scales of the
+    integrand, to the error of the tanh-sinh rule at its step (1e-9)."""
+    ot = oracle.tables(qs_chi_min=chi[0], qs_chi_max=chi[1], qs_n_chi=n_chi, qs_n_xi=n_xi, qs_xi_min=xi_min,
+                       bw_chi_min=chi[0], bw_chi_max=chi[1], bw_n_chi=n_chi, bw_n_xi=n_xi)
+    g = api.qed_tables_copy_to_host(api.qed_tables_generate(_params(api, ot)))
+    assert np.max(np.abs(g["qs_lnG"] - ot.qs_lnG)) < tol
+    assert np.max(np.abs(g["bw_lnT"] - ot.bw_lnT)) < tol
+    assert np.all(np.abs(g["qs_lnP"] - ot.qs_lnP) <= tol * np.maximum(1.0, np.abs(ot.qs_lnP)))
+    assert np.all(np.abs(g["bw_P"] - ot.bw_P) <= tol * ot.bw_P + 1e-15)

@@ -262,13 +262,11 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1)
     long long *s_n = s_end + n_seg;
     __shared__ __align__(8) uint64_t s_full[S];
     __shared__ __align__(8) uint64_t s_empty[S];
-    __shared__ float s_qs[QED_MAX_TABLE_N];
-    __shared__ float s_bw[QED_MAX_TABLE_N];
+    __shared__ RateSmem<float> rs;
     __shared__ long long s_warp[THREADS / 32];
     __shared__ int s_abort;
 
-    for (int i = threadIdx.x; i < tab.qs_G.n; i += THREADS) s_qs[i] = tab.qs_G.ln_f[i];
-    for (int i = threadIdx.x; i < tab.bw_T.n; i += THREADS) s_bw[i] = tab.bw_T.ln_f[i];
+    stage_rates(rs, tab, THREADS);
     if (threadIdx.x == 0) {
         s_abort = 0;
         for (int k = 0; k < S; ++k) {
@@ -362,7 +360,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1)
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&s_empty[st]);
-        evolve_regs<float, 4>(sg, n, i0, full4, px, py, pz, ex, ey, ez, bx, by, bz, tau, tc, s_qs, s_bw, tab, dt,
+        evolve_regs<float, 4>(sg, n, i0, full4, px, py, pz, ex, ey, ez, bx, by, bz, tau, tc, rs, tab, dt,
                               sg.proc == QED_PROC_QS ? cut_qs : cut_bw, stats, dry, bad);
     }
     if (!dry) warp_count_err(stats ? stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);

@@ -12,6 +12,7 @@
 #include <cstdio>
 #include <string>
 
+#include "fixed64.cuh"
 #include "qed.h"
 
 namespace qed {
@@ -122,6 +123,7 @@ struct Table1D {
     T inv_d;         // (n - 1) / (ln chi_max - ln chi_min)
     T chi_min, chi_max;
     int n;
+    FixAxis fix;     // the axis on integers (the FP64 evolution, fixed64.cuh)
 };
 
 // bins of the guide tables that bracket the inverse-CDF search
@@ -219,6 +221,7 @@ struct qed_tables {
     float *f_qs_dlnP, *f_bw_dP;
     // guide tables of the 2-D tables' inverse-CDF search, one per precision
     int32_t *d_qs_guide, *d_bw_guide, *f_qs_guide, *f_bw_guide;
+    qed::FixAxis qs_fix, bw_fix;  // the 1-D tables' axes on integers
 };
 
 namespace qed {

@@ -20,8 +20,8 @@ namespace qed {
 // One tile: THREADS x VEC consecutive particles of segment `sg` starting at
 // tile index `first`, loaded straight from global memory.
 template <typename T, int VEC, int THREADS>
-__device__ __forceinline__ void evolve_tile(const EvolveSeg<T> &sg, int64_t n, long long first, const T *s_qs,
-                                            const T *s_bw, const TablesView<T> &tab, T dt, T cut, long long *stats,
+__device__ __forceinline__ void evolve_tile(const EvolveSeg<T> &sg, int64_t n, long long first, const RateSmem<T> &rs,
+                                            const TablesView<T> &tab, T dt, T cut, long long *stats,
                                             int dry, int &bad)
 {
     const int64_t i0 = first * ((int64_t)THREADS * VEC) + (int64_t)threadIdx.x * VEC;
@@ -42,7 +42,7 @@ __device__ __forceinline__ void evolve_tile(const EvolveSeg<T> &sg, int64_t n, l
     } else {
         load_scalar<T, VEC>(sg, n, i0, px, py, pz, ex, ey, ez, bx, by, bz, tau, tc);
     }
-    evolve_regs<T, VEC>(sg, n, i0, full, px, py, pz, ex, ey, ez, bx, by, bz, tau, tc, s_qs, s_bw, tab, dt, cut,
+    evolve_regs<T, VEC>(sg, n, i0, full, px, py, pz, ex, ey, ez, bx, by, bz, tau, tc, rs, tab, dt, cut,
                         stats, dry, bad);
 }
 
@@ -70,14 +70,12 @@ template <typename T, int VEC, int MAXSEG, int MINB = 3>
 __global__ void __launch_bounds__(kEvolveThreads, MINB)
     evolve_kernel(const __grid_constant__ EvolveArgs<T, MAXSEG> a)
 {
-    __shared__ T s_qs[QED_MAX_TABLE_N];
-    __shared__ T s_bw[QED_MAX_TABLE_N];
+    __shared__ RateSmem<T> rs;
     __shared__ long long s_end[MAXSEG];  // inclusive prefix of tile counts
     __shared__ long long s_n[MAXSEG];
     constexpr int64_t tile = kEvolveTile<T, VEC>;
 
-    for (int i = threadIdx.x; i < a.tab.qs_G.n; i += blockDim.x) s_qs[i] = a.tab.qs_G.ln_f[i];
-    for (int i = threadIdx.x; i < a.tab.bw_T.n; i += blockDim.x) s_bw[i] = a.tab.bw_T.ln_f[i];
+    stage_rates(rs, a.tab, blockDim.x);
     if (threadIdx.x == 0) {
         long long acc = 0;
         for (int s = 0; s < a.n_seg; ++s) {
@@ -94,7 +92,7 @@ __global__ void __launch_bounds__(kEvolveThreads, MINB)
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {
         int s = 0;
         while (t >= s_end[s]) ++s;
-        evolve_tile<T, VEC, kEvolveThreads>(a.seg[s], s_n[s], t - (s ? s_end[s - 1] : 0), s_qs, s_bw, a.tab, a.dt,
+        evolve_tile<T, VEC, kEvolveThreads>(a.seg[s], s_n[s], t - (s ? s_end[s - 1] : 0), rs, a.tab, a.dt,
                                             a.chi_cut[a.seg[s].proc], a.stats, 0, bad);
     }
     warp_count_err(a.stats ? a.stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
@@ -152,14 +150,12 @@ __global__ void __launch_bounds__((CW + 1) * 32, MINB)
     extern __shared__ __align__(128) float s_stage[];  // [S][kBulkArrays][TP]
     __shared__ __align__(8) uint64_t s_full[S];
     __shared__ __align__(8) uint64_t s_empty[S];
-    __shared__ float s_qs[QED_MAX_TABLE_N];
-    __shared__ float s_bw[QED_MAX_TABLE_N];
+    __shared__ RateSmem<float> rs;
     __shared__ long long s_end[MAXSEG];
     __shared__ long long s_n[MAXSEG];
     __shared__ int s_abort;
 
-    for (int i = threadIdx.x; i < a.tab.qs_G.n; i += blockDim.x) s_qs[i] = a.tab.qs_G.ln_f[i];
-    for (int i = threadIdx.x; i < a.tab.bw_T.n; i += blockDim.x) s_bw[i] = a.tab.bw_T.ln_f[i];
+    stage_rates(rs, a.tab, blockDim.x);
     if (threadIdx.x == 0) {
         long long acc = 0;
         for (int s = 0; s < a.n_seg; ++s) {
@@ -267,7 +263,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, MINB)
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&s_empty[st]);
-        evolve_regs<float, 4>(sg, n, i0, full4, px, py, pz, ex, ey, ez, bx, by, bz, tau, tc, s_qs, s_bw, a.tab,
+        evolve_regs<float, 4>(sg, n, i0, full4, px, py, pz, ex, ey, ez, bx, by, bz, tau, tc, rs, a.tab,
                               a.dt, a.chi_cut[sg.proc], a.stats, 0, bad);
     }
     warp_count_err(a.stats ? a.stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
@@ -298,24 +294,22 @@ static qed_status launch_bulk(const EvolveArgs<float, MAXSEG> &a, int64_t capaci
 // by binary search.
 template <typename T, int VEC, int THREADS>
 __global__ void __launch_bounds__(THREADS, 768 / THREADS)
-    evolve_seg_kernel(const EvolveSeg<T> *__restrict__ segs, int n_seg, TablesView<T> tab, T dt, T cut_qs, T cut_bw,
+    evolve_seg_kernel(const EvolveSeg<T> *__restrict__ segs, int n_seg, const __grid_constant__ TablesView<T> tab, T dt, T cut_qs, T cut_bw,
                       long long *stats, int dry)
 {
-    __shared__ T s_qs[QED_MAX_TABLE_N];
-    __shared__ T s_bw[QED_MAX_TABLE_N];
+    __shared__ RateSmem<T> rs;
     __shared__ long long s_warp[THREADS / 32];
     extern __shared__ long long s_dyn[];  // [n_seg] inclusive tile prefix, [n_seg] counts
     long long *s_end = s_dyn, *s_n = s_dyn + n_seg;
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
-    for (int i = threadIdx.x; i < tab.qs_G.n; i += THREADS) s_qs[i] = tab.qs_G.ln_f[i];
-    for (int i = threadIdx.x; i < tab.bw_T.n; i += THREADS) s_bw[i] = tab.bw_T.ln_f[i];
+    stage_rates(rs, tab, THREADS);
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);
     int bad = 0;
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {
         const int lo = find_segment(s_end, n_seg, t);
         const EvolveSeg<T> &sg = segs[lo];
-        evolve_tile<T, VEC, THREADS>(sg, s_n[lo], t - (lo ? s_end[lo - 1] : 0), s_qs, s_bw, tab, dt,
+        evolve_tile<T, VEC, THREADS>(sg, s_n[lo], t - (lo ? s_end[lo - 1] : 0), rs, tab, dt,
                                      sg.proc == QED_PROC_QS ? cut_qs : cut_bw, stats, dry, bad);
     }
     if (!dry) warp_count_err(stats ? stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
@@ -434,10 +428,15 @@ qed_status launch_evolve(const EvolveArgs<T, MAXSEG> &a, bool vec_ok, int64_t ca
     }
     if (vec_ok) {
         constexpr int V = sizeof(T) == 4 ? 4 : 2;
-        if (sizeof(T) == 4 && ctas_per_sm != 3) {  // 64 registers: 32 warps per SM (the faster)
-            const int g = grid_override > 0 ? grid_override : evolve_grid<T, V, MAXSEG, 4>(capacity_sum);
-            evolve_kernel<T, V, MAXSEG, 4><<<g, kEvolveThreads, 0, st>>>(a);
-        } else {
+        bool done = false;
+        if constexpr (sizeof(T) == 4) {
+            if (ctas_per_sm != 3) {  // 64 registers: 32 warps per SM (the faster)
+                const int g = grid_override > 0 ? grid_override : evolve_grid<T, V, MAXSEG, 4>(capacity_sum);
+                evolve_kernel<T, V, MAXSEG, 4><<<g, kEvolveThreads, 0, st>>>(a);
+                done = true;
+            }
+        }
+        if (!done) {
             const int g = grid_override > 0 ? grid_override : evolve_grid<T, V, MAXSEG>(capacity_sum);
             evolve_kernel<T, V, MAXSEG><<<g, kEvolveThreads, 0, st>>>(a);
         }

@@ -57,38 +57,147 @@ __device__ __forceinline__ void store_vec(T *p, int64_t i, const T (&in)[VEC])
     }
 }
 
-// one particle: chi, rate, optical-depth decrement; returns fire
+// The 1-D rate tables of both processes in shared memory: FP32 as they are, FP64
+// as 64-bit integers (units of 2^-53) with the tables of the integer logarithm
+// and exponential (fixed64.cuh).
 template <typename T>
-__device__ __forceinline__ bool evolve_one(int proc, const T *s_qs, const T *s_bw, const TablesView<T> &tv,
-                                           T px, T py, T pz, T ex, T ey, T ez, T bx, T by, T bz, T dt, T cut,
-                                           T &tau, T &tc, T &chi_out, int &bad)
+struct RateSmem;
+template <>
+struct RateSmem<float> {
+    float qs[QED_MAX_TABLE_N], bw[QED_MAX_TABLE_N];
+};
+template <>
+struct RateSmem<double> {
+    long long qs[QED_MAX_TABLE_N], bw[QED_MAX_TABLE_N];
+    long long ln[256], ex[256];
+    int r[256];
+    int off[2];  // per process: nonzero if a value or a step of its table does not fit the integers
+};
+
+__device__ __forceinline__ void stage_rates(RateSmem<float> &s, const TablesView<float> &tab, int threads)
 {
-    T chi, rate;
+    for (int i = threadIdx.x; i < tab.qs_G.n; i += threads) s.qs[i] = tab.qs_G.ln_f[i];
+    for (int i = threadIdx.x; i < tab.bw_T.n; i += threads) s.bw[i] = tab.bw_T.ln_f[i];
+}
+
+// x in units of 2^-53 (to nearest) from its bits, |x| < 700
+__device__ __forceinline__ long long fix_from_ln(double x)
+{
+    const int hi = __double2hiint(x), sh = 1032 - ((hi >> 20) & 0x7ff);  // the 53 bits << 11 have the unit 2^-63 at 2^9
+    uint64_t m = ((uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(x)) << 11;
+    m = sh > 60 ? 0 : ((m >> sh) + 1) >> 1;
+    return hi < 0 ? -(long long)m : (long long)m;
+}
+
+// the table on integers; nonzero where it does not fit: |ln f| < 700, steps below 500
+__device__ __forceinline__ int stage_fix(long long *out, const Table1D<double> &t, int threads)
+{
+    const auto below = [](double x, int hi_limit) { return (__double2hiint(x) & 0x7fffffff) < hi_limit; };
+    int off = 0;
+    for (int i = threadIdx.x; i < t.n; i += threads) {
+        const double x = t.ln_f[i];
+        off |= below(x, 0x4085e000) ? 0 : 1;                                  // 700
+        if (i + 1 < t.n) off |= below(t.ln_f[i + 1] - x, 0x407f4000) ? 0 : 1;  // 500
+        out[i] = fix_from_ln(x);
+    }
+    return off;
+}
+
+// every thread of the CTA; the caller's next barrier publishes it
+__device__ __forceinline__ void stage_rates(RateSmem<double> &s, const TablesView<double> &tab, int threads)
+{
+    if (threadIdx.x < 2) s.off[threadIdx.x] = 0;
+    __syncthreads();
+    if (stage_fix(s.qs, tab.qs_G, threads)) s.off[0] = 1;
+    if (stage_fix(s.bw, tab.bw_T, threads)) s.off[1] = 1;
+    for (int i = threadIdx.x; i < 256; i += threads) s.ln[i] = kFixLog[i], s.ex[i] = kFixExp[i], s.r[i] = kFixLogR[i];
+}
+
+// one particle: chi, rate, optical-depth decrement; returns fire
+__device__ __forceinline__ bool evolve_one(int proc, const RateSmem<float> &rs, const TablesView<float> &tv, float px,
+                                           float py, float pz, float ex, float ey, float ez, float bx, float by,
+                                           float bz, float dt, float cut, float &tau, float &tc, float &chi_out,
+                                           int &bad)
+{
+    float chi, rate;
     if (proc == QED_PROC_QS) {
-        T gamma, inv;
+        float gamma, inv;
         chi = chi_lepton(px, py, pz, ex, ey, ez, bx, by, bz, gamma, inv);
-        rate = qs_rate(s_qs, tv.qs_G, chi, gamma, inv);
+        rate = qs_rate(rs.qs, tv.qs_G, chi, gamma, inv);
     } else {
-        T pm, inv;
+        float pm, inv;
         chi = chi_photon(px, py, pz, ex, ey, ez, bx, by, bz, pm, inv);
-        rate = bw_rate(s_bw, tv.bw_T, chi, pm, inv);
+        rate = bw_rate(rs.bw, tv.bw_T, chi, pm, inv);
     }
     const bool ok = isfinite(chi) && !isnan(tau) && isfinite(rate);
     bad += ok ? 0 : 1;
-    if (!ok || chi < cut) rate = T(0);  // below the process's chi threshold: no evolution
+    if (!ok || chi < cut) rate = 0.0f;  // below the process's chi threshold: no evolution
     chi_out = chi;
-    if constexpr (sizeof(T) == 4) {
-        // Kahan-compensated decrement; tau - tc is the optical depth
-        if (!isfinite(tau)) return false;  // removed particle (tau = +inf)
-        const T y = d_fma(-rate, dt, -tc);
-        const T t = tau + y;
-        tc = (t - tau) - y;
-        tau = t;
-        return ok && (t < T(0) || (t == T(0) && tc > T(0)));
+    // Kahan-compensated decrement; tau - tc is the optical depth
+    if (!isfinite(tau)) return false;  // removed particle (tau = +inf)
+    const float y = d_fma(-rate, dt, -tc);
+    const float t = tau + y;
+    tc = (t - tau) - y;
+    tau = t;
+    return ok && (t < 0.0f || (t == 0.0f && tc > 0.0f));
+}
+
+struct EvolvedFp64 {
+    double tau, chi;
+    int fire, bad;
+};
+
+// The same in FP64 throughout, out of line: the particles that the integers of
+// fixed64.cuh leave to it (blocks of subnormal or huge values, infinities, NaN,
+// a force far below its terms, chi at a table's end or at the cut-off).
+static __device__ __noinline__ EvolvedFp64 evolve_one_fp64(int proc, const Table1D<double> &tb, double px, double py,
+                                                           double pz, double ex, double ey, double ez, double bx,
+                                                           double by, double bz, double dt, double cut, double tau)
+{
+    double chi, rate, en, inv;
+    if (proc == QED_PROC_QS) {
+        chi = chi_lepton(px, py, pz, ex, ey, ez, bx, by, bz, en, inv);
+        rate = qs_rate(tb.ln_f, tb, chi, en, inv);
     } else {
-        tau = tau - rate * dt;
-        return ok && tau < T(0);
+        chi = chi_photon(px, py, pz, ex, ey, ez, bx, by, bz, en, inv);
+        rate = bw_rate(tb.ln_f, tb, chi, en, inv);
     }
+    const bool ok = isfinite(chi) && !isnan(tau) && isfinite(rate);
+    if (!ok || chi < cut) rate = 0.0;  // below the process's chi threshold: no evolution
+    tau = tau - rate * dt;
+    return EvolvedFp64{tau, chi, ok && tau < 0.0, ok ? 0 : 1};
+}
+
+__device__ __forceinline__ bool evolve_one(int proc, const RateSmem<double> &rs, const TablesView<double> &tv,
+                                           double px, double py, double pz, double ex, double ey, double ez, double bx,
+                                           double by, double bz, double dt, double cut, double &tau, double &,
+                                           double &chi_out, int &bad)
+{
+    const bool qs = proc == QED_PROC_QS;
+    const Table1D<double> &tb = qs ? tv.qs_G : tv.bw_T;
+    FixOut o;
+    bool fast = fix_particle(qs, px, py, pz, ex, ey, ez, bx, by, bz, tb.fix, qs ? rs.qs : rs.bw, rs.r, rs.ln, rs.ex, o);
+    // (tau = 0 or NaN: a rate that the integers drop as below 1e-290 could decide)
+    const long long tb_bits = __double_as_longlong(tau) & 0x7fffffffffffffffll;
+    fast = fast && rs.off[qs ? 0 : 1] == 0 && tb_bits != 0 && tb_bits <= 0x7ff0000000000000ll && !(cut > 0.0);
+    if (!fast) {
+        const auto mag = [](double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; };
+        const long long inf = 0x7ff0000000000000ll;
+        if (!(mag(ex) | mag(ey) | mag(ez) | mag(bx) | mag(by) | mag(bz)) && mag(px) < inf && mag(py) < inf &&
+            mag(pz) < inf && tb_bits <= inf) {  // no field: chi = 0, nothing evolves
+            chi_out = 0.0;
+            return __double_as_longlong(tau) < 0 && tb_bits != 0;
+        }
+        const EvolvedFp64 r = evolve_one_fp64(proc, tb, px, py, pz, ex, ey, ez, bx, by, bz, dt, cut, tau);
+        tau = r.tau, chi_out = r.chi;
+        bad += r.bad;
+        return r.fire != 0;
+    }
+    // the only FP64 instruction: tau - (rate / coef) (coef dt)
+    tau = fma(-o.rate, (qs ? 2.0 / 3.0 * kAlpha : kAlpha) * dt, tau);
+    const bool fire = __double_as_longlong(tau) < 0 && __double_as_longlong(tau) != (long long)0x8000000000000000ull;
+    if (fire) chi_out = sqrt(scalbn((double)o.s, o.s_e));
+    return fire;
 }
 
 // warp-ballot compaction of the firing particles among [i0, i0 + VEC) (cnt of
@@ -134,7 +243,7 @@ __device__ __forceinline__ void evolve_regs(const EvolveSeg<T> &sg, int64_t n, i
                                             const T (&px)[VEC], const T (&py)[VEC], const T (&pz)[VEC],
                                             const T (&ex)[VEC], const T (&ey)[VEC], const T (&ez)[VEC],
                                             const T (&bx)[VEC], const T (&by)[VEC], const T (&bz)[VEC], T (&tau)[VEC],
-                                            T (&tc)[VEC], const T *s_qs, const T *s_bw, const TablesView<T> &tab,
+                                            T (&tc)[VEC], const RateSmem<T> &rs, const TablesView<T> &tab,
                                             T dt, T cut, long long *stats, int dry, int &bad)
 {
     bool fire[VEC];
@@ -143,7 +252,7 @@ __device__ __forceinline__ void evolve_regs(const EvolveSeg<T> &sg, int64_t n, i
 #pragma unroll
     for (int j = 0; j < VEC; ++j) {
         T c = sizeof(T) == 4 ? tc[j] : T(0);
-        fire[j] = evolve_one<T>(sg.proc, s_qs, s_bw, tab, px[j], py[j], pz[j], ex[j], ey[j], ez[j], bx[j], by[j],
+        fire[j] = evolve_one(sg.proc, rs, tab, px[j], py[j], pz[j], ex[j], ey[j], ez[j], bx[j], by[j],
                                 bz[j], dt, cut, tau[j], c, chi[j], bad);
         tc[j] = c;
         fire[j] = fire[j] && (i0 + j < n);

@@ -40,18 +40,16 @@ __device__ __forceinline__ void store_live(T *p, int64_t i0, int64_t n, bool ful
 template <typename T, int VEC, int THREADS>
 __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     push_evolve_kernel(const EvolveSeg<T> *__restrict__ segs, const PushSeg<T> *__restrict__ psegs, int n_seg,
-                       TablesView<T> tab, WaveParams w, double t0, double dt_d, const int64_t *d_step, int64_t step,
+                       const __grid_constant__ TablesView<T> tab, WaveParams w, double t0, double dt_d, const int64_t *d_step, int64_t step,
                        T cut_qs, T cut_bw, long long *stats, int store_fields)
 {
-    __shared__ T s_qs[QED_MAX_TABLE_N];
-    __shared__ T s_bw[QED_MAX_TABLE_N];
+    __shared__ RateSmem<T> rs;
     __shared__ long long s_warp[THREADS / 32];
     extern __shared__ long long s_dyn[];  // [n_seg] inclusive tile prefix, [n_seg] counts
     long long *s_end = s_dyn, *s_n = s_dyn + n_seg;
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
-    for (int i = threadIdx.x; i < tab.qs_G.n; i += THREADS) s_qs[i] = tab.qs_G.ln_f[i];
-    for (int i = threadIdx.x; i < tab.bw_T.n; i += THREADS) s_bw[i] = tab.bw_T.ln_f[i];
+    stage_rates(rs, tab, THREADS);
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);
     const WaveT<T> wt = wave_at<T>(w, t0 + (double)(d_step ? *d_step : step) * dt_d);
     const T dt = (T)dt_d;
@@ -97,7 +95,7 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
                 pg.bx[i0 + j] = bx, pg.by[i0 + j] = by, pg.bz[i0 + j] = bz;
             }
             T c = tc[j];
-            fire[j] = evolve_one<T>(sg.proc, s_qs, s_bw, tab, px[j], py[j], pz[j], ex, ey, ez, bx, by, bz, dt, cut,
+            fire[j] = evolve_one(sg.proc, rs, tab, px[j], py[j], pz[j], ex, ey, ez, bx, by, bz, dt, cut,
                                     tau[j], c, chi[j], bad);
             tc[j] = c;
             fire[j] = fire[j] && (i0 + j < n);

@@ -90,11 +90,37 @@ static void free_tables(qed_tables *t)
 static size_t n_qs2(const qed_table_params &p) { return (size_t)p.qs.n_chi * p.qs.n_xi; }
 static size_t n_bw2(const qed_table_params &p) { return (size_t)p.bw.n_chi * p.bw.n_xi; }
 
+// a 1-D table's axis on integers (fixed64.cuh), in extended precision; a table
+// whose logarithms the integers cannot hold (ok = 0) takes the FP64 path
+static FixAxis fix_axis(const qed_table_axis &a)
+{
+    FixAxis f;
+    memset(&f, 0, sizeof(f));
+    const long double one = 9007199254740992.0L;  // 2^53
+    const long double l0 = std::log((long double)a.chi_min), l1 = std::log((long double)a.chi_max);
+    f.n = a.n_chi;
+    if (!(l0 > -700.0L) || !(l1 < 700.0L)) return f;
+    f.ln_min = (long long)rintl(l0 * one);
+    f.ln_max = (long long)rintl(l1 * one);
+    if (f.ln_max - f.ln_min < 4096) return f;
+    const uint64_t d = (uint64_t)(f.ln_max - f.ln_min);
+    int bits = 0;
+    while ((a.n_chi - 1) >> bits) ++bits;
+    while ((d << (f.shift + 1)) < (1ull << 62)) ++f.shift;
+    f.frac = 60 - bits;
+    f.scale = fix_limbs((int64_t)rintl((long double)(a.n_chi - 1) / ((long double)d * std::ldexp(1.0L, f.shift)) *
+                                       std::ldexp(1.0L, f.frac + 62)));
+    f.ok = 1;
+    return f;
+}
+
 qed_status alloc_tables(const qed_table_params *p, qed_tables **out)
 {
     qed_tables *t = new qed_tables();
     memset(t, 0, sizeof(*t));
     t->params = *p;
+    t->qs_fix = fix_axis(p->qs);
+    t->bw_fix = fix_axis(p->bw);
     cudaGetDevice(&t->device);
     const size_t sz[6] = {(size_t)p->qs.n_chi, n_qs2(*p), (size_t)p->bw.n_chi, n_bw2(*p), n_qs2(*p), n_bw2(*p)};
     double **dp[6] = {&t->d_qs_lnG, &t->d_qs_lnP, &t->d_bw_lnT, &t->d_bw_P, &t->d_qs_dlnP, &t->d_bw_dP};
@@ -147,7 +173,7 @@ qed_status finish_tables(qed_tables *t, cudaStream_t st)
 }
 
 template <typename T>
-static Table1D<T> view1(const T *f, const qed_table_axis &a)
+static Table1D<T> view1(const T *f, const qed_table_axis &a, const FixAxis &fix)
 {
     Table1D<T> v;
     v.ln_f = f;
@@ -157,6 +183,7 @@ static Table1D<T> view1(const T *f, const qed_table_axis &a)
     v.chi_min = (T)a.chi_min;
     v.chi_max = (T)a.chi_max;
     v.n = a.n_chi;
+    v.fix = fix;
     return v;
 }
 
@@ -188,8 +215,8 @@ template <>
 TablesView<double> make_view<double>(const qed_tables *t)
 {
     TablesView<double> v;
-    v.qs_G = view1<double>(t->d_qs_lnG, t->params.qs);
-    v.bw_T = view1<double>(t->d_bw_lnT, t->params.bw);
+    v.qs_G = view1<double>(t->d_qs_lnG, t->params.qs, t->qs_fix);
+    v.bw_T = view1<double>(t->d_bw_lnT, t->params.bw, t->bw_fix);
     v.qs_P = view2<double>(t->d_qs_lnP, t->d_qs_dlnP, t->d_qs_guide, t->params.qs, true);
     v.bw_P = view2<double>(t->d_bw_P, t->d_bw_dP, t->d_bw_guide, t->params.bw, false);
     return v;
@@ -199,8 +226,8 @@ template <>
 TablesView<float> make_view<float>(const qed_tables *t)
 {
     TablesView<float> v;
-    v.qs_G = view1<float>(t->f_qs_lnG, t->params.qs);
-    v.bw_T = view1<float>(t->f_bw_lnT, t->params.bw);
+    v.qs_G = view1<float>(t->f_qs_lnG, t->params.qs, t->qs_fix);
+    v.bw_T = view1<float>(t->f_bw_lnT, t->params.bw, t->bw_fix);
     v.qs_P = view2<float>(t->f_qs_lnP, t->f_qs_dlnP, t->f_qs_guide, t->params.qs, true);
     v.bw_P = view2<float>(t->f_bw_P, t->f_bw_dP, t->f_bw_guide, t->params.bw, false);
     return v;

@@ -223,3 +223,38 @@ def test_bw_asymptotes_against_oracle(api):
         assert np.all(np.abs(rate - 0.3) < 1e-3)
         assert np.allclose(tau_eff(got, prec == api.QED_F32), tau_new, rtol=tol, atol=0)
         assert len(fidx) == 0 and st["nonfinite"] == 0
+
+
+@pytest.mark.parametrize("proc", [0, 1])
+def test_evolve_fp64_particles_of_both_paths(api, tabs, proc):
+    """FP64 particles that the integer evaluation takes side by side with those it leaves to the FP64 path (no field, at
+    rest, a force far below its terms, scales far apart, magnitudes beyond 2^+-400, chi at the table's ends): one step
+    against the oracle."""
+    ot, t = tabs
+    n = 4096 + 3
+    host = _workload("bench", n, 77)
+    p, f = ("px", "py", "pz"), ("ex", "ey", "ez", "bx", "by", "bz")
+    i = np.arange(n)
+    kind = np.where(i < 3000, i % 16, 99)  # in one warp, then without any
+    r = np.random.default_rng(3)
+    for k in p:
+        host[k] = np.where(kind == 1, 1e-3 * host[k], host[k])
+        host[k] = np.where(kind == 2, host[k] * 10.0 ** r.uniform(-8, 0, n), host[k])
+        host[k] = np.where(kind == 3, 0.0 if proc == 0 else host[k], host[k])
+        host[k] = np.where(kind == 4, host[k] * 1e-130, host[k])
+    for a, b in zip(("bx", "by", "bz"), p):  # B along p within 1e-3
+        host[a] = np.where(kind == 5, 1e-5 * host[b] + 1e-3 * host[a], host[a])
+    for k in f:
+        host[k] = np.where(kind == 6, 0.0, host[k])
+        host[k] = np.where(kind == 7, host[k] * 10.0 ** r.uniform(-2, 6, n), host[k])
+        host[k] = np.where(kind == 8, host[k] * 1e130 * (1.0 if proc else 0.0), host[k])
+        host[k] = np.where((kind == 5) & np.isin(k, ("ex", "ey", "ez")), 0.0, host[k])
+    # a photon (lepton: to rounding) along x in a field across it with chi on a table end
+    for k in p + f:
+        host[k] = np.where((kind == 9) | (kind == 10), 0.0, host[k])
+    host["px"] = np.where((kind == 9) | (kind == 10), 64.0, host["px"])
+    host["ey"] = np.where(kind == 9, 2e-2 / 64.0, np.where(kind == 10, 1e3 / 64.0, host["ey"]))
+    got, fidx, fchi, st = _run(api, t, proc, host, api.QED_F64, 10.0)
+    diff = compare_evolve("evolve", tau_eff(got, False), fidx, fchi, as_f64(host, np.float64), proc, ot, 10.0,
+                          TOL["f64"], True)
+    assert len(diff) == 0 and st["nonfinite"] == 0 and len(fidx) > 100

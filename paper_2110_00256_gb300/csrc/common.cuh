@@ -222,6 +222,7 @@ struct qed_tables {
     // guide tables of the 2-D tables' inverse-CDF search, one per precision
     int32_t *d_qs_guide, *d_bw_guide, *f_qs_guide, *f_bw_guide;
     qed::FixAxis qs_fix, bw_fix;  // the 1-D tables' axes on integers
+    void *block, *derived;        // the one allocation that holds them all; where those formed from the FP64 tables begin
 };
 
 namespace qed {

@@ -33,7 +33,7 @@
 namespace qed {
 
 qed_status check_params(const qed_table_params *p);
-qed_status alloc_tables(const qed_table_params *p, qed_tables **out);
+qed_status alloc_tables(const qed_table_params *p, qed_tables **out, size_t scratch = 0);
 qed_status finish_tables(qed_tables *t, cudaStream_t st);
 
 constexpr double kPi = 3.14159265358979323846;
@@ -93,19 +93,49 @@ __device__ double bw_integrand(double chi, double xi)
 constexpr int kPieceOct = -30, kPieceOcts = 40, kPieces = 4 * kPieceOcts, kPieceCoef = 14;
 constexpr int kPieceRow = 2 * kPieceCoef;  // both functions of a piece
 
-// one warp per piece of one process; blockIdx.y: QS (nu 5/3, 2/3) or BW (1/3, 2/3)
+// One warp per piece, both processes (they share K_{2/3}).  The trapezoid rule
+// takes the step of the piece's largest argument, so its nodes t_k, and all
+// factors but exp(-x (cosh t_k - 1)), are the same for the 14 arguments: the
+// lanes form them 32 at a time, then each of 14 lanes runs one argument's sum
+// (one exponential and three FMAs a step; with the factors formed by every lane
+// in every step, ~130 FP64 instructions, the launch took 362 us).
+constexpr int kPieceT = 160;  // trapezoid nodes: (ln(2 (40 + 5/3 t) / 2^-30) / (1/4) = 106 at the lower end
 __global__ void __launch_bounds__(32) bessel_pieces_kernel(double *out)
 {
+    __shared__ double s_c1[kPieceT], s_f[3][kPieceT];  // cosh t - 1; cosh(nu t)/cosh t for nu = 5/3, 1/3; cosh(2t/3)
     const int piece = blockIdx.x, lane = threadIdx.x;
     const double scale = ldexp(1.0, kPieceOct + piece / 4);
-    double f[2] = {0.0, 0.0};
+    const double hi = scale * (1.0 + (2 * (piece % 4) + 2) / 8.0), lo = scale * (1.0 + (2 * (piece % 4)) / 8.0);
+    const double h = fmin(0.25, 0.6 / sqrt(hi));
+    int n = 0;  // steps: until lo (cosh t - 1) leaves every integrand below e^-40
+    for (int base = 0; base < kPieceT; base += 32) {
+        const int k = base + lane + 1;
+        const double t = k * h, s = sinh(0.5 * t), c1 = 2.0 * s * s;
+        const double e1 = exp(t / 3.0), i1 = 1.0 / e1, e2 = e1 * e1, i2 = i1 * i1;
+        const double ch = 1.0 / (e2 * e1 + i2 * i1);  // 1/(2 cosh t)
+        s_c1[k - 1] = c1;
+        s_f[0][k - 1] = (e2 * e2 * e1 + i2 * i2 * i1) * ch;
+        s_f[1][k - 1] = (e1 + i1) * ch;
+        s_f[2][k - 1] = 0.5 * (e2 + i2);
+        const bool live = !(lo * c1 > 40.0 && lo * c1 - 5.0 / 3.0 * t > 40.0);
+        n += __popc(__ballot_sync(0xffffffffu, live));
+        if (!__any_sync(0xffffffffu, live)) break;
+    }
+    __syncwarp();
+    double f[3] = {0.0, 0.0, 0.0};
     if (lane < kPieceCoef) {
-        const double x = cospi((lane + 0.5) / kPieceCoef);  // Chebyshev node in [-1, 1]
-        bessel_scaled(scale * (1.0 + (2 * (piece % 4) + 1 + x) / 8.0), (blockIdx.y ? 1.0 : 5.0) / 3.0, 2.0 / 3.0, f[0],
-                      f[1]);
+        const double x = scale * (1.0 + (2 * (piece % 4) + 1 + cospi((lane + 0.5) / kPieceCoef)) / 8.0);  // Chebyshev node
+        double sum[3] = {0.5, 0.5, 0.5};
+        for (int k = 0; k < n; ++k) {
+            const double e = exp_tang(fmax(-x * s_c1[k], -700.0));
+#pragma unroll
+            for (int i = 0; i < 3; ++i) sum[i] = fma(e, s_f[i][k], sum[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; ++i) f[i] = h * sum[i];
     }
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k < 3; ++k) {
         // lane i: Chebyshev coefficient i, then the coefficient of x^i by the
         // recurrence T_k = 2 x T_{k-1} - T_{k-2}
         double c = 0.0;
@@ -116,13 +146,18 @@ __global__ void __launch_bounds__(32) bessel_pieces_kernel(double *out)
         c *= (lane ? 2.0 : 1.0) / kPieceCoef;
         double t0 = lane == 0 ? 1.0 : 0.0, t1 = lane == 1 ? 1.0 : 0.0;  // T_0, T_1
         double p = __shfl_sync(0xffffffffu, c, 0) * t0 + __shfl_sync(0xffffffffu, c, 1) * t1;
-        for (int n = 2; n < kPieceCoef; ++n) {
+        for (int i = 2; i < kPieceCoef; ++i) {
             const double up = __shfl_up_sync(0xffffffffu, t1, 1);
             const double t2 = 2.0 * (lane ? up : 0.0) - t0;
-            p += __shfl_sync(0xffffffffu, c, n) * t2;
+            p += __shfl_sync(0xffffffffu, c, i) * t2;
             t0 = t1, t1 = t2;
         }
-        if (lane < kPieceCoef) out[((size_t)blockIdx.y * kPieces + piece) * kPieceRow + k * kPieceCoef + lane] = p;
+        if (lane < kPieceCoef) {
+            double *qs = out + (size_t)piece * kPieceRow + lane, *bw = qs + (size_t)kPieces * kPieceRow;
+            if (k == 0) qs[0] = p;
+            if (k == 1) bw[0] = p;
+            if (k == 2) qs[kPieceCoef] = bw[kPieceCoef] = p;
+        }
     }
 }
 
@@ -189,7 +224,7 @@ struct GenArgs {
     double qs_l0, qs_l1, qs_xi_min, bw_l0, bw_l1;
     int qs_n_chi, qs_n_xi, bw_n_chi, bw_n_xi;
     double *pieces;  // [2][kPieces][kPieceRow]: the Bessel functions
-    double *nodes;   // [2][3][kGl][QED_MAX_TABLE_N]: q, w va, w vb at the Gauss-Legendre nodes of every interval
+    double *nodes;   // [2][3][kGl][n_xi]: q, w va, w vb at the Gauss-Legendre nodes of every interval
 };
 
 // interval j of a row: QS j = 0 is [xi_min e^-100, xi_min] in ln xi, j >= 1 is
@@ -205,48 +240,64 @@ __device__ __forceinline__ void row_interval(bool qs, double ln_xi_min, int M, i
     }
 }
 
-// Gauss-Legendre (16 points, weights and nodes of the reference interval by
-// value): where the integrand's singularity (QS: ln xi = 0, where 1 - xi
+// Gauss-Legendre (weights and nodes of the reference interval by value) with 16
+// points where the integrand's singularity (QS: ln xi = 0, where 1 - xi
 // vanishes; BW: xi = 0) lies at least twice the interval's half-width from its
 // centre (the error falls like (2 + sqrt 3)^-32 = 5e-19), the interval is not
 // wide against the integrand's own scale in ln xi, and e^-Y falls by at most
-// e^-12 across it (the error of e^-6t on [-1, 1] is 2e-20).
-constexpr int kGl = 16;
+// e^-12 across it (the error of e^-6t on [-1, 1] is 2e-20); with 8 points where
+// the singularity lies 8 half-widths away ((8 + sqrt 63)^-16 = 6e-20) and e^-Y
+// falls by at most e^-2 (2e-18).  QS interval 0, below xi_min, is integrated
+// in w = xi^(1/3), S growing like w there: with 16 points if Y(xi_min) <= 1/2 and
+// xi_min <= 1/5 (xi = 1 then lies 2.4 half-widths from the centre).
+constexpr int kGl = 16, kGlFew = 8;
 struct GaussLegendre16 {
-    double x[kGl], w[kGl];
+    double x[kGl], w[kGl], xf[kGlFew], wf[kGlFew];
 };
 
-__device__ __forceinline__ bool gl_smooth(bool qs, double lo, double hi)
+// points of the rule that the interval's place allows: 16, 8 or 0 (tanh-sinh)
+__device__ __forceinline__ int gl_points(bool qs, int j, double lo, double hi)
 {
-    const double c = 0.5 * (lo + hi), h = 0.5 * (hi - lo);
-    return qs ? (-c >= 2.0 * h && h <= 0.5) : (c >= 2.0 * h);
+    if (j == 0) return qs && hi <= -1.6095 ? kGl : 0;  // ln(1/5)
+    const double c = qs ? -0.5 * (lo + hi) : 0.5 * (lo + hi), h = 0.5 * (hi - lo);
+    if (c < 2.0 * h || (qs && h > 0.5)) return 0;
+    return c >= 8.0 * h && !(qs && h > 0.1) ? kGlFew : kGl;
 }
 
-// the nodes that every row of a process shares: thread = interval, blockIdx.y = process
+// the nodes that every row of a process shares: thread = (interval, node), blockIdx.y = process
 __global__ void __launch_bounds__(128) row_nodes_kernel(const __grid_constant__ GenArgs a,
                                                          const __grid_constant__ GaussLegendre16 g)
 {
     const bool qs = blockIdx.y == 0;
     const int M = qs ? a.qs_n_xi : a.bw_n_xi;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < 1 || j >= M) return;
+    const int j = blockIdx.x * 8 + threadIdx.x / kGl, k = threadIdx.x % kGl;
+    if (j >= M) return;
     double lo, hi;
     row_interval(qs, log(a.qs_xi_min), M, j, lo, hi);
-    double *out = a.nodes + (size_t)blockIdx.y * 3 * kGl * QED_MAX_TABLE_N;
-    const double c = 0.5 * (lo + hi), h = 0.5 * (hi - lo);
-    for (int k = 0; k < kGl; ++k) {
-        double q, va, vb;
-        node_terms(qs, fma(h, g.x[k], c), q, va, vb);
-        out[(size_t)k * QED_MAX_TABLE_N + j] = q;
-        out[(size_t)(kGl + k) * QED_MAX_TABLE_N + j] = g.w[k] * h * va;
-        out[(size_t)(2 * kGl + k) * QED_MAX_TABLE_N + j] = g.w[k] * h * vb;
+    const int points = gl_points(qs, j, lo, hi);
+    if (k >= points) return;
+    double *out = a.nodes + (qs ? 0 : (size_t)3 * kGl * a.qs_n_xi);
+    double x, w;
+    if (j == 0) {  // w^3 = xi from 0 to xi_min: S du = (3 S / w) dw
+        const double top = cbrt(a.qs_xi_min), v = 0.5 * top * (1.0 + g.x[k]);
+        x = 3.0 * log(v);
+        w = 0.5 * top * g.w[k] * 3.0 / v;
+    } else {
+        const double c = 0.5 * (lo + hi), h = 0.5 * (hi - lo);
+        x = fma(h, points == kGl ? g.x[k] : g.xf[k], c);
+        w = h * (points == kGl ? g.w[k] : g.wf[k]);
     }
+    double q, va, vb;
+    node_terms(qs, x, q, va, vb);
+    out[(size_t)k * M + j] = q;
+    out[(size_t)(kGl + k) * M + j] = w * va;
+    out[(size_t)(2 * kGl + k) * M + j] = w * vb;
 }
 
 // One CTA per row.  Bound by the FP64 pipe: ~60 FP64 instructions per
-// Gauss-Legendre node, 256 x 16 nodes in a row of the 256 x 256 tables, and the
-// tanh-sinh intervals (two at the ends, and the few per row across which e^-Y
-// falls steeply), whose nodes and weights on [-1, 1] are shared too.
+// Gauss-Legendre node, ~256 x 8 nodes in a row of the 256 x 256 tables, and the
+// tanh-sinh intervals (one at the end, and ~4 per row across which e^-Y falls
+// steeply), whose nodes and weights on [-1, 1] are shared too.
 __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__ GenArgs a)
 {
     __shared__ double acc[QED_MAX_TABLE_N], tail[QED_MAX_TABLE_N];
@@ -276,7 +327,7 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__
     if (threadIdx.x == 0) s_n_hard = 0;
     __syncthreads();
 
-    const double *nodes = a.nodes + (qs ? 0 : (size_t)3 * kGl * QED_MAX_TABLE_N);
+    const double *nodes = a.nodes + (qs ? 0 : (size_t)3 * kGl * a.qs_n_xi);
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
         double lo, hi;
         row_interval(qs, lxm, M, j, lo, hi);
@@ -284,22 +335,22 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__
             acc[0] = 0.0;
             continue;
         }
-        bool smooth = j > 0 && gl_smooth(qs, lo, hi);
-        if (smooth) {
-            // the outermost nodes lie within 1 % of the ends: Y's fall between them
-            const double q0 = nodes[j], q1 = nodes[(size_t)(kGl - 1) * QED_MAX_TABLE_N + j];
-            if (fmin(q0, q1) * inv_chi > 800.0) {  // e^-Y is zero on all of it
+        int points = gl_points(qs, j, lo, hi);
+        if (points) {
+            // the outermost nodes lie within 2 % of the ends: Y's fall between them
+            const double q0 = nodes[j], q1 = nodes[(size_t)(points - 1) * M + j];
+            if (fmin(q0, q1) * inv_chi > 800.0 && j > 0) {  // e^-Y is zero on all of it
                 acc[j] = 0.0;
                 continue;
             }
-            smooth = fabs(q1 - q0) * inv_chi <= 11.5;
+            const double fall = fabs(q1 - q0) * inv_chi;
+            if (fall > (j == 0 ? 0.5 : (points == kGl ? 11.5 : 1.9))) points = 0;
         }
-        if (smooth) {
+        if (points) {
             double part = 0.0;
-            for (int k = 0; k < kGl; ++k) {
-                const double *p = nodes + (size_t)k * QED_MAX_TABLE_N + j;
-                part += row_integrand(s_c, qs, inv_chi, p[0], p[(size_t)kGl * QED_MAX_TABLE_N],
-                                      p[(size_t)2 * kGl * QED_MAX_TABLE_N]);
+            for (int k = 0; k < points; ++k) {
+                const double *p = nodes + (size_t)k * M + j;
+                part += row_integrand(s_c, qs, inv_chi, p[0], p[(size_t)kGl * M], p[(size_t)2 * kGl * M]);
             }
             acc[j] = part;
         } else {
@@ -574,10 +625,9 @@ __global__ void __launch_bounds__(128) exact_draw_kernel(int qs, const double *_
 }
 
 // Gauss-Legendre nodes and weights, n points (Newton's method on the three-term recurrence)
-template <typename G, int n>
-static G gauss_legendre()
+template <int n>
+static void gauss_legendre(double (&gx)[n], double (&gw)[n])
 {
-    G g;
     for (int i = 0; i < n; ++i) {
         double x = std::cos(kPi * (i + 0.75) / (n + 0.5));
         double dp = 1.0;
@@ -592,10 +642,9 @@ static G gauss_legendre()
             x -= dx;
             if (std::fabs(dx) < 1e-16) break;
         }
-        g.x[i] = x;
-        g.w[i] = 2.0 / ((1.0 - x * x) * dp * dp);
+        gx[i] = x;
+        gw[i] = 2.0 / ((1.0 - x * x) * dp * dp);
     }
-    return g;
 }
 
 }  // namespace qed
@@ -615,7 +664,11 @@ extern "C" qed_status qed_exact_sample(qed_process proc, const double *d_chi, in
         QED_FAIL(QED_ERR_INVALID_ARG, "d_work holds %lld doubles, %lld needed", (long long)work_capacity,
                  (long long)QED_EXACT_WORK(m));
     static_assert(QED_EXACT_WORK(1) == kExactRowStride, "work layout");
-    static const GaussLegendre8 gl = gauss_legendre<GaussLegendre8, 8>();
+    static const GaussLegendre8 gl = [] {
+        GaussLegendre8 g;
+        gauss_legendre<8>(g.x, g.w);
+        return g;
+    }();
     cudaStream_t st = as_stream(stream);
     const int qs = proc == QED_PROC_QS;
     exact_rows_kernel<<<(unsigned)m, 256, 0, st>>>(qs, d_chi, d_work, gl);
@@ -638,7 +691,9 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
     qed_status s = check_params(params);
     if (s) return s;
     qed_tables *t = nullptr;
-    if ((s = alloc_tables(params, &t))) return s;
+    const size_t scratch =
+        ((size_t)2 * kPieces * kPieceRow + (size_t)3 * kGl * (params->qs.n_xi + params->bw.n_xi)) * sizeof(double);
+    if ((s = alloc_tables(params, &t, scratch))) return s;
     cudaStream_t st = as_stream(stream);
     GenArgs a;
     a.qs_lnG = t->d_qs_lnG, a.qs_lnP = t->d_qs_lnP, a.bw_lnT = t->d_bw_lnT, a.bw_P = t->d_bw_P;
@@ -647,25 +702,25 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
     a.bw_l0 = std::log(params->bw.chi_min), a.bw_l1 = std::log(params->bw.chi_max);
     a.qs_n_chi = params->qs.n_chi, a.qs_n_xi = params->qs.n_xi;
     a.bw_n_chi = params->bw.n_chi, a.bw_n_xi = params->bw.n_xi;
-    // scratch of this call: the pieces and the shared nodes
-    constexpr size_t n_pieces = (size_t)2 * kPieces * kPieceRow, n_nodes = (size_t)2 * 3 * kGl * QED_MAX_TABLE_N;
-    double *work = nullptr;
-    cudaError_t e = cudaMalloc((void **)&work, (n_pieces + n_nodes) * sizeof(double));
+    // scratch (the pieces, the shared nodes) in the room of the derived tables, which finish_tables fills afterwards
+    a.pieces = (double *)t->derived;
+    a.nodes = a.pieces + (size_t)2 * kPieces * kPieceRow;
+    static const GaussLegendre16 gl = [] {
+        GaussLegendre16 g;
+        gauss_legendre<kGl>(g.x, g.w);
+        gauss_legendre<kGlFew>(g.xf, g.wf);
+        return g;
+    }();
+    const int m = params->qs.n_xi > params->bw.n_xi ? params->qs.n_xi : params->bw.n_xi;
+    constexpr int dyn = kPieces * kPieceRow * (int)sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(table_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) {
-        a.pieces = work, a.nodes = work + n_pieces;
-        static const GaussLegendre16 gl = gauss_legendre<GaussLegendre16, kGl>();
-        const int m = params->qs.n_xi > params->bw.n_xi ? params->qs.n_xi : params->bw.n_xi;
-        bessel_pieces_kernel<<<dim3(kPieces, 2), 32, 0, st>>>(work);
-        row_nodes_kernel<<<dim3((m + 127) / 128, 2), 128, 0, st>>>(a, gl);
-        constexpr int dyn = kPieces * kPieceRow * (int)sizeof(double);
-        e = cudaFuncSetAttribute(table_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
-        if (e == cudaSuccess) {
-            table_rows_kernel<<<params->qs.n_chi + params->bw.n_chi, 256, dyn, st>>>(a);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        cudaFree(work);
+        bessel_pieces_kernel<<<kPieces, 32, 0, st>>>(a.pieces);
+        row_nodes_kernel<<<dim3((m + 7) / 8, 2), 8 * kGl, 0, st>>>(a, gl);
+        table_rows_kernel<<<params->qs.n_chi + params->bw.n_chi, 256, dyn, st>>>(a);
+        e = cudaGetLastError();
     }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         qed_tables_destroy(t);
         QED_FAIL(QED_ERR_CUDA, "table generation failed: %s", cudaGetErrorString(e));

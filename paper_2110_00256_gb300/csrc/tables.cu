@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -21,6 +22,8 @@ static qed_status check_axis(const qed_table_axis &a, const char *name, bool qs)
         QED_FAIL(QED_ERR_INVALID_ARG, "%s: need 0 < xi_min < 1 (got %g)", name, a.xi_min);
     return QED_OK;
 }
+
+qed_status alloc_tables(const qed_table_params *p, qed_tables **out, size_t scratch = 0);
 
 qed_status check_params(const qed_table_params *p)
 {
@@ -79,11 +82,7 @@ __global__ void guide_kernel(const T *__restrict__ v, int n_xi, bool qs, int32_t
 static void free_tables(qed_tables *t)
 {
     if (!t) return;
-    void *ptrs[] = {t->d_qs_lnG, t->d_qs_lnP, t->d_bw_lnT, t->d_bw_P, t->f_qs_lnG, t->f_qs_lnP, t->f_bw_lnT, t->f_bw_P,
-                    t->d_qs_dlnP, t->d_bw_dP, t->f_qs_dlnP, t->f_bw_dP, t->d_qs_guide, t->d_bw_guide,
-                    t->f_qs_guide, t->f_bw_guide};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
+    if (t->block) cudaFree(t->block);
     delete t;
 }
 
@@ -114,7 +113,7 @@ static FixAxis fix_axis(const qed_table_axis &a)
     return f;
 }
 
-qed_status alloc_tables(const qed_table_params *p, qed_tables **out)
+qed_status alloc_tables(const qed_table_params *p, qed_tables **out, size_t scratch)
 {
     qed_tables *t = new qed_tables();
     memset(t, 0, sizeof(*t));
@@ -122,23 +121,30 @@ qed_status alloc_tables(const qed_table_params *p, qed_tables **out)
     t->qs_fix = fix_axis(p->qs);
     t->bw_fix = fix_axis(p->bw);
     cudaGetDevice(&t->device);
-    const size_t sz[6] = {(size_t)p->qs.n_chi, n_qs2(*p), (size_t)p->bw.n_chi, n_bw2(*p), n_qs2(*p), n_bw2(*p)};
-    double **dp[6] = {&t->d_qs_lnG, &t->d_qs_lnP, &t->d_bw_lnT, &t->d_bw_P, &t->d_qs_dlnP, &t->d_bw_dP};
-    float **fp[6] = {&t->f_qs_lnG, &t->f_qs_lnP, &t->f_bw_lnT, &t->f_bw_P, &t->f_qs_dlnP, &t->f_bw_dP};
-    for (int k = 0; k < 6; ++k) {
-        cudaError_t e1 = cudaMalloc((void **)dp[k], sz[k] * sizeof(double));
-        cudaError_t e2 = cudaMalloc((void **)fp[k], sz[k] * sizeof(float));
-        if (e1 != cudaSuccess || e2 != cudaSuccess) {
-            free_tables(t);
-            QED_FAIL(QED_ERR_CUDA, "table allocation failed: %s", cudaGetErrorString(e1 != cudaSuccess ? e1 : e2));
-        }
-    }
-    const size_t ng[2] = {(size_t)p->qs.n_chi * (kGuideBins + 1), (size_t)p->bw.n_chi * (kGuideBins + 1)};
-    int32_t **gp[4] = {&t->d_qs_guide, &t->f_qs_guide, &t->d_bw_guide, &t->f_bw_guide};
-    for (int k = 0; k < 4; ++k) {
-        cudaError_t e = cudaMalloc((void **)gp[k], ng[k / 2] * sizeof(int32_t));
+    // one allocation (an allocation and a release each for the 16 arrays were
+    // most of a table generation's host time): the four FP64 tables, then what is
+    // formed from them, with at least `scratch` bytes there
+    size_t size = 0;
+    const auto place = [&](auto *&ptr, size_t n) {  // offsets first (block == NULL), then addresses
+        ptr = (std::remove_reference_t<decltype(ptr)>)((uintptr_t)t->block + size);
+        size += (n * sizeof(*ptr) + 255) / 256 * 256;
+    };
+    const size_t n1[2] = {(size_t)p->qs.n_chi, (size_t)p->bw.n_chi}, n2[2] = {n_qs2(*p), n_bw2(*p)};
+    for (int pass = 0; pass < 2; ++pass) {
+        size = 0;
+        place(t->d_qs_lnG, n1[0]), place(t->d_qs_lnP, n2[0]), place(t->d_bw_lnT, n1[1]), place(t->d_bw_P, n2[1]);
+        t->derived = (void *)((uintptr_t)t->block + size);
+        const size_t least = size + scratch;
+        place(t->d_qs_dlnP, n2[0]), place(t->d_bw_dP, n2[1]);
+        place(t->f_qs_lnG, n1[0]), place(t->f_qs_lnP, n2[0]), place(t->f_bw_lnT, n1[1]), place(t->f_bw_P, n2[1]);
+        place(t->f_qs_dlnP, n2[0]), place(t->f_bw_dP, n2[1]);
+        place(t->d_qs_guide, n1[0] * (kGuideBins + 1)), place(t->f_qs_guide, n1[0] * (kGuideBins + 1));
+        place(t->d_bw_guide, n1[1] * (kGuideBins + 1)), place(t->f_bw_guide, n1[1] * (kGuideBins + 1));
+        if (size < least) size = least;
+        if (pass) break;
+        const cudaError_t e = cudaMalloc(&t->block, size);
         if (e != cudaSuccess) {
-            free_tables(t);
+            delete t;
             QED_FAIL(QED_ERR_CUDA, "table allocation failed: %s", cudaGetErrorString(e));
         }
     }

@@ -158,6 +158,44 @@ __device__ __forceinline__ void fix_sqrt(uint64_t g2, int64_t &sq, uint64_t &inv
     inv_e = s / 2 + 2 - 125;  // 1/(g 2^-(s/2+2)) = (y 2^-62 2^-63) 2^(s/2+2)
 }
 
+// the double nearest to v 2^e for |v| < 2^63 (normal results; 0 for v = 0)
+__device__ __forceinline__ double fix_to_double(int64_t v, int e)
+{
+    const uint64_t a = v < 0 ? 0 - (uint64_t)v : (uint64_t)v;
+    if (a == 0) return 0.0;
+    const int lz = __clzll((long long)a);
+    const uint64_t n = a << lz;
+    uint64_t t = n >> 11;
+    const uint32_t rest = (uint32_t)n & 0x7ffu;
+    t += rest > 0x400u || (rest == 0x400u && (t & 1)) ? 1 : 0;  // to nearest, ties to even (2^53 carries into the exponent)
+    const uint64_t bits = ((uint64_t)(unsigned)(e - lz + 11 + 52 + 1022) << 52) + t;
+    return __hiloint2double((int)(bits >> 32) | (v < 0 ? (int)0x80000000 : 0), (int)(uint32_t)bits);
+}
+
+// ln(n 2^e) as a double for n in [2^63, 2^64), |ln| < 62: the reduction of
+// fix_half_ln with the cubic term to 2^-58; within 2^-57 absolute, and 2^-53
+// relative (one rounding) above 1/8.  No FP64 instruction: one costs as much as
+// 76 issue slots, this function ~60.
+__device__ __forceinline__ double fix_ln(uint64_t n, int e)
+{
+    const int j = (int)(n >> 55) & 255;
+    const uint32_t r = (uint32_t)__ldg(&kFixLogR[j]);
+    const int64_t u = (int64_t)((uwide((uint32_t)(n >> 32), r) << 17) + (uwide((uint32_t)n, r) >> 15));  // 2^-64
+    const int a = (int)(u >> 25);                  // 2^-39
+    const int b = (int)((uint32_t)u & 0x1ffffffu);  // 2^-64
+    const int64_t h2 = (wide(a, a) + (wide(a, b) >> 24)) >> 15;  // u^2/2, 2^-64
+    int t = 429496730 - (__mulhi(a, 357913941) >> 7);            // 1/3 - u/4 + u^2/5 - u^3/6, 2^-31
+    t = 536870912 - (__mulhi(a, t) >> 7);
+    t = 715827883 - (__mulhi(a, t) >> 7);
+    const int64_t c3 = wide((int)(h2 >> 15), (int)(wide(a, t) >> 29)) >> 25;  // u^3 t, 2^-64
+    const int64_t l = __ldg(&kFixLog[j]) + ((u - h2 + c3) >> 1);              // ln m, 2^-63
+    const int k = 63 + e;
+    if (k == 0 || k == -1) return fix_to_double(k ? l - 2 * kHalfLn2 : l, -63);
+    // k ln 2 in 2^-57
+    const int64_t kl = (wide(k, (int)(kHalfLn2 >> 32)) << 27) + (wide(k, (int)((uint32_t)kHalfLn2 >> 1)) >> 4);
+    return fix_to_double(kl + (l >> 6), -57);
+}
+
 // ---------------------------------------------------------------------------
 // One process's 1-D rate table on the integers (filled by the host when the
 // tables are made): logarithms in units of 2^-53.  ok: the axis fits.

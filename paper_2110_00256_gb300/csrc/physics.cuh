@@ -25,11 +25,21 @@ __device__ __forceinline__ double r_log(double x) { return log_tang(x); }
 __device__ __forceinline__ float r_exp(float x) { return __expf(x); }
 __device__ __forceinline__ double r_exp(double x) { return exp_tang(x); }
 __device__ __forceinline__ double d_fma(double a, double b, double c) { return fma(a, b, c); }
+// ln x on the integers (fixed64.cuh) for x in [2^-86, 2^86]; Tang's beyond
+__device__ __forceinline__ double log_int(double x)
+{
+    const int hi = __double2hiint(x);
+    if ((unsigned)(hi - (937 << 20)) >= (172u << 20)) return log_tang(x);  // (also zero, negative, NaN)
+    const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(x);
+    return fix_ln(m << 11, (hi >> 20) - 1023 - 63);
+}
+
 // logarithm and exponential of the 2-D inverse-CDF sampling: FP32 the library
-// forms; FP64 Tang's (ln chi and ln r are interpolation coordinates, where the
-// logarithm's 2^-57 absolute error near 1 is far below the tables' spacing)
+// forms; FP64 the integer logarithm (ln chi and ln r are interpolation
+// coordinates, where its 2^-57 absolute error near 1 is far below the tables'
+// spacing) and Tang's exponential
 __device__ __forceinline__ float s_log(float x) { return logf(x); }
-__device__ __forceinline__ double s_log(double x) { return log_tang(x); }
+__device__ __forceinline__ double s_log(double x) { return log_int(x); }
 __device__ __forceinline__ float s_exp(float x) { return expf(x); }
 __device__ __forceinline__ double s_exp(double x) { return exp_tang(x); }
 
@@ -351,10 +361,10 @@ __device__ __forceinline__ void store_tau<float>(float *tau, float *tau_c, int64
     tau_c[i] = c;
 }
 
-// -ln U in FP64 for U in [2^-54, 1]: Tang's logarithm (within 2 ulp); above
+// -ln U to FP64 for U in [2^-54, 1]: the integer logarithm (fixed64.cuh); above
 // 1 - 2^-8, where ln U is small and that logarithm's error no longer shrinks
 // with it, the Taylor series of log1p(d) with d = U - 1 (exact: U >= 1/2), whose
-// remainder d^8/8 is below 2^-59 of the result.  The optical-depth resets are
+// remainder d^8/8 is below 2^-59 of the result.  The optical-depth resets were
 // the event kernels' largest FP64 cost, and GB300's FP64 pipe their bound when
 // many particles fire.
 static __device__ __noinline__ double neg_log1p_series(double u)
@@ -372,10 +382,11 @@ __device__ __forceinline__ double neg_log_u(double u)
 {
     // (positive doubles order as their bit patterns: the test costs no FP64
     // instruction; the series is out of line, so that the other 99.6 % of the
-    // draws do not issue it predicated off; U >= 2^-54 is normal, so Tang's core
-    // needs no range check)
+    // draws do not issue it predicated off; U >= 2^-54 is normal)
     if (__double_as_longlong(u) > __double_as_longlong(1.0 - 0x1p-8)) return neg_log1p_series(u);
-    return -log_tang_core(u, 0);
+    const int hi = __double2hiint(u);
+    const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(u);
+    return -fix_ln(m << 11, (hi >> 20) - 1023 - 63);
 }
 
 // tau = -ln U, U the 53-bit uniform of (seed, (id, step, purpose)), in FP64 (§3)

@@ -24,10 +24,16 @@ static inline unsigned long long __umul64hi(unsigned long long a, unsigned long 
 {
     return (unsigned long long)(((unsigned __int128)a * b) >> 64);
 }
+template <class T> static inline T __ldg(const T *p) { return *p; }
 static int g_skew;  // rsqrtf on the GPU is within 2 ulp: skewed either way here
 static inline float rsqrtf(float x) { return (1.0f / sqrtf(x)) * (1.0f + 1.2e-7f * (float)(g_skew++ % 3 - 1)); }
 
 #include "fixed64.cuh"
+
+extern "C" void fixed_ln(int64_t n, const uint64_t *m, const int *e, double *out)
+{
+    for (int64_t i = 0; i < n; ++i) out[i] = qed::fix_ln(m[i], e[i]);
+}
 
 // n particles (rows px py pz ex ey ez bx by bz of p); the table of n_tab values on [chi_min, chi_max]
 extern "C" void fixed_rates(int qs, int64_t n, const double *p, double chi_min, double chi_max, int n_tab,

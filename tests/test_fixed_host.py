@@ -145,3 +145,27 @@ def test_table_ends_of_the_pair_rate_are_left_to_fp64(lib):
     p[4] = [2e-2, 1e3, 2.1e-2, 1.9e-2]
     ok = run(lib, False, p)[3]
     assert list(ok) == [False, False, True, True]
+
+
+def test_logarithm_against_extended_precision(lib):
+    """The resets' and the sampling's logarithm: within 2^-57 absolute and one rounding (2^-53 and the integers' 2^-57) where
+    the result is not small, over the significands next to every table edge, next to 1 and at random."""
+    r = np.random.default_rng(2)
+    m = r.integers(1 << 63, 1 << 64, 400_000, dtype=np.uint64)
+    edge = (np.arange(256, dtype=np.uint64) << np.uint64(55)) + np.uint64(1 << 63)
+    near = np.concatenate([edge, edge - np.uint64(1), edge + np.uint64(1 << 11)])
+    near = near[near >= 1 << 63]
+    m = np.concatenate([np.repeat(near, 8), (np.uint64(2 ** 64 - 1) - np.arange(1 << 12, dtype=np.uint64) * np.uint64(2048)), m])
+    e = r.integers(-63 - 85, -63 + 85, m.size).astype(np.int32)
+    e[::3] = -63
+    e[1::3] = -64
+    out = np.zeros(m.size)
+    ptr = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    lib.fixed_ln(ctypes.c_int64(m.size), ptr(m), ptr(e), ptr(out))
+    k = e.astype(np.int64) + 64  # n 2^e = (n 2^-64) 2^k, n 2^-64 in [1/2, 1)
+    x = m.astype(LD) / LD(2) ** 64
+    # (ln x taken from 1 where k = 0, so that the reference keeps its digits there)
+    ref = np.where(k == 0, np.log1p((m - np.uint64(2 ** 63)).astype(LD) / LD(2) ** 64 - LD(0.5)),
+                   np.log(x) + k * np.log(LD(2)))
+    err = np.abs(out - ref).astype(np.float64)
+    assert np.all(err <= 2.0 ** -57 + 2.0 ** -53 * np.abs(ref).astype(np.float64))

@@ -51,29 +51,54 @@ __global__ void mlp_to_bf16_kernel(const float *p, __nv_bfloat16 *w)
 }
 
 // ---------------------------------------------------------------------------
-// training: one CTA of kTrainThreads threads takes kTrainThreads samples at a
-// time (one per thread) and accumulates the gradient of the mean squared error
-// in shared memory; each CTA stores its sums (gradient and loss) in a slot of
-// its own, and mlp_reduce_kernel adds the slots in CTA order, so that a
-// training run gives the same bits every time (atomic adds across CTAs would
-// round in the order the CTAs arrive).
+// training: a CTA of 256 threads takes 32 samples at a time, so that a minibatch
+// of 4096 spreads over 128 SMs (one thread per sample, 128 to a CTA, put it on
+// 32 of them and took 60 us, bound by shared-memory reads: two for each FMA).
+// The three 64 x 64 products are register tiles: layer 2 and its transpose take
+// 4 neurons x 2 samples per thread, the weight gradient 4 x 4 weights, held in
+// registers over all of the CTA's samples.  Each CTA stores its sums (gradient
+// and loss) in a slot of its own, and mlp_reduce_kernel adds the slots in a fixed
+// order, so that a training run gives the same bits every time (atomic adds
+// across CTAs would round in the order the CTAs arrive).
 // ---------------------------------------------------------------------------
-constexpr int kTrainThreads = 128;
-constexpr int kTS = kTrainThreads + 1;  // padded sample stride of the [64][samples] buffers
+constexpr int kTrainThreads = 256;
+constexpr int kTrainBatch = 32;   // samples of a CTA's pass
+constexpr int kTW = kMlpH + 4;    // row stride of the [.][64] buffers: 16-byte aligned, rows on different banks
 
 struct TrainSmem {
-    alignas(8) float w1a[kMlpH];
-    alignas(8) float w1b[kMlpH];
-    alignas(8) float b1[kMlpH];
-    float w2[kMlpH * kMlpH], b2[kMlpH], w3[kMlpH], b3;
-    float g[kMlpParams];       // gradient accumulator of this CTA
-    float h1[kMlpH * kTS];     // bf16-rounded h1, [k][s]
-    float z2[kMlpH * kTS];     // z2, then d2 = dL/dz2
-    float q[kMlpH * kTS];      // dy * h2, then d1 = dL/dz1
-    float x[2][kTrainThreads], dy[kTrainThreads];
+    alignas(16) float w1a[kMlpH];
+    alignas(16) float w1b[kMlpH];
+    alignas(16) float b1[kMlpH];
+    alignas(16) float b2[kMlpH];
+    alignas(16) float w3[kMlpH];
+    alignas(16) float w2[kMlpH * kTW];      // [j][k]
+    alignas(16) float w2t[kMlpH * kTW];     // [k][j]
+    alignas(16) float h1[kTrainBatch * kTW];  // bf16-rounded h1, [sample][k]
+    alignas(16) float d2[kTrainBatch * kTW];  // dL/dz2, [sample][j]
+    float x[2][kTrainBatch], tgt[kTrainBatch];
+    float sums[8][6 * kMlpH + 2];           // per warp: dW1 (two columns), db1, db2, dW3, (unused), db3, loss
 };
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+
+// acc[a][b] = sum over c of m[c][4 q + a] v[2 p + b][c], c ascending from the given start
+__device__ __forceinline__ void tile_4x2(float (&acc)[4][2], const float *m, const float *v, int q, int p)
+{
+    const float *v0 = v + (2 * p) * kTW, *v1 = v0 + kTW;
+#pragma unroll 4
+    for (int c = 0; c < kMlpH; c += 4) {
+        const float4 a = *reinterpret_cast<const float4 *>(v0 + c), b = *reinterpret_cast<const float4 *>(v1 + c);
+        const float va[4] = {a.x, a.y, a.z, a.w}, vb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 w = *reinterpret_cast<const float4 *>(m + (c + i) * kTW + 4 * q);
+            acc[0][0] = fmaf(w.x, va[i], acc[0][0]), acc[0][1] = fmaf(w.x, vb[i], acc[0][1]);
+            acc[1][0] = fmaf(w.y, va[i], acc[1][0]), acc[1][1] = fmaf(w.y, vb[i], acc[1][1]);
+            acc[2][0] = fmaf(w.z, va[i], acc[2][0]), acc[2][1] = fmaf(w.z, vb[i], acc[2][1]);
+            acc[3][0] = fmaf(w.w, va[i], acc[3][0]), acc[3][1] = fmaf(w.w, vb[i], acc[3][1]);
+        }
+    }
+}
 
 __global__ void __launch_bounds__(kTrainThreads) mlp_train_kernel(MlpView v, const double *__restrict__ chi,
                                                                     const double *__restrict__ uu,
@@ -82,149 +107,181 @@ __global__ void __launch_bounds__(kTrainThreads) mlp_train_kernel(MlpView v, con
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     TrainSmem &S = *reinterpret_cast<TrainSmem *>(smem_raw);
-    const int tid = threadIdx.x;
-    for (int i = tid; i < kMlpH; i += blockDim.x) {
-        S.w1a[i] = __bfloat162float(v.w[kOffW1 + 2 * i]);
-        S.w1b[i] = __bfloat162float(v.w[kOffW1 + 2 * i + 1]);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid < kMlpH) {
+        S.w1a[tid] = __bfloat162float(v.w[kOffW1 + 2 * tid]);
+        S.w1b[tid] = __bfloat162float(v.w[kOffW1 + 2 * tid + 1]);
+        S.b1[tid] = __bfloat162float(v.w[kOffB1 + tid]);
+        S.b2[tid] = __bfloat162float(v.w[kOffB2 + tid]);
+        S.w3[tid] = __bfloat162float(v.w[kOffW3 + tid]);
     }
-    for (int i = tid; i < kMlpH * kMlpH; i += blockDim.x) S.w2[i] = __bfloat162float(v.w[kOffW2 + i]);
-    for (int i = tid; i < kMlpH; i += blockDim.x) {
-        S.b1[i] = __bfloat162float(v.w[kOffB1 + i]);
-        S.b2[i] = __bfloat162float(v.w[kOffB2 + i]);
-        S.w3[i] = __bfloat162float(v.w[kOffW3 + i]);
+    for (int i = tid; i < kMlpH * kMlpH; i += kTrainThreads) {
+        const float w = __bfloat162float(v.w[kOffW2 + i]);
+        S.w2[(i / kMlpH) * kTW + i % kMlpH] = w;
+        S.w2t[(i % kMlpH) * kTW + i / kMlpH] = w;
     }
-    for (int i = tid; i < kMlpParams; i += blockDim.x) S.g[i] = 0.f;
-    if (tid == 0) S.b3 = __bfloat162float(v.w[kOffB3]);
-    __syncthreads();
+    const float b3 = __bfloat162float(v.w[kOffB3]);
     const float inv_n = 1.0f / (float)n;
-    float my_loss = 0.f;
+    const int q = tid & 15, p = tid >> 4;  // neurons 4 q .. 4 q + 3 of samples 2 p, 2 p + 1
+    float gw2[4][4] = {};                  // dW2[4 p + a][4 q + b]
+    float ga[4] = {}, gb[4] = {}, g1[4] = {}, g2[4] = {}, g3[4] = {};  // dW1, db1, db2, dW3 of the neurons 4 q ..
+    float gb3 = 0.0f, my_loss = 0.0f;
 
-    for (int64_t base = (int64_t)blockIdx.x * kTrainThreads; base < n; base += (int64_t)gridDim.x * kTrainThreads) {
-        const int64_t i = base + tid;
-        const bool valid = i < n;
-        float x1 = 0.f, x2 = 0.f, tgt = 0.f;
-        if (valid) {
-            const MlpIn in = mlp_input(v, chi[i], uu[i]);
-            x1 = in.x1, x2 = in.x2;
-            tgt = mlp_target(v.proc, xi[i], in);
+    for (int64_t base = (int64_t)blockIdx.x * kTrainBatch; base < n; base += (int64_t)gridDim.x * kTrainBatch) {
+        __syncthreads();  // (the weights are staged; the last pass's buffers are free)
+        if (tid < kTrainBatch) {
+            const int64_t i = base + tid;
+            const bool valid = i < n;
+            const MlpIn in = mlp_input(v, valid ? chi[i] : 1.0, valid ? uu[i] : 0.5);
+            S.x[0][tid] = valid ? in.x1 : 0.0f;
+            S.x[1][tid] = valid ? in.x2 : 0.0f;
+            S.tgt[tid] = valid ? mlp_target(v.proc, xi[i], in) : 0.0f;
         }
-        S.x[0][tid] = x1;
-        S.x[1][tid] = x2;
-        // forward, with the inference kernels' arithmetic (pairs of neurons)
-        const uint64_t x1x1 = f2(x1, x1), x2x2 = f2(x2, x2);
-        for (int k = 0; k < kMlpH; k += 2) {
-            const float2 g = f2u(layer1_pair(S.w1a, S.w1b, S.b1, k, x1x1, x2x2));
-            S.h1[k * kTS + tid] = bf16r(g.x);
-            S.h1[(k + 1) * kTS + tid] = bf16r(g.y);
-        }
-        float y = S.b3;
-        for (int j = 0; j < kMlpH; j += 2) {
-            float z0 = S.b2[j], z1 = S.b2[j + 1];
-            for (int k = 0; k < kMlpH; ++k) {
-                const float h = S.h1[k * kTS + tid];
-                z0 = fmaf(S.w2[j * kMlpH + k], h, z0);
-                z1 = fmaf(S.w2[(j + 1) * kMlpH + k], h, z1);
+        __syncthreads();
+        {  // layer 1 with the inference kernels' arithmetic (pairs of neurons): 8 neurons of one sample per thread
+            const int s = tid >> 3, k0 = (tid & 7) * 8;
+            const uint64_t x1x1 = f2(S.x[0][s], S.x[0][s]), x2x2 = f2(S.x[1][s], S.x[1][s]);
+#pragma unroll
+            for (int k = k0; k < k0 + 8; k += 2) {
+                const float2 g = f2u(layer1_pair(S.w1a, S.w1b, S.b1, k, x1x1, x2x2));
+                *reinterpret_cast<float2 *>(S.h1 + s * kTW + k) = make_float2(bf16r(g.x), bf16r(g.y));
             }
-            S.z2[j * kTS + tid] = z0;
-            S.z2[(j + 1) * kTS + tid] = z1;
-            const float2 g = f2u(gelu2(f2(z0, z1)));
-            S.q[j * kTS + tid] = g.x;
-            S.q[(j + 1) * kTS + tid] = g.y;
-            y = fmaf(S.w3[j + 1], g.y, fmaf(S.w3[j], g.x, y));
-        }
-        const float r = valid ? y - tgt : 0.f;
-        my_loss += r * r;
-        const float dy = 2.f * r * inv_n;
-        S.dy[tid] = dy;
-        for (int j = 0; j < kMlpH; ++j) {
-            const float z = S.z2[j * kTS + tid];
-            S.q[j * kTS + tid] *= dy;                             // dy h2, for dW3
-            S.z2[j * kTS + tid] = dy * S.w3[j] * gelu_grad(z);    // d2
         }
         __syncthreads();
-        // dW2 = d2^T h1, db2 = sum d2, dW3 = sum dy h2, db3 = sum dy
-        for (int e = tid; e < kMlpH * kMlpH; e += blockDim.x) {
-            const int j = e / kMlpH, k = e % kMlpH;
-            float acc = 0.f;
-            for (int s = 0; s < kTrainThreads; ++s) acc = fmaf(S.z2[j * kTS + s], S.h1[k * kTS + s], acc);
-            S.g[kOffW2 + e] += acc;
-        }
-        if (tid < kMlpH) {
-            float a = 0.f, b = 0.f;
-            for (int s = 0; s < kTrainThreads; ++s) {
-                a += S.z2[tid * kTS + s];
-                b += S.q[tid * kTS + s];
+        // layer 2 and 3
+        float z[4][2], h2[4][2], y[2] = {0.0f, 0.0f};
+#pragma unroll
+        for (int a = 0; a < 4; ++a) z[a][0] = z[a][1] = S.b2[4 * q + a];
+        tile_4x2(z, S.w2t, S.h1, q, p);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+#pragma unroll
+            for (int a = 0; a < 4; a += 2) {
+                const float2 g = f2u(gelu2(f2(z[a][b], z[a + 1][b])));
+                h2[a][b] = g.x, h2[a + 1][b] = g.y;
+                y[b] = fmaf(S.w3[4 * q + a + 1], g.y, fmaf(S.w3[4 * q + a], g.x, y[b]));
             }
-            S.g[kOffB2 + tid] += a;
-            S.g[kOffW3 + tid] += b;
-        } else if (tid == kMlpH) {
-            float a = 0.f;
-            for (int s = 0; s < kTrainThreads; ++s) a += S.dy[s];
-            S.g[kOffB3] += a;
+#pragma unroll
+            for (int o = 1; o < 16; o <<= 1) y[b] += __shfl_xor_sync(0xffffffffu, y[b], o);  // over the 16 q's
         }
-        __syncthreads();
-        // d1 = (W2^T d2) * gelu'(z1), per sample
-        for (int k = 0; k < kMlpH; ++k) {
-            float acc = 0.f;
-            for (int j = 0; j < kMlpH; ++j) acc = fmaf(S.w2[j * kMlpH + k], S.z2[j * kTS + tid], acc);
-            const float z1 = fmaf(S.w1a[k], x1, fmaf(S.w1b[k], x2, S.b1[k]));
-            S.q[k * kTS + tid] = acc * gelu_grad(z1);
-        }
-        __syncthreads();
-        // dW1 = d1^T x, db1 = sum d1
-        if (tid < kMlpH) {
-            float a0 = 0.f, a1 = 0.f, b = 0.f;
-            for (int s = 0; s < kTrainThreads; ++s) {
-                const float d = S.q[tid * kTS + s];
-                a0 = fmaf(d, S.x[0][s], a0);
-                a1 = fmaf(d, S.x[1][s], a1);
-                b += d;
+        // d2, db2, dW3, db3
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int s = 2 * p + b;
+            const float r = base + s < n ? y[b] + b3 - S.tgt[s] : 0.0f;
+            const float dy = 2.0f * r * inv_n;
+            my_loss += r * r;
+            gb3 += dy;
+            float d[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                d[a] = dy * S.w3[4 * q + a] * gelu_grad(z[a][b]);
+                g3[a] = fmaf(dy, h2[a][b], g3[a]);
+                g2[a] += d[a];
             }
-            S.g[kOffW1 + 2 * tid] += a0;
-            S.g[kOffW1 + 2 * tid + 1] += a1;
-            S.g[kOffB1 + tid] += b;
+            *reinterpret_cast<float4 *>(S.d2 + s * kTW + 4 * q) = make_float4(d[0], d[1], d[2], d[3]);
         }
         __syncthreads();
+        // dW2 = d2^T h1
+#pragma unroll 4
+        for (int s = 0; s < kTrainBatch; ++s) {
+            const float4 d = *reinterpret_cast<const float4 *>(S.d2 + s * kTW + 4 * p);
+            const float4 h = *reinterpret_cast<const float4 *>(S.h1 + s * kTW + 4 * q);
+            const float dd[4] = {d.x, d.y, d.z, d.w}, hh[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) gw2[a][b] = fmaf(dd[a], hh[b], gw2[a][b]);
+        }
+        // d1 = (W2^T d2) gelu'(z1); dW1 = d1^T x, db1 = sum d1
+        float acc[4][2] = {};
+        tile_4x2(acc, S.w2, S.d2, q, p);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const float x1 = S.x[0][2 * p + b], x2 = S.x[1][2 * p + b];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const int k = 4 * q + a;
+                const float d = acc[a][b] * gelu_grad(fmaf(S.w1a[k], x1, fmaf(S.w1b[k], x2, S.b1[k])));
+                ga[a] = fmaf(d, x1, ga[a]);
+                gb[a] = fmaf(d, x2, gb[a]);
+                g1[a] += d;
+            }
+        }
     }
-    S.dy[tid] = my_loss;  // (the per-sample buffer is free after the last pass)
-    __syncthreads();
+    // the slot: dW2 from the tiles; the sums over samples across the warp's two
+    // p's and then the eight warps, in order
     float *slot = part + (size_t)blockIdx.x * (kMlpParams + 1);
-    for (int i = tid; i < kMlpParams; i += blockDim.x) slot[i] = S.g[i];
-    if (tid == 0) {
-        float l = 0.f;
-        for (int s = 0; s < kTrainThreads; ++s) l += S.dy[s];
-        slot[kMlpParams] = l * inv_n;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) slot[kOffW2 + (4 * p + a) * kMlpH + 4 * q + b] = gw2[a][b];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        float w[5] = {ga[a], gb[a], g1[a], g2[a], g3[a]};
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            w[i] += __shfl_xor_sync(0xffffffffu, w[i], 16);
+            if (lane < 16) S.sums[warp][i * kMlpH + 4 * q + a] = w[i];
+        }
+    }
+    gb3 += __shfl_xor_sync(0xffffffffu, gb3, 16);
+    my_loss += __shfl_xor_sync(0xffffffffu, my_loss, 16);
+    if (lane == 0) S.sums[warp][5 * kMlpH] = gb3, S.sums[warp][5 * kMlpH + 1] = my_loss;
+    __syncthreads();
+    for (int i = tid; i < 5 * kMlpH + 2; i += kTrainThreads) {
+        float t = 0.0f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += S.sums[w][i];
+        const int kind = i / kMlpH, k = i % kMlpH;
+        const int at = kind == 0 ? kOffW1 + 2 * k : kind == 1 ? kOffW1 + 2 * k + 1 : kind == 2 ? kOffB1 + k
+                       : kind == 3 ? kOffB2 + k : kind == 4 ? kOffW3 + k : k == 0 ? kOffB3 : kMlpParams;
+        slot[at] = at == kMlpParams ? t * inv_n : t;
     }
 }
 
-// the training kernel's per-CTA slots summed in CTA order: the gradient, and
-// the batch's mean loss into loss_out
-__global__ void mlp_reduce_kernel(const float *__restrict__ part, int slots, float *grad, float *loss_out)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > kMlpParams) return;
-    float a = 0.f;
-    for (int c = 0; c < slots; ++c) a += part[(size_t)c * (kMlpParams + 1) + i];
-    if (i < kMlpParams)
-        grad[i] = a;
-    else
-        *loss_out = a;
-}
+// what a training step changes: the master parameters, Adam's moments, the bf16 copy
+struct MlpAdam {
+    float *p, *m, *v;
+    __nv_bfloat16 *w;
+    float lr, bc1, bc2;
+};
 
-// Adam (Kingma & Ba 2015); refreshes the bf16 copy and clears the gradient
-__global__ void mlp_adam_kernel(float *p, float *m, float *v, float *g, __nv_bfloat16 *w, float lr, float bc1,
-                                float bc2)
+// The training kernel's per-CTA slots added in a fixed order (eight threads per
+// parameter take every eighth slot, so that their loads are in flight together,
+// and their sums are added in order): the gradient into grad_out (may be NULL),
+// the batch's mean loss into loss_out (may be NULL), and with ADAM the parameters'
+// step from it (Kingma & Ba 2015) and their bf16 copy.
+template <bool ADAM>
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float *__restrict__ part, int slots, float *grad_out,
+                                                          float *loss_out, MlpAdam u)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kMlpParams; i += gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = 0.9f * m[i] + 0.1f * gi;
-        const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float pi = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + 1e-8f);
-        p[i] = pi;
-        w[i] = __float2bfloat16_rn(pi);
-        g[i] = 0.f;
+    __shared__ float s_sum[8][32];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    float a = 0.0f;
+    if (i <= kMlpParams) {
+#pragma unroll 4
+        for (int c = g; c < slots; c += 8) a += part[(size_t)c * (kMlpParams + 1) + i];
+    }
+    s_sum[g][lane] = a;
+    __syncthreads();
+    if (g || i > kMlpParams) return;
+    float t = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t += s_sum[k][lane];
+    if (i == kMlpParams) {
+        if (loss_out) *loss_out = t;
+        return;
+    }
+    if (grad_out) grad_out[i] = t;
+    if constexpr (ADAM) {
+        const float mi = 0.9f * u.m[i] + 0.1f * t;
+        const float vi = 0.999f * u.v[i] + 0.001f * t * t;
+        u.m[i] = mi;
+        u.v[i] = vi;
+        const float pi = u.p[i] - u.lr * (mi / u.bc1) / (sqrtf(vi / u.bc2) + 1e-8f);
+        u.p[i] = pi;
+        u.w[i] = __float2bfloat16_rn(pi);
     }
 }
 
@@ -530,7 +587,7 @@ static void free_mlp(qed_mlp *m)
 {
     if (!m) return;
     for (int p = 0; p < 2; ++p) {
-        void *ptrs[] = {m->master[p], m->adam_m[p], m->adam_v[p], m->grad[p], m->part[p], m->loss[p], m->w[p]};
+        void *ptrs[] = {m->master[p], m->adam_m[p], m->adam_v[p], m->part[p], m->w[p]};
         for (void *x : ptrs)
             if (x) cudaFree(x);
     }
@@ -548,17 +605,14 @@ static qed_status create_mlp(const double chi_min[2], const double chi_max[2], u
     m->part_slots = sm_count();
     for (int p = 0; p < 2; ++p) {
         cudaError_t e = cudaSuccess;
-        float **fp[] = {&m->master[p], &m->adam_m[p], &m->adam_v[p], &m->grad[p]};
+        float **fp[] = {&m->master[p], &m->adam_m[p], &m->adam_v[p]};
         for (float **f : fp)
             if (e == cudaSuccess) e = cudaMalloc((void **)f, kMlpParams * sizeof(float));
-        if (e == cudaSuccess) e = cudaMalloc((void **)&m->loss[p], sizeof(float));
         if (e == cudaSuccess)
             e = cudaMalloc((void **)&m->part[p], (size_t)m->part_slots * (kMlpParams + 1) * sizeof(float));
         if (e == cudaSuccess) e = cudaMalloc((void **)&m->w[p], kMlpParams * sizeof(__nv_bfloat16));
         if (e == cudaSuccess) e = cudaMemsetAsync(m->adam_m[p], 0, kMlpParams * sizeof(float), st);
         if (e == cudaSuccess) e = cudaMemsetAsync(m->adam_v[p], 0, kMlpParams * sizeof(float), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(m->grad[p], 0, kMlpParams * sizeof(float), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(m->loss[p], 0, sizeof(float), st);
         if (e != cudaSuccess) {
             free_mlp(m);
             QED_FAIL(QED_ERR_CUDA, "mlp allocation failed: %s", cudaGetErrorString(e));
@@ -700,8 +754,9 @@ extern "C" qed_status qed_mlp_set_params(qed_mlp *m, qed_process proc, const flo
     return QED_OK;
 }
 
+// the batch's gradient and loss: into grad_out / loss_out, or with `adam` into the parameters
 static qed_status launch_train(qed_mlp *m, int proc, const double *chi, const double *u, const double *xi, int64_t n,
-                               cudaStream_t st)
+                               float *grad_out, float *loss_out, const MlpAdam *adam, cudaStream_t st)
 {
     static bool attr = false;
     const size_t sm = sizeof(TrainSmem);
@@ -709,13 +764,16 @@ static qed_status launch_train(qed_mlp *m, int proc, const double *chi, const do
         QED_CUDA_TRY(cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
         attr = true;
     }
-    int64_t blocks = (n + kTrainThreads - 1) / kTrainThreads;
+    int64_t blocks = (n + kTrainBatch - 1) / kTrainBatch;
     const int64_t cap = (int64_t)m->part_slots;
     blocks = blocks < 1 ? 1 : (blocks > cap ? cap : blocks);
     mlp_train_kernel<<<(int)blocks, kTrainThreads, sm, st>>>(mlp_view(m, proc), chi, u, xi, n, m->part[proc]);
     QED_LAUNCH_CHECK();
-    mlp_reduce_kernel<<<(kMlpParams + 1 + 255) / 256, 256, 0, st>>>(m->part[proc], (int)blocks, m->grad[proc],
-                                                                   m->loss[proc]);
+    constexpr int g = (kMlpParams + 1 + 31) / 32;
+    if (adam)
+        mlp_reduce_kernel<true><<<g, 256, 0, st>>>(m->part[proc], (int)blocks, grad_out, loss_out, *adam);
+    else
+        mlp_reduce_kernel<false><<<g, 256, 0, st>>>(m->part[proc], (int)blocks, grad_out, loss_out, MlpAdam{});
     QED_LAUNCH_CHECK();
     return QED_OK;
 }
@@ -737,12 +795,7 @@ extern "C" qed_status qed_mlp_gradients(qed_mlp *m, qed_process proc, const doub
     if ((s = check_batch(d_chi, d_u, d_xi, n))) return s;
     if (!d_grad) QED_FAIL(QED_ERR_INVALID_ARG, "d_grad is NULL");
     cudaStream_t st = as_stream(stream);
-    QED_CUDA_TRY(cudaMemsetAsync(m->grad[proc], 0, kMlpParams * sizeof(float), st));
-    if ((s = launch_train(m, proc, d_chi, d_u, d_xi, n, st))) return s;
-    QED_CUDA_TRY(cudaMemcpyAsync(d_grad, m->grad[proc], kMlpParams * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    if (d_loss) QED_CUDA_TRY(cudaMemcpyAsync(d_loss, m->loss[proc], sizeof(float), cudaMemcpyDeviceToDevice, st));
-    QED_CUDA_TRY(cudaMemsetAsync(m->grad[proc], 0, kMlpParams * sizeof(float), st));
-    return QED_OK;
+    return launch_train(m, proc, d_chi, d_u, d_xi, n, d_grad, d_loss, nullptr, st);
 }
 
 extern "C" qed_status qed_mlp_train_step(qed_mlp *m, qed_process proc, const double *d_chi, const double *d_u,
@@ -754,13 +807,11 @@ extern "C" qed_status qed_mlp_train_step(qed_mlp *m, qed_process proc, const dou
     if ((s = check_batch(d_chi, d_u, d_xi, n))) return s;
     if (!(lr > 0.f)) QED_FAIL(QED_ERR_INVALID_ARG, "learning rate must be positive");
     cudaStream_t st = as_stream(stream);
-    if ((s = launch_train(m, proc, d_chi, d_u, d_xi, n, st))) return s;
-    const int64_t k = ++m->step[proc];
-    const float bc1 = 1.f - powf(0.9f, (float)k), bc2 = 1.f - powf(0.999f, (float)k);
-    mlp_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, st>>>(m->master[proc], m->adam_m[proc], m->adam_v[proc],
-                                                              m->grad[proc], m->w[proc], lr, bc1, bc2);
-    QED_LAUNCH_CHECK();
-    if (d_loss) QED_CUDA_TRY(cudaMemcpyAsync(d_loss, m->loss[proc], sizeof(float), cudaMemcpyDeviceToDevice, st));
+    const int64_t k = m->step[proc] + 1;
+    const MlpAdam u{m->master[proc], m->adam_m[proc], m->adam_v[proc], m->w[proc], lr, 1.f - powf(0.9f, (float)k),
+                    1.f - powf(0.999f, (float)k)};
+    if ((s = launch_train(m, proc, d_chi, d_u, d_xi, n, nullptr, d_loss, &u, st))) return s;
+    m->step[proc] = k;
     return QED_OK;
 }
 

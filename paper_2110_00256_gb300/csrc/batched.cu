@@ -266,7 +266,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1)
     __shared__ long long s_warp[THREADS / 32];
     __shared__ int s_abort;
 
-    stage_rates(rs, tab, THREADS);
+    stage_rates(rs, tab, dt, THREADS);
     if (threadIdx.x == 0) {
         s_abort = 0;
         for (int k = 0; k < S; ++k) {

@@ -17,7 +17,7 @@ struct EventArgs {
 };
 
 template <typename T, bool MLP>
-__global__ void __launch_bounds__(256) qs_event_kernel(const __grid_constant__ EventArgs<T> a)
+__global__ void __launch_bounds__(256, (MLP || sizeof(T) == 8) ? 1 : 4) qs_event_kernel(const __grid_constant__ EventArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);
@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(256) qs_event_kernel(const __grid_constant__ E
 }
 
 template <typename T, bool MLP>
-__global__ void __launch_bounds__(256) bw_event_kernel(const __grid_constant__ EventArgs<T> a)
+__global__ void __launch_bounds__(256, (MLP || sizeof(T) == 8) ? 1 : 4) bw_event_kernel(const __grid_constant__ EventArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kEvolveThreads, MINB)
     __shared__ long long s_n[MAXSEG];
     constexpr int64_t tile = kEvolveTile<T, VEC>;
 
-    stage_rates(rs, a.tab, blockDim.x);
+    stage_rates(rs, a.tab, a.dt, blockDim.x);
     if (threadIdx.x == 0) {
         long long acc = 0;
         for (int s = 0; s < a.n_seg; ++s) {
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, MINB)
     __shared__ long long s_n[MAXSEG];
     __shared__ int s_abort;
 
-    stage_rates(rs, a.tab, blockDim.x);
+    stage_rates(rs, a.tab, a.dt, blockDim.x);
     if (threadIdx.x == 0) {
         long long acc = 0;
         for (int s = 0; s < a.n_seg; ++s) {
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS)
     long long *s_end = s_dyn, *s_n = s_dyn + n_seg;
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
-    stage_rates(rs, tab, THREADS);
+    stage_rates(rs, tab, dt, THREADS);
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);
     int bad = 0;
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {

@@ -72,9 +72,10 @@ struct RateSmem<double> {
     long long ln[256], ex[256];
     int r[256];
     int off[2];  // per process: nonzero if a value or a step of its table does not fit the integers
+    double coef_dt[2];  // per process: the rate's constant factor times dt
 };
 
-__device__ __forceinline__ void stage_rates(RateSmem<float> &s, const TablesView<float> &tab, int threads)
+__device__ __forceinline__ void stage_rates(RateSmem<float> &s, const TablesView<float> &tab, float, int threads)
 {
     for (int i = threadIdx.x; i < tab.qs_G.n; i += threads) s.qs[i] = tab.qs_G.ln_f[i];
     for (int i = threadIdx.x; i < tab.bw_T.n; i += threads) s.bw[i] = tab.bw_T.ln_f[i];
@@ -104,9 +105,9 @@ __device__ __forceinline__ int stage_fix(long long *out, const Table1D<double> &
 }
 
 // every thread of the CTA; the caller's next barrier publishes it
-__device__ __forceinline__ void stage_rates(RateSmem<double> &s, const TablesView<double> &tab, int threads)
+__device__ __forceinline__ void stage_rates(RateSmem<double> &s, const TablesView<double> &tab, double dt, int threads)
 {
-    if (threadIdx.x < 2) s.off[threadIdx.x] = 0;
+    if (threadIdx.x < 2) s.off[threadIdx.x] = 0, s.coef_dt[threadIdx.x] = (threadIdx.x ? kAlpha : 2.0 / 3.0 * kAlpha) * dt;
     __syncthreads();
     if (stage_fix(s.qs, tab.qs_G, threads)) s.off[0] = 1;
     if (stage_fix(s.bw, tab.bw_T, threads)) s.off[1] = 1;
@@ -179,7 +180,8 @@ __device__ __forceinline__ bool evolve_one(int proc, const RateSmem<double> &rs,
     bool fast = fix_particle(qs, px, py, pz, ex, ey, ez, bx, by, bz, tb.fix, qs ? rs.qs : rs.bw, rs.r, rs.ln, rs.ex, o);
     // (tau = 0 or NaN: a rate that the integers drop as below 1e-290 could decide)
     const long long tb_bits = __double_as_longlong(tau) & 0x7fffffffffffffffll;
-    fast = fast && rs.off[qs ? 0 : 1] == 0 && tb_bits != 0 && tb_bits <= 0x7ff0000000000000ll && !(cut > 0.0);
+    fast = fast && rs.off[qs ? 0 : 1] == 0 && tb_bits != 0 && tb_bits <= 0x7ff0000000000000ll &&
+           __double_as_longlong(cut) <= 0;  // (no cut-off; compared as bits: no FP64 instruction)
     if (!fast) {
         const auto mag = [](double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; };
         const long long inf = 0x7ff0000000000000ll;
@@ -194,7 +196,7 @@ __device__ __forceinline__ bool evolve_one(int proc, const RateSmem<double> &rs,
         return r.fire != 0;
     }
     // the only FP64 instruction: tau - (rate / coef) (coef dt)
-    tau = fma(-o.rate, (qs ? 2.0 / 3.0 * kAlpha : kAlpha) * dt, tau);
+    tau = fma(-o.rate, rs.coef_dt[qs ? 0 : 1], tau);
     const bool fire = __double_as_longlong(tau) < 0 && __double_as_longlong(tau) != (long long)0x8000000000000000ull;
     if (fire) chi_out = sqrt(scalbn((double)o.s, o.s_e));
     return fire;

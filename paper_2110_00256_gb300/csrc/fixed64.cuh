@@ -172,11 +172,12 @@ __device__ __forceinline__ double fix_to_double(int64_t v, int e)
     return __hiloint2double((int)(bits >> 32) | (v < 0 ? (int)0x80000000 : 0), (int)(uint32_t)bits);
 }
 
-// ln(n 2^e) as a double for n in [2^63, 2^64), |ln| < 62: the reduction of
+// ln(n 2^e) (minus it with `neg`: an FP64 sign change is an FP64 instruction) as a
+// double for n in [2^63, 2^64), |ln| < 62: the reduction of
 // fix_half_ln with the cubic term to 2^-58; within 2^-57 absolute, and 2^-53
 // relative (one rounding) above 1/8.  No FP64 instruction: one costs as much as
 // 76 issue slots, this function ~60.
-__device__ __forceinline__ double fix_ln(uint64_t n, int e)
+__device__ __forceinline__ double fix_ln(uint64_t n, int e, bool neg = false)
 {
     const int j = (int)(n >> 55) & 255;
     const uint32_t r = (uint32_t)__ldg(&kFixLogR[j]);
@@ -190,10 +191,11 @@ __device__ __forceinline__ double fix_ln(uint64_t n, int e)
     const int64_t c3 = wide((int)(h2 >> 15), (int)(wide(a, t) >> 29)) >> 25;  // u^3 t, 2^-64
     const int64_t l = __ldg(&kFixLog[j]) + ((u - h2 + c3) >> 1);              // ln m, 2^-63
     const int k = 63 + e;
-    if (k == 0 || k == -1) return fix_to_double(k ? l - 2 * kHalfLn2 : l, -63);
-    // k ln 2 in 2^-57
+    // k ln 2 + ln m in 2^-57, or in 2^-63 where k is 0 or -1
+    const bool fine = k == 0 || k == -1;
     const int64_t kl = (wide(k, (int)(kHalfLn2 >> 32)) << 27) + (wide(k, (int)((uint32_t)kHalfLn2 >> 1)) >> 4);
-    return fix_to_double(kl + (l >> 6), -57);
+    const int64_t v = fine ? (k ? l - 2 * kHalfLn2 : l) : kl + (l >> 6);
+    return fix_to_double(neg ? -v : v, fine ? -63 : -57);
 }
 
 // ---------------------------------------------------------------------------

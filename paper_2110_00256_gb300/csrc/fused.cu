@@ -40,7 +40,8 @@ __device__ __forceinline__ void store_live(T *p, int64_t i0, int64_t n, bool ful
 template <typename T, int VEC, int THREADS>
 __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     push_evolve_kernel(const EvolveSeg<T> *__restrict__ segs, const PushSeg<T> *__restrict__ psegs, int n_seg,
-                       const __grid_constant__ TablesView<T> tab, WaveParams w, double t0, double dt_d, const int64_t *d_step, int64_t step,
+                       const __grid_constant__ TablesView<T> tab, WaveT<T> wt, double t0, double dt_d,
+                       const int64_t *d_step, int64_t step,
                        T cut_qs, T cut_bw, long long *stats, int store_fields)
 {
     __shared__ RateSmem<T> rs;
@@ -49,10 +50,10 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     long long *s_end = s_dyn, *s_n = s_dyn + n_seg;
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
-    stage_rates(rs, tab, THREADS);
+    stage_rates(rs, tab, wt.dt, THREADS);
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);
-    const WaveT<T> wt = wave_at<T>(w, t0 + (double)(d_step ? *d_step : step) * dt_d);
-    const T dt = (T)dt_d;
+    wt.t = (T)(t0 + (double)(d_step ? *d_step : step) * dt_d);
+    const T dt = wt.dt;
     int bad = 0;
     int s = 0;
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {
@@ -136,7 +137,7 @@ static qed_status launch_fused_impl(const EvolveSeg<T> *segs, const PushSeg<T> *
         attr = true;
     }
     push_evolve_kernel<T, VEC, kThreads><<<sm_count() * per_sm, kThreads, dyn, st>>>(
-        segs, psegs, n_seg, tab, w, t0, dt, d_step, step, cut_qs, cut_bw, stats, store_fields);
+        segs, psegs, n_seg, tab, wave_in<T>(w, dt), t0, dt, d_step, step, cut_qs, cut_bw, stats, store_fields);
     QED_LAUNCH_CHECK();
     return QED_OK;
 }

@@ -326,13 +326,19 @@ __device__ __forceinline__ void store_tau<double>(double *tau, double *, int64_t
 // times 2^(e - 52), exact in FP64, rounded once by the integer-to-float
 // conversion and scaled exactly.  Elsewhere (0, tiny, huge, infinite, NaN) by
 // FP64 conversions, with the same results.
+static __device__ __noinline__ float2 split_f32_pair_fp64(double x)  // (out of line: never predicated into the others)
+{
+    const float h = __double2float_rn(x);
+    return make_float2(h, __double2float_rn((double)h - x));
+}
+
 __device__ __forceinline__ void split_f32_pair(double x, float &h, float &c)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int e = (int)((b >> 52) & 0x7ffu) - 1023;
     if (e < -74 || e > 126) {
-        h = __double2float_rn(x);
-        c = __double2float_rn((double)h - x);
+        const float2 p = split_f32_pair_fp64(x);
+        h = p.x, c = p.y;
         return;
     }
     const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;  // 53 significant bits
@@ -386,7 +392,7 @@ __device__ __forceinline__ double neg_log_u(double u)
     if (__double_as_longlong(u) > __double_as_longlong(1.0 - 0x1p-8)) return neg_log1p_series(u);
     const int hi = __double2hiint(u);
     const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(u);
-    return -fix_ln(m << 11, (hi >> 20) - 1023 - 63);
+    return fix_ln(m << 11, (hi >> 20) - 1023 - 63, true);
 }
 
 // tau = -ln U, U the 53-bit uniform of (seed, (id, step, purpose)), in FP64 (§3)

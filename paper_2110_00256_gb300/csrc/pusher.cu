@@ -42,7 +42,7 @@ __device__ __forceinline__ void push_one(const PushSeg<T> &g, int64_t i, const W
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) push_kernel(const PushSeg<T> *__restrict__ segs, int n_seg, WaveParams w,
+__global__ void __launch_bounds__(256) push_kernel(const PushSeg<T> *__restrict__ segs, int n_seg, WaveT<T> wt,
                                                     double t0, double dt, const int64_t *d_step, int64_t step)
 {
     extern __shared__ long long s_dyn[];  // [n_seg] inclusive prefix of particle counts
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) push_kernel(const PushSeg<T> *__restrict_
     }
     __syncthreads();
     const long long total = s_dyn[n_seg - 1];
-    const WaveT<T> wt = wave_at<T>(w, t0 + (double)(d_step ? *d_step : step) * dt);
+    wt.t = (T)(t0 + (double)(d_step ? *d_step : step) * dt);
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total;
          k += (long long)gridDim.x * blockDim.x) {
         int lo = 0, hi = n_seg - 1;
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(256) push_kernel(const PushSeg<T> *__restrict_
             else
                 lo = mid + 1;
         }
-        push_one<T>(segs[lo], k - (lo ? s_dyn[lo - 1] : 0), wt, (T)dt);
+        push_one<T>(segs[lo], k - (lo ? s_dyn[lo - 1] : 0), wt, wt.dt);
     }
 }
 
@@ -106,24 +106,22 @@ template PushSeg<double> push_seg<double>(const qed_species *, double);
 
 // one species, its descriptor as a kernel parameter
 template <typename T>
-__global__ void __launch_bounds__(256) push_single_kernel(const __grid_constant__ PushSeg<T> g, WaveParams w,
-                                                          double t, double dt)
+__global__ void __launch_bounds__(256) push_single_kernel(const __grid_constant__ PushSeg<T> g, const WaveT<T> wt)
 {
-    const WaveT<T> wt = wave_at<T>(w, t);
     int64_t n = *g.count;
     n = n < 0 ? 0 : (n > g.cap ? g.cap : n);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        push_one<T>(g, i, wt, (T)dt);
+        push_one<T>(g, i, wt, wt.dt);
 }
 
 // fields already stored in the species (uniform fields, or gathered by the caller)
 template <typename T>
-__global__ void __launch_bounds__(256) push_stored_kernel(const __grid_constant__ PushSeg<T> g, double dt)
+__global__ void __launch_bounds__(256) push_stored_kernel(const __grid_constant__ PushSeg<T> g, T dt)
 {
     int64_t n = *g.count;
     n = n < 0 ? 0 : (n > g.cap ? g.cap : n);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        advance<T>(g, i, g.x[i], g.ex[i], g.ey[i], g.ez[i], g.bx[i], g.by[i], g.bz[i], (T)dt);
+        advance<T>(g, i, g.x[i], g.ex[i], g.ey[i], g.ez[i], g.bx[i], g.by[i], g.bz[i], dt);
 }
 
 template <typename T>
@@ -139,7 +137,7 @@ qed_status launch_push(const void *d_segs, int n_seg, const WaveParams &w, doubl
         attr = true;
     }
     push_kernel<T><<<resident_grid<push_kernel<T>>(256, 3 * QED_MAX_PATCHES * sizeof(long long), capacity), 256, dyn,
-                     st>>>((const PushSeg<T> *)d_segs, n_seg, w, t0, dt, d_step, step);
+                     st>>>((const PushSeg<T> *)d_segs, n_seg, wave_in<T>(w, dt), t0, dt, d_step, step);
     QED_LAUNCH_CHECK();
     return QED_OK;
 }
@@ -179,10 +177,10 @@ extern "C" qed_status qed_push_plane_wave(const qed_species *sp, double charge, 
     cudaStream_t st = as_stream(stream);
     if (prec == QED_F32)
         push_single_kernel<float><<<resident_grid<push_single_kernel<float>>(256, 0, sp->capacity), 256, 0, st>>>(
-            push_seg<float>(sp, charge), wave_params(wave), t, dt);
+            push_seg<float>(sp, charge), wave_in<float>(wave_params(wave), dt, t));
     else
         push_single_kernel<double><<<resident_grid<push_single_kernel<double>>(256, 0, sp->capacity), 256, 0, st>>>(
-            push_seg<double>(sp, charge), wave_params(wave), t, dt);
+            push_seg<double>(sp, charge), wave_in<double>(wave_params(wave), dt, t));
     QED_LAUNCH_CHECK();
     return QED_OK;
 }
@@ -199,7 +197,7 @@ extern "C" qed_status qed_push_stored_fields(const qed_species *sp, double charg
     cudaStream_t st = as_stream(stream);
     if (prec == QED_F32)
         push_stored_kernel<float><<<resident_grid<push_stored_kernel<float>>(256, 0, sp->capacity), 256, 0, st>>>(
-            push_seg<float>(sp, charge), dt);
+            push_seg<float>(sp, charge), (float)dt);
     else
         push_stored_kernel<double><<<resident_grid<push_stored_kernel<double>>(256, 0, sp->capacity), 256, 0, st>>>(
             push_seg<double>(sp, charge), dt);

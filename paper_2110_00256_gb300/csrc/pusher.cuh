@@ -24,18 +24,21 @@ struct PushSeg {
 __device__ __forceinline__ void d_sincospi(float u, float *s, float *c) { sincospif(u, s, c); }
 __device__ __forceinline__ void d_sincospi(double u, double *s, double *c) { sincospi(u, s, c); }
 
-// the wave's parameters and the time in the working precision, converted once
-// per thread (conversions from FP64 run on GB300's narrow FP64 pipe)
+// The wave's parameters, the time and the time step in the working precision.
+// The host converts the parameters and the step: a kernel that takes them as
+// FP64 arguments converts them again at every use once registers are short (the
+// fused cascade kernel held GB300's narrow FP64 pipe 54 % busy with nothing but
+// those conversions).  The batched kernels set t from the step counter.
 template <typename T>
 struct WaveT {
-    T omega_pi, phase0_pi, e0, d, t;
+    T omega_pi, phase0_pi, e0, d, t, dt;
     int circular;
 };
 
 template <typename T>
-__device__ __forceinline__ WaveT<T> wave_at(const WaveParams &w, double t)
+inline WaveT<T> wave_in(const WaveParams &w, double dt, double t = 0.0)
 {
-    return WaveT<T>{(T)w.omega_pi, (T)w.phase0_pi, (T)w.e0, (T)w.direction, (T)t, w.circular};
+    return WaveT<T>{(T)w.omega_pi, (T)w.phase0_pi, (T)w.e0, (T)w.direction, (T)t, (T)dt, w.circular};
 }
 
 // phase phi = omega (t - d x) + phase0; E = E0 (0, cos phi, [sin phi]); B = d x-hat cross E.

@@ -164,9 +164,11 @@ typedef struct {
  * the default (8 consumer warps, 4 stages, 1 CTA per SM).  DIRECT in FP32
  * runs 4 CTAs of 256 threads per SM (64 registers), or 3 (80 registers) with
  * evolve_ctas_per_sm 3.  All give identical results.  DEFAULT (with
- * evolve_threads and evolve_ctas_per_sm 0) is a bulk-copy pipeline with 15
- * consumer warps and 2 stages in FP32 when the arrays are 16-byte aligned, the
- * fastest on GB300, and DIRECT otherwise. */
+ * evolve_threads and evolve_ctas_per_sm 0) goes by the particles (the sum of the
+ * capacities) per SM, as measured on GB300: one particle per thread up to 1024
+ * (1.6e5 particles), direct loads up to 49152 (7e6), and beyond a bulk-copy
+ * pipeline with 15 consumer warps and 2 stages in FP32 when the arrays are
+ * 16-byte aligned, DIRECT otherwise. */
 enum { QED_EVOLVE_DEFAULT = 0, QED_EVOLVE_DIRECT = 1, QED_EVOLVE_BULK = 2 };
 
 /* ------------------------------------------------------------------------- */
@@ -301,11 +303,12 @@ qed_status qed_generate_pairs(const qed_tables *t, const qed_species *photons,
                               const qed_fire_list *fire, uint64_t seed, int64_t step,
                               const qed_substep_opts *opts, qed_precision prec, void *stream);
 
-/* The whole substep on three species in four launches: zero the firing
+/* The whole substep on three species in three launches: zero the firing
  * counts; one evolution launch over electrons (QS), positrons (QS) and photons
  * (BW); one event launch for the three firing lists (photon emission of both
- * leptons and pair production side by side: they touch disjoint particles;
- * with the learned sampler, one launch per list); clamp the counts.  fire[0..2]
+ * leptons and pair production side by side: they touch disjoint particles),
+ * whose last CTA clamps the counts (with the learned sampler, one launch per list
+ * and one for the counts).  fire[0..2]
  * are the firing lists of the three species in that order.  Products are
  * appended after the live particles and are first evolved in the next call.
  * Graph-capturable. */
@@ -393,15 +396,16 @@ qed_status qed_batch_create(const qed_patch *patches, int32_t n_patches, qed_pre
                             qed_batch **out, void *stream);
 qed_status qed_batch_destroy(qed_batch *b);
 
-/* qed_substep for every patch of `b` (§3, §5), in four launches whatever the
- * number of patches: zero the firing counts (and add the live counts to
- * QED_STAT_EVOLVED); one persistent evolution launch over all 3 x n species
+/* qed_substep for every patch of `b` (§3, §5), in two launches whatever the
+ * number of patches: one persistent evolution launch over all 3 x n species
  * segments (tiles of every segment form one index space, so uneven patches
  * share the grid; FP32 with aligned arrays streams them through shared memory
- * by default); one event launch over all firing lists (photon emission of the
- * leptons and pair production of the photons side by side; with the learned
- * sampler, one launch per process); one launch clamping the counts (and
- * advancing opts->d_step).  Stream-ordered, allocates nothing,
+ * by default; it adds the live counts to QED_STAT_EVOLVED); one event launch over
+ * all firing lists (photon emission of the leptons and pair production of the
+ * photons side by side; with the learned sampler, one launch per process),
+ * which at its end clamps the counts and advances opts->d_step.  The firing
+ * counts are kept in `b` during the step and written to the lists' d_count at
+ * its end, so steps of one batch do not overlap.  Stream-ordered, allocates nothing,
  * graph-capturable.  Results per patch are those of qed_substep on that patch. */
 qed_status qed_substep_batched(const qed_tables *t, const qed_batch *b, double dt, uint64_t seed,
                                int64_t step, const qed_substep_opts *opts, void *stream);

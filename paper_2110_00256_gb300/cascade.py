@@ -3,8 +3,8 @@ counter-propagating a linearly polarised plane wave whose fields are evaluated
 analytically at each particle, the substep (photon emission, pair production)
 after every push, all steps captured in one CUDA graph with a device step
 counter.  By default the push is fused into the evolution
-(qed_push_substep_batched: one pass per particle, 4 launches per step);
-fused=False runs the separate push and substep (5 launches per step) with the
+(qed_push_substep_batched: one pass per particle, 2 launches per step);
+fused=False runs the separate push and substep (3 launches per step) with the
 evolution launch shape chosen by qed_tune_evolve.  Every 50 steps the photons
 that pair production removed are compacted out of the arrays.
 
@@ -120,7 +120,7 @@ def run(tables: api.Tables, steps: int = 2000, scale: float = 1.0, photon_factor
     # particle-steps: each step adds the live count of every species of every
     # patch, as the evolution reads it, to the 'evolved' counter
     particle_steps = s["evolved"]
-    per_step = 4 if fused else 5
+    per_step = 2 if fused else 3
     extra = (4 * len(patches) / compact_every) if compact_every else 0.0
     return {"patches": int(len(counts)), "electrons": int(counts.sum()), "steps": steps, "ms": ms,
             "particle_steps": particle_steps, "value": particle_steps / (ms * 1e-3), "n_start": n0, "n_end": n1,

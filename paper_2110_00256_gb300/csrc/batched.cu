@@ -1,9 +1,11 @@
 // batched.cu -- the substep over many patches (each with its own electrons,
-// positrons and photons of uneven size) in four launches per step, whatever
-// the number of patches: zero the firing counts, one evolution launch over all
-// 3 x n segments, one event launch over all firing lists (photon emission of
-// the leptons, pair production of the photons; with the learned sampler, one
-// launch per process), one clamp.  The segment
+// positrons and photons of uneven size) in two launches per step, whatever
+// the number of patches: one evolution launch over all 3 x n segments and one
+// event launch over all firing lists (photon emission of the leptons, pair
+// production of the photons; with the learned sampler, one launch per process),
+// whose last CTA writes the firing counts out, keeps the species counts within
+// their capacities and advances the step.  The firing counts are kept in the
+// batch meanwhile and left at zero for the next step.  The segment
 // descriptors live in device memory owned by a qed_batch (made once), so the
 // step allocates nothing and can be captured in a CUDA graph; with
 // opts->d_step a captured step replays as many steps.  qed_tune_evolve picks
@@ -37,54 +39,54 @@ struct qed_batch {
     void *d_evolve;    // EvolveSeg<T>[3 n]: electrons, positrons, photons of patch 0, 1, ...
     void *d_qs;        // EventSeg<T>[2 n]: electrons -> photons, positrons -> photons
     void *d_bw;        // EventSeg<T>[n]: photons -> electrons, positrons
-    int64_t **d_zero;  // [3 n] firing counts to zero
-    qed::ClampEntry *d_clamp;  // [6 n] species and firing counts to clamp
+    qed::ClampEntry *d_clamp;  // [6 n] per patch: the species' and the firing lists' counts and capacities
+    unsigned long long *d_count;  // [3 n] firing counts of the step in flight (zero between steps), then a ticket
     void *d_push;      // PushSeg<T>[3 n] when every species has positions, else NULL
     bool vec;
     bool push_vec;     // vec, and the positions 16-byte aligned too
     int64_t capacity_sum, fire_capacity_max;
-    int threads, ctas_per_sm;  // tuned evolution launch shape (0: default)
+    int threads, ctas_per_sm;  // tuned evolution launch shape (0: the bulk-copy kernel)
+    bool tuned;
 };
 
 namespace qed {
 
-// one CTA of 256: zero the n firing counts; with stats, add the live counts of
-// the species (the first three of every six clamp entries), clamped as the
-// evolution clamps them, to QED_STAT_EVOLVED: the particles this step evolves,
-// less the photons removed by pair production that are still in the arrays
-// (QED_STAT_PAIRS - QED_STAT_COMPACTED: they are read, but not evolved)
-__global__ void __launch_bounds__(256) zero_counts_kernel(int64_t *const *p, int n, const ClampEntry *e,
-                                                          int n_patches, long long *stats)
+// What ends a step, done by the last CTA of its last event launch (a launch of
+// its own took 3.5 us, as did zeroing the counts before the step): the firing
+// counts, clamped, to the caller's lists, the batch's own back to zero, the
+// species counts within their capacities (the reservations overshoot), the step
+// counter advanced.
+struct StepEnd {
+    const ClampEntry *entries;  // [6 n]
+    unsigned long long *count;  // [3 n], then the ticket; NULL: another event launch follows
+    int n_patches;
+    int64_t *step;
+};
+
+__device__ __forceinline__ void end_step(const StepEnd &f)
 {
-    __shared__ long long s_sum[8];
-    for (int i = threadIdx.x; i < n; i += blockDim.x) *p[i] = 0;
-    if (!stats) return;
-    long long live = 0;
-    for (int i = threadIdx.x; i < 3 * n_patches; i += blockDim.x) {
-        const ClampEntry &c = e[6 * (i / 3) + i % 3];
-        const long long v = (long long)*c.count;  // as the evolution reads it
-        live += v < 0 ? 0 : (v > c.cap ? c.cap : v);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) live += __shfl_xor_sync(0xffffffffu, live, o);
-    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = live;
+    __shared__ bool s_last;
+    if (!f.count) return;
+    const int n = 3 * f.n_patches;
     __syncthreads();
     if (threadIdx.x == 0) {
-        long long t = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s_sum[w];
-        long long removed = stats[QED_STAT_PAIRS] - stats[QED_STAT_COMPACTED];
-        removed = removed < 0 ? 0 : (removed > t ? t : removed);
-        atomicAdd((unsigned long long *)(stats + QED_STAT_EVOLVED), (unsigned long long)(t - removed));
+        __threadfence();
+        s_last = atomicAdd(f.count + n, 1ull) == gridDim.x - 1;
     }
-}
-
-__global__ void clamp_batch_kernel(const ClampEntry *e, int n, int64_t *step)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        unsigned long long *c = e[i].count;
-        if (*c > (unsigned long long)e[i].cap) *c = e[i].cap;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const ClampEntry sp = f.entries[6 * (i / 3) + i % 3], fi = f.entries[6 * (i / 3) + 3 + i % 3];
+        if (__ldcg(sp.count) > (unsigned long long)sp.cap) *sp.count = sp.cap;
+        const unsigned long long v = __ldcg(f.count + i);
+        *fi.count = v > (unsigned long long)fi.cap ? fi.cap : v;
+        f.count[i] = 0;
     }
-    if (step && blockIdx.x == 0 && threadIdx.x == 0) *step += 1;
+    if (threadIdx.x == 0) {
+        f.count[n] = 0;
+        if (f.step) *f.step += 1;
+    }
 }
 
 // Block-wide prefix of the 32-entry chunk counts of n_seg firing lists into
@@ -137,7 +139,8 @@ __device__ __forceinline__ int find_seg(const long long *s_end, int n_seg, long 
 // dynamic shared memory: [InferSmem if MLP][s_end n][s_n n]
 template <typename T, bool MLP, bool QS>
 __global__ void __launch_bounds__(256, (MLP || sizeof(T) == 8) ? 1 : 4)
-    event_batched_kernel(const EventSeg<T> *__restrict__ segs, int n_seg, const __grid_constant__ EventCommon<T> c)
+    event_batched_kernel(const EventSeg<T> *__restrict__ segs, int n_seg, const __grid_constant__ EventCommon<T> c,
+                         const StepEnd end)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long s_warp[8];
@@ -160,6 +163,7 @@ __global__ void __launch_bounds__(256, (MLP || sizeof(T) == 8) ? 1 : 4)
             bw_event_chunk<T, MLP>(segs[s], c, step, base, s_n[s], S, k);
     }
     flush_counts(c.stats, k, QS);
+    end_step(end);
 }
 
 // Both processes in one launch (table sampler): the photon emission of every
@@ -170,7 +174,7 @@ template <typename T>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 4)
     event_batched_all_kernel(const EventSeg<T> *__restrict__ qs, int n_qs, const EventSeg<T> *__restrict__ bw,
                              int n_bw, const __grid_constant__ EventCommon<T> cq,
-                             const __grid_constant__ EventCommon<T> cb)
+                             const __grid_constant__ EventCommon<T> cb, const StepEnd end)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long s_warp[8];
@@ -194,6 +198,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 4)
     }
     flush_counts(cq.stats, kq, true);
     flush_counts(cb.stats, kb, false);
+    end_step(end);
 }
 
 // ---------------------------------------------------------------------------
@@ -364,6 +369,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1)
                               sg.proc == QED_PROC_QS ? cut_qs : cut_bw, stats, dry, bad);
     }
     if (!dry) warp_count_err(stats ? stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
+    if (stats && !dry && blockIdx.x == 0 && warp == 0) count_evolved(s_n, n_seg, stats);
 }
 
 // 15 consumer warps + the producer (16 warps, one CTA per SM), 2 stages, as the single-call default
@@ -397,7 +403,8 @@ static int resident_grid(int64_t warps, int per_sm)
 }
 
 template <typename T, bool QS>
-static qed_status launch_events_batched(const qed_batch *b, const EventCommon<T> &c, bool mlp, cudaStream_t st)
+static qed_status launch_events_batched(const qed_batch *b, const EventCommon<T> &c, const StepEnd &end, bool mlp,
+                                        cudaStream_t st)
 {
     const int n_seg = QS ? 2 * b->n_patches : b->n_patches;
     const EventSeg<T> *segs = (const EventSeg<T> *)(QS ? b->d_qs : b->d_bw);
@@ -415,7 +422,7 @@ static qed_status launch_events_batched(const qed_batch *b, const EventCommon<T>
             QED_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, kMaxDyn));
             attr = true;
         }
-        k<<<resident_grid(warps, per_sm), 256, dyn, st>>>(segs, n_seg, c);
+        k<<<resident_grid(warps, per_sm), 256, dyn, st>>>(segs, n_seg, c, end);
     } else {
         auto k = event_batched_kernel<T, false, QS>;
         static bool attr = false;
@@ -426,7 +433,7 @@ static qed_status launch_events_batched(const qed_batch *b, const EventCommon<T>
                                                                                       (int)sizeof(long long)));
             attr = true;
         }
-        k<<<resident_grid(warps, per_sm), 256, dyn, st>>>(segs, n_seg, c);
+        k<<<resident_grid(warps, per_sm), 256, dyn, st>>>(segs, n_seg, c, end);
     }
     QED_LAUNCH_CHECK();
     return QED_OK;
@@ -434,7 +441,7 @@ static qed_status launch_events_batched(const qed_batch *b, const EventCommon<T>
 
 template <typename T>
 static qed_status launch_events_batched_all(const qed_batch *b, const EventCommon<T> &cq, const EventCommon<T> &cb,
-                                           cudaStream_t st)
+                                           const StepEnd &end, cudaStream_t st)
 {
     const int n_qs = 2 * b->n_patches, n_bw = b->n_patches;
     const size_t dyn = (size_t)(n_qs + n_bw) * 2 * sizeof(long long);
@@ -449,7 +456,7 @@ static qed_status launch_events_batched_all(const qed_batch *b, const EventCommo
         attr = true;
     }
     k<<<resident_grid(warps, per_sm), 256, dyn, st>>>((const EventSeg<T> *)b->d_qs, n_qs,
-                                                      (const EventSeg<T> *)b->d_bw, n_bw, cq, cb);
+                                                      (const EventSeg<T> *)b->d_bw, n_bw, cq, cb, end);
     QED_LAUNCH_CHECK();
     return QED_OK;
 }
@@ -459,8 +466,10 @@ static qed_status build_batch(const qed_patch *patches, int n, qed_batch *b, cud
 {
     std::vector<EvolveSeg<T>> ev(3 * (size_t)n);
     std::vector<EventSeg<T>> qs(2 * (size_t)n), bw((size_t)n);
-    std::vector<int64_t *> zero(3 * (size_t)n);
     std::vector<ClampEntry> clamp(6 * (size_t)n);
+    const size_t count_bytes = (3 * (size_t)n + 1) * sizeof(unsigned long long);
+    QED_CUDA_TRY(cudaMalloc((void **)&b->d_count, count_bytes));
+    QED_CUDA_TRY(cudaMemsetAsync(b->d_count, 0, count_bytes, st));
     bool vec = true;
     int64_t capsum = 0, fmax = 0;
     for (int i = 0; i < n; ++i) {
@@ -469,7 +478,7 @@ static qed_status build_batch(const qed_patch *patches, int n, qed_batch *b, cud
         const int proc[3] = {QED_PROC_QS, QED_PROC_QS, QED_PROC_BW};
         for (int k = 0; k < 3; ++k) {
             vec = fill_seg<T>(ev[3 * i + k], sp[k], proc[k], &p.fire[k]) && vec;
-            zero[3 * i + k] = p.fire[k].d_count;
+            ev[3 * i + k].fire_count = b->d_count + 3 * i + k;
             clamp[6 * i + k] = ClampEntry{(unsigned long long *)sp[k]->d_count, sp[k]->capacity};
             clamp[6 * i + 3 + k] = ClampEntry{(unsigned long long *)p.fire[k].d_count, p.fire[k].capacity};
             capsum += sp[k]->capacity;
@@ -480,7 +489,8 @@ static qed_status build_batch(const qed_patch *patches, int n, qed_batch *b, cud
             memset(&g, 0, sizeof(g));
             g.parent = ptrs<T>(sp[k]);
             g.out0 = ptrs<T>(&p.photons);
-            g.fire_idx = p.fire[k].idx, g.fire_chi = p.fire[k].chi, g.fire_count = p.fire[k].d_count;
+            g.fire_idx = p.fire[k].idx, g.fire_chi = p.fire[k].chi;
+            g.fire_count = (const int64_t *)b->d_count + 3 * i + k;
             g.fire_cap = p.fire[k].capacity;
         }
         EventSeg<T> &g = bw[i];
@@ -488,7 +498,8 @@ static qed_status build_batch(const qed_patch *patches, int n, qed_batch *b, cud
         g.parent = ptrs<T>(&p.photons);
         g.out0 = ptrs<T>(&p.electrons);
         g.out1 = ptrs<T>(&p.positrons);
-        g.fire_idx = p.fire[2].idx, g.fire_chi = p.fire[2].chi, g.fire_count = p.fire[2].d_count;
+        g.fire_idx = p.fire[2].idx, g.fire_chi = p.fire[2].chi;
+        g.fire_count = (const int64_t *)b->d_count + 3 * i + 2;
         g.fire_cap = p.fire[2].capacity;
     }
     bool positions = true, pos_al16 = true;
@@ -512,10 +523,9 @@ static qed_status build_batch(const qed_patch *patches, int n, qed_batch *b, cud
         void **dst;
         const void *src;
         size_t bytes;
-    } ups[5] = {{&b->d_evolve, ev.data(), ev.size() * sizeof(EvolveSeg<T>)},
+    } ups[4] = {{&b->d_evolve, ev.data(), ev.size() * sizeof(EvolveSeg<T>)},
                 {&b->d_qs, qs.data(), qs.size() * sizeof(EventSeg<T>)},
                 {&b->d_bw, bw.data(), bw.size() * sizeof(EventSeg<T>)},
-                {(void **)&b->d_zero, zero.data(), zero.size() * sizeof(int64_t *)},
                 {(void **)&b->d_clamp, clamp.data(), clamp.size() * sizeof(ClampEntry)}};
     for (const Up &u : ups) {
         QED_CUDA_TRY(cudaMalloc(u.dst, u.bytes));
@@ -538,14 +548,19 @@ static qed_status substep_batched_impl(const qed_tables *t, const qed_batch *b, 
 {
     const int n = b->n_patches;
     long long *stats = o ? (long long *)o->d_stats : nullptr;
-    zero_counts_kernel<<<1, 256, 0, st>>>(b->d_zero, 3 * n, b->d_clamp, n, stats);
-    QED_LAUNCH_CHECK();
     const int threads = (o && o->evolve_threads) ? o->evolve_threads : (b->threads ? b->threads : 256);
     const int ctas = (o && o->evolve_ctas_per_sm) ? o->evolve_ctas_per_sm : b->ctas_per_sm;
     // the default shape (nothing asked for, nothing tuned) of an FP32 batch with
-    // aligned arrays: the bulk-copy kernel
+    // aligned arrays: the bulk-copy kernel for many particles (kDirectPerSm; the
+    // block of 2e6: 29.5 us a step with it, 26.6 with direct loads); few
+    // particles one per thread (kSmallPerSm)
+    const bool open = !(o && (o->evolve_threads || o->evolve_ctas_per_sm)) && !b->tuned &&
+                      !(o && o->wait_limit_cycles);
+    const int64_t per_sm = b->capacity_sum / sm_count();
+    const bool small = open && !(o && o->evolve_pipeline != QED_EVOLVE_DEFAULT) && per_sm < kSmallPerSm;
+    const bool few = open && !(o && o->evolve_pipeline == QED_EVOLVE_BULK) && per_sm < kDirectPerSm;
     const bool bulk = sizeof(T) == 4 && b->vec && !(o && (o->evolve_threads || o->evolve_ctas_per_sm)) &&
-                      !(o && o->evolve_pipeline == QED_EVOLVE_DIRECT) && b->threads == 0 && b->ctas_per_sm == 0;
+                      !(o && o->evolve_pipeline == QED_EVOLVE_DIRECT) && b->threads == 0 && b->ctas_per_sm == 0 && !few;
     if (o && o->evolve_begin) QED_CUDA_TRY(cudaEventRecord((cudaEvent_t)o->evolve_begin, st));
     const T cut_qs = o ? (T)o->qs_chi_cut : T(0), cut_bw = o ? (T)o->bw_chi_cut : T(0);
     qed_status s;
@@ -557,35 +572,36 @@ static qed_status substep_batched_impl(const qed_tables *t, const qed_batch *b, 
         s = bulk ? launch_evolve_seg_bulk((const EvolveSeg<float> *)b->d_evolve, 3 * n, make_view<float>(t),
                                           (float)dt, cut_qs, cut_bw, stats, 0, o ? o->wait_limit_cycles : 0, st)
                  : launch_evolve_segments<T>((const EvolveSeg<T> *)b->d_evolve, 3 * n, make_view<T>(t), (T)dt,
-                                             cut_qs, cut_bw, stats, 0, b->vec, threads, ctas, st);
+                                             cut_qs, cut_bw, stats, 0, b->vec && !small, small ? 128 : threads,
+                                             ctas, st);
     } else {
         s = launch_evolve_segments<T>((const EvolveSeg<T> *)b->d_evolve, 3 * n, make_view<T>(t), (T)dt, cut_qs,
-                                      cut_bw, stats, 0, b->vec, threads, ctas, st);
+                                      cut_bw, stats, 0, b->vec && !small, small ? 128 : threads, ctas, st);
     }
     if (s) return s;
     if (o && o->evolve_end) QED_CUDA_TRY(cudaEventRecord((cudaEvent_t)o->evolve_end, st));
     const bool mlp = o && o->sampler == 1;
+    const StepEnd end{b->d_clamp, b->d_count, n, o ? o->d_step : nullptr};
     if (mlp) {
-        if ((s = launch_events_batched<T, false>(b, event_common<T>(t, QED_PROC_BW, seed, step, o), true, st)))
-            return s;
-        if ((s = launch_events_batched<T, true>(b, event_common<T>(t, QED_PROC_QS, seed, step, o), true, st)))
-            return s;
+        s = launch_events_batched<T, false>(b, event_common<T>(t, QED_PROC_BW, seed, step, o), StepEnd{}, true, st);
+        if (s == QED_OK)
+            s = launch_events_batched<T, true>(b, event_common<T>(t, QED_PROC_QS, seed, step, o), end, true, st);
     } else {
         // the push fused into the evolution without stored fields computes every
         // particle's fields itself: the photons emitted get none
         EventCommon<T> cq = event_common<T>(t, QED_PROC_QS, seed, step, o);
         cq.copy_fields = (wave && !store_fields) ? 0 : 1;
-        if ((s = launch_events_batched_all<T>(b, cq, event_common<T>(t, QED_PROC_BW, seed, step, o), st))) return s;
+        s = launch_events_batched_all<T>(b, cq, event_common<T>(t, QED_PROC_BW, seed, step, o), end, st);
     }
-    clamp_batch_kernel<<<(6 * n + 255) / 256, 256, 0, st>>>(b->d_clamp, 6 * n, o ? o->d_step : nullptr);
-    QED_LAUNCH_CHECK();
-    return QED_OK;
+    // (a step that was not ended leaves its firing counts behind)
+    if (s) cudaMemsetAsync(b->d_count, 0, (3 * (size_t)n + 1) * sizeof(unsigned long long), st);
+    return s;
 }
 
 static void free_batch(qed_batch *b)
 {
     if (!b) return;
-    void *p[] = {b->d_evolve, b->d_qs, b->d_bw, b->d_zero, b->d_clamp, b->d_push};
+    void *p[] = {b->d_evolve, b->d_qs, b->d_bw, b->d_count, b->d_clamp, b->d_push};
     for (void *x : p)
         if (x) cudaFree(x);
     delete b;
@@ -727,6 +743,7 @@ extern "C" qed_status qed_tune_evolve(const qed_tables *t, qed_batch *b, int32_t
     if (s) return s;
     b->threads = bt;
     b->ctas_per_sm = bc;
+    b->tuned = true;
     if (threads_out) *threads_out = bt;
     if (ctas_per_sm_out) *ctas_per_sm_out = bc;
     if (ms_out) *ms_out = best;

@@ -60,11 +60,24 @@ __global__ void __launch_bounds__(256, (MLP || sizeof(T) == 8) ? 1 : 4) bw_event
 // parents below the pre-step counts and appends to another species), so their
 // chunks of 32 entries run side by side; the chunk index runs over the three
 // lists one after the other.
+// The last CTA to finish keeps the device counts within their capacities (the
+// reservations overshoot) and advances the step counter, which saves a launch:
+// the CTAs take tickets in the top 16 bits of the first list's count, which the
+// substep zeroes, and which nobody else reads before the launch has ended.
 template <typename T>
 struct Events3Args {
     EventSeg<T> seg[3];  // electrons -> photons, positrons -> photons, photons -> pairs
     EventCommon<T> qs, bw;
+    int64_t *step;       // the device step counter, or NULL
 };
+
+constexpr int kTicketShift = 48;
+constexpr unsigned long long kCountMask = (1ull << kTicketShift) - 1;
+
+__device__ __forceinline__ void clamp1(unsigned long long *c, int64_t cap)
+{
+    if (c && *c > (unsigned long long)cap) *c = cap;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(256) events3_kernel(const __grid_constant__ Events3Args<T> a)
@@ -73,7 +86,10 @@ __global__ void __launch_bounds__(256) events3_kernel(const __grid_constant__ Ev
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);  // (not touched without the learned sampler)
     int64_t nf[3], c1, c2, c3;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) nf[k] = fire_n(a.seg[k].fire_count, a.seg[k].fire_cap);
+    for (int k = 0; k < 3; ++k) {
+        nf[k] = (int64_t)((unsigned long long)*a.seg[k].fire_count & kCountMask);
+        nf[k] = nf[k] > a.seg[k].fire_cap ? a.seg[k].fire_cap : nf[k];
+    }
     c1 = (nf[0] + 31) / 32;
     c2 = c1 + (nf[1] + 31) / 32;
     c3 = c2 + (nf[2] + 31) / 32;
@@ -91,16 +107,26 @@ __global__ void __launch_bounds__(256) events3_kernel(const __grid_constant__ Ev
     }
     flush_counts(a.qs.stats, kq, true);
     flush_counts(a.bw.stats, kb, false);
+    __syncthreads();
+    if (threadIdx.x) return;
+    __threadfence();
+    unsigned long long *first = (unsigned long long *)a.seg[0].fire_count;
+    if (atomicAdd(first, 1ull << kTicketShift) >> kTicketShift != gridDim.x - 1) return;
+    __threadfence();
+    const int64_t cap[3] = {a.seg[0].parent.cap, a.seg[1].parent.cap, a.seg[2].parent.cap};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        unsigned long long *sp = a.seg[k].parent.count, *fi = (unsigned long long *)a.seg[k].fire_count;
+        if (__ldcg(sp) > (unsigned long long)cap[k]) *sp = cap[k];
+        const unsigned long long n = __ldcg(fi) & kCountMask;
+        *fi = n > (unsigned long long)a.seg[k].fire_cap ? a.seg[k].fire_cap : n;
+    }
+    if (a.step) *a.step += 1;
 }
 
 __global__ void zero3(int64_t *a, int64_t *b, int64_t *c)
 {
     if (threadIdx.x == 0) *a = 0, *b = 0, *c = 0;
-}
-
-__device__ __forceinline__ void clamp1(unsigned long long *c, int64_t cap)
-{
-    if (c && *c > (unsigned long long)cap) *c = cap;
 }
 
 // keep the device counts within their capacities after the reservations of the
@@ -296,9 +322,11 @@ static qed_status substep_impl(const qed_tables *t, const qed_species *e, const 
         ea.seg[2].out1 = ptrs<T>(p);
         ea.qs = event_common<T>(t, QED_PROC_QS, seed, step, o);
         ea.bw = event_common<T>(t, QED_PROC_BW, seed, step, o);
+        ea.step = o ? o->d_step : nullptr;
         const int g3 = event_grid<events3_kernel<T>>(0, fire[0].capacity + fire[1].capacity + fire[2].capacity);
         events3_kernel<T><<<g3, 256, 0, st>>>(ea);
         QED_LAUNCH_CHECK();
+        return QED_OK;
     }
     clamp_all<<<1, 32, 0, st>>>(ptrs<T>(e).count, e->capacity, ptrs<T>(p).count, p->capacity, ptrs<T>(g).count,
                                 g->capacity, (unsigned long long *)fire[0].d_count, fire[0].capacity,

@@ -66,14 +66,14 @@ __device__ __forceinline__ const T *seg_array(const EvolveSeg<T> &g, int k)
 }
 
 // segments as kernel parameters (a few species); MINB resident CTAs per SM
-template <typename T, int VEC, int MAXSEG, int MINB = 3>
-__global__ void __launch_bounds__(kEvolveThreads, MINB)
+template <typename T, int VEC, int MAXSEG, int MINB = 3, int THREADS = kEvolveThreads>
+__global__ void __launch_bounds__(THREADS, MINB)
     evolve_kernel(const __grid_constant__ EvolveArgs<T, MAXSEG> a)
 {
     __shared__ RateSmem<T> rs;
     __shared__ long long s_end[MAXSEG];  // inclusive prefix of tile counts
     __shared__ long long s_n[MAXSEG];
-    constexpr int64_t tile = kEvolveTile<T, VEC>;
+    constexpr int64_t tile = (int64_t)THREADS * VEC;
 
     stage_rates(rs, a.tab, a.dt, blockDim.x);
     if (threadIdx.x == 0) {
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kEvolveThreads, MINB)
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {
         int s = 0;
         while (t >= s_end[s]) ++s;
-        evolve_tile<T, VEC, kEvolveThreads>(a.seg[s], s_n[s], t - (s ? s_end[s - 1] : 0), rs, a.tab, a.dt,
+        evolve_tile<T, VEC, THREADS>(a.seg[s], s_n[s], t - (s ? s_end[s - 1] : 0), rs, a.tab, a.dt,
                                             a.chi_cut[a.seg[s].proc], a.stats, 0, bad);
     }
     warp_count_err(a.stats ? a.stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
@@ -313,6 +313,7 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS)
                                      sg.proc == QED_PROC_QS ? cut_qs : cut_bw, stats, dry, bad);
     }
     if (!dry) warp_count_err(stats ? stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
+    if (stats && !dry && blockIdx.x == 0 && threadIdx.x < 32) count_evolved(s_n, n_seg, stats);
 }
 
 template <typename T, int THREADS>
@@ -393,16 +394,17 @@ int sm_count()
     return g_sm_count;
 }
 
-template <typename T, int VEC, int MAXSEG, int MINB = 3>
+template <typename T, int VEC, int MAXSEG, int MINB = 3, int THREADS = kEvolveThreads>
 static int evolve_grid(int64_t total_particles)
 {
     static int blocks_per_sm = 0;
     if (blocks_per_sm == 0) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, evolve_kernel<T, VEC, MAXSEG, MINB>,
-                                                      kEvolveThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, evolve_kernel<T, VEC, MAXSEG, MINB, THREADS>,
+                                                      THREADS, 0);
         if (blocks_per_sm <= 0) blocks_per_sm = 1;
     }
-    const int64_t tiles = (total_particles + kEvolveTile<T, VEC> - 1) / kEvolveTile<T, VEC>;
+    constexpr int64_t tile = (int64_t)THREADS * VEC;
+    const int64_t tiles = (total_particles + tile - 1) / tile;
     int64_t g = (int64_t)sm_count() * blocks_per_sm;
     if (tiles < g) g = tiles < 1 ? 1 : tiles;
     return (int)g;
@@ -414,12 +416,21 @@ qed_status launch_evolve(const EvolveArgs<T, MAXSEG> &a, bool vec_ok, int64_t ca
 {
     // the grid is sized from the capacities (counts live on the device); idle
     // CTAs exit after reading the counts
+    if (pipeline == QED_EVOLVE_DEFAULT && threads == 0 && ctas_per_sm == 0 && grid_override <= 0 &&
+        a.wait_cycles == 0 && capacity_sum <= (int64_t)sm_count() * kSmallPerSm) {
+        // few particles: one per thread in CTAs of 64 (kSmallPerSm)
+        const int g = evolve_grid<T, 1, MAXSEG, 8, 64>(capacity_sum);
+        evolve_kernel<T, 1, MAXSEG, 8, 64><<<g, 64, 0, st>>>(a);
+        QED_LAUNCH_CHECK();
+        return QED_OK;
+    }
     if constexpr (sizeof(T) == 4) {
-        // the default: bulk copies, 15 consumer warps + the producer (16 warps, 4 per
+        // the default for many particles: bulk copies, 15 consumer warps + the producer (16 warps, 4 per
         // scheduler), 2 stages of 1920-particle tiles: the fastest of 7 .. 18 consumer
         // warps and 2 .. 4 stages measured on GB300
         const bool dflt = pipeline == QED_EVOLVE_DEFAULT && threads == 0 && ctas_per_sm == 0;
-        if (vec_ok && (pipeline == QED_EVOLVE_BULK || dflt) && grid_override <= 0) {
+        const bool few = dflt && a.wait_cycles == 0 && capacity_sum <= (int64_t)sm_count() * kDirectPerSm;
+        if (vec_ok && (pipeline == QED_EVOLVE_BULK || (dflt && !few)) && grid_override <= 0) {
             if (dflt) return launch_bulk<15, 2, 1, MAXSEG>(a, capacity_sum, st);
             if (threads == 512) return launch_bulk<16, 2, 1, MAXSEG>(a, capacity_sum, st);
             if (ctas_per_sm == 2) return launch_bulk<8, 2, 2, MAXSEG>(a, capacity_sum, st);

@@ -9,8 +9,16 @@
 namespace qed {
 
 constexpr int kEvolveThreads = 256;
-template <typename T, int VEC>
-constexpr int64_t kEvolveTile = (int64_t)kEvolveThreads * VEC;
+// The evolution's form by the particles (capacities) per SM, where nothing else
+// is asked for.  Measured on GB300 (152 SMs), us per FP32 substep in a graph:
+//   particles                  1.2e5   4e5   1.6e6   6.4e6   1.28e7
+//   one per thread, CTAs of 64   9.4  12.5    25.6    71       151
+//   direct loads, 4 per thread  11.1  12.7    22.4    53.2     120
+//   bulk copies                 13.8  15.2    24.8    58.4     112
+// and per FP64 substep, one per thread / two per thread: 13.7 / 16.0 (1e4),
+// 18.4 / 18.9 (1.2e5), 28.8 / 28.1 (4e5).  Few particles want a short chain per
+// thread and all SMs; the bulk pipeline pays from several tiles per CTA on.
+constexpr int64_t kSmallPerSm = 1024, kDirectPerSm = 49152;
 
 template <typename T>
 struct EvolveSeg {

@@ -339,6 +339,25 @@ __device__ __forceinline__ long long tile_prefix(const EvolveSeg<T> *__restrict_
     return n_seg ? s_end[n_seg - 1] : 0;
 }
 
+// The batched step's particle count: one warp adds the live counts s_n of all
+// segments, as the evolution reads them, to QED_STAT_EVOLVED, less the photons
+// removed by pair production that are still in the arrays (QED_STAT_PAIRS -
+// QED_STAT_COMPACTED: they are read, but not evolved).  After a
+// kernel's loop, which it then costs no registers (before it, the cascade kernel
+// spilled and lost 5 %), and before the step's events.
+__device__ __forceinline__ void count_evolved(const long long *s_n, int n_seg, long long *stats)
+{
+    long long live = 0;
+    for (int i = threadIdx.x & 31; i < n_seg; i += 32) live += s_n[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) live += __shfl_xor_sync(0xffffffffu, live, o);
+    if ((threadIdx.x & 31) == 0) {
+        long long removed = stats[QED_STAT_PAIRS] - stats[QED_STAT_COMPACTED];
+        removed = removed < 0 ? 0 : (removed > live ? live : removed);
+        atomicAdd((unsigned long long *)(stats + QED_STAT_EVOLVED), (unsigned long long)(live - removed));
+    }
+}
+
 // the segment of tile t: the first s with s_end[s] > t
 __device__ __forceinline__ int find_segment(const long long *s_end, int n_seg, long long t)
 {

@@ -115,6 +115,7 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
         compact_fire<T, VEC>(sg, i0, fire, chi, cnt, stats);
     }
     warp_count_err(stats ? stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
+    if (stats && blockIdx.x == 0 && threadIdx.x < 32) count_evolved(s_n, n_seg, stats);
 }
 
 template <typename T, int VEC>

@@ -376,3 +376,38 @@ def test_full_size_batched_workload_sampled(api, tabs):
         assert np.all(np.abs(post_tau[quiet] - tau_new[quiet]) <= bound[quiet]), (i, k)
         fired_total += int(f.sum())
     assert fired_total > 0
+
+
+@pytest.mark.parametrize("prec_name", ["f32", "f64"])
+@pytest.mark.parametrize("per_sm", [1024, 49152])
+@pytest.mark.parametrize("more", [0, 1])
+def test_evolution_forms_at_the_lines_of_the_default(api, tables, prec_name, per_sm, more):
+    """The default evolution on either side of the particle counts where its form changes gives the bits of direct loads."""
+    _, t = tables
+    prec = api.QED_F64 if prec_name == "f64" else api.QED_F32
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    caps = sms * per_sm + more
+    if caps > 10 ** 6 and prec_name == "f64":
+        pytest.skip("one form on both sides")
+    from paper_2110_00256_gb300 import workloads
+    n = caps // 2
+    live = [n - n // 50, caps - n - 4096 - n // 50]  # (room for every product)
+    runs = []
+    for pipeline in (api.QED_EVOLVE_DEFAULT, api.QED_EVOLVE_DIRECT):
+        e, g = api.SpeciesBuffers(n, prec), api.SpeciesBuffers(caps - n - 4096, prec)
+        p = api.SpeciesBuffers(4096, prec)
+        for sp, m, first in ((e, live[0], 0), (g, live[1], 10 ** 12)):
+            sp.set(workloads.paper_benchmark_torch(m, 5 + first % 7, first, dtype=torch.float64))
+        fire = [api.FireBuffers(s.capacity) for s in (e, p, g)]
+        d = torch.zeros(1, dtype=torch.int64, device="cuda")
+        st = api.Stats()
+        call = api.SubstepCall(t, e, p, g, fire, 10.0, 3, stats=st, pipeline=pipeline)
+        call.opts.d_step = d.data_ptr()
+        call(0)
+        torch.cuda.synchronize()
+        assert d.item() == 1 and st.as_dict()["dropped_capacity"] == 0
+        runs.append(([f.n() for f in fire], st.as_dict(), e["tau"][:live[0]].clone(), g["tau"][:live[1]].clone(),
+                     e["px"][:live[0]].clone()))
+    assert runs[0][:2] == runs[1][:2] and runs[0][0][0] > 0
+    for a, b in zip(runs[0][2:], runs[1][2:]):
+        assert torch.equal(a, b)

@@ -132,18 +132,13 @@ __device__ __forceinline__ void qs_event_chunk(const EventSeg<T> &g, const Event
     }
 
     const T p2 = px * px + py * py + pz * pz;
-    T inv;  // 1/|p|
-    if constexpr (sizeof(T) == 8) {
-        inv = p2 > T(0) ? rsqrt(p2) : T(0);  // (within 1 ulp; no FP64 division)
-    } else {
-        const T pm = d_sqrt(p2);
-        inv = pm > T(0) ? T(1) / pm : T(0);
-    }
-    const T gamma = d_sqrt(T(1) + p2);
+    T pm, inv;  // |p|, 1/|p|
+    e_norm(p2, pm, inv);
+    const T gamma = e_sqrt(T(1) + p2);
     const T gg = (gamma - T(1)) * xi;  // photon energy (§2.2)
     const T g1 = gamma - gg;            // lepton energy after emission
     const T q = (g1 - T(1)) * (g1 + T(1));
-    const T pn = d_sqrt(q > T(0) ? q : T(0));
+    const T pn = e_sqrt(q > T(0) ? q : T(0));
     const T nx = px * inv, ny = py * inv, nz = pz * inv;
 
     // (the FP32 test against the float threshold decides as the FP64 one does,
@@ -204,16 +199,17 @@ __device__ __forceinline__ void bw_event_chunk(const EventSeg<T> &g, const Event
     }
 
     const T p2 = px * px + py * py + pz * pz;
-    const T gg = d_sqrt(p2);  // photon energy (IEEE: it decides whether a pair is made, as in the oracle)
-    T inv;
-    if constexpr (sizeof(T) == 8)
-        inv = p2 > T(0) ? rsqrt(p2) : T(0);  // (within 1 ulp; no FP64 division)
-    else
-        inv = gg > T(0) ? T(1) / gg : T(0);
+    T gg, inv;  // photon energy, 1/|p|
+    e_norm(p2, gg, inv);
+    // (the IEEE root where it decides whether a pair is made, as in the oracle)
+    if constexpr (sizeof(T) == 8) {
+        const long long lo = __double_as_longlong(2.0 - 1e-9), hi = __double_as_longlong(2.0 + 1e-9);
+        if (__double_as_longlong(gg) > lo && __double_as_longlong(gg) < hi) gg = d_sqrt(p2);
+    }
     const bool pair = valid && gg > T(2);  // below 2 m_e c^2 no pair
     const T nx = px * inv, ny = py * inv, nz = pz * inv;
     const T km = (gg - T(2)) * xm, kp = (gg - T(2)) * xp;  // kinetic energies (§2.1)
-    const T pmm = d_sqrt(km * (km + T(2))), pmp = d_sqrt(kp * (kp + T(2)));
+    const T pmm = e_sqrt(km * (km + T(2))), pmp = e_sqrt(kp * (kp + T(2)));
 
     const long long se = warp_reserve(E.count, pair);
     const long long sq = warp_reserve(Q.count, pair);

@@ -38,15 +38,28 @@ __host__ __device__ __forceinline__ Fix fix_limbs(int64_t v)
     return Fix{(int)(v >> 32), (int)((uint32_t)v >> 2)};
 }
 
-// a double on the block exponent eb (biased, the largest of its block): v 2^(eb - 1084)
-__device__ __forceinline__ Fix fix_from(double x, int eb)
+// v >> d, 0 for d >= 64 (PTX clamps the amount)
+__device__ __forceinline__ uint64_t fix_shr(uint64_t v, int d)
+{
+#ifdef __CUDA_ARCH__
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(d));
+    return r;
+#else
+    return d > 63 ? 0 : v >> d;
+#endif
+}
+
+// a double on the block exponent eb (biased, the largest of its block): v 2^(eb - 1084);
+// top: eb in the exponent's place with ones below it
+__device__ __forceinline__ Fix fix_from(double x, int top)
 {
     const int hi = __double2hiint(x);
     const uint32_t lo = (uint32_t)__double2loint(x);
-    const int d = eb - ((hi >> 20) & 0x7ff);
+    const int d = (top - (hi & 0x7fffffff)) >> 20;  // eb - the exponent
     const uint32_t mh = ((uint32_t)hi & 0x000fffffu) | 0x00100000u;
-    uint64_t v = (uint64_t)__funnelshift_l(lo, mh, 9) << 32 | (lo << 9);  // 53 bits << 9
-    v >>= d > 63 ? 63 : d;  // (a zero or subnormal among larger values is shifted out: eb >= 128)
+    // 53 bits << 9 (a zero or subnormal among larger values is shifted out: eb >= 128)
+    const uint64_t v = fix_shr((uint64_t)__funnelshift_l(lo, mh, 9) << 32 | (lo << 9), d);
     const int s = (hi >> 31) | 1;
     return Fix{(int)(v >> 32) * s, (int)((uint32_t)v >> 2) * s};
 }
@@ -172,6 +185,64 @@ __device__ __forceinline__ double fix_to_double(int64_t v, int e)
     return __hiloint2double((int)(bits >> 32) | (v < 0 ? (int)0x80000000 : 0), (int)(uint32_t)bits);
 }
 
+// x = g 2^e with e even, g in [2^59, 2^61), for a positive normal x
+__device__ __forceinline__ uint64_t fix_even(double x, int &e)
+{
+    const int hi = __double2hiint(x), be = hi >> 20;
+    const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(x);
+    const int s = be & 1 ? 8 : 7;  // be - 1075 - s is even
+    e = be - 1075 - s;
+    return m << s;
+}
+
+// whether x is positive, normal and within 2^+-500 (the integer forms below)
+__device__ __forceinline__ bool fix_plain(double x)
+{
+    return (unsigned)(__double2hiint(x) - (523 << 20)) < (1000u << 20);
+}
+
+// sqrt(x) and 1/sqrt(x) for fix_plain(x): within 2^-59 before the rounding to FP64
+__device__ __forceinline__ void fix_sqrt_double(double x, double &root, double &inv_root)
+{
+    int e, ie;
+    const uint64_t g = fix_even(x, e);
+    int64_t sq;
+    uint64_t inv;
+    fix_sqrt(g, sq, inv, ie);
+    const int h = e / 2 - 30;  // sqrt(x) = sq 2^h
+    root = fix_to_double(sq, h);
+    inv_root = fix_to_double((int64_t)(inv >> 1), ie + 1 - h);  // (inv may be 2^63)
+}
+
+__device__ __forceinline__ double fix_sqrt_double(double x)
+{
+    double r, i;
+    fix_sqrt_double(x, r, i);
+    return r;
+}
+
+// a / b for fix_plain(|a|), fix_plain(b): within 2^-58 before the rounding to
+// FP64.  The reciprocal of b's significand by two Newton steps from the 22-bit
+// one (as in fix_sqrt), times a's.
+__device__ __forceinline__ double fix_div(double a, double b)
+{
+    const int ha = __double2hiint(a), hb = __double2hiint(b);
+    const uint64_t ma = (uint64_t)((ha & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(a);
+    const uint64_t mb = (uint64_t)((hb & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(b);
+    const uint64_t g = mb << 10;  // [2^62, 2^63): g 2^-63 in [1/2, 1)
+    const uint32_t fh = (uint32_t)(g >> 32), fl = (uint32_t)g;
+    const float y = __frcp_rn((float)fh * 0x1p-31f);
+    const int y0 = (int)fminf(y * 0x1p30f, 2147483520.0f);  // 2^-30, [1, 2)
+    const int64_t e0 = (int64_t)((1ull << 61) - uwide(fh, (uint32_t)y0) - (uwide(fl, (uint32_t)y0) >> 32));
+    const uint64_t y1 = ((uint64_t)y0 << 32) + (uint64_t)(wide(y0, (int)(e0 >> 10)) >> 19);  // 2^-62
+    const uint32_t yh = (uint32_t)(y1 >> 32), yl = (uint32_t)y1;
+    const int64_t e1 = -(int64_t)((uwide(fh, yh) << 32) + uwide(fh, yl) + uwide(fl, yh) + (uwide(fl, yl) >> 32));
+    const uint64_t inv = y1 + (uint64_t)(wide((int)yh, (int)(e1 >> 21)) >> 40);  // 1/(g 2^-63), 2^-62
+    const uint64_t p = __umul64hi(ma << 10, inv);  // (ma 2^-53)(2^53/mb) 2^61
+    const int64_t q = (ha ^ hb) < 0 ? -(int64_t)p : (int64_t)p;
+    return fix_to_double(q, ((ha >> 20) & 0x7ff) - ((hb >> 20) & 0x7ff) - 61);
+}
+
 // ln(n 2^e) (minus it with `neg`: an FP64 sign change is an FP64 instruction) as a
 // double for n in [2^63, 2^64), |ln| < 62: the reduction of
 // fix_half_ln with the cubic term to 2^-58; within 2^-57 absolute, and 2^-53
@@ -240,14 +311,15 @@ __device__ __forceinline__ bool fix_particle(bool qs, double px, double py, doub
                                              const int *tab_r, const long long *tab_ln, const long long *tab_ex,
                                              FixOut &o)
 {
-    const auto ebits = [](double x) { return (__double2hiint(x) >> 20) & 0x7ff; };
+    const auto mag_hi = [](double x) { return __double2hiint(x) & 0x7fffffff; };
     const auto imax = [](int a, int b) { return a > b ? a : b; };
-    int ep = imax(imax(ebits(px), ebits(py)), ebits(pz));
-    const int ef = imax(imax(imax(ebits(ex), ebits(ey)), imax(ebits(ez), ebits(bx))), imax(ebits(by), ebits(bz)));
+    int ep = imax(imax(mag_hi(px), mag_hi(py)), mag_hi(pz)) >> 20;
+    const int ef = imax(imax(imax(mag_hi(ex), mag_hi(ey)), imax(mag_hi(ez), mag_hi(bx))), imax(mag_hi(by), mag_hi(bz))) >> 20;
     // blocks within 2^+-400 (no infinity, NaN or subnormal, and no overflow that FP64 would see)
     bool ok = ax.ok && (unsigned)(ep - 623) <= 800u && (unsigned)(ef - 623) <= 800u;
     if (qs) ep = imax(ep, 1023);  // gamma^2 = 1 + p^2 on one scale
-    const Fix x = fix_from(px, ep), y = fix_from(py, ep), z = fix_from(pz, ep);
+    const int tp = ep << 20 | 0xfffff, tf = ef << 20 | 0xfffff;
+    const Fix x = fix_from(px, tp), y = fix_from(py, tp), z = fix_from(pz, tp);
     Acc a{wide(x.h, x.h) + wide(y.h, y.h) + wide(z.h, z.h), wide(x.h, x.l) + wide(y.h, y.l) + wide(z.h, z.l)};
     uint64_t g2 = (uint64_t)(a.hh + (a.m >> 29));
     const int sh = 58 - 2 * (ep - 1023);
@@ -258,8 +330,8 @@ __device__ __forceinline__ bool fix_particle(bool qs, double px, double py, doub
     int inv_e;
     fix_sqrt(g2, sq, inv, inv_e);
     const Fix g{(int)(sq >> 30), (int)(sq & 0x3fffffff)};
-    const Fix e0 = fix_from(ex, ef), e1 = fix_from(ey, ef), e2 = fix_from(ez, ef);
-    const Fix b0 = fix_from(bx, ef), b1 = fix_from(by, ef), b2 = fix_from(bz, ef);
+    const Fix e0 = fix_from(ex, tf), e1 = fix_from(ey, tf), e2 = fix_from(ez, tf);
+    const Fix b0 = fix_from(bx, tf), b1 = fix_from(by, tf), b2 = fix_from(bz, tf);
     Acc f0{0, 0}, f1{0, 0}, f2{0, 0}, pe{0, 0};
     mac(f0, g, e0), mac(f0, y, b2), msc(f0, z, b1);
     mac(f1, g, e1), mac(f1, z, b0), msc(f1, x, b2);

@@ -25,6 +25,35 @@ __device__ __forceinline__ double r_log(double x) { return log_tang(x); }
 __device__ __forceinline__ float r_exp(float x) { return __expf(x); }
 __device__ __forceinline__ double r_exp(double x) { return exp_tang(x); }
 __device__ __forceinline__ double d_fma(double a, double b, double c) { return fma(a, b, c); }
+// square root, reciprocal square root and quotient of the event kernels: FP32 as
+// they are; FP64 on the integers (fixed64.cuh) where the arguments are ordinary (an
+// FP64 square root or division is ~10 FP64 instructions of 76 issue slots
+// each), within 2^-58 before the last rounding, so that now and then the last
+// bit differs from the IEEE operation's
+__device__ __forceinline__ float e_sqrt(float x) { return sqrtf(x); }
+__device__ __forceinline__ double e_sqrt(double x) { return fix_plain(x) ? fix_sqrt_double(x) : sqrt(x); }
+__device__ __forceinline__ float e_div(float a, float b) { return a / b; }
+__device__ __forceinline__ double e_div(double a, double b)
+{
+    return fix_plain(__longlong_as_double(__double_as_longlong(a) & 0x7fffffffffffffffll)) && fix_plain(b) ? fix_div(a, b)
+                                                                                                          : a / b;
+}
+// |p| and 1/|p| (0 for p = 0) from p^2
+__device__ __forceinline__ void e_norm(float p2, float &p, float &inv)
+{
+    p = sqrtf(p2);
+    inv = p > 0.0f ? 1.0f / p : 0.0f;
+}
+__device__ __forceinline__ void e_norm(double p2, double &p, double &inv)
+{
+    if (fix_plain(p2)) {
+        fix_sqrt_double(p2, p, inv);
+    } else {
+        p = sqrt(p2);
+        inv = p2 > 0.0 ? rsqrt(p2) : 0.0;
+    }
+}
+
 // ln x on the integers (fixed64.cuh) for x in [2^-86, 2^86]; Tang's beyond
 __device__ __forceinline__ double log_int(double x)
 {
@@ -275,7 +304,7 @@ __device__ __forceinline__ T qs_sample_xi(const Table2D<T> &tb, T chi, T r)
     const T x0 = tb.x0 + T(m) * tb.dx;
     const T x1 = (m + 1 == tb.n_xi - 1) ? T(0) : tb.x0 + T(m + 1) * tb.dx;
     if (!(dp > T(0))) return s_exp(x0);
-    T lx = x0 + (lr - p0) * (x1 - x0) / dp;
+    T lx = x0 + e_div((lr - p0) * (x1 - x0), dp);
     lx = lx > T(0) ? T(0) : lx;
     return s_exp(lx);
 }
@@ -307,7 +336,7 @@ __device__ __forceinline__ T bw_sample_xi(const Table2D<T> &tb, T chi, double u,
     const T x0 = T(m) * tb.dx;
     const T x1 = (m + 1 == tb.n_xi - 1) ? T(0.5) : T(m + 1) * tb.dx;
     if (!(dp > T(0))) return x0;
-    T x = x0 + (r - p0) * (x1 - x0) / dp;
+    T x = x0 + e_div((r - p0) * (x1 - x0), dp);
     return x > T(0.5) ? T(0.5) : (x < T(0) ? T(0) : x);
 }
 

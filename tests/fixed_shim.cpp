@@ -24,11 +24,22 @@ static inline unsigned long long __umul64hi(unsigned long long a, unsigned long 
 {
     return (unsigned long long)(((unsigned __int128)a * b) >> 64);
 }
+static inline float __frcp_rn(float x) { return 1.0f / x; }
 template <class T> static inline T __ldg(const T *p) { return *p; }
 static int g_skew;  // rsqrtf on the GPU is within 2 ulp: skewed either way here
 static inline float rsqrtf(float x) { return (1.0f / sqrtf(x)) * (1.0f + 1.2e-7f * (float)(g_skew++ % 3 - 1)); }
 
 #include "fixed64.cuh"
+
+extern "C" void fixed_roots(int64_t n, const double *a, const double *b, double *root, double *inv, double *quot, int *ok)
+{
+    for (int64_t i = 0; i < n; ++i) {
+        ok[i] = qed::fix_plain(b[i]);
+        if (!ok[i]) continue;
+        qed::fix_sqrt_double(b[i], root[i], inv[i]);
+        quot[i] = qed::fix_div(a[i], b[i]);
+    }
+}
 
 extern "C" void fixed_ln(int64_t n, const uint64_t *m, const int *e, double *out)
 {

@@ -169,3 +169,31 @@ def test_logarithm_against_extended_precision(lib):
                    np.log(x) + k * np.log(LD(2)))
     err = np.abs(out - ref).astype(np.float64)
     assert np.all(err <= 2.0 ** -57 + 2.0 ** -53 * np.abs(ref).astype(np.float64))
+
+
+def test_roots_and_quotients_against_extended_precision(lib):
+    """sqrt, 1/sqrt and a/b: one rounding (2^-53) and the integers' 2^-58; exact squares and powers of two; what is not
+    ordinary is refused."""
+    r = np.random.default_rng(4)
+    n = 300_000
+    b = r.uniform(1, 2, n) * 2.0 ** r.integers(-499, 499, n)
+    b[:1000] = np.arange(1, 1001, dtype=np.float64) ** 2
+    b[1000:1900] = 2.0 ** np.arange(-450, 450)
+    b[1900:2900] = 4.0 + np.arange(-500, 500) * 2.0 ** -50
+    b[2900:3900] = np.nextafter(1.0, 0.0) - np.arange(1000) * 2.0 ** -53
+    a = r.uniform(-2, 2, n) * 2.0 ** r.integers(-400, 400, n)
+    a[:1900] = b[:1900] * r.integers(1, 100, 1900)  # exact products
+    a[2900:3900] = 1.0
+    a = np.where(a == 0, 1.0, a)
+    bad = [0.0, -1.0, np.nan, np.inf, 1e-310, 1e200, 1e-200]
+    b[-len(bad):] = bad
+    root, inv, quot, ok = np.zeros(n), np.zeros(n), np.zeros(n), np.zeros(n, dtype=np.int32)
+    ptr = lambda v: v.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    lib.fixed_roots(ctypes.c_int64(n), ptr(a), ptr(b), ptr(root), ptr(inv), ptr(quot), ptr(ok))
+    assert not ok[-len(bad):].any() and ok[:-len(bad)].all()
+    a, b, root, inv, quot = (v[:-len(bad)] for v in (a, b, root, inv, quot))
+    tol = 2.0 ** -53 + 2.0 ** -58
+    s = np.sqrt(b.astype(LD))
+    assert np.all(np.abs(root / s - 1) <= tol) and np.all(np.abs(inv * s - 1) <= tol)
+    assert np.all(np.abs(quot / (a.astype(LD) / b.astype(LD)) - 1) <= tol)
+    assert np.array_equal(root[:1000], np.arange(1, 1001)) and np.array_equal(quot[:1900], a[:1900] / b[:1900])

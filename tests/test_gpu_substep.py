@@ -381,9 +381,9 @@ def test_full_size_batched_workload_sampled(api, tabs):
 @pytest.mark.parametrize("prec_name", ["f32", "f64"])
 @pytest.mark.parametrize("per_sm", [1024, 49152])
 @pytest.mark.parametrize("more", [0, 1])
-def test_evolution_forms_at_the_lines_of_the_default(api, tables, prec_name, per_sm, more):
+def test_evolution_forms_at_the_lines_of_the_default(api, tabs, prec_name, per_sm, more):
     """The default evolution on either side of the particle counts where its form changes gives the bits of direct loads."""
-    _, t = tables
+    _, t = tabs
     prec = api.QED_F64 if prec_name == "f64" else api.QED_F32
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     caps = sms * per_sm + more

@@ -720,26 +720,22 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
         table_rows_kernel<<<params->qs.n_chi + params->bw.n_chi, 256, dyn, st>>>(a);
         e = cudaGetLastError();
     }
+    // every entry must be finite (a chi range whose rates underflow FP64 is
+    // rejected): ln G and ln T lie next to each other, one copy
+    const size_t n_g = params->qs.n_chi, off_t = t->d_bw_lnT - t->d_qs_lnG, n_one = off_t + params->bw.n_chi;
+    std::vector<double> one(n_one);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(one.data(), t->d_qs_lnG, n_one * sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         qed_tables_destroy(t);
         QED_FAIL(QED_ERR_CUDA, "table generation failed: %s", cudaGetErrorString(e));
     }
-    // every entry must be finite (a chi range whose rates underflow FP64 is rejected)
-    std::vector<double> g(params->qs.n_chi), tt(params->bw.n_chi);
-    if ((s = qed_tables_copy_to_host(t, g.data(), nullptr, tt.data(), nullptr))) {
-        qed_tables_destroy(t);
-        return s;
-    }
-    for (double v : g)
-        if (!std::isfinite(v)) {
+    for (size_t i = 0; i < n_one; ++i)
+        if ((i < n_g || i >= off_t) && !std::isfinite(one[i])) {
             qed_tables_destroy(t);
-            QED_FAIL(QED_ERR_NUMERIC, "ln G is not finite over the requested chi range");
-        }
-    for (double v : tt)
-        if (!std::isfinite(v)) {
-            qed_tables_destroy(t);
-            QED_FAIL(QED_ERR_NUMERIC, "ln T is not finite over the requested chi_gamma range");
+            QED_FAIL(QED_ERR_NUMERIC, "ln %s is not finite over the requested %s range", i < n_g ? "G" : "T",
+                     i < n_g ? "chi" : "chi_gamma");
         }
     if ((s = finish_tables(t, st))) {
         qed_tables_destroy(t);

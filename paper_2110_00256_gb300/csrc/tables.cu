@@ -33,20 +33,28 @@ qed_status check_params(const qed_table_params *p)
     return check_axis(p->bw, "bw", false);
 }
 
-// d[n][m] = v[n][m+1] - v[n][m] in FP64, 0 in the last column
-__global__ void col_diff_kernel(const double *__restrict__ v, double *__restrict__ d, int64_t rows, int cols)
-{
-    const int64_t n = rows * cols;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int m = (int)(i % cols);
-        d[i] = (m + 1 < cols) ? v[i + 1] - v[i] : 0.0;
-    }
-}
+// Everything formed entry by entry from the FP64 tables, in one launch: the
+// column differences d[n][m] = v[n][m+1] - v[n][m] of both 2-D tables in FP64 (0
+// in the last column) and the FP32 copies of all six.  blockIdx.y: process.
+struct Derived {
+    const double *one[2], *two[2];
+    double *diff[2];
+    float *f_one[2], *f_two[2], *f_diff[2];
+    int n_chi[2], n_xi[2];
+};
 
-__global__ void to_f32_kernel(const double *__restrict__ in, float *__restrict__ out, int64_t n)
+__global__ void derive_kernel(const Derived t)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = __double2float_rn(in[i]);
+    const int p = blockIdx.y, cols = t.n_xi[p];
+    const int64_t n = (int64_t)t.n_chi[p] * cols;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double v = t.two[p][i];
+        const double d = (int)(i % cols) + 1 < cols ? t.two[p][i + 1] - v : 0.0;
+        t.diff[p][i] = d;
+        t.f_diff[p][i] = __double2float_rn(d);
+        t.f_two[p][i] = __double2float_rn(v);
+        if (i < t.n_chi[p]) t.f_one[p][i] = __double2float_rn(t.one[p][i]);
+    }
 }
 
 // Guide table of one 2-D table: for row n and edge e of kGuideBins equal bins
@@ -54,10 +62,9 @@ __global__ void to_f32_kernel(const double *__restrict__ in, float *__restrict__
 // largest m with v[n][m] <= edge (0 if none); edge 0 is -inf, the last +inf.
 // A draw in bin b then lies between the rows' guides at b and b + 1.
 template <typename T>
-__global__ void guide_kernel(const T *__restrict__ v, int n_xi, bool qs, int32_t *__restrict__ g)
+__device__ void guide_entry(const T *__restrict__ v, int n_xi, bool qs, int32_t *__restrict__ g)
 {
     const int n = blockIdx.x, e = threadIdx.x;
-    if (e > kGuideBins) return;
     int32_t out;
     if (e == 0) {
         out = 0;
@@ -77,6 +84,17 @@ __global__ void guide_kernel(const T *__restrict__ v, int n_xi, bool qs, int32_t
         out = lo;
     }
     g[(size_t)n * (kGuideBins + 1) + e] = out;
+}
+
+// row blockIdx.x, process blockIdx.y, precision blockIdx.z
+__global__ void guide_kernel(const Derived t, int32_t *qs_d, int32_t *bw_d, int32_t *qs_f, int32_t *bw_f)
+{
+    const int p = blockIdx.y;
+    if ((int)blockIdx.x >= t.n_chi[p] || threadIdx.x > kGuideBins) return;
+    if (blockIdx.z)
+        guide_entry<float>(t.f_two[p], t.n_xi[p], p == 0, p ? bw_f : qs_f);
+    else
+        guide_entry<double>(t.two[p], t.n_xi[p], p == 0, p ? bw_d : qs_d);
 }
 
 static void free_tables(qed_tables *t)
@@ -132,7 +150,7 @@ qed_status alloc_tables(const qed_table_params *p, qed_tables **out, size_t scra
     const size_t n1[2] = {(size_t)p->qs.n_chi, (size_t)p->bw.n_chi}, n2[2] = {n_qs2(*p), n_bw2(*p)};
     for (int pass = 0; pass < 2; ++pass) {
         size = 0;
-        place(t->d_qs_lnG, n1[0]), place(t->d_qs_lnP, n2[0]), place(t->d_bw_lnT, n1[1]), place(t->d_bw_P, n2[1]);
+        place(t->d_qs_lnG, n1[0]), place(t->d_bw_lnT, n1[1]), place(t->d_qs_lnP, n2[0]), place(t->d_bw_P, n2[1]);
         t->derived = (void *)((uintptr_t)t->block + size);
         const size_t least = size + scratch;
         place(t->d_qs_dlnP, n2[0]), place(t->d_bw_dP, n2[1]);
@@ -156,23 +174,16 @@ qed_status alloc_tables(const qed_table_params *p, qed_tables **out, size_t scra
 qed_status finish_tables(qed_tables *t, cudaStream_t st)
 {
     const qed_table_params &p = t->params;
-    col_diff_kernel<<<256, 256, 0, st>>>(t->d_qs_lnP, t->d_qs_dlnP, p.qs.n_chi, p.qs.n_xi);
+    const Derived d{{t->d_qs_lnG, t->d_bw_lnT}, {t->d_qs_lnP, t->d_bw_P},     {t->d_qs_dlnP, t->d_bw_dP},
+                    {t->f_qs_lnG, t->f_bw_lnT}, {t->f_qs_lnP, t->f_bw_P},     {t->f_qs_dlnP, t->f_bw_dP},
+                    {p.qs.n_chi, p.bw.n_chi},   {p.qs.n_xi, p.bw.n_xi}};
+    const size_t most = n_qs2(p) > n_bw2(p) ? n_qs2(p) : n_bw2(p);
+    const unsigned blocks = (unsigned)((most + 255) / 256 < 1024 ? (most + 255) / 256 : 1024);
+    derive_kernel<<<dim3(blocks, 2), 256, 0, st>>>(d);
     QED_LAUNCH_CHECK();
-    col_diff_kernel<<<256, 256, 0, st>>>(t->d_bw_P, t->d_bw_dP, p.bw.n_chi, p.bw.n_xi);
-    QED_LAUNCH_CHECK();
-    const size_t sz[6] = {(size_t)p.qs.n_chi, n_qs2(p), (size_t)p.bw.n_chi, n_bw2(p), n_qs2(p), n_bw2(p)};
-    const double *d[6] = {t->d_qs_lnG, t->d_qs_lnP, t->d_bw_lnT, t->d_bw_P, t->d_qs_dlnP, t->d_bw_dP};
-    float *f[6] = {t->f_qs_lnG, t->f_qs_lnP, t->f_bw_lnT, t->f_bw_P, t->f_qs_dlnP, t->f_bw_dP};
-    for (int k = 0; k < 6; ++k) {
-        int blocks = (int)((sz[k] + 255) / 256);
-        if (blocks > 1024) blocks = 1024;
-        to_f32_kernel<<<blocks, 256, 0, st>>>(d[k], f[k], (int64_t)sz[k]);
-        QED_LAUNCH_CHECK();
-    }
-    guide_kernel<double><<<p.qs.n_chi, kGuideBins + 1, 0, st>>>(t->d_qs_lnP, p.qs.n_xi, true, t->d_qs_guide);
-    guide_kernel<float><<<p.qs.n_chi, kGuideBins + 1, 0, st>>>(t->f_qs_lnP, p.qs.n_xi, true, t->f_qs_guide);
-    guide_kernel<double><<<p.bw.n_chi, kGuideBins + 1, 0, st>>>(t->d_bw_P, p.bw.n_xi, false, t->d_bw_guide);
-    guide_kernel<float><<<p.bw.n_chi, kGuideBins + 1, 0, st>>>(t->f_bw_P, p.bw.n_xi, false, t->f_bw_guide);
+    const unsigned rows = (unsigned)(p.qs.n_chi > p.bw.n_chi ? p.qs.n_chi : p.bw.n_chi);
+    guide_kernel<<<dim3(rows, 2, 2), kGuideBins + 1, 0, st>>>(d, t->d_qs_guide, t->d_bw_guide, t->f_qs_guide,
+                                                              t->f_bw_guide);
     QED_LAUNCH_CHECK();
     QED_CUDA_TRY(cudaStreamSynchronize(st));
     return QED_OK;

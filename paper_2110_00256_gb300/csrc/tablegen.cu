@@ -93,23 +93,27 @@ __device__ double bw_integrand(double chi, double xi)
 constexpr int kPieceOct = -30, kPieceOcts = 40, kPieces = 4 * kPieceOcts, kPieceCoef = 14;
 constexpr int kPieceRow = 2 * kPieceCoef;  // both functions of a piece
 
-// One warp per piece, both processes (they share K_{2/3}).  The trapezoid rule
+// One CTA per piece, both processes (they share K_{2/3}).  The trapezoid rule
 // takes the step of the piece's largest argument, so its nodes t_k, and all
 // factors but exp(-x (cosh t_k - 1)), are the same for the 14 arguments: the
-// lanes form them 32 at a time, then each of 14 lanes runs one argument's sum
-// (one exponential and three FMAs a step; with the factors formed by every lane
-// in every step, ~130 FP64 instructions, the launch took 362 us).
+// threads form them once, then eight threads to an argument each run every
+// eighth step of its sum (one exponential and three FMAs).  Bound by FP64
+// latency: with the factors formed in every step (~130 FP64 instructions) the
+// launch took 362 us, with one warp per piece 148 us.
 constexpr int kPieceT = 160;  // trapezoid nodes: (ln(2 (40 + 5/3 t) / 2^-30) / (1/4) = 106 at the lower end
-__global__ void __launch_bounds__(32) bessel_pieces_kernel(double *out)
+__global__ void __launch_bounds__(128) bessel_pieces_kernel(double *out)
 {
     __shared__ double s_c1[kPieceT], s_f[3][kPieceT];  // cosh t - 1; cosh(nu t)/cosh t for nu = 5/3, 1/3; cosh(2t/3)
-    const int piece = blockIdx.x, lane = threadIdx.x;
+    __shared__ double s_cos[4 * kPieceCoef], s_part[3][8][16];
+    __shared__ int s_live;
+    const int piece = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const double scale = ldexp(1.0, kPieceOct + piece / 4);
     const double hi = scale * (1.0 + (2 * (piece % 4) + 2) / 8.0), lo = scale * (1.0 + (2 * (piece % 4)) / 8.0);
     const double h = fmin(0.25, 0.6 / sqrt(hi));
-    int n = 0;  // steps: until lo (cosh t - 1) leaves every integrand below e^-40
-    for (int base = 0; base < kPieceT; base += 32) {
-        const int k = base + lane + 1;
+    if (tid == 0) s_live = 0;
+    if (tid < 4 * kPieceCoef) s_cos[tid] = cospi((double)tid / (2 * kPieceCoef));
+    __syncthreads();
+    for (int k = tid + 1; k <= kPieceT; k += 128) {  // (whole warps)
         const double t = k * h, s = sinh(0.5 * t), c1 = 2.0 * s * s;
         const double e1 = exp(t / 3.0), i1 = 1.0 / e1, e2 = e1 * e1, i2 = i1 * i1;
         const double ch = 1.0 / (e2 * e1 + i2 * i1);  // 1/(2 cosh t)
@@ -117,47 +121,54 @@ __global__ void __launch_bounds__(32) bessel_pieces_kernel(double *out)
         s_f[0][k - 1] = (e2 * e2 * e1 + i2 * i2 * i1) * ch;
         s_f[1][k - 1] = (e1 + i1) * ch;
         s_f[2][k - 1] = 0.5 * (e2 + i2);
-        const bool live = !(lo * c1 > 40.0 && lo * c1 - 5.0 / 3.0 * t > 40.0);
-        n += __popc(__ballot_sync(0xffffffffu, live));
-        if (!__any_sync(0xffffffffu, live)) break;
+        // steps needed: until lo (cosh t - 1) leaves every integrand below e^-40
+        const unsigned live = __ballot_sync(0xffffffffu, !(lo * c1 > 40.0 && lo * c1 - 5.0 / 3.0 * t > 40.0));
+        if (lane == 0) atomicAdd(&s_live, __popc(live));
     }
-    __syncwarp();
-    double f[3] = {0.0, 0.0, 0.0};
+    __syncthreads();
+    {
+        const int i = tid & 15, part = tid >> 4, n = s_live;
+        double sum[3] = {0.0, 0.0, 0.0};
+        if (i < kPieceCoef) {
+            const double x = scale * (1.0 + (2 * (piece % 4) + 1 + s_cos[2 * i + 1]) / 8.0);  // Chebyshev node
+            for (int k = part; k < n; k += 8) {
+                const double e = exp_tang(fmax(-x * s_c1[k], -700.0));
+#pragma unroll
+                for (int f = 0; f < 3; ++f) sum[f] = fma(e, s_f[f][k], sum[f]);
+            }
+        }
+#pragma unroll
+        for (int f = 0; f < 3; ++f) s_part[f][part][i] = sum[f];
+    }
+    __syncthreads();
+    const int f = tid >> 5;  // a warp per function
+    if (f == 3) return;
+    double v = 0.0;
     if (lane < kPieceCoef) {
-        const double x = scale * (1.0 + (2 * (piece % 4) + 1 + cospi((lane + 0.5) / kPieceCoef)) / 8.0);  // Chebyshev node
-        double sum[3] = {0.5, 0.5, 0.5};
-        for (int k = 0; k < n; ++k) {
-            const double e = exp_tang(fmax(-x * s_c1[k], -700.0));
+        v = 0.5;  // the term t = 0
 #pragma unroll
-            for (int i = 0; i < 3; ++i) sum[i] = fma(e, s_f[i][k], sum[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) f[i] = h * sum[i];
+        for (int p = 0; p < 8; ++p) v += s_part[f][p][lane];
+        v *= h;
     }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        // lane i: Chebyshev coefficient i, then the coefficient of x^i by the
-        // recurrence T_k = 2 x T_{k-1} - T_{k-2}
-        double c = 0.0;
-        for (int i = 0; i < kPieceCoef; ++i) {
-            const int turn = (2 * i + 1) * lane % (4 * kPieceCoef);  // the angle in units of pi / (2 kPieceCoef)
-            c += __shfl_sync(0xffffffffu, f[k], i) * cospi((double)turn / (2 * kPieceCoef));
-        }
-        c *= (lane ? 2.0 : 1.0) / kPieceCoef;
-        double t0 = lane == 0 ? 1.0 : 0.0, t1 = lane == 1 ? 1.0 : 0.0;  // T_0, T_1
-        double p = __shfl_sync(0xffffffffu, c, 0) * t0 + __shfl_sync(0xffffffffu, c, 1) * t1;
-        for (int i = 2; i < kPieceCoef; ++i) {
-            const double up = __shfl_up_sync(0xffffffffu, t1, 1);
-            const double t2 = 2.0 * (lane ? up : 0.0) - t0;
-            p += __shfl_sync(0xffffffffu, c, i) * t2;
-            t0 = t1, t1 = t2;
-        }
-        if (lane < kPieceCoef) {
-            double *qs = out + (size_t)piece * kPieceRow + lane, *bw = qs + (size_t)kPieces * kPieceRow;
-            if (k == 0) qs[0] = p;
-            if (k == 1) bw[0] = p;
-            if (k == 2) qs[kPieceCoef] = bw[kPieceCoef] = p;
-        }
+    // lane i: Chebyshev coefficient i, then the coefficient of x^i by the
+    // recurrence T_k = 2 x T_{k-1} - T_{k-2}
+    double c = 0.0;
+    for (int i = 0; i < kPieceCoef; ++i)  // (the angle in units of pi / (2 kPieceCoef))
+        c += __shfl_sync(0xffffffffu, v, i) * s_cos[(2 * i + 1) * lane % (4 * kPieceCoef)];
+    c *= (lane ? 2.0 : 1.0) / kPieceCoef;
+    double t0 = lane == 0 ? 1.0 : 0.0, t1 = lane == 1 ? 1.0 : 0.0;  // T_0, T_1
+    double p = __shfl_sync(0xffffffffu, c, 0) * t0 + __shfl_sync(0xffffffffu, c, 1) * t1;
+    for (int i = 2; i < kPieceCoef; ++i) {
+        const double up = __shfl_up_sync(0xffffffffu, t1, 1);
+        const double t2 = 2.0 * (lane ? up : 0.0) - t0;
+        p += __shfl_sync(0xffffffffu, c, i) * t2;
+        t0 = t1, t1 = t2;
+    }
+    if (lane < kPieceCoef) {
+        double *qs = out + (size_t)piece * kPieceRow + lane, *bw = qs + (size_t)kPieces * kPieceRow;
+        if (f == 0) qs[0] = p;
+        if (f == 1) bw[0] = p;
+        if (f == 2) qs[kPieceCoef] = bw[kPieceCoef] = p;
     }
 }
 
@@ -197,15 +208,24 @@ constexpr double kQsFactor = 0.27566444771089600;  // sqrt(3) / (2 pi)
 __device__ __forceinline__ void node_terms(bool qs, double x, double &q, double &va, double &vb)
 {
     if (qs) {
-        const double xi = exp(x), om = -expm1(x);  // 1 - xi
-        q = (2.0 / 3.0) * xi / om;
+        // xi and om = 1 - xi, each without cancellation, from one exponential
+        double xi, om;
+        if (x > -0.7) {
+            om = -expm1(x);
+            xi = 1.0 - om;
+        } else {
+            xi = exp_tang(x);
+            om = 1.0 - xi;
+        }
+        const double r = xi / om;
+        q = (2.0 / 3.0) * r;
         va = kQsFactor * xi;
-        vb = va * (xi * xi / om);
+        vb = va * (xi * r);
     } else {
-        const double om = 1.0 - x;
-        q = (2.0 / 3.0) / (x * om);
+        const double om = 1.0 - x, r = 1.0 / (x * om);
+        q = (2.0 / 3.0) * r;
         va = 1.0;
-        vb = x / om + om / x;
+        vb = (x * x + om * om) * r;  // x/om + om/x
     }
 }
 
@@ -221,8 +241,10 @@ __device__ __forceinline__ double row_integrand(const double *c, bool qs, double
 
 struct GenArgs {
     double *qs_lnG, *qs_lnP, *bw_lnT, *bw_P;
-    double qs_l0, qs_l1, qs_xi_min, bw_l0, bw_l1;
+    double qs_l0, qs_l1, qs_xi_min, qs_ln_xi_min, bw_l0, bw_l1;
     int qs_n_chi, qs_n_xi, bw_n_chi, bw_n_xi;
+    int *points;  // [2][n_xi]: points of the rule that an interval's place allows
+    double ts_end[kTsHalf + 1], ts_w[kTsHalf + 1];  // tanh-sinh: distance of node k from the nearer end, weight (half-widths)
     double *pieces;  // [2][kPieces][kPieceRow]: the Bessel functions
     double *nodes;   // [2][3][kGl][n_xi]: q, w va, w vb at the Gauss-Legendre nodes of every interval
 };
@@ -273,8 +295,9 @@ __global__ void __launch_bounds__(128) row_nodes_kernel(const __grid_constant__ 
     const int j = blockIdx.x * 8 + threadIdx.x / kGl, k = threadIdx.x % kGl;
     if (j >= M) return;
     double lo, hi;
-    row_interval(qs, log(a.qs_xi_min), M, j, lo, hi);
+    row_interval(qs, a.qs_ln_xi_min, M, j, lo, hi);
     const int points = gl_points(qs, j, lo, hi);
+    if (k == 0) a.points[(qs ? 0 : a.qs_n_xi) + j] = points;
     if (k >= points) return;
     double *out = a.nodes + (qs ? 0 : (size_t)3 * kGl * a.qs_n_xi);
     double x, w;
@@ -300,42 +323,36 @@ __global__ void __launch_bounds__(128) row_nodes_kernel(const __grid_constant__ 
 // steeply), whose nodes and weights on [-1, 1] are shared too.
 __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__ GenArgs a)
 {
-    __shared__ double acc[QED_MAX_TABLE_N], tail[QED_MAX_TABLE_N];
+    __shared__ double acc[QED_MAX_TABLE_N], tail[QED_MAX_TABLE_N], cum[QED_MAX_TABLE_N];
     extern __shared__ double s_c[];  // [kPieces][kPieceRow]
-    __shared__ double s_ts[2][kTsHalf + 1];  // tanh-sinh: distance of node k from the nearer end, weight (half-widths)
     __shared__ short s_hard[QED_MAX_TABLE_N];
     __shared__ int s_n_hard;
-    __shared__ double s_tot;
+    __shared__ double s_chi[2];
     const bool qs = blockIdx.x < (unsigned)a.qs_n_chi;
     const int row = qs ? blockIdx.x : blockIdx.x - a.qs_n_chi;
     const int N = qs ? a.qs_n_chi : a.bw_n_chi;
     const int M = qs ? a.qs_n_xi : a.bw_n_xi;
-    const double l0 = qs ? a.qs_l0 : a.bw_l0, l1 = qs ? a.qs_l1 : a.bw_l1;
-    const double chi = exp(row == N - 1 ? l1 : l0 + row * (l1 - l0) / (N - 1));
-    const double inv_chi = 1.0 / chi;
-    const double lxm = log(a.qs_xi_min);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
 
+    if (threadIdx.x == 0) {
+        const double l0 = qs ? a.qs_l0 : a.bw_l0, l1 = qs ? a.qs_l1 : a.bw_l1;
+        s_chi[0] = exp(row == N - 1 ? l1 : l0 + row * (l1 - l0) / (N - 1));
+        s_chi[1] = 1.0 / s_chi[0];
+        s_n_hard = 0;
+    }
     const double *pieces = a.pieces + (qs ? 0 : (size_t)kPieces * kPieceRow);
     for (int i = threadIdx.x; i < kPieces * kPieceRow; i += blockDim.x) s_c[i] = pieces[i];
-    if (threadIdx.x <= kTsHalf) {
-        const double tk = threadIdx.x * kTsStep;
-        const double s = 0.5 * kPi * sinh(tk), ch = cosh(s);
-        s_ts[0][threadIdx.x] = 2.0 / (1.0 + exp(2.0 * s));
-        s_ts[1][threadIdx.x] = kTsStep * 0.5 * kPi * cosh(tk) / (ch * ch);
-    }
-    if (threadIdx.x == 0) s_n_hard = 0;
     __syncthreads();
+    const double chi = s_chi[0], inv_chi = s_chi[1];
 
     const double *nodes = a.nodes + (qs ? 0 : (size_t)3 * kGl * a.qs_n_xi);
+    const int *allowed = a.points + (qs ? 0 : a.qs_n_xi);
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
-        double lo, hi;
-        row_interval(qs, lxm, M, j, lo, hi);
         if (!qs && j == 0) {
             acc[0] = 0.0;
             continue;
         }
-        int points = gl_points(qs, j, lo, hi);
+        int points = allowed[j];
         if (points) {
             // the outermost nodes lie within 2 % of the ends: Y's fall between them
             const double q0 = nodes[j], q1 = nodes[(size_t)(points - 1) * M + j];
@@ -361,23 +378,23 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__
     for (int i = warp; i < s_n_hard; i += nw) {
         const int j = s_hard[i];
         double lo, hi;
-        row_interval(qs, lxm, M, j, lo, hi);
+        row_interval(qs, a.qs_ln_xi_min, M, j, lo, hi);
         const double r = 0.5 * (hi - lo);
         double part = 0.0;
         for (int k = lane - kTsHalf; k <= kTsHalf; k += 32) {
-            const double d = r * s_ts[0][abs(k)];  // offset from the nearer end, exact near the ends
+            const double d = r * a.ts_end[abs(k)];  // offset from the nearer end, exact near the ends
             const double x = k < 0 ? lo + d : (k > 0 ? hi - d : 0.5 * (lo + hi));
             if (!qs && !(x > 0.0)) continue;
             double q, va, vb;
             node_terms(qs, x, q, va, vb);
-            part += s_ts[1][abs(k)] * row_integrand(s_c, qs, inv_chi, q, va, vb);
+            part += a.ts_w[abs(k)] * row_integrand(s_c, qs, inv_chi, q, va, vb);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
         if (lane == 0) acc[j] = r * part;
     }
     __syncthreads();
-    // running sums from both ends, in order (one thread each)
+    // running sums from both ends, in order (one thread each, in two warps)
     if (threadIdx.x == 0) {
         double c = 0.0;
         for (int m = M - 1; m >= 0; --m) {
@@ -386,31 +403,25 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__
         }
     } else if (threadIdx.x == 32) {
         double c = 0.0;
-        for (int m = 0; m < M; ++m) c += acc[m];
-        s_tot = c;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double c = 0.0;
         for (int m = 0; m < M; ++m) {
             c += acc[m];
-            acc[m] = c;
+            cum[m] = c;
         }
     }
     __syncthreads();
-    const double tot = s_tot;
+    const double tot = cum[M - 1];
     if (qs) {
         // ln P = ln(C/G), except near P = 1 where log1p(-tail/G) keeps the relative accuracy
         double *out = a.qs_lnP + (size_t)row * M;
         for (int m = threadIdx.x; m < M; m += blockDim.x) {
             const double t = tail[m] / tot;
-            out[m] = m == M - 1 ? 0.0 : (t < 0.5 ? log1p(-t) : log(acc[m] / tot));
+            out[m] = m == M - 1 ? 0.0 : (t < 0.5 ? log1p(-t) : log(cum[m] / tot));
         }
         if (threadIdx.x == 0) a.qs_lnG[row] = log(tot);
     } else {
         double *out = a.bw_P + (size_t)row * M;
         for (int m = threadIdx.x; m < M; m += blockDim.x) {
-            double v = tot > 0.0 ? acc[m] / (2.0 * tot) : 0.0;
+            double v = tot > 0.0 ? cum[m] / (2.0 * tot) : 0.0;
             if (m == 0) v = 0.0;
             if (m == M - 1 && tot > 0.0) v = 0.5;
             out[m] = v;
@@ -692,19 +703,27 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
     if (s) return s;
     qed_tables *t = nullptr;
     const size_t scratch =
-        ((size_t)2 * kPieces * kPieceRow + (size_t)3 * kGl * (params->qs.n_xi + params->bw.n_xi)) * sizeof(double);
+        ((size_t)2 * kPieces * kPieceRow + (size_t)3 * kGl * (params->qs.n_xi + params->bw.n_xi)) * sizeof(double) +
+        (size_t)(params->qs.n_xi + params->bw.n_xi) * sizeof(int);
     if ((s = alloc_tables(params, &t, scratch))) return s;
     cudaStream_t st = as_stream(stream);
     GenArgs a;
     a.qs_lnG = t->d_qs_lnG, a.qs_lnP = t->d_qs_lnP, a.bw_lnT = t->d_bw_lnT, a.bw_P = t->d_bw_P;
     a.qs_l0 = std::log(params->qs.chi_min), a.qs_l1 = std::log(params->qs.chi_max);
     a.qs_xi_min = params->qs.xi_min;
+    a.qs_ln_xi_min = std::log(params->qs.xi_min);
+    for (int k = 0; k <= kTsHalf; ++k) {
+        const double tk = k * kTsStep, sh = 0.5 * kPi * std::sinh(tk), ch = std::cosh(sh);
+        a.ts_end[k] = 2.0 / (1.0 + std::exp(2.0 * sh));
+        a.ts_w[k] = kTsStep * 0.5 * kPi * std::cosh(tk) / (ch * ch);
+    }
     a.bw_l0 = std::log(params->bw.chi_min), a.bw_l1 = std::log(params->bw.chi_max);
     a.qs_n_chi = params->qs.n_chi, a.qs_n_xi = params->qs.n_xi;
     a.bw_n_chi = params->bw.n_chi, a.bw_n_xi = params->bw.n_xi;
     // scratch (the pieces, the shared nodes) in the room of the derived tables, which finish_tables fills afterwards
     a.pieces = (double *)t->derived;
     a.nodes = a.pieces + (size_t)2 * kPieces * kPieceRow;
+    a.points = (int *)(a.nodes + (size_t)3 * kGl * (params->qs.n_xi + params->bw.n_xi));
     static const GaussLegendre16 gl = [] {
         GaussLegendre16 g;
         gauss_legendre<kGl>(g.x, g.w);
@@ -715,7 +734,7 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
     constexpr int dyn = kPieces * kPieceRow * (int)sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(table_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) {
-        bessel_pieces_kernel<<<kPieces, 32, 0, st>>>(a.pieces);
+        bessel_pieces_kernel<<<kPieces, 128, 0, st>>>(a.pieces);
         row_nodes_kernel<<<dim3((m + 7) / 8, 2), 8 * kGl, 0, st>>>(a, gl);
         table_rows_kernel<<<params->qs.n_chi + params->bw.n_chi, 256, dyn, st>>>(a);
         e = cudaGetLastError();

@@ -341,8 +341,8 @@ class Mlp:
                                        loss.data_ptr() if loss is not None else None, _stream(stream)))
 
     def gradients(self, proc: int, chi: torch.Tensor, u: torch.Tensor, xi: torch.Tensor, stream=None):
-        g = torch.zeros(self.NPARAM, dtype=torch.float32, device=chi.device)
-        loss = torch.zeros(1, dtype=torch.float32, device=chi.device)
+        g = torch.empty(self.NPARAM, dtype=torch.float32, device=chi.device)
+        loss = torch.empty(1, dtype=torch.float32, device=chi.device)
         check(lib().qed_mlp_gradients(self.handle, proc, chi.data_ptr(), u.data_ptr(), xi.data_ptr(),
                                       int(chi.numel()), g.data_ptr(), loss.data_ptr(), _stream(stream)))
         return g, loss

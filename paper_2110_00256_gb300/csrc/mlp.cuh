@@ -25,7 +25,7 @@
 
 #include <cuda_bf16.h>
 
-#include "common.cuh"
+#include "physics.cuh"
 
 namespace qed {
 
@@ -172,13 +172,16 @@ __device__ __forceinline__ double mlp_output(int proc, float y, const MlpIn &in)
     return in.low ? (double)xs : 1.0 - (double)xs;  // (1 - xs in FP64 keeps a small xs)
 }
 
-// the output y whose map gives xi (the training target of a sample)
+// the output y whose map gives xi (the training target of a sample); with the
+// integer logarithm and quotient (physics.cuh): the library's log and log1p were a
+// serial chain of ~100 FP64 instructions ahead of every minibatch.  1 - xi rounds
+// by at most 2^-54, far below the FP32 result.
 __device__ __forceinline__ float mlp_target(int proc, double xi, const MlpIn &in)
 {
-    if (proc == QED_PROC_QS) return (float)(log(xi) - log1p(-xi)) - fmaf(3.0f, in.lnu, in.base);
+    if (proc == QED_PROC_QS) return (float)(log_int(xi) - log_int(1.0 - xi)) - fmaf(3.0f, in.lnu, in.base);
     double xs = in.low ? xi : 1.0 - xi;
     xs = xs < 1e-300 ? 1e-300 : (xs > 0.5 ? 0.5 : xs);
-    return (float)((log1p(-xs) - log(xs)) / (4.0 * (double)in.base));
+    return (float)e_div(log_int(1.0 - xs) - log_int(xs), 4.0 * (double)in.base);
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)

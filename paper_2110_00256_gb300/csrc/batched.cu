@@ -16,6 +16,7 @@
 
 #include "events.cuh"
 #include "evolve_core.cuh"
+#include "launch.cuh"
 #include "pipeline.cuh"
 #include "pusher.cuh"
 
@@ -182,6 +183,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : 4)
     const int n_seg = n_qs + n_bw;
     long long *s_end = reinterpret_cast<long long *>(smem_raw);
     long long *s_n = s_end + n_seg;
+    allow_next();
+    wait_previous();
     chunk_prefix<T>(qs, n_qs, bw, n_seg, s_end, s_n, s_warp);
     const long long total = s_end[n_seg - 1];
     const int64_t step = event_step(cq.d_step, cq.step);
@@ -272,6 +275,8 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1)
     __shared__ int s_abort;
 
     stage_rates(rs, tab, dt, THREADS);
+    allow_next();
+    wait_previous();
     if (threadIdx.x == 0) {
         s_abort = 0;
         for (int k = 0; k < S; ++k) {
@@ -388,9 +393,8 @@ static qed_status launch_evolve_seg_bulk(const EvolveSeg<float> *segs, int n_seg
                                           (int)(stage + 3 * QED_MAX_PATCHES * 2 * sizeof(long long))));
         attr = true;
     }
-    k<<<sm_count(), (kSegBulkCW + 1) * 32, dyn, st>>>(segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry,
-                                                       wait_cycles);
-    QED_LAUNCH_CHECK();
+    QED_CUDA_TRY(launch_next(false, k, sm_count(), (kSegBulkCW + 1) * 32, dyn, st, segs, n_seg, tab, dt, cut_qs, cut_bw, stats,
+                             dry, wait_cycles));
     return QED_OK;
 }
 
@@ -455,9 +459,8 @@ static qed_status launch_events_batched_all(const qed_batch *b, const EventCommo
         QED_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 256, kMaxDyn));
         attr = true;
     }
-    k<<<resident_grid(warps, per_sm), 256, dyn, st>>>((const EventSeg<T> *)b->d_qs, n_qs,
-                                                      (const EventSeg<T> *)b->d_bw, n_bw, cq, cb, end);
-    QED_LAUNCH_CHECK();
+    QED_CUDA_TRY(launch_next(few_particles(b->capacity_sum), k, resident_grid(warps, per_sm), 256, dyn, st, (const EventSeg<T> *)b->d_qs, n_qs,
+                             (const EventSeg<T> *)b->d_bw, n_bw, cq, cb, end));
     return QED_OK;
 }
 
@@ -556,9 +559,9 @@ static qed_status substep_batched_impl(const qed_tables *t, const qed_batch *b, 
     // particles one per thread (kSmallPerSm)
     const bool open = !(o && (o->evolve_threads || o->evolve_ctas_per_sm)) && !b->tuned &&
                       !(o && o->wait_limit_cycles);
-    const int64_t per_sm = b->capacity_sum / sm_count();
-    const bool small = open && !(o && o->evolve_pipeline != QED_EVOLVE_DEFAULT) && per_sm < kSmallPerSm;
-    const bool few = open && !(o && o->evolve_pipeline == QED_EVOLVE_BULK) && per_sm < kDirectPerSm;
+    const bool small = open && !(o && o->evolve_pipeline != QED_EVOLVE_DEFAULT) && few_particles(b->capacity_sum);
+    const bool few = open && !(o && o->evolve_pipeline == QED_EVOLVE_BULK) &&
+                     b->capacity_sum <= (int64_t)sm_count() * kDirectPerSm;
     const bool bulk = sizeof(T) == 4 && b->vec && !(o && (o->evolve_threads || o->evolve_ctas_per_sm)) &&
                       !(o && o->evolve_pipeline == QED_EVOLVE_DIRECT) && b->threads == 0 && b->ctas_per_sm == 0 && !few;
     if (o && o->evolve_begin) QED_CUDA_TRY(cudaEventRecord((cudaEvent_t)o->evolve_begin, st));
@@ -573,10 +576,10 @@ static qed_status substep_batched_impl(const qed_tables *t, const qed_batch *b, 
                                           (float)dt, cut_qs, cut_bw, stats, 0, o ? o->wait_limit_cycles : 0, st)
                  : launch_evolve_segments<T>((const EvolveSeg<T> *)b->d_evolve, 3 * n, make_view<T>(t), (T)dt,
                                              cut_qs, cut_bw, stats, 0, b->vec && !small, small ? 128 : threads,
-                                             ctas, st);
+                                             ctas, st, small);
     } else {
         s = launch_evolve_segments<T>((const EvolveSeg<T> *)b->d_evolve, 3 * n, make_view<T>(t), (T)dt, cut_qs,
-                                      cut_bw, stats, 0, b->vec && !small, small ? 128 : threads, ctas, st);
+                                      cut_bw, stats, 0, b->vec && !small, small ? 128 : threads, ctas, st, small);
     }
     if (s) return s;
     if (o && o->evolve_end) QED_CUDA_TRY(cudaEventRecord((cudaEvent_t)o->evolve_end, st));

@@ -7,6 +7,7 @@
 
 #include "events.cuh"
 #include "evolve.cuh"
+#include "launch.cuh"
 
 namespace qed {
 
@@ -84,6 +85,8 @@ __global__ void __launch_bounds__(256) events3_kernel(const __grid_constant__ Ev
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);  // (not touched without the learned sampler)
+    allow_next();
+    wait_previous();
     int64_t nf[3], c1, c2, c3;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -126,6 +129,8 @@ __global__ void __launch_bounds__(256) events3_kernel(const __grid_constant__ Ev
 
 __global__ void zero3(int64_t *a, int64_t *b, int64_t *c)
 {
+    allow_next();
+    wait_previous();
     if (threadIdx.x == 0) *a = 0, *b = 0, *c = 0;
 }
 
@@ -291,8 +296,8 @@ static qed_status substep_impl(const qed_tables *t, const qed_species *e, const 
     bool vec = fill_seg<T>(a.seg[0], e, QED_PROC_QS, &fire[0]);
     vec = fill_seg<T>(a.seg[1], p, QED_PROC_QS, &fire[1]) && vec;
     vec = fill_seg<T>(a.seg[2], g, QED_PROC_BW, &fire[2]) && vec;
-    zero3<<<1, 32, 0, st>>>(fire[0].d_count, fire[1].d_count, fire[2].d_count);
-    QED_LAUNCH_CHECK();
+    const bool early = few_particles(e->capacity + p->capacity + g->capacity);
+    QED_CUDA_TRY(launch_next(early, zero3, 1, 32, 0, st, fire[0].d_count, fire[1].d_count, fire[2].d_count));
     if (o && o->evolve_begin) QED_CUDA_TRY(cudaEventRecord((cudaEvent_t)o->evolve_begin, st));
     qed_status s = launch_evolve<T, 4>(a, vec, e->capacity + p->capacity + g->capacity, 0, st,
                                        o ? o->evolve_pipeline : 0, o ? o->evolve_threads : 0,
@@ -324,8 +329,7 @@ static qed_status substep_impl(const qed_tables *t, const qed_species *e, const 
         ea.bw = event_common<T>(t, QED_PROC_BW, seed, step, o);
         ea.step = o ? o->d_step : nullptr;
         const int g3 = event_grid<events3_kernel<T>>(0, fire[0].capacity + fire[1].capacity + fire[2].capacity);
-        events3_kernel<T><<<g3, 256, 0, st>>>(ea);
-        QED_LAUNCH_CHECK();
+        QED_CUDA_TRY(launch_next(early, events3_kernel<T>, g3, 256, 0, st, ea));
         return QED_OK;
     }
     clamp_all<<<1, 32, 0, st>>>(ptrs<T>(e).count, e->capacity, ptrs<T>(p).count, p->capacity, ptrs<T>(g).count,

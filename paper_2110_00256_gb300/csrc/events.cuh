@@ -67,7 +67,7 @@ struct EventCounts {
 
 template <typename T>
 __device__ __forceinline__ void write_particle(const SpeciesPtrs<T> &d, int64_t k, T px, T py, T pz, T ex, T ey,
-                                               T ez, T bx, T by, T bz, T w, uint64_t id, double tau,
+                                               T ez, T bx, T by, T bz, T w, uint64_t id,
                                                bool fields = true)
 {
     d.px[k] = px, d.py[k] = py, d.pz[k] = pz;
@@ -77,7 +77,6 @@ __device__ __forceinline__ void write_particle(const SpeciesPtrs<T> &d, int64_t 
     }
     d.w[k] = w;
     d.id[k] = id;
-    store_tau<T>(d.tau, d.tau_c, k, tau);
 }
 
 // the product sits where its parent is
@@ -91,8 +90,8 @@ __device__ __forceinline__ void copy_position(const SpeciesPtrs<T> &d, int64_t k
 template <typename T>
 __device__ __forceinline__ void write_dead(const SpeciesPtrs<T> &d, int64_t k)
 {
-    write_particle<T>(d, k, T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), ~0ull,
-                      (double)INFINITY);
+    write_particle<T>(d, k, T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), ~0ull);
+    store_tau<T>(d.tau, d.tau_c, k, (double)INFINITY);
     if (d.x) d.x[k] = T(0), d.y[k] = T(0), d.z[k] = T(0);
 }
 
@@ -154,12 +153,13 @@ __device__ __forceinline__ void qs_event_chunk(const EventSeg<T> &g, const Event
         const bool f = c.copy_fields != 0;
         write_particle<T>(G, slot, gg * nx, gg * ny, gg * nz, f ? P.ex[i] : T(0), f ? P.ey[i] : T(0),
                           f ? P.ez[i] : T(0), f ? P.bx[i] : T(0), f ? P.by[i] : T(0), f ? P.bz[i] : T(0), P.w[i],
-                          child, tau_draw(c.seed, child, step, kTauInit), f);
+                          child, f);
+        store_draw(G.tau, G.tau_c, slot, c.seed, child, step, kTauInit);
         copy_position<T>(G, slot, P, i);
     }
     if (exec) {
         P.px[i] = pn * nx, P.py[i] = pn * ny, P.pz[i] = pn * nz;
-        store_tau<T>(P.tau, P.tau_c, i, tau_draw(c.seed, pid, step, kTauReset));
+        store_draw(P.tau, P.tau_c, i, c.seed, pid, step, kTauReset);
     }
     k.exec += exec ? 1 : 0;
     k.kept += (keep && room) ? 1 : 0;
@@ -226,10 +226,10 @@ __device__ __forceinline__ void bw_event_chunk(const EventSeg<T> &g, const Event
         const uint64_t ide = ((uint64_t)cid.y << 32) | cid.x;
         const uint64_t idp = ((uint64_t)cid.w << 32) | cid.z;
         const T ex = P.ex[i], ey = P.ey[i], ez = P.ez[i], bx = P.bx[i], by = P.by[i], bz = P.bz[i], wt = P.w[i];
-        write_particle<T>(E, se, pmm * nx, pmm * ny, pmm * nz, ex, ey, ez, bx, by, bz, wt, ide,
-                          tau_draw(c.seed, ide, step, kTauInit));
-        write_particle<T>(Q, sq, pmp * nx, pmp * ny, pmp * nz, ex, ey, ez, bx, by, bz, wt, idp,
-                          tau_draw(c.seed, idp, step, kTauInit));
+        write_particle<T>(E, se, pmm * nx, pmm * ny, pmm * nz, ex, ey, ez, bx, by, bz, wt, ide);
+        store_draw(E.tau, E.tau_c, se, c.seed, ide, step, kTauInit);
+        write_particle<T>(Q, sq, pmp * nx, pmp * ny, pmp * nz, ex, ey, ez, bx, by, bz, wt, idp);
+        store_draw(Q.tau, Q.tau_c, sq, c.seed, idp, step, kTauInit);
         copy_position<T>(E, se, P, i);
         copy_position<T>(Q, sq, P, i);
         // the photon is removed
@@ -237,7 +237,7 @@ __device__ __forceinline__ void bw_event_chunk(const EventSeg<T> &g, const Event
         P.tau[i] = T(INFINITY);
         if (sizeof(T) == 4) P.tau_c[i] = T(0);
     }
-    if (valid && !pair) store_tau<T>(P.tau, P.tau_c, i, tau_draw(c.seed, pid, step, kTauReset));
+    if (valid && !pair) store_draw(P.tau, P.tau_c, i, c.seed, pid, step, kTauReset);
     k.exec += exec ? 1 : 0;
     k.pairs += (pair && room) ? 1 : 0;
     k.nopair += (valid && !pair) ? 1 : 0;

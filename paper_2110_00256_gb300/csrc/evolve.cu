@@ -76,6 +76,8 @@ __global__ void __launch_bounds__(THREADS, MINB)
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
     stage_rates(rs, a.tab, a.dt, blockDim.x);
+    allow_next();
+    wait_previous();
     if (threadIdx.x == 0) {
         long long acc = 0;
         for (int s = 0; s < a.n_seg; ++s) {
@@ -156,6 +158,8 @@ __global__ void __launch_bounds__((CW + 1) * 32, MINB)
     __shared__ int s_abort;
 
     stage_rates(rs, a.tab, a.dt, blockDim.x);
+    allow_next();
+    wait_previous();
     if (threadIdx.x == 0) {
         long long acc = 0;
         for (int s = 0; s < a.n_seg; ++s) {
@@ -283,8 +287,7 @@ static qed_status launch_bulk(const EvolveArgs<float, MAXSEG> &a, int64_t capaci
     const int64_t tiles = (capacity_sum + tp - 1) / tp;
     int64_t g = (int64_t)sm_count() * MINB;
     if (tiles < g) g = tiles < 1 ? 1 : tiles;
-    evolve_bulk_kernel<CW, S, MINB, MAXSEG><<<(int)g, (CW + 1) * 32, dyn, st>>>(a);
-    QED_LAUNCH_CHECK();
+    QED_CUDA_TRY(launch_next(false, evolve_bulk_kernel<CW, S, MINB, MAXSEG>, (int)g, (CW + 1) * 32, dyn, st, a));
     return QED_OK;
 }
 
@@ -304,6 +307,8 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS)
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
     stage_rates(rs, tab, dt, THREADS);
+    allow_next();
+    wait_previous();
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);
     int bad = 0;
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {
@@ -318,7 +323,8 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS)
 
 template <typename T, int THREADS>
 static qed_status launch_seg_impl(const EvolveSeg<T> *segs, int n_seg, const TablesView<T> &tab, T dt, T cut_qs,
-                                  T cut_bw, long long *stats, int dry, bool vec, int ctas_per_sm, cudaStream_t st)
+                                  T cut_bw, long long *stats, int dry, bool vec, int ctas_per_sm, cudaStream_t st,
+                                  bool early)
 {
     const size_t dyn = (size_t)n_seg * 2 * sizeof(long long);
     int grid = sm_count() * (ctas_per_sm > 0 ? ctas_per_sm : 768 / THREADS);
@@ -332,8 +338,8 @@ static qed_status launch_seg_impl(const EvolveSeg<T> *segs, int n_seg, const Tab
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
             attr = true;
         }
-        evolve_seg_kernel<T, V, THREADS><<<grid, THREADS, dyn, st>>>(segs, n_seg, tab, dt, cut_qs, cut_bw, stats,
-                                                                      dry);
+        QED_CUDA_TRY(launch_next(false, evolve_seg_kernel<T, V, THREADS>, grid, THREADS, dyn, st, segs, n_seg, tab, dt, cut_qs,
+                                 cut_bw, stats, dry));
     } else {
         static bool attr = false;
         if (!attr) {
@@ -341,8 +347,8 @@ static qed_status launch_seg_impl(const EvolveSeg<T> *segs, int n_seg, const Tab
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn));
             attr = true;
         }
-        evolve_seg_kernel<T, 1, THREADS><<<grid, THREADS, dyn, st>>>(segs, n_seg, tab, dt, cut_qs, cut_bw, stats,
-                                                                      dry);
+        QED_CUDA_TRY(launch_next(early, evolve_seg_kernel<T, 1, THREADS>, grid, THREADS, dyn, st, segs, n_seg, tab, dt, cut_qs,
+                                 cut_bw, stats, dry));
     }
     QED_LAUNCH_CHECK();
     return QED_OK;
@@ -351,24 +357,27 @@ static qed_status launch_seg_impl(const EvolveSeg<T> *segs, int n_seg, const Tab
 template <typename T>
 qed_status launch_evolve_segments(const EvolveSeg<T> *d_segs, int n_seg, const TablesView<T> &tab, T dt, T cut_qs,
                                   T cut_bw, long long *stats, int dry, bool vec, int threads, int ctas_per_sm,
-                                  cudaStream_t st)
+                                  cudaStream_t st, bool early)
 {
     if (n_seg <= 0) return QED_OK;
     switch (threads) {
     case 128:
-        return launch_seg_impl<T, 128>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st);
+        return launch_seg_impl<T, 128>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st,
+                                       early);
     case 512:
-        return launch_seg_impl<T, 512>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st);
+        return launch_seg_impl<T, 512>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st,
+                                       early);
     default:
-        return launch_seg_impl<T, 256>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st);
+        return launch_seg_impl<T, 256>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st,
+                                       early);
     }
 }
 
 template qed_status launch_evolve_segments<float>(const EvolveSeg<float> *, int, const TablesView<float> &, float,
-                                                  float, float, long long *, int, bool, int, int, cudaStream_t);
+                                                  float, float, long long *, int, bool, int, int, cudaStream_t, bool);
 template qed_status launch_evolve_segments<double>(const EvolveSeg<double> *, int, const TablesView<double> &,
                                                    double, double, double, long long *, int, bool, int, int,
-                                                   cudaStream_t);
+                                                   cudaStream_t, bool);
 
 // clamp the firing counters to their capacity once the evolution is done
 __global__ void clamp_fire_counts(unsigned long long *c0, int64_t cap0, unsigned long long *c1, int64_t cap1,
@@ -417,11 +426,10 @@ qed_status launch_evolve(const EvolveArgs<T, MAXSEG> &a, bool vec_ok, int64_t ca
     // the grid is sized from the capacities (counts live on the device); idle
     // CTAs exit after reading the counts
     if (pipeline == QED_EVOLVE_DEFAULT && threads == 0 && ctas_per_sm == 0 && grid_override <= 0 &&
-        a.wait_cycles == 0 && capacity_sum <= (int64_t)sm_count() * kSmallPerSm) {
+        a.wait_cycles == 0 && few_particles(capacity_sum)) {
         // few particles: one per thread in CTAs of 64 (kSmallPerSm)
         const int g = evolve_grid<T, 1, MAXSEG, 8, 64>(capacity_sum);
-        evolve_kernel<T, 1, MAXSEG, 8, 64><<<g, 64, 0, st>>>(a);
-        QED_LAUNCH_CHECK();
+        QED_CUDA_TRY(launch_next(true, evolve_kernel<T, 1, MAXSEG, 8, 64>, g, 64, 0, st, a));
         return QED_OK;
     }
     if constexpr (sizeof(T) == 4) {
@@ -443,17 +451,17 @@ qed_status launch_evolve(const EvolveArgs<T, MAXSEG> &a, bool vec_ok, int64_t ca
         if constexpr (sizeof(T) == 4) {
             if (ctas_per_sm != 3) {  // 64 registers: 32 warps per SM (the faster)
                 const int g = grid_override > 0 ? grid_override : evolve_grid<T, V, MAXSEG, 4>(capacity_sum);
-                evolve_kernel<T, V, MAXSEG, 4><<<g, kEvolveThreads, 0, st>>>(a);
+                QED_CUDA_TRY(launch_next(false, evolve_kernel<T, V, MAXSEG, 4>, g, kEvolveThreads, 0, st, a));
                 done = true;
             }
         }
         if (!done) {
             const int g = grid_override > 0 ? grid_override : evolve_grid<T, V, MAXSEG>(capacity_sum);
-            evolve_kernel<T, V, MAXSEG><<<g, kEvolveThreads, 0, st>>>(a);
+            QED_CUDA_TRY(launch_next(false, evolve_kernel<T, V, MAXSEG>, g, kEvolveThreads, 0, st, a));
         }
     } else {
         const int g = grid_override > 0 ? grid_override : evolve_grid<T, 1, MAXSEG>(capacity_sum);
-        evolve_kernel<T, 1, MAXSEG><<<g, kEvolveThreads, 0, st>>>(a);
+        QED_CUDA_TRY(launch_next(false, evolve_kernel<T, 1, MAXSEG>, g, kEvolveThreads, 0, st, a));
     }
     QED_LAUNCH_CHECK();
     return QED_OK;
@@ -509,7 +517,7 @@ __global__ void init_tau_kernel(T *tau, T *tau_c, const uint64_t *id, const int6
     int64_t n = *count;
     n = n < 0 ? 0 : (n > capacity ? capacity : n);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        store_tau<T>(tau, tau_c, i, tau_draw(seed, id[i], step, kTauInit));
+        store_draw(tau, tau_c, i, seed, id[i], step, kTauInit);
 }
 
 }  // namespace qed

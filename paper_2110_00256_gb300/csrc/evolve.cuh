@@ -19,6 +19,8 @@ constexpr int kEvolveThreads = 256;
 // 18.4 / 18.9 (1.2e5), 28.8 / 28.1 (4e5).  Few particles want a short chain per
 // thread and all SMs; the bulk pipeline pays from several tiles per CTA on.
 constexpr int64_t kSmallPerSm = 1024, kDirectPerSm = 49152;
+int sm_count();
+inline bool few_particles(int64_t capacity_sum) { return capacity_sum <= (int64_t)sm_count() * kSmallPerSm; }
 
 template <typename T>
 struct EvolveSeg {
@@ -61,7 +63,7 @@ bool fill_seg(EvolveSeg<T> &g, const qed_species *sp, int proc, const qed_fire_l
 template <typename T>
 qed_status launch_evolve_segments(const EvolveSeg<T> *d_segs, int n_seg, const TablesView<T> &tab, T dt, T cut_qs,
                                   T cut_bw, long long *stats, int dry, bool vec, int threads, int ctas_per_sm,
-                                  cudaStream_t st);
+                                  cudaStream_t st, bool early = false);
 
 qed_status check_fire(const qed_fire_list *f, const char *name);
 

@@ -243,12 +243,11 @@ __device__ __forceinline__ double fix_div(double a, double b)
     return fix_to_double(q, ((ha >> 20) & 0x7ff) - ((hb >> 20) & 0x7ff) - 61);
 }
 
-// ln(n 2^e) (minus it with `neg`: an FP64 sign change is an FP64 instruction) as a
-// double for n in [2^63, 2^64), |ln| < 62: the reduction of
+// ln(n 2^e) = v 2^unit for n in [2^63, 2^64), |ln| < 62: the reduction of
 // fix_half_ln with the cubic term to 2^-58; within 2^-57 absolute, and 2^-53
 // relative (one rounding) above 1/8.  No FP64 instruction: one costs as much as
 // 76 issue slots, this function ~60.
-__device__ __forceinline__ double fix_ln(uint64_t n, int e, bool neg = false)
+__device__ __forceinline__ int64_t fix_ln_value(uint64_t n, int e, int &unit)
 {
     const int j = (int)(n >> 55) & 255;
     const uint32_t r = (uint32_t)__ldg(&kFixLogR[j]);
@@ -265,8 +264,15 @@ __device__ __forceinline__ double fix_ln(uint64_t n, int e, bool neg = false)
     // k ln 2 + ln m in 2^-57, or in 2^-63 where k is 0 or -1
     const bool fine = k == 0 || k == -1;
     const int64_t kl = (wide(k, (int)(kHalfLn2 >> 32)) << 27) + (wide(k, (int)((uint32_t)kHalfLn2 >> 1)) >> 4);
-    const int64_t v = fine ? (k ? l - 2 * kHalfLn2 : l) : kl + (l >> 6);
-    return fix_to_double(neg ? -v : v, fine ? -63 : -57);
+    unit = fine ? -63 : -57;
+    return fine ? (k ? l - 2 * kHalfLn2 : l) : kl + (l >> 6);
+}
+
+__device__ __forceinline__ double fix_ln(uint64_t n, int e)
+{
+    int unit;
+    const int64_t v = fix_ln_value(n, e, unit);
+    return fix_to_double(v, unit);
 }
 
 // ---------------------------------------------------------------------------

@@ -157,6 +157,42 @@ __device__ __forceinline__ double chi_photon(double px, double py, double pz, do
     return sqrt(s < 0.0 ? 0.0 : s);
 }
 
+// The same in fields with only Ey and Bz (a linearly polarised wave along x), the
+// terms with a zero factor left out (the compiler may not do that by itself): a
+// product of a finite number and zero added to another number changes nothing
+// but the sign of a zero, and every sum below is squared, so a finite
+// particle's chi has the same bits, with the roundings as the full forms
+// contract; a momentum component that is not finite still gives a chi that is not.
+__device__ __forceinline__ float chi_lepton_yz(float px, float py, float pz, float ey, float bz, float &gamma,
+                                               float &inv_gamma)
+{
+    const float p2 = px * px + py * py + pz * pz;
+    gamma = sqrtf(1.0f + p2);
+    inv_gamma = 1.0f / gamma;
+    const float pm = sqrtf(p2);
+    const float inv = pm > 0.0f ? 1.0f / pm : 0.0f;
+    const float nx = px * inv, ny = py * inv, nz = pz * inv;
+    const float ne = __fmul_rn(ny, ey);
+    const float fx = fmaf(gamma, -__fmul_rn(ne, nx), __fmul_rn(py, bz));
+    const float fy = fmaf(gamma, fmaf(-ne, ny, ey), -__fmul_rn(px, bz));
+    const float fz = __fmul_rn(gamma, -__fmul_rn(ne, nz));
+    const float s = fx * fx + fy * fy + fz * fz + (p2 > 0.0f ? ne * ne : ey * ey);
+    return sqrtf(s);
+}
+
+__device__ __forceinline__ float chi_photon_yz(float px, float py, float pz, float ey, float bz, float &pm, float &inv_pm)
+{
+    const float p2 = px * px + py * py + pz * pz;
+    inv_pm = p2 > 0.0f ? rsqrtf(p2) : 0.0f;
+    pm = p2 * inv_pm;
+    const float nx = px * inv_pm, ny = py * inv_pm, nz = pz * inv_pm;
+    const float ne = __fmul_rn(ny, ey);
+    const float fx = fmaf(pm, -__fmul_rn(ne, nx), __fmul_rn(py, bz));
+    const float fy = fmaf(pm, fmaf(-ne, ny, ey), -__fmul_rn(px, bz));
+    const float fz = __fmul_rn(pm, -__fmul_rn(ne, nz));
+    return sqrtf(fx * fx + fy * fy + fz * fz);
+}
+
 // log-log interpolation of a 1-D table held in `tab` (shared or global):
 // ln f(chi) = ln f_n + (ln chi - ln chi_n) (ln f_{n+1} - ln f_n) / (ln chi_{n+1} - ln chi_n),
 // n = clamp(floor((ln chi - ln chi_min) / d), 0, N - 2); chi clamped into the table.
@@ -413,22 +449,65 @@ static __device__ __noinline__ double neg_log1p_series(double u)
     return fma(d * d, q, -d);  // -(d - d^2/2 + d^3/3 - ... - d^7/7)
 }
 
-__device__ __forceinline__ double neg_log_u(double u)
+// -ln U = v 2^unit for the 53-bit uniform U of the words (uniform53: M 2^-k, M from
+// the words' bits), without assembling U; false: U above 1 - 2^-8, by the series
+__device__ __forceinline__ bool neg_log_words(const U4 &w, int64_t &v, int &unit)
 {
-    // (positive doubles order as their bit patterns: the test costs no FP64
-    // instruction; the series is out of line, so that the other 99.6 % of the
-    // draws do not issue it predicated off; U >= 2^-54 is normal)
-    if (__double_as_longlong(u) > __double_as_longlong(1.0 - 0x1p-8)) return neg_log1p_series(u);
-    const int hi = __double2hiint(u);
-    const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(u);
-    return fix_ln(m << 11, (hi >> 20) - 1023 - 63, true);
+    const uint64_t d = (((uint64_t)w.y << 32) | w.x) >> 11;
+    const bool big = d >= (1ull << 52);
+    const uint64_t m = big ? d + (d & 1ull) : 2ull * d + 1ull;
+    const int lz = __clzll((long long)m), e = (big ? -53 : -54) - lz;
+    const uint64_t n = m << lz;  // U = n 2^e
+    if (e >= -64 && (e > -64 || (n >> 56) == 255)) return false;
+    v = -fix_ln_value(n, e, unit);
+    return true;
 }
 
-// tau = -ln U, U the 53-bit uniform of (seed, (id, step, purpose)), in FP64 (§3)
+// tau = -ln U, U the 53-bit uniform of (seed, (id, step, purpose)), to FP64 (§3)
 __device__ __forceinline__ double tau_draw(uint64_t seed, uint64_t id, int64_t step, uint32_t purpose)
 {
     const U4 w = draw(seed, id, step, purpose);
-    return neg_log_u(uniform53(w.x, w.y));
+    int64_t v;
+    int unit;
+    if (!neg_log_words(w, v, unit)) return neg_log1p_series(uniform53(w.x, w.y));
+    return fix_to_double(v, unit);
+}
+
+// (h, c) = (fl32(x), fl32(h - x)) of x = v 2^unit, v > 0 with x far inside the
+// normal floats: the top 24 of v's bits, rounded to nearest even, and the residual
+// (its upper 31 bits) by one integer-to-float conversion
+__device__ __forceinline__ void split_fixed(int64_t v, int unit, float &h, float &c)
+{
+    const int lz = __clzll((long long)v);
+    const uint64_t n = (uint64_t)v << lz, rem = n & 0xffffffffffull;  // the other 40
+    unsigned int keep = (unsigned int)(n >> 40);
+    const bool up = rem > 0x8000000000ull || (rem == 0x8000000000ull && (keep & 1u));
+    const int64_t diff = up ? (int64_t)(0x10000000000ull - rem) : -(int64_t)rem;  // (h - x) / 2^(unit - lz)
+    keep += up ? 1u : 0u;  // (2^24 carries into the exponent)
+    const int e = unit - lz;
+    h = __uint_as_float(((unsigned int)(e + 63 + 126) << 23) + keep);
+    c = __int2float_rn((int)(diff >> 9)) * __uint_as_float((unsigned int)(e + 9 + 127) << 23);
+}
+
+// store tau = -ln U of (seed, (id, step, purpose)): FP64 as is, FP32 as the float pair
+__device__ __forceinline__ void store_draw(double *tau, double *, int64_t i, uint64_t seed, uint64_t id, int64_t step,
+                                           uint32_t purpose)
+{
+    tau[i] = tau_draw(seed, id, step, purpose);
+}
+__device__ __forceinline__ void store_draw(float *tau, float *tau_c, int64_t i, uint64_t seed, uint64_t id,
+                                           int64_t step, uint32_t purpose)
+{
+    const U4 w = draw(seed, id, step, purpose);
+    int64_t v;
+    int unit;
+    float h, c;
+    if (neg_log_words(w, v, unit))
+        split_fixed(v, unit, h, c);
+    else
+        split_f32_pair(neg_log1p_series(uniform53(w.x, w.y)), h, c);
+    tau[i] = h;
+    tau_c[i] = c;
 }
 
 }  // namespace qed

@@ -114,6 +114,39 @@ __device__ __forceinline__ void stage_rates(RateSmem<double> &s, const TablesVie
     for (int i = threadIdx.x; i < 256; i += threads) s.ln[i] = kFixLog[i], s.ex[i] = kFixExp[i], s.r[i] = kFixLogR[i];
 }
 
+// the FP32 decrement of one particle's optical depth by its rate; returns fire
+__device__ __forceinline__ bool decrement(float chi, float rate, float dt, float cut, float &tau, float &tc,
+                                          float &chi_out, int &bad)
+{
+    const bool ok = isfinite(chi) && !isnan(tau) && isfinite(rate);
+    bad += ok ? 0 : 1;
+    if (!ok || chi < cut) rate = 0.0f;  // below the process's chi threshold: no evolution
+    chi_out = chi;
+    // Kahan-compensated decrement; tau - tc is the optical depth
+    if (!isfinite(tau)) return false;  // removed particle (tau = +inf)
+    const float y = d_fma(-rate, dt, -tc);
+    const float t = tau + y;
+    tc = (t - tau) - y;
+    tau = t;
+    return ok && (t < 0.0f || (t == 0.0f && tc > 0.0f));
+}
+
+// one particle in the linearly polarised wave's fields (Ey, Bz)
+__device__ __forceinline__ bool evolve_one_yz(int proc, const RateSmem<float> &rs, const TablesView<float> &tv,
+                                              float px, float py, float pz, float ey, float bz, float dt, float cut,
+                                              float &tau, float &tc, float &chi_out, int &bad)
+{
+    float chi, rate, en, inv;
+    if (proc == QED_PROC_QS) {
+        chi = chi_lepton_yz(px, py, pz, ey, bz, en, inv);
+        rate = qs_rate(rs.qs, tv.qs_G, chi, en, inv);
+    } else {
+        chi = chi_photon_yz(px, py, pz, ey, bz, en, inv);
+        rate = bw_rate(rs.bw, tv.bw_T, chi, en, inv);
+    }
+    return decrement(chi, rate, dt, cut, tau, tc, chi_out, bad);
+}
+
 // one particle: chi, rate, optical-depth decrement; returns fire
 __device__ __forceinline__ bool evolve_one(int proc, const RateSmem<float> &rs, const TablesView<float> &tv, float px,
                                            float py, float pz, float ex, float ey, float ez, float bx, float by,
@@ -130,17 +163,7 @@ __device__ __forceinline__ bool evolve_one(int proc, const RateSmem<float> &rs, 
         chi = chi_photon(px, py, pz, ex, ey, ez, bx, by, bz, pm, inv);
         rate = bw_rate(rs.bw, tv.bw_T, chi, pm, inv);
     }
-    const bool ok = isfinite(chi) && !isnan(tau) && isfinite(rate);
-    bad += ok ? 0 : 1;
-    if (!ok || chi < cut) rate = 0.0f;  // below the process's chi threshold: no evolution
-    chi_out = chi;
-    // Kahan-compensated decrement; tau - tc is the optical depth
-    if (!isfinite(tau)) return false;  // removed particle (tau = +inf)
-    const float y = d_fma(-rate, dt, -tc);
-    const float t = tau + y;
-    tc = (t - tau) - y;
-    tau = t;
-    return ok && (t < 0.0f || (t == 0.0f && tc > 0.0f));
+    return decrement(chi, rate, dt, cut, tau, tc, chi_out, bad);
 }
 
 struct EvolvedFp64 {

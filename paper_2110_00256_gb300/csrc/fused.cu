@@ -7,7 +7,10 @@
 // arithmetic is the separate kernels' own (pusher.cuh, evolve_core.cuh), so
 // the particles end with the same bits; only the field arrays are left alone
 // unless asked for.
+#include <type_traits>
+
 #include "evolve_core.cuh"
+#include "launch.cuh"
 #include "pusher.cuh"
 
 namespace qed {
@@ -35,9 +38,13 @@ __device__ __forceinline__ void store_live(T *p, int64_t i0, int64_t n, bool ful
     }
 }
 
+// YZ (FP32): the linearly polarised wave, whose only fields are Ey and Bz, with the
+// zero terms of the push and of chi left out; the particles end with the same
+// bits.  The kernel is bound by its instruction issue, 10:1 photons to electrons
+// in the cascade: 308 instructions per particle without.
 // FP32: two particles per thread, 4 CTAs of 256 per SM (64 registers), the
 // fastest of VEC 1 / 2 / 4 x 2 .. 4 CTAs per SM measured on GB300
-template <typename T, int VEC, int THREADS>
+template <typename T, int VEC, int THREADS, bool YZ>
 __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     push_evolve_kernel(const EvolveSeg<T> *__restrict__ segs, const PushSeg<T> *__restrict__ psegs, int n_seg,
                        const __grid_constant__ TablesView<T> tab, WaveT<T> wt, double t0, double dt_d,
@@ -51,6 +58,8 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
     stage_rates(rs, tab, wt.dt, THREADS);
+    allow_next();
+    wait_previous();
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);
     wt.t = (T)(t0 + (double)(d_step ? *d_step : step) * dt_d);
     const T dt = wt.dt;
@@ -86,18 +95,28 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
 #pragma unroll
         for (int j = 0; j < VEC; ++j) {
             T ex, ey, ez, bx, by, bz, vx, vy, vz;
-            wave_fields<T>(wt, x[j], ex, ey, ez, bx, by, bz);
-            boris_move<T>(pg.q, dt, ex, ey, ez, bx, by, bz, px[j], py[j], pz[j], vx, vy, vz);
+            if constexpr (YZ) {
+                wave_fields_yz(wt, x[j], ey, bz);
+                boris_move_yz(pg.q, dt, ey, bz, px[j], py[j], pz[j], vx, vy, vz);
+            } else {
+                wave_fields<T>(wt, x[j], ex, ey, ez, bx, by, bz);
+                boris_move<T>(pg.q, dt, ex, ey, ez, bx, by, bz, px[j], py[j], pz[j], vx, vy, vz);
+            }
             x[j] = x[j] + vx * dt;
             y[j] = y[j] + vy * dt;
             z[j] = z[j] + vz * dt;
-            if (store_fields && i0 + j < n) {
-                pg.ex[i0 + j] = ex, pg.ey[i0 + j] = ey, pg.ez[i0 + j] = ez;
-                pg.bx[i0 + j] = bx, pg.by[i0 + j] = by, pg.bz[i0 + j] = bz;
+            if constexpr (!YZ) {
+                if (store_fields && i0 + j < n) {
+                    pg.ex[i0 + j] = ex, pg.ey[i0 + j] = ey, pg.ez[i0 + j] = ez;
+                    pg.bx[i0 + j] = bx, pg.by[i0 + j] = by, pg.bz[i0 + j] = bz;
+                }
             }
             T c = tc[j];
-            fire[j] = evolve_one(sg.proc, rs, tab, px[j], py[j], pz[j], ex, ey, ez, bx, by, bz, dt, cut,
-                                    tau[j], c, chi[j], bad);
+            if constexpr (YZ)
+                fire[j] = evolve_one_yz(sg.proc, rs, tab, px[j], py[j], pz[j], ey, bz, dt, cut, tau[j], c, chi[j], bad);
+            else
+                fire[j] = evolve_one(sg.proc, rs, tab, px[j], py[j], pz[j], ex, ey, ez, bx, by, bz, dt, cut, tau[j], c,
+                                     chi[j], bad);
             tc[j] = c;
             fire[j] = fire[j] && (i0 + j < n);
             cnt += fire[j] ? 1 : 0;
@@ -118,7 +137,7 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     if (stats && blockIdx.x == 0 && threadIdx.x < 32) count_evolved(s_n, n_seg, stats);
 }
 
-template <typename T, int VEC>
+template <typename T, int VEC, bool YZ>
 static qed_status launch_fused_impl(const EvolveSeg<T> *segs, const PushSeg<T> *psegs, int n_seg,
                                     const TablesView<T> &tab, const WaveParams &w, double t0, double dt,
                                     const int64_t *d_step, int64_t step, T cut_qs, T cut_bw, long long *stats,
@@ -129,17 +148,16 @@ static qed_status launch_fused_impl(const EvolveSeg<T> *segs, const PushSeg<T> *
     static bool attr = false;
     static int per_sm = 0;
     if (!attr) {
-        QED_CUDA_TRY(cudaFuncSetAttribute(push_evolve_kernel<T, VEC, kThreads>,
+        QED_CUDA_TRY(cudaFuncSetAttribute(push_evolve_kernel<T, VEC, kThreads, YZ>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           3 * QED_MAX_PATCHES * 2 * (int)sizeof(long long)));
-        QED_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, push_evolve_kernel<T, VEC, kThreads>,
+        QED_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, push_evolve_kernel<T, VEC, kThreads, YZ>,
                                                                    kThreads, dyn));
         if (per_sm < 1) per_sm = 1;
         attr = true;
     }
-    push_evolve_kernel<T, VEC, kThreads><<<sm_count() * per_sm, kThreads, dyn, st>>>(
-        segs, psegs, n_seg, tab, wave_in<T>(w, dt), t0, dt, d_step, step, cut_qs, cut_bw, stats, store_fields);
-    QED_LAUNCH_CHECK();
+    QED_CUDA_TRY(launch_next(false, push_evolve_kernel<T, VEC, kThreads, YZ>, sm_count() * per_sm, kThreads, dyn, st, segs, psegs,
+                             n_seg, tab, wave_in<T>(w, dt), t0, dt, d_step, step, cut_qs, cut_bw, stats, store_fields));
     return QED_OK;
 }
 
@@ -150,13 +168,16 @@ qed_status launch_push_evolve(const EvolveSeg<T> *d_segs, const void *d_push, in
 {
     if (n_seg <= 0) return QED_OK;
     const PushSeg<T> *p = (const PushSeg<T> *)d_push;
-    if (vec) {
-        constexpr int V = 2;
-        return launch_fused_impl<T, V>(d_segs, p, n_seg, tab, w, t0, dt, d_step, step, cut_qs, cut_bw, stats,
-                                       store_fields, st);
+    const auto launch = [&](auto v, auto yz) {
+        return launch_fused_impl<T, v.value, yz.value>(d_segs, p, n_seg, tab, w, t0, dt, d_step, step, cut_qs, cut_bw,
+                                                       stats, store_fields, st);
+    };
+    using One = std::integral_constant<int, 1>;
+    using Two = std::integral_constant<int, 2>;
+    if constexpr (sizeof(T) == 4) {
+        if (!w.circular && !store_fields) return vec ? launch(Two{}, std::true_type{}) : launch(One{}, std::true_type{});
     }
-    return launch_fused_impl<T, 1>(d_segs, p, n_seg, tab, w, t0, dt, d_step, step, cut_qs, cut_bw, stats,
-                                   store_fields, st);
+    return vec ? launch(Two{}, std::false_type{}) : launch(One{}, std::false_type{});
 }
 
 template qed_status launch_push_evolve<float>(const EvolveSeg<float> *, const void *, int, const TablesView<float> &,

@@ -58,6 +58,16 @@ __device__ __forceinline__ void wave_fields(const WaveT<T> &w, T x, T &ex, T &ey
     bz = w.d * ey;
 }
 
+// the linearly polarised wave's fields that are not zero (without the sine)
+__device__ __forceinline__ void wave_fields_yz(const WaveT<float> &w, float x, float &ey, float &bz)
+{
+    const float u = w.omega_pi * (w.t - w.d * x) + w.phase0_pi;
+    float s, c;
+    d_sincospi(u, &s, &c);
+    ey = w.e0 * c;
+    bz = w.d * ey;
+}
+
 // reciprocal square root: FP32 rsqrtf (within 2 ulp), FP64 rsqrt (within 1 ulp);
 // the push is not part of the paper's method, and its arithmetic budget is the
 // fused cascade kernel's limit
@@ -87,6 +97,30 @@ __device__ __forceinline__ void boris_move(T q, T dt, T ex, T ey, T ez, T bx, T 
     py = my + (qz * sx - qx * sz) + h * ey;
     pz = mz + (qx * sy - qy * sx) + h * ez;
     const T ig = d_rsqrt(T(1) + px * px + py * py + pz * pz);
+    vx = px * ig, vy = py * ig, vz = pz * ig;
+}
+
+// the same in fields with only Ey and Bz, the terms with a zero factor left out
+// (bit for bit the same for finite momenta, see chi_lepton_yz)
+__device__ __forceinline__ void boris_move_yz(float q, float dt, float ey, float bz, float &px, float &py, float &pz,
+                                              float &vx, float &vy, float &vz)
+{
+    if (q == 0.0f) {
+        const float p2 = px * px + py * py + pz * pz;
+        const float inv = p2 > 0.0f ? d_rsqrt(p2) : 0.0f;
+        vx = px * inv, vy = py * inv, vz = pz * inv;
+        return;
+    }
+    const float h = 0.5f * q * dt;
+    const float my = fmaf(h, ey, py);  // half electric kick
+    const float hg = h * d_rsqrt(1.0f + px * px + my * my + pz * pz);
+    const float tz = __fmul_rn(hg, bz);
+    const float f = 2.0f / fmaf(tz, tz, 1.0f);
+    const float sz = __fmul_rn(f, tz);
+    const float qx = __fadd_rn(px, __fmul_rn(my, tz)), qy = __fadd_rn(my, -__fmul_rn(px, tz));
+    px = __fadd_rn(px, __fmul_rn(qy, sz));
+    py = fmaf(h, ey, __fadd_rn(my, -__fmul_rn(qx, sz)));
+    const float ig = d_rsqrt(1.0f + px * px + py * py + pz * pz);
     vx = px * ig, vy = py * ig, vz = pz * ig;
 }
 

@@ -92,11 +92,31 @@ __device__ __forceinline__ void end_step(const StepEnd &f)
 
 // Block-wide prefix of the 32-entry chunk counts of n_seg firing lists into
 // s_end (inclusive); s_n receives the clamped list lengths.  The lists are
-// a[0 .. na) followed by b[0 .. n_seg - na).
+// a[0 .. na) followed by b[0 .. n_seg - na).  Up to 32 lists: by the first warp,
+// one list per lane, with one barrier.
 template <typename T>
 __device__ void chunk_prefix(const EventSeg<T> *a, int na, const EventSeg<T> *b, int n_seg, long long *s_end,
                              long long *s_n, long long *s_warp)
 {
+    if (n_seg <= 32) {
+        if (threadIdx.x < 32) {
+            const int s = threadIdx.x;
+            long long n = 0;
+            if (s < n_seg) {
+                const EventSeg<T> &g = s < na ? a[s] : b[s - na];
+                n = fire_n(g.fire_count, g.fire_cap);
+            }
+            long long incl = (n + 31) / 32;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (s >= o) incl += v;
+            }
+            if (s < n_seg) s_n[s] = n, s_end[s] = incl;
+        }
+        __syncthreads();
+        return;
+    }
     const int per = (n_seg + blockDim.x - 1) / blockDim.x;
     const int s0 = threadIdx.x * per, s1 = min(n_seg, s0 + per);
     long long local = 0;

@@ -61,8 +61,10 @@ struct EventCommon {
     int copy_fields;          // 0: products get no field values (the caller computes them, see qed_push_substep_batched)
 };
 
+// per-lane event counts; worked (the same in the whole warp): some chunk was run
 struct EventCounts {
     int exec = 0, kept = 0, disc = 0, drop = 0, pairs = 0, nopair = 0;
+    bool worked = false;
 };
 
 template <typename T>
@@ -161,6 +163,7 @@ __device__ __forceinline__ void qs_event_chunk(const EventSeg<T> &g, const Event
         P.px[i] = pn * nx, P.py[i] = pn * ny, P.pz[i] = pn * nz;
         store_draw(P.tau, P.tau_c, i, c.seed, pid, step, kTauReset);
     }
+    k.worked = true;
     k.exec += exec ? 1 : 0;
     k.kept += (keep && room) ? 1 : 0;
     k.disc += (exec && !keep) ? 1 : 0;
@@ -238,6 +241,7 @@ __device__ __forceinline__ void bw_event_chunk(const EventSeg<T> &g, const Event
         if (sizeof(T) == 4) P.tau_c[i] = T(0);
     }
     if (valid && !pair) store_draw(P.tau, P.tau_c, i, c.seed, pid, step, kTauReset);
+    k.worked = true;
     k.exec += exec ? 1 : 0;
     k.pairs += (pair && room) ? 1 : 0;
     k.nopair += (valid && !pair) ? 1 : 0;
@@ -245,6 +249,9 @@ __device__ __forceinline__ void bw_event_chunk(const EventSeg<T> &g, const Event
 
 __device__ __forceinline__ void flush_counts(long long *stats, const EventCounts &k, bool qs)
 {
+    // (in a sparse step nearly every warp is idle, and these reductions would be
+    // most of its instructions)
+    if (!k.worked) return;
     if (k.drop) note_error(QED_EW_CAPACITY);
     if (!stats) return;
     if (qs) {

@@ -243,10 +243,10 @@ struct GenArgs {
     double *qs_lnG, *qs_lnP, *bw_lnT, *bw_P;
     double qs_l0, qs_l1, qs_xi_min, qs_ln_xi_min, bw_l0, bw_l1;
     int qs_n_chi, qs_n_xi, bw_n_chi, bw_n_xi;
-    int *points;  // [2][n_xi]: points of the rule that an interval's place allows
+    int *points;  // [2][n_xi]: the fewest points that an interval's place allows
     double ts_end[kTsHalf + 1], ts_w[kTsHalf + 1];  // tanh-sinh: distance of node k from the nearer end, weight (half-widths)
     double *pieces;  // [2][kPieces][kPieceRow]: the Bessel functions
-    double *nodes;   // [2][3][kGl][n_xi]: q, w va, w vb at the Gauss-Legendre nodes of every interval
+    double *nodes;   // [2][3][kGlSlots][n_xi]: q, w va, w vb at the Gauss-Legendre nodes of every interval
 };
 
 // interval j of a row: QS j = 0 is [xi_min e^-100, xi_min] in ln xi, j >= 1 is
@@ -262,44 +262,50 @@ __device__ __forceinline__ void row_interval(bool qs, double ln_xi_min, int M, i
     }
 }
 
-// Gauss-Legendre (weights and nodes of the reference interval by value) with 16
-// points where the integrand's singularity (QS: ln xi = 0, where 1 - xi
-// vanishes; BW: xi = 0) lies at least twice the interval's half-width from its
-// centre (the error falls like (2 + sqrt 3)^-32 = 5e-19), the interval is not
-// wide against the integrand's own scale in ln xi, and e^-Y falls by at most
-// e^-12 across it (the error of e^-6t on [-1, 1] is 2e-20); with 8 points where
-// the singularity lies 8 half-widths away ((8 + sqrt 63)^-16 = 6e-20) and e^-Y
-// falls by at most e^-2 (2e-18).  QS interval 0, below xi_min, is integrated
-// in w = xi^(1/3), S growing like w there: with 16 points if Y(xi_min) <= 1/2 and
-// xi_min <= 1/5 (xi = 1 then lies 2.4 half-widths from the centre).
-constexpr int kGl = 16, kGlFew = 8;
-struct GaussLegendre16 {
-    double x[kGl], w[kGl], xf[kGlFew], wf[kGlFew];
+// Gauss-Legendre rules (weights and nodes of the reference interval by value).
+// What bounds a rule is the place of the integrand's singularity (QS: ln xi = 0,
+// where 1 - xi vanishes; BW: xi = 0), c half-widths from the interval's centre
+// (the error of n points falls like (c + sqrt(c^2 - 1))^-2n), the interval's
+// width in ln xi against the integrand's own scale, and how far e^-Y falls across
+// it, e^-f (the error of e^(-f t/2) on [-1, 1]):
+//   16 points: c >= 2 (5e-19), f <= 12 (2e-20);
+//    8 points: c >= 8 (6e-20), f <= 2 (2e-18);
+//    5 points: c >= 40 (9e-20), f <= 0.3 (5e-18).
+// QS interval 0, below xi_min, is integrated in w = xi^(1/3), S growing like w
+// there: with 16 points if Y(xi_min) <= 1/2 and xi_min <= 1/5 (xi = 1 then lies 2.4
+// half-widths from the centre).
+constexpr int kGl = 16, kGl8 = 8, kGl5 = 5;
+constexpr int kGlSlots = kGl + kGl8 + kGl5;  // the three rules' nodes of an interval, one after the other
+struct GaussLegendreRules {
+    double x[kGl], w[kGl], x8[kGl8], w8[kGl8], x5[kGl5], w5[kGl5];
 };
 
-// points of the rule that the interval's place allows: 16, 8 or 0 (tanh-sinh)
+// the fewest points that the interval's place allows: 16, 8, 5, or 0 (tanh-sinh)
 __device__ __forceinline__ int gl_points(bool qs, int j, double lo, double hi)
 {
     if (j == 0) return qs && hi <= -1.6095 ? kGl : 0;  // ln(1/5)
     const double c = qs ? -0.5 * (lo + hi) : 0.5 * (lo + hi), h = 0.5 * (hi - lo);
     if (c < 2.0 * h || (qs && h > 0.5)) return 0;
-    return c >= 8.0 * h && !(qs && h > 0.1) ? kGlFew : kGl;
+    if (c < 8.0 * h || (qs && h > 0.1)) return kGl;
+    return c < 40.0 * h ? kGl8 : kGl5;
 }
 
 // the nodes that every row of a process shares: thread = (interval, node), blockIdx.y = process
 __global__ void __launch_bounds__(128) row_nodes_kernel(const __grid_constant__ GenArgs a,
-                                                         const __grid_constant__ GaussLegendre16 g)
+                                                         const __grid_constant__ GaussLegendreRules g)
 {
     const bool qs = blockIdx.y == 0;
     const int M = qs ? a.qs_n_xi : a.bw_n_xi;
-    const int j = blockIdx.x * 8 + threadIdx.x / kGl, k = threadIdx.x % kGl;
-    if (j >= M) return;
+    const int j = blockIdx.x * 4 + threadIdx.x / 32, k = threadIdx.x % 32;
+    if (j >= M || k >= kGlSlots) return;
     double lo, hi;
     row_interval(qs, a.qs_ln_xi_min, M, j, lo, hi);
     const int points = gl_points(qs, j, lo, hi);
     if (k == 0) a.points[(qs ? 0 : a.qs_n_xi) + j] = points;
-    if (k >= points) return;
-    double *out = a.nodes + (qs ? 0 : (size_t)3 * kGl * a.qs_n_xi);
+    // (a rule with more points than the place asks for serves the rows where e^-Y falls faster)
+    const int n = k < kGl ? kGl : k < kGl + kGl8 ? kGl8 : kGl5;
+    if (points == 0 || n < points) return;
+    double *out = a.nodes + (qs ? 0 : (size_t)3 * kGlSlots * a.qs_n_xi);
     double x, w;
     if (j == 0) {  // w^3 = xi from 0 to xi_min: S du = (3 S / w) dw
         const double top = cbrt(a.qs_xi_min), v = 0.5 * top * (1.0 + g.x[k]);
@@ -307,24 +313,25 @@ __global__ void __launch_bounds__(128) row_nodes_kernel(const __grid_constant__ 
         w = 0.5 * top * g.w[k] * 3.0 / v;
     } else {
         const double c = 0.5 * (lo + hi), h = 0.5 * (hi - lo);
-        x = fma(h, points == kGl ? g.x[k] : g.xf[k], c);
-        w = h * (points == kGl ? g.w[k] : g.wf[k]);
+        x = fma(h, n == kGl ? g.x[k] : n == kGl8 ? g.x8[k - kGl] : g.x5[k - kGl - kGl8], c);
+        w = h * (n == kGl ? g.w[k] : n == kGl8 ? g.w8[k - kGl] : g.w5[k - kGl - kGl8]);
     }
     double q, va, vb;
     node_terms(qs, x, q, va, vb);
     out[(size_t)k * M + j] = q;
-    out[(size_t)(kGl + k) * M + j] = w * va;
-    out[(size_t)(2 * kGl + k) * M + j] = w * vb;
+    out[(size_t)(kGlSlots + k) * M + j] = w * va;
+    out[(size_t)(2 * kGlSlots + k) * M + j] = w * vb;
 }
 
 // One CTA per row.  Bound by the FP64 pipe: ~60 FP64 instructions per
-// Gauss-Legendre node, ~256 x 8 nodes in a row of the 256 x 256 tables, and the
+// Gauss-Legendre node, ~256 x 6 nodes in a row of the 256 x 256 tables, and the
 // tanh-sinh intervals (one at the end, and ~4 per row across which e^-Y falls
-// steeply), whose nodes and weights on [-1, 1] are shared too.
+// steeply), whose nodes and weights on [-1, 1] are shared too.  Shared memory by
+// the row's length, so that all 512 rows are resident at once (three to an SM
+// left 56 rows for a second wave).
 __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__ GenArgs a)
 {
-    __shared__ double acc[QED_MAX_TABLE_N], tail[QED_MAX_TABLE_N], cum[QED_MAX_TABLE_N];
-    extern __shared__ double s_c[];  // [kPieces][kPieceRow]
+    extern __shared__ double s_c[];  // [kPieces][kPieceRow], then acc, tail, cum [M]
     __shared__ short s_hard[QED_MAX_TABLE_N];
     __shared__ int s_n_hard;
     __shared__ double s_chi[2];
@@ -332,6 +339,7 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__
     const int row = qs ? blockIdx.x : blockIdx.x - a.qs_n_chi;
     const int N = qs ? a.qs_n_chi : a.bw_n_chi;
     const int M = qs ? a.qs_n_xi : a.bw_n_xi;
+    double *const acc = s_c + kPieces * kPieceRow, *const tail = acc + M, *const cum = tail + M;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
 
     if (threadIdx.x == 0) {
@@ -345,7 +353,7 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__
     __syncthreads();
     const double chi = s_chi[0], inv_chi = s_chi[1];
 
-    const double *nodes = a.nodes + (qs ? 0 : (size_t)3 * kGl * a.qs_n_xi);
+    const double *nodes = a.nodes + (qs ? 0 : (size_t)3 * kGlSlots * a.qs_n_xi);
     const int *allowed = a.points + (qs ? 0 : a.qs_n_xi);
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
         if (!qs && j == 0) {
@@ -354,21 +362,22 @@ __global__ void __launch_bounds__(256) table_rows_kernel(const __grid_constant__
         }
         int points = allowed[j];
         if (points) {
-            // the outermost nodes lie within 2 % of the ends: Y's fall between them
-            const double q0 = nodes[j], q1 = nodes[(size_t)(points - 1) * M + j];
+            // the fall of e^-Y between the outermost nodes of 16, which lie within 1 % of the ends
+            const double q0 = nodes[j], q1 = nodes[(size_t)(kGl - 1) * M + j];
             if (fmin(q0, q1) * inv_chi > 800.0 && j > 0) {  // e^-Y is zero on all of it
                 acc[j] = 0.0;
                 continue;
             }
             const double fall = fabs(q1 - q0) * inv_chi;
-            if (fall > (j == 0 ? 0.5 : (points == kGl ? 11.5 : 1.9))) points = 0;
+            if (points == kGl5 && fall > 0.29) points = kGl8;
+            if (points == kGl8 && fall > 1.9) points = kGl;
+            if (fall > (j == 0 ? 0.5 : 11.5)) points = 0;
         }
         if (points) {
+            const double *p = nodes + (size_t)(points == kGl ? 0 : points == kGl8 ? kGl : kGl + kGl8) * M + j;
             double part = 0.0;
-            for (int k = 0; k < points; ++k) {
-                const double *p = nodes + (size_t)k * M + j;
-                part += row_integrand(s_c, qs, inv_chi, p[0], p[(size_t)kGl * M], p[(size_t)2 * kGl * M]);
-            }
+            for (int k = 0; k < points; ++k, p += M)
+                part += row_integrand(s_c, qs, inv_chi, p[0], p[(size_t)kGlSlots * M], p[(size_t)2 * kGlSlots * M]);
             acc[j] = part;
         } else {
             s_hard[atomicAdd(&s_n_hard, 1)] = (short)j;
@@ -703,7 +712,7 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
     if (s) return s;
     qed_tables *t = nullptr;
     const size_t scratch =
-        ((size_t)2 * kPieces * kPieceRow + (size_t)3 * kGl * (params->qs.n_xi + params->bw.n_xi)) * sizeof(double) +
+        ((size_t)2 * kPieces * kPieceRow + (size_t)3 * kGlSlots * (params->qs.n_xi + params->bw.n_xi)) * sizeof(double) +
         (size_t)(params->qs.n_xi + params->bw.n_xi) * sizeof(int);
     if ((s = alloc_tables(params, &t, scratch))) return s;
     cudaStream_t st = as_stream(stream);
@@ -723,19 +732,20 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
     // scratch (the pieces, the shared nodes) in the room of the derived tables, which finish_tables fills afterwards
     a.pieces = (double *)t->derived;
     a.nodes = a.pieces + (size_t)2 * kPieces * kPieceRow;
-    a.points = (int *)(a.nodes + (size_t)3 * kGl * (params->qs.n_xi + params->bw.n_xi));
-    static const GaussLegendre16 gl = [] {
-        GaussLegendre16 g;
+    a.points = (int *)(a.nodes + (size_t)3 * kGlSlots * (params->qs.n_xi + params->bw.n_xi));
+    static const GaussLegendreRules gl = [] {
+        GaussLegendreRules g;
         gauss_legendre<kGl>(g.x, g.w);
-        gauss_legendre<kGlFew>(g.xf, g.wf);
+        gauss_legendre<kGl8>(g.x8, g.w8);
+        gauss_legendre<kGl5>(g.x5, g.w5);
         return g;
     }();
     const int m = params->qs.n_xi > params->bw.n_xi ? params->qs.n_xi : params->bw.n_xi;
-    constexpr int dyn = kPieces * kPieceRow * (int)sizeof(double);
+    const int dyn = (kPieces * kPieceRow + 3 * m) * (int)sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(table_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     if (e == cudaSuccess) {
         bessel_pieces_kernel<<<kPieces, 128, 0, st>>>(a.pieces);
-        row_nodes_kernel<<<dim3((m + 7) / 8, 2), 8 * kGl, 0, st>>>(a, gl);
+        row_nodes_kernel<<<dim3((m + 3) / 4, 2), 128, 0, st>>>(a, gl);
         table_rows_kernel<<<params->qs.n_chi + params->bw.n_chi, 256, dyn, st>>>(a);
         e = cudaGetLastError();
     }

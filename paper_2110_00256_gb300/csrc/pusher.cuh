@@ -59,20 +59,38 @@ __device__ __forceinline__ void wave_fields(const WaveT<T> &w, T x, T &ex, T &ey
 }
 
 // the linearly polarised wave's fields that are not zero (without the sine)
-__device__ __forceinline__ void wave_fields_yz(const WaveT<float> &w, float x, float &ey, float &bz)
+template <typename T>
+__device__ __forceinline__ void wave_fields_yz(const WaveT<T> &w, T x, T &ey, T &bz)
 {
-    const float u = w.omega_pi * (w.t - w.d * x) + w.phase0_pi;
-    float s, c;
+    const T u = w.omega_pi * (w.t - w.d * x) + w.phase0_pi;
+    T s, c;
     d_sincospi(u, &s, &c);
     ey = w.e0 * c;
     bz = w.d * ey;
 }
 
-// reciprocal square root: FP32 rsqrtf (within 2 ulp), FP64 rsqrt (within 1 ulp);
-// the push is not part of the paper's method, and its arithmetic budget is the
-// fused cascade kernel's limit
+// reciprocal square root: FP32 rsqrtf (within 2 ulp), FP64 on the integers (within
+// 1 ulp, fixed64.cuh: an FP64 instruction of a warp takes 76 issue slots), and the
+// quotient 2/x likewise; the push is not part of the paper's method, and its
+// arithmetic budget is the fused cascade kernel's limit
 __device__ __forceinline__ float d_rsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double d_rsqrt(double x) { return rsqrt(x); }
+__device__ __forceinline__ double d_rsqrt(double x)
+{
+    if (!fix_plain(x)) return rsqrt(x);
+    double root, inv;
+    fix_sqrt_double(x, root, inv);
+    return inv;
+}
+__device__ __forceinline__ float two_over(float x) { return 2.0f / x; }
+__device__ __forceinline__ double two_over(double x) { return fix_plain(x) ? fix_div(2.0, x) : 2.0 / x; }
+
+// products and sums that are not contracted
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return fma(a, b, c); }
 
 // one step of the momentum of a particle of charge q (relativistic Boris
 // rotation; q = 0: a photon, unchanged) and the velocity it then moves with
@@ -90,7 +108,7 @@ __device__ __forceinline__ void boris_move(T q, T dt, T ex, T ey, T ez, T bx, T 
     const T mx = px + h * ex, my = py + h * ey, mz = pz + h * ez;  // half electric kick
     const T hg = h * d_rsqrt(T(1) + mx * mx + my * my + mz * mz);
     const T tx = hg * bx, ty = hg * by, tz = hg * bz;
-    const T f = T(2) / (T(1) + tx * tx + ty * ty + tz * tz);
+    const T f = two_over(T(1) + tx * tx + ty * ty + tz * tz);
     const T sx = f * tx, sy = f * ty, sz = f * tz;
     const T qx = mx + (my * tz - mz * ty), qy = my + (mz * tx - mx * tz), qz = mz + (mx * ty - my * tx);
     px = mx + (qy * sz - qz * sy) + h * ex;
@@ -102,25 +120,25 @@ __device__ __forceinline__ void boris_move(T q, T dt, T ex, T ey, T ez, T bx, T 
 
 // the same in fields with only Ey and Bz, the terms with a zero factor left out
 // (bit for bit the same for finite momenta, see chi_lepton_yz)
-__device__ __forceinline__ void boris_move_yz(float q, float dt, float ey, float bz, float &px, float &py, float &pz,
-                                              float &vx, float &vy, float &vz)
+template <typename T>
+__device__ __forceinline__ void boris_move_yz(T q, T dt, T ey, T bz, T &px, T &py, T &pz, T &vx, T &vy, T &vz)
 {
-    if (q == 0.0f) {
-        const float p2 = px * px + py * py + pz * pz;
-        const float inv = p2 > 0.0f ? d_rsqrt(p2) : 0.0f;
+    if (q == T(0)) {
+        const T p2 = px * px + py * py + pz * pz;
+        const T inv = p2 > T(0) ? d_rsqrt(p2) : T(0);
         vx = px * inv, vy = py * inv, vz = pz * inv;
         return;
     }
-    const float h = 0.5f * q * dt;
-    const float my = fmaf(h, ey, py);  // half electric kick
-    const float hg = h * d_rsqrt(1.0f + px * px + my * my + pz * pz);
-    const float tz = __fmul_rn(hg, bz);
-    const float f = 2.0f / fmaf(tz, tz, 1.0f);
-    const float sz = __fmul_rn(f, tz);
-    const float qx = __fadd_rn(px, __fmul_rn(my, tz)), qy = __fadd_rn(my, -__fmul_rn(px, tz));
-    px = __fadd_rn(px, __fmul_rn(qy, sz));
-    py = fmaf(h, ey, __fadd_rn(my, -__fmul_rn(qx, sz)));
-    const float ig = d_rsqrt(1.0f + px * px + py * py + pz * pz);
+    const T h = T(0.5) * q * dt;
+    const T my = fma_rn(h, ey, py);  // half electric kick
+    const T hg = h * d_rsqrt(T(1) + px * px + my * my + pz * pz);
+    const T tz = mul_rn(hg, bz);
+    const T f = two_over(fma_rn(tz, tz, T(1)));
+    const T sz = mul_rn(f, tz);
+    const T qx = add_rn(px, mul_rn(my, tz)), qy = add_rn(my, -mul_rn(px, tz));
+    px = add_rn(px, mul_rn(qy, sz));
+    py = fma_rn(h, ey, add_rn(my, -mul_rn(qx, sz)));
+    const T ig = d_rsqrt(T(1) + px * px + py * py + pz * pz);
     vx = px * ig, vy = py * ig, vz = pz * ig;
 }
 

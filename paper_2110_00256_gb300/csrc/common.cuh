@@ -138,6 +138,9 @@ struct Table2D {
     T ln_min, inv_d, chi_min, chi_max;
     T x0, dx;        // xi axis: QS ln xi_min and step in ln xi; BW 0 and step in xi
     int n_chi, n_xi;
+    FixAxis fix;     // the chi axis on integers
+    Fix dx_fix;      // dx 2^dx_shift in [2^61, 2^62) (QS: dx_shift >= 63, or 0: the integers cannot hold it)
+    int dx_shift;
 };
 
 template <typename T>

@@ -18,7 +18,7 @@ struct EventArgs {
 };
 
 template <typename T, bool MLP>
-__global__ void __launch_bounds__(256, (MLP || sizeof(T) == 8) ? 1 : 4) qs_event_kernel(const __grid_constant__ EventArgs<T> a)
+__global__ void __launch_bounds__(256, MLP ? 1 : 4) qs_event_kernel(const __grid_constant__ EventArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);
@@ -36,8 +36,10 @@ __global__ void __launch_bounds__(256, (MLP || sizeof(T) == 8) ? 1 : 4) qs_event
     flush_counts(a.com.stats, k, true);
 }
 
+// (four CTAs of 64 registers per SM: 2e6 FP64 decays, with the caller's ordering of
+// the products, 612 us; three 631, two 686 -- the table's rows are loads in a chain)
 template <typename T, bool MLP>
-__global__ void __launch_bounds__(256, (MLP || sizeof(T) == 8) ? 1 : 4) bw_event_kernel(const __grid_constant__ EventArgs<T> a)
+__global__ void __launch_bounds__(256, MLP ? 1 : 4) bw_event_kernel(const __grid_constant__ EventArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);

@@ -221,15 +221,10 @@ __device__ __forceinline__ double fix_sqrt_double(double x)
     return r;
 }
 
-// a / b for fix_plain(|a|), fix_plain(b): within 2^-58 before the rounding to
-// FP64.  The reciprocal of b's significand by two Newton steps from the 22-bit
-// one (as in fix_sqrt), times a's.
-__device__ __forceinline__ double fix_div(double a, double b)
+// 1/(g 2^-63) in 2^-62 for g in [2^62, 2^63), within 2^-58: two Newton steps from
+// the 22-bit reciprocal (as in fix_sqrt)
+__device__ __forceinline__ uint64_t fix_recip(uint64_t g)
 {
-    const int ha = __double2hiint(a), hb = __double2hiint(b);
-    const uint64_t ma = (uint64_t)((ha & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(a);
-    const uint64_t mb = (uint64_t)((hb & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(b);
-    const uint64_t g = mb << 10;  // [2^62, 2^63): g 2^-63 in [1/2, 1)
     const uint32_t fh = (uint32_t)(g >> 32), fl = (uint32_t)g;
     const float y = __frcp_rn((float)fh * 0x1p-31f);
     const int y0 = (int)fminf(y * 0x1p30f, 2147483520.0f);  // 2^-30, [1, 2)
@@ -237,7 +232,17 @@ __device__ __forceinline__ double fix_div(double a, double b)
     const uint64_t y1 = ((uint64_t)y0 << 32) + (uint64_t)(wide(y0, (int)(e0 >> 10)) >> 19);  // 2^-62
     const uint32_t yh = (uint32_t)(y1 >> 32), yl = (uint32_t)y1;
     const int64_t e1 = -(int64_t)((uwide(fh, yh) << 32) + uwide(fh, yl) + uwide(fl, yh) + (uwide(fl, yl) >> 32));
-    const uint64_t inv = y1 + (uint64_t)(wide((int)yh, (int)(e1 >> 21)) >> 40);  // 1/(g 2^-63), 2^-62
+    return y1 + (uint64_t)(wide((int)yh, (int)(e1 >> 21)) >> 40);
+}
+
+// a / b for fix_plain(|a|), fix_plain(b): within 2^-58 before the rounding to
+// FP64 (the reciprocal of b's significand times a's)
+__device__ __forceinline__ double fix_div(double a, double b)
+{
+    const int ha = __double2hiint(a), hb = __double2hiint(b);
+    const uint64_t ma = (uint64_t)((ha & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(a);
+    const uint64_t mb = (uint64_t)((hb & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(b);
+    const uint64_t inv = fix_recip(mb << 10);       // 1/(mb 2^-53), 2^-62
     const uint64_t p = __umul64hi(ma << 10, inv);  // (ma 2^-53)(2^53/mb) 2^61
     const int64_t q = (ha ^ hb) < 0 ? -(int64_t)p : (int64_t)p;
     return fix_to_double(q, ((ha >> 20) & 0x7ff) - ((hb >> 20) & 0x7ff) - 61);
@@ -289,18 +294,26 @@ struct FixAxis {
 constexpr long long kFixLnTSmall = -13251786775133077ll;  // ln of T's asymptotes (kLnTSmall, kLnTLarge), 2^-53
 constexpr long long kFixLnTLarge = -8724416322236899ll;
 
-// the table's logarithms at ln chi = lc (clamped into the axis): ln f_i + f (ln f_{i+1} - ln f_i)
-__device__ __forceinline__ int64_t fix_table(const FixAxis &ax, const long long *tab, int64_t lc)
+// the interval of the axis at ln chi = lc (clamped into it) and the fraction of it, 2^-62
+__device__ __forceinline__ Fix fix_locate(const FixAxis &ax, int64_t lc, int &i)
 {
     int64_t d = lc - ax.ln_min;
     const int64_t dmax = ax.ln_max - ax.ln_min;
     d = d < 0 ? 0 : (d > dmax ? dmax : d);
     // t = d (n - 1) / dmax in units of 2^-frac (below 2^60): the difference shifted below 2^62 times the scale
     const int64_t t = mul_q62(fix_limbs(d << ax.shift), ax.scale);
-    int i = (int)(t >> ax.frac);
+    i = (int)(t >> ax.frac);
     i = i > ax.n - 2 ? ax.n - 2 : i;
+    return fix_limbs((t - ((int64_t)i << ax.frac)) << (62 - ax.frac));
+}
+
+// the table's logarithms at ln chi = lc (clamped into the axis): ln f_i + f (ln f_{i+1} - ln f_i)
+__device__ __forceinline__ int64_t fix_table(const FixAxis &ax, const long long *tab, int64_t lc)
+{
+    int i;
+    const Fix f = fix_locate(ax, lc, i);
     const int64_t a = tab[i];
-    return a + mul_q62(fix_limbs((t - ((int64_t)i << ax.frac)) << (62 - ax.frac)), fix_limbs(tab[i + 1] - a));
+    return a + mul_q62(f, fix_limbs(tab[i + 1] - a));
 }
 
 struct FixOut {

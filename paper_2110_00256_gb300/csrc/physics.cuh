@@ -18,8 +18,9 @@ __device__ __forceinline__ float d_fma(float a, float b, float c) { return fmaf(
 // logarithm and exponential of the 1-D rate lookups: in FP32 the hardware's
 // approximate forms (__logf: absolute error ~2^-21 near 1; __expf: ~2 + 1.2 |x|
 // ulp), whose ~1e-6 relative effect on a rate is far below the tables'
-// interpolation error; in FP64 Tang's table-driven forms (fp64_math.cuh, within
-// 2 ulp), which take fewer FP64 instructions than the library functions
+// interpolation error; in FP64 (the path behind the integer one of fixed64.cuh)
+// Tang's table-driven forms (fp64_math.cuh, within 2 ulp), which take fewer FP64
+// instructions than the library functions
 __device__ __forceinline__ float r_log(float x) { return __logf(x); }
 __device__ __forceinline__ double r_log(double x) { return log_tang(x); }
 __device__ __forceinline__ float r_exp(float x) { return __expf(x); }
@@ -64,9 +65,9 @@ __device__ __forceinline__ double log_int(double x)
 }
 
 // logarithm and exponential of the 2-D inverse-CDF sampling: FP32 the library
-// forms; FP64 the integer logarithm (ln chi and ln r are interpolation
-// coordinates, where its 2^-57 absolute error near 1 is far below the tables'
-// spacing) and Tang's exponential
+// forms; the general FP64 forms the integer logarithm (ln chi and ln r are
+// interpolation coordinates, where its 2^-57 absolute error near 1 is far below
+// the tables' spacing) and Tang's exponential
 __device__ __forceinline__ float s_log(float x) { return logf(x); }
 __device__ __forceinline__ double s_log(double x) { return log_int(x); }
 __device__ __forceinline__ float s_exp(float x) { return expf(x); }
@@ -292,20 +293,27 @@ __device__ __forceinline__ void locate_2d(const Table2D<T> &tb, T chi, const T *
     r1 = r0 + tb.n_xi;
 }
 
+// where the search of a row starts: the bracket that the guide tables of the two
+// rows give for bin b of the draw (both rows' answers, hence the interpolated
+// row's, lie between their guides at b and b + 1), widened by one entry on each
+// side against rounding at the edges.  Invariant: P_lo <= x (or lo == 0), P_hi > x
+// (hi == M: sentinel).
+__device__ __forceinline__ void search_bracket(const int32_t *g0, const int32_t *g1, int b, int M, int &lo, int &hi)
+{
+    const int a0 = __ldg(g0 + b), a1 = __ldg(g1 + b), c0 = __ldg(g0 + b + 1), c1 = __ldg(g1 + b + 1);
+    lo = (a0 < a1 ? a0 : a1) - 1, hi = (c0 > c1 ? c0 : c1) + 2;
+    lo = lo < 0 ? 0 : lo;
+    hi = hi > M ? M : hi;
+}
+
 // largest m in [0, M-1] with P_m <= x on the interpolated row (binary search;
 // the row is non-decreasing), then clamped to [0, M-2]; m = 0 when x < P_0.
-// The search starts from the bracket that the guide tables of the two rows give
-// for bin b of the draw (both rows' answers, hence the interpolated row's, lie
-// between their guides at b and b + 1), widened by one entry on each side
-// against rounding at the edges.
 template <typename T>
 __device__ __forceinline__ int search_row(const T *r0, const T *r1, T w, int M, T x, const int32_t *g0,
                                           const int32_t *g1, int b)
 {
-    const int a0 = __ldg(g0 + b), a1 = __ldg(g1 + b), c0 = __ldg(g0 + b + 1), c1 = __ldg(g1 + b + 1);
-    int lo = (a0 < a1 ? a0 : a1) - 1, hi = (c0 > c1 ? c0 : c1) + 2;
-    lo = lo < 0 ? 0 : lo;
-    hi = hi > M ? M : hi;  // invariant: P_lo <= x (or lo == 0), P_hi > x (hi == M: sentinel)
+    int lo, hi;
+    search_bracket(g0, g1, b, M, lo, hi);
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (row_val(r0, r1, w, mid) <= x)
@@ -316,6 +324,121 @@ __device__ __forceinline__ int search_row(const T *r0, const T *r1, T w, int M, 
     return lo > M - 2 ? M - 2 : lo;
 }
 
+// ---------------------------------------------------------------------------
+// The FP64 inverse CDFs on 64-bit integers: chi's interval as in the rates, the
+// draw and the row's values in one unit (BW: P and r in 2^-62; QS: ln P and ln r in
+// 2^-58 to 2^-63), the quotient to 2^-58.  The general forms below take ~55 FP64 instructions
+// of 76 issue slots each for an event, these none (2e6 photons all decaying, with the
+// caller's ordering of the products: 727 -> 613 us).
+// They return false, for the general forms: chi outside [2^-86, 2^86], a table that
+// the units cannot hold, a draw off its row's ends or on a flat stretch, and small
+// draws -- BW r < 2^-9 (1 in 256), where FP64 holds more than the unit does, QS
+// r < 2^-20 -- and QS xi above e^(-1/8).
+// ---------------------------------------------------------------------------
+struct UnitBW {  // a value in [0, 1], rounded down; anything else: ok = false
+    static __device__ __forceinline__ int64_t of(double x, int, bool &ok)
+    {
+        const uint32_t hi = (uint32_t)__double2hiint(x);
+        ok = ok && hi <= 0x3ff00000u;  // (1 + a fraction below 2^-20 passes, and stays below 2^63)
+        const uint64_t m = (uint64_t)((hi & 0x000fffffu) | 0x00100000u) << 32 | (uint32_t)__double2loint(x);
+        return (int64_t)fix_shr(m << 10, 1023 - (int)(hi >> 20));  // (zero and subnormal values: 0)
+    }
+};
+struct UnitQS {  // in 2^-(58 + s), +-2^(4 - s) for values beyond (ok = false)
+    static __device__ __forceinline__ int64_t of(double x, int s, bool &ok)
+    {
+        const int hi = __double2hiint(x), d = 1026 - s - ((hi >> 20) & 0x7ff);
+        const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(x);
+        ok = ok && d >= 0;
+        const int64_t v = d >= 0 ? (int64_t)fix_shr(m << 9, d) : (1ll << 62) - 1;
+        return hi < 0 ? -v : v;
+    }
+};
+
+template <typename U>
+__device__ __forceinline__ int64_t fix_row(const double *r0, const double *r1, const Fix &w, int m, int s, bool &ok)
+{
+    const int64_t a = U::of(__ldg(r0 + m), s, ok), b = U::of(__ldg(r1 + m), s, ok);
+    return a + mul_q62(w, fix_limbs(b - a));
+}
+
+// the column m of draw x (guide bin b) on the row at chi, and (x - P_m) / (P_{m+1} - P_m)
+// in 2^-61.  Entries beyond the unit compare as its ends; rows do not decrease, so
+// that they matter only where the columns at m hold one.
+template <typename U>
+__device__ __forceinline__ bool fix_column(const Table2D<double> &tb, double chi, int64_t x, int s, int b, int &m,
+                                           int64_t &f)
+{
+    const int hi = __double2hiint(chi);
+    bool ok = tb.fix.ok && (unsigned)(hi - (937 << 20)) < (172u << 20);
+    if (!ok) return false;
+    const uint64_t mc = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(chi);
+    int unit, row;
+    const int64_t lc = fix_ln_value(mc << 11, (hi >> 20) - 1023 - 63, unit);
+    const Fix w = fix_locate(tb.fix, unit == -63 ? (lc + 512) >> 10 : (lc + 8) >> 4, row);
+    const double *r0 = tb.v + (size_t)row * tb.n_xi, *r1 = r0 + tb.n_xi;
+    const int32_t *g0 = tb.guide + (size_t)row * (kGuideBins + 1), *g1 = g0 + kGuideBins + 1;
+    b = b > kGuideBins - 1 ? kGuideBins - 1 : b;
+    int hi_m;
+    search_bracket(g0, g1, b, tb.n_xi, m, hi_m);
+    bool any = true;
+    while (hi_m - m > 1) {
+        const int mid = (m + hi_m) >> 1;
+        if (fix_row<U>(r0, r1, w, mid, s, any) <= x)
+            m = mid;
+        else
+            hi_m = mid;
+    }
+    m = m > tb.n_xi - 2 ? tb.n_xi - 2 : m;
+    const int64_t p0 = fix_row<U>(r0, r1, w, m, s, ok), dp = fix_row<U>(r0, r1, w, m + 1, s, ok) - p0, d = x - p0;
+    if (!ok || d < 0 || d >= dp) return false;
+    const int z = __clzll(dp) - 1;
+    f = (int64_t)__umul64hi((uint64_t)d << z, fix_recip((uint64_t)dp << z));
+    return true;
+}
+
+__device__ __forceinline__ bool bw_sample_fixed(const Table2D<double> &tb, double chi, double u, double &x)
+{
+    bool ok = true;
+    int64_t r = UnitBW::of(u, 0, ok), f;
+    r = r > (1ll << 61) ? (1ll << 62) - r : r;
+    int m;
+    if (!ok || r < (1ll << 53) || !fix_column<UnitBW>(tb, chi, r, 0, (int)(r >> 55), m, f)) return false;
+    // (m + f) dx, rounded once
+    const int k = 32 - __clz(m);
+    const int64_t c = ((int64_t)m << (61 - k)) + (f >> k);
+    if (c == 0) return false;
+    const int z = __clzll(c) - 2;
+    x = fix_to_double(mul_q62(fix_limbs(c << z), tb.dx_fix), 1 + k - z - tb.dx_shift);
+    if (__double_as_longlong(x) > __double_as_longlong(0.5)) x = 0.5;
+    return true;
+}
+
+__device__ __forceinline__ bool qs_sample_fixed(const Table2D<double> &tb, double chi, double r, double &xi)
+{
+    const int hi = __double2hiint(r);
+    bool ok = true;
+    const int64_t v = UnitBW::of(r, 0, ok);
+    if (!ok || hi < 0x3eb00000 || !tb.dx_shift) return false;  // 2^-20 <= r <= 1
+    const uint64_t mr = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(r);
+    int unit, m, k;
+    int64_t f;
+    const int64_t lr = fix_ln_value(mr << 11, (hi >> 20) - 1023 - 63, unit);
+    // the unit with |ln r|: 2^-58 below r = 1/2, up to 2^-63, so that it is finer than
+    // FP64's roundings of ln P until the logarithm's own error is all there is
+    const int z = __clzll(-lr), s = unit == -63 ? (z < 5 ? z : 5) : 0;
+    if (!fix_column<UnitQS>(tb, chi, unit == -63 ? lr >> (5 - s) : 2 * lr, s, (int)(v >> 56), m, f)) return false;
+    // ln xi = -(n - 1 - m - f) dx, 2^-53
+    const int64_t c = ((int64_t)(tb.n_xi - 1 - m) << 52) - ((f + 256) >> 9);
+    const int sh = tb.dx_shift - 63;
+    const int64_t y = (mul_q62(fix_limbs(c), tb.dx_fix) + ((1ll << sh) >> 1)) >> sh;
+    // near xi = 1 the lepton keeps gamma (1 - xi), a rounding of xi over 1 - xi: as before
+    if (y < (1ll << 50)) return false;
+    xi = fix_to_double(fix_exp(-y, k, kFixExp), k - 62);
+    return true;
+}
+static_assert(kGuideBins == 64, "the guide's bin is the top 6 bits of r");
+
 // QS inverse CDF (§3.2): ln P interpolated in ln chi, binary search on ln r, then
 // ln xi = ln xi_m + (ln r - ln P_m)(ln xi_{m+1} - ln xi_m)/(ln P_{m+1} - ln P_m).
 // The denominator is interpolated from the FP64-formed column differences, so
@@ -323,7 +446,7 @@ __device__ __forceinline__ int search_row(const T *r0, const T *r1, T w, int M, 
 // entries share most of their digits); the same holds below xi_min, where the
 // first segment is extrapolated.
 template <typename T>
-__device__ __forceinline__ T qs_sample_xi(const Table2D<T> &tb, T chi, T r)
+__device__ __forceinline__ T qs_sample_row(const Table2D<T> &tb, T chi, T r)
 {
     const T *r0, *r1;
     T w;
@@ -345,19 +468,30 @@ __device__ __forceinline__ T qs_sample_xi(const Table2D<T> &tb, T chi, T r)
     return s_exp(lx);
 }
 
+// (out of line: the few draws that the integer forms leave)
+static __device__ __noinline__ double qs_sample_fp64(const Table2D<double> &tb, double chi, double r)
+{
+    return qs_sample_row<double>(tb, chi, r);
+}
+
+template <typename T>
+__device__ __forceinline__ T qs_sample_xi(const Table2D<T> &tb, T chi, T r)
+{
+    if constexpr (sizeof(T) == 8) {
+        double xi;
+        return qs_sample_fixed(tb, chi, r, xi) ? xi : qs_sample_fp64(tb, chi, r);
+    } else {
+        return qs_sample_row<T>(tb, chi, r);
+    }
+}
+
+
 // BW inverse CDF (§3.1): r <= 1/2 samples the electron, otherwise the positron
 // with r -> 1 - r; P interpolated in ln chi_g, binary search on r, linear in xi
 // (denominator from the column differences, as for QS).
 template <typename T>
-__device__ __forceinline__ T bw_sample_xi(const Table2D<T> &tb, T chi, double u, bool &electron)
+__device__ __forceinline__ T bw_sample_row(const Table2D<T> &tb, T chi, T r)
 {
-    // split on the FP64 draw, then round the folded value (keeps 1 - u accurate)
-    electron = __double_as_longlong(u) <= __double_as_longlong(0.5);  // u <= 1/2 (u > 0: the bits order as the values)
-    T r;
-    if constexpr (sizeof(T) == 4)
-        r = electron ? sample_uniform<T>(u) : one_minus_rz(u);
-    else
-        r = electron ? u : 1.0 - u;
     const T *r0, *r1;
     T w;
     size_t off;
@@ -374,6 +508,25 @@ __device__ __forceinline__ T bw_sample_xi(const Table2D<T> &tb, T chi, double u,
     if (!(dp > T(0))) return x0;
     T x = x0 + e_div((r - p0) * (x1 - x0), dp);
     return x > T(0.5) ? T(0.5) : (x < T(0) ? T(0) : x);
+}
+
+static __device__ __noinline__ double bw_sample_fp64(const Table2D<double> &tb, double chi, double r)
+{
+    return bw_sample_row<double>(tb, chi, r);
+}
+
+template <typename T>
+__device__ __forceinline__ T bw_sample_xi(const Table2D<T> &tb, T chi, double u, bool &electron)
+{
+    // split on the FP64 draw, then round the folded value (keeps 1 - u accurate)
+    electron = __double_as_longlong(u) <= __double_as_longlong(0.5);  // u <= 1/2 (u > 0: the bits order as the values)
+    if constexpr (sizeof(T) == 4) {
+        return bw_sample_row<T>(tb, chi, electron ? sample_uniform<T>(u) : one_minus_rz(u));
+    } else {
+        double x;
+        if (bw_sample_fixed(tb, chi, u, x)) return x;
+        return bw_sample_fp64(tb, chi, electron ? u : 1.0 - u);
+    }
 }
 
 

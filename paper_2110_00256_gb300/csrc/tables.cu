@@ -205,9 +205,13 @@ static Table1D<T> view1(const T *f, const qed_table_axis &a, const FixAxis &fix)
 }
 
 template <typename T>
-static Table2D<T> view2(const T *f, const T *df, const int32_t *guide, const qed_table_axis &a, bool qs)
+static Table2D<T> view2(const T *f, const T *df, const int32_t *guide, const qed_table_axis &a, const FixAxis &fix,
+                        bool qs)
 {
     Table2D<T> v;
+    v.fix = fix;
+    v.dx_fix = Fix{0, 0};
+    v.dx_shift = 0;
     v.v = f;
     v.dv = df;
     v.guide = guide;
@@ -218,13 +222,11 @@ static Table2D<T> view2(const T *f, const T *df, const int32_t *guide, const qed
     v.chi_max = (T)a.chi_max;
     v.n_chi = a.n_chi;
     v.n_xi = a.n_xi;
-    if (qs) {
-        v.x0 = (T)std::log(a.xi_min);
-        v.dx = (T)(-std::log(a.xi_min) / (a.n_xi - 1));
-    } else {
-        v.x0 = (T)0;
-        v.dx = (T)(0.5 / (a.n_xi - 1));
-    }
+    const double dx = qs ? -std::log(a.xi_min) / (a.n_xi - 1) : 0.5 / (a.n_xi - 1);
+    v.x0 = qs ? (T)std::log(a.xi_min) : (T)0;
+    v.dx = (T)dx;
+    const int s = 61 - std::ilogb(dx);
+    if (s <= 100 && (s >= 63 || !qs)) v.dx_shift = s, v.dx_fix = fix_limbs((int64_t)std::ldexp(dx, s));
     return v;
 }
 
@@ -234,8 +236,9 @@ TablesView<double> make_view<double>(const qed_tables *t)
     TablesView<double> v;
     v.qs_G = view1<double>(t->d_qs_lnG, t->params.qs, t->qs_fix);
     v.bw_T = view1<double>(t->d_bw_lnT, t->params.bw, t->bw_fix);
-    v.qs_P = view2<double>(t->d_qs_lnP, t->d_qs_dlnP, t->d_qs_guide, t->params.qs, true);
-    v.bw_P = view2<double>(t->d_bw_P, t->d_bw_dP, t->d_bw_guide, t->params.bw, false);
+    v.qs_P = view2<double>(t->d_qs_lnP, t->d_qs_dlnP, t->d_qs_guide, t->params.qs, t->qs_fix,
+                           true);
+    v.bw_P = view2<double>(t->d_bw_P, t->d_bw_dP, t->d_bw_guide, t->params.bw, t->bw_fix, false);
     return v;
 }
 
@@ -245,8 +248,9 @@ TablesView<float> make_view<float>(const qed_tables *t)
     TablesView<float> v;
     v.qs_G = view1<float>(t->f_qs_lnG, t->params.qs, t->qs_fix);
     v.bw_T = view1<float>(t->f_bw_lnT, t->params.bw, t->bw_fix);
-    v.qs_P = view2<float>(t->f_qs_lnP, t->f_qs_dlnP, t->f_qs_guide, t->params.qs, true);
-    v.bw_P = view2<float>(t->f_bw_P, t->f_bw_dP, t->f_bw_guide, t->params.bw, false);
+    v.qs_P = view2<float>(t->f_qs_lnP, t->f_qs_dlnP, t->f_qs_guide, t->params.qs, t->qs_fix,
+                           true);
+    v.bw_P = view2<float>(t->f_bw_P, t->f_bw_dP, t->f_bw_guide, t->params.bw, t->bw_fix, false);
     return v;
 }
 

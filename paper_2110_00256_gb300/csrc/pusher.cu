@@ -41,8 +41,10 @@ __device__ __forceinline__ void push_one(const PushSeg<T> &g, int64_t i, const W
     advance<T>(g, i, x, ex, ey, ez, bx, by, bz, dt);
 }
 
+// FP32 six CTAs of 40 registers per SM, with the wave's constants as parameters: its
+// loads bound it (a cascade's 100 separate steps: 47.6 ms, five CTAs of 48 49.9)
 template <typename T>
-__global__ void __launch_bounds__(256) push_kernel(const PushSeg<T> *__restrict__ segs, int n_seg, WaveT<T> wt,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 4) push_kernel(const PushSeg<T> *__restrict__ segs, int n_seg, WaveT<T> wt,
                                                     double t0, double dt, const int64_t *d_step, int64_t step)
 {
     extern __shared__ long long s_dyn[];  // [n_seg] inclusive prefix of particle counts

@@ -36,10 +36,13 @@ __global__ void __launch_bounds__(256, MLP ? 1 : 4) qs_event_kernel(const __grid
     flush_counts(a.com.stats, k, true);
 }
 
-// (four CTAs of 64 registers per SM: 2e6 FP64 decays, with the caller's ordering of
-// the products, 612 us; three 631, two 686 -- the table's rows are loads in a chain)
+// FP64 four CTAs of 64 registers per SM: 2e6 decays, with the caller's ordering of
+// the products, 612 us; three 631, two 686 (1e8 decays: 10.2 ms, three 10.8) -- the
+// table's rows are loads in a chain.  FP32 three: a decay there is bound by its
+// writes to 26 arrays, and more warps in flight scatter them (1e8 decays: 5.78 ms,
+// four 9.47; 2e6 with the ordering: 475 us, four 450)
 template <typename T, bool MLP>
-__global__ void __launch_bounds__(256, MLP ? 1 : 4) bw_event_kernel(const __grid_constant__ EventArgs<T> a)
+__global__ void __launch_bounds__(256, MLP ? 1 : (sizeof(T) == 8 ? 4 : 3)) bw_event_kernel(const __grid_constant__ EventArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);

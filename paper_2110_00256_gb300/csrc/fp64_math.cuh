@@ -1,7 +1,7 @@
-// fp64_math.cuh -- table-driven FP64 exponential and logarithm for the 1-D rate
-// lookups of the FP64 evolution.  GB300's FP64 pipe bounds that kernel, so its
-// speed is its FP64 instruction count, and these two functions are a quarter
-// of it.  Both take P. T. P. Tang's table-driven reductions (ACM TOMS 15 (1989)
+// fp64_math.cuh -- table-driven FP64 exponential and logarithm: of the FP64 forms
+// behind the integer ones (fixed64.cuh: particles and draws that the integers
+// cannot hold) and of table generation.  GB300's FP64 pipe bounds those, so their
+// speed is their FP64 instruction count.  Both take P. T. P. Tang's table-driven reductions (ACM TOMS 15 (1989)
 // 144 for the exponential, 16 (1990) 378 for the logarithm) with Taylor
 // polynomials of the reduced argument; the tables hold correctly rounded values
 // (fp64_tables.h, written by gen_fp64_tables.py).  Every table index and the

@@ -1,5 +1,5 @@
-// measure.cu -- standalone throughput probes: the FP64 peak against which the
-// FP64 evolution kernel (bound by GB300's FP64 pipe) is judged, measured by a
+// measure.cu -- standalone throughput probes: the FP64 pipe's peak, which bounds
+// FP64 instructions (and why the FP64 path runs on integers), measured by a
 // kernel that does nothing but dependent chains of fused multiply-adds; the
 // special-function unit's tanh.approx.f32 rate, which bounds the learned
 // sampler's GELUs; and an evaluation of the rate lookups' FP64 logarithm and

@@ -89,7 +89,8 @@ constexpr double kLnTLarge = -0.9686047877362934;  // ln kTLarge
 // form when chi is small against gamma |E| + |p| |B|; a particle at rest has
 // chi = |E|.  FP64 keeps the difference form: its cancellation error, 1e-16
 // (S/chi)^2 relative, is below the FP64 tolerance, and it saves the FP64
-// square root and division of n, FP64 being GB300's scarce unit.
+// square root and division of n (as does the integer form that runs first,
+// fixed64.cuh).
 // The rate multiplies by 1/gamma.  FP64 takes gamma and 1/gamma from one
 // reciprocal square root (within 1 ulp); FP32 keeps IEEE square roots and
 // divisions here (with reciprocal square roots the HBM-bound evolution kernel

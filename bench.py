@@ -96,7 +96,7 @@ def peaks():
 
 
 KERNEL_SOURCES = ("evolve.cu", "evolve.cuh", "evolve_core.cuh", "physics.cuh", "common.cuh", "pipeline.cuh",
-                  "fp64_math.cuh", "fp64_tables.h")
+                  "fp64_math.cuh", "fp64_tables.h", "fixed64.cuh", "fixed_tables.h", "launch.cuh")
 
 
 def kernel_hash() -> str:
@@ -982,15 +982,16 @@ def gpu_main(args):
         result["paths"]["fp64_table"]["fp64_fma_probe"] = {
             "fma_per_s": probe["fma_per_s"], "per_sm_per_clock": round(probe["fma_per_s"] / (sms * mhz * 1e6), 3),
             "clock_mhz_assumed": mhz, "ms": round(probe["ms"], 3)}
-        ipp = profile_record("evolve_kernel_fp64_insts.txt", "fp64_inst_per_particle")
+        # the evolution runs on 64-bit integers: its bound is the instruction issue
+        ipp = profile_record("evolve_kernel_fp64_insts.txt", "warp_inst_per_particle")
         if ipp:
-            peak64 = probe["fma_per_s"]
+            peak64 = 4.0 * sms * mhz * 1e6
             ach_i = ipp * r64["n_before"] / (ev64 * 1e-3)
             result["paths"]["fp64_table"]["roofline"] = {
-                "bound": "alu", "kernel": "evolve_kernel<double,2,4,3>", "unit": "FP64 instructions/s",
+                "bound": "issue", "kernel": "evolve_kernel<double,2,256>", "unit": "warp instructions/s",
                 "achieved": ach_i, "peak": peak64, "frac": round(ach_i / peak64, 4),
-                "peak_kind": "measured: qed_probe_fp64_fma (dependent DFMA chains) on this GPU",
-                "fp64_inst_per_particle": ipp}
+                "peak_kind": "four issue slots per SM and clock at the sampled clock",
+                "warp_inst_per_particle": ipp}
         bufs, fire = b64, f64
         del b64, f64
         torch.cuda.empty_cache()

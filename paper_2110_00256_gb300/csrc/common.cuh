@@ -131,13 +131,14 @@ constexpr int kGuideBins = 64;
 
 template <typename T>
 struct Table2D {
-    const T *v;      // [n_chi][n_xi], ln P (QS) or P (BW)
-    const T *dv;     // [n_chi][n_xi], v[n][m+1] - v[n][m] formed in FP64 (last column 0)
+    const T *v;      // [n_chi][pitch], ln P (QS) or P (BW)
+    const T *dv;     // [n_chi][pitch], v[n][m+1] - v[n][m] formed in FP64 (last column 0)
     const int32_t *guide;  // [n_chi][kGuideBins + 1]: per row, the largest m with v[n][m] at or
                            // below each edge of kGuideBins equal bins of the uniform draw r
     T ln_min, inv_d, chi_min, chi_max;
     T x0, dx;        // xi axis: QS ln xi_min and step in ln xi; BW 0 and step in xi
     int n_chi, n_xi;
+    int pitch;       // from row to row of v and dv (FP32: padded, see tables.cu)
     FixAxis fix;     // the chi axis on integers
     Fix dx_fix;      // dx 2^dx_shift in [2^61, 2^62) (QS: dx_shift >= 63, or 0: the integers cannot hold it)
     int dx_shift;

@@ -289,9 +289,9 @@ __device__ __forceinline__ void locate_2d(const Table2D<T> &tb, T chi, const T *
     n = n > tb.n_chi - 2 ? tb.n_chi - 2 : n;
     w = t - T(n);
     row = n;
-    off = (size_t)n * tb.n_xi;
+    off = (size_t)n * tb.pitch;
     r0 = tb.v + off;
-    r1 = r0 + tb.n_xi;
+    r1 = r0 + tb.pitch;
 }
 
 // where the search of a row starts: the bracket that the guide tables of the two
@@ -377,7 +377,7 @@ __device__ __forceinline__ bool fix_column(const Table2D<double> &tb, double chi
     int unit, row;
     const int64_t lc = fix_ln_value(mc << 11, (hi >> 20) - 1023 - 63, unit);
     const Fix w = fix_locate(tb.fix, unit == -63 ? (lc + 512) >> 10 : (lc + 8) >> 4, row);
-    const double *r0 = tb.v + (size_t)row * tb.n_xi, *r1 = r0 + tb.n_xi;
+    const double *r0 = tb.v + (size_t)row * tb.pitch, *r1 = r0 + tb.pitch;
     const int32_t *g0 = tb.guide + (size_t)row * (kGuideBins + 1), *g1 = g0 + kGuideBins + 1;
     b = b > kGuideBins - 1 ? kGuideBins - 1 : b;
     int hi_m;
@@ -460,7 +460,7 @@ __device__ __forceinline__ T qs_sample_row(const Table2D<T> &tb, T chi, T r)
     b = b > kGuideBins - 1 ? kGuideBins - 1 : (b < 0 ? 0 : b);
     const int m = search_row(r0, r1, w, tb.n_xi, lr, g0, g0 + kGuideBins + 1, b);
     const T p0 = row_val(r0, r1, w, m);
-    const T dp = row_val(tb.dv + off, tb.dv + off + tb.n_xi, w, m);  // P_{m+1} - P_m
+    const T dp = row_val(tb.dv + off, tb.dv + off + tb.pitch, w, m);  // P_{m+1} - P_m
     const T x0 = tb.x0 + T(m) * tb.dx;
     const T x1 = (m + 1 == tb.n_xi - 1) ? T(0) : tb.x0 + T(m + 1) * tb.dx;
     if (!(dp > T(0))) return s_exp(x0);
@@ -503,7 +503,7 @@ __device__ __forceinline__ T bw_sample_row(const Table2D<T> &tb, T chi, T r)
     b = b > kGuideBins - 1 ? kGuideBins - 1 : (b < 0 ? 0 : b);
     const int m = search_row(r0, r1, w, tb.n_xi, r, g0, g0 + kGuideBins + 1, b);
     const T p0 = row_val(r0, r1, w, m);
-    const T dp = row_val(tb.dv + off, tb.dv + off + tb.n_xi, w, m);
+    const T dp = row_val(tb.dv + off, tb.dv + off + tb.pitch, w, m);
     const T x0 = T(m) * tb.dx;
     const T x1 = (m + 1 == tb.n_xi - 1) ? T(0.5) : T(m + 1) * tb.dx;
     if (!(dp > T(0))) return x0;

@@ -33,6 +33,15 @@ qed_status check_params(const qed_table_params *p)
     return check_axis(p->bw, "bw", false);
 }
 
+// Rows of the FP32 2-D tables lie pitch32() apart: a draw's hot columns (where P is
+// large) are one or two of a row's 128-byte lines, and at a power-of-two distance
+// the rows' hot lines share a fraction of the cache's sets -- how large a one then
+// hangs on where the arrays happen to lie.  1e8 FP32 draws from 256x256 tables: ln P
+// 3.85e10 -> 5.35e10 per second (256 floats apart, as separate allocations: 4.06e10),
+// P 3.47e10 -> 3.9e10 to 4.2e10 with each process's arrays side by side (3.4e10 to
+// 3.6e10 scattered or with the guide between them; separate allocations 4.1e10 to 4.4e10).
+static int pitch32(int n_xi) { return (n_xi + 31) / 32 * 32 + 32; }
+
 // Everything formed entry by entry from the FP64 tables, in one launch: the
 // column differences d[n][m] = v[n][m+1] - v[n][m] of both 2-D tables in FP64 (0
 // in the last column) and the FP32 copies of all six.  blockIdx.y: process.
@@ -40,7 +49,7 @@ struct Derived {
     const double *one[2], *two[2];
     double *diff[2];
     float *f_one[2], *f_two[2], *f_diff[2];
-    int n_chi[2], n_xi[2];
+    int n_chi[2], n_xi[2], pitch32[2];
 };
 
 __global__ void derive_kernel(const Derived t)
@@ -51,8 +60,9 @@ __global__ void derive_kernel(const Derived t)
         const double v = t.two[p][i];
         const double d = (int)(i % cols) + 1 < cols ? t.two[p][i + 1] - v : 0.0;
         t.diff[p][i] = d;
-        t.f_diff[p][i] = __double2float_rn(d);
-        t.f_two[p][i] = __double2float_rn(v);
+        const int64_t k = i / cols * t.pitch32[p] + i % cols;
+        t.f_diff[p][k] = __double2float_rn(d);
+        t.f_two[p][k] = __double2float_rn(v);
         if (i < t.n_chi[p]) t.f_one[p][i] = __double2float_rn(t.one[p][i]);
     }
 }
@@ -62,7 +72,7 @@ __global__ void derive_kernel(const Derived t)
 // largest m with v[n][m] <= edge (0 if none); edge 0 is -inf, the last +inf.
 // A draw in bin b then lies between the rows' guides at b and b + 1.
 template <typename T>
-__device__ void guide_entry(const T *__restrict__ v, int n_xi, bool qs, int32_t *__restrict__ g)
+__device__ void guide_entry(const T *__restrict__ v, int n_xi, int pitch, bool qs, int32_t *__restrict__ g)
 {
     const int n = blockIdx.x, e = threadIdx.x;
     int32_t out;
@@ -72,7 +82,7 @@ __device__ void guide_entry(const T *__restrict__ v, int n_xi, bool qs, int32_t 
         out = n_xi - 1;
     } else {
         const T x = qs ? d_log(T(e) / T(kGuideBins)) : T(e) / T(2 * kGuideBins);
-        const T *row = v + (size_t)n * n_xi;
+        const T *row = v + (size_t)n * pitch;
         int lo = 0, hi = n_xi;  // largest m with row[m] <= x: row[lo] <= x (or lo == 0), row[hi] > x
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
@@ -92,9 +102,9 @@ __global__ void guide_kernel(const Derived t, int32_t *qs_d, int32_t *bw_d, int3
     const int p = blockIdx.y;
     if ((int)blockIdx.x >= t.n_chi[p] || threadIdx.x > kGuideBins) return;
     if (blockIdx.z)
-        guide_entry<float>(t.f_two[p], t.n_xi[p], p == 0, p ? bw_f : qs_f);
+        guide_entry<float>(t.f_two[p], t.n_xi[p], t.pitch32[p], p == 0, p ? bw_f : qs_f);
     else
-        guide_entry<double>(t.two[p], t.n_xi[p], p == 0, p ? bw_d : qs_d);
+        guide_entry<double>(t.two[p], t.n_xi[p], t.n_xi[p], p == 0, p ? bw_d : qs_d);
 }
 
 static void free_tables(qed_tables *t)
@@ -153,11 +163,12 @@ qed_status alloc_tables(const qed_table_params *p, qed_tables **out, size_t scra
         place(t->d_qs_lnG, n1[0]), place(t->d_bw_lnT, n1[1]), place(t->d_qs_lnP, n2[0]), place(t->d_bw_P, n2[1]);
         t->derived = (void *)((uintptr_t)t->block + size);
         const size_t least = size + scratch;
-        place(t->d_qs_dlnP, n2[0]), place(t->d_bw_dP, n2[1]);
-        place(t->f_qs_lnG, n1[0]), place(t->f_qs_lnP, n2[0]), place(t->f_bw_lnT, n1[1]), place(t->f_bw_P, n2[1]);
-        place(t->f_qs_dlnP, n2[0]), place(t->f_bw_dP, n2[1]);
-        place(t->d_qs_guide, n1[0] * (kGuideBins + 1)), place(t->f_qs_guide, n1[0] * (kGuideBins + 1));
-        place(t->d_bw_guide, n1[1] * (kGuideBins + 1)), place(t->f_bw_guide, n1[1] * (kGuideBins + 1));
+        const size_t f2[2] = {n1[0] * pitch32(p->qs.n_xi), n1[1] * pitch32(p->bw.n_xi)};
+        place(t->f_qs_lnG, n1[0]), place(t->f_bw_lnT, n1[1]);
+        place(t->f_qs_lnP, f2[0]), place(t->f_qs_dlnP, f2[0]), place(t->f_qs_guide, n1[0] * (kGuideBins + 1));
+        place(t->f_bw_P, f2[1]), place(t->f_bw_dP, f2[1]), place(t->f_bw_guide, n1[1] * (kGuideBins + 1));
+        place(t->d_qs_dlnP, n2[0]), place(t->d_qs_guide, n1[0] * (kGuideBins + 1));
+        place(t->d_bw_dP, n2[1]), place(t->d_bw_guide, n1[1] * (kGuideBins + 1));
         if (size < least) size = least;
         if (pass) break;
         const cudaError_t e = cudaMalloc(&t->block, size);
@@ -176,7 +187,8 @@ qed_status finish_tables(qed_tables *t, cudaStream_t st)
     const qed_table_params &p = t->params;
     const Derived d{{t->d_qs_lnG, t->d_bw_lnT}, {t->d_qs_lnP, t->d_bw_P},     {t->d_qs_dlnP, t->d_bw_dP},
                     {t->f_qs_lnG, t->f_bw_lnT}, {t->f_qs_lnP, t->f_bw_P},     {t->f_qs_dlnP, t->f_bw_dP},
-                    {p.qs.n_chi, p.bw.n_chi},   {p.qs.n_xi, p.bw.n_xi}};
+                    {p.qs.n_chi, p.bw.n_chi},   {p.qs.n_xi, p.bw.n_xi},
+                    {pitch32(p.qs.n_xi), pitch32(p.bw.n_xi)}};
     const size_t most = n_qs2(p) > n_bw2(p) ? n_qs2(p) : n_bw2(p);
     const unsigned blocks = (unsigned)((most + 255) / 256 < 1024 ? (most + 255) / 256 : 1024);
     derive_kernel<<<dim3(blocks, 2), 256, 0, st>>>(d);
@@ -222,6 +234,7 @@ static Table2D<T> view2(const T *f, const T *df, const int32_t *guide, const qed
     v.chi_max = (T)a.chi_max;
     v.n_chi = a.n_chi;
     v.n_xi = a.n_xi;
+    v.pitch = sizeof(T) == 4 ? pitch32(a.n_xi) : a.n_xi;
     const double dx = qs ? -std::log(a.xi_min) / (a.n_xi - 1) : 0.5 / (a.n_xi - 1);
     v.x0 = qs ? (T)std::log(a.xi_min) : (T)0;
     v.dx = (T)dx;

@@ -435,7 +435,8 @@ __device__ __forceinline__ bool qs_sample_fixed(const Table2D<double> &tb, doubl
     const int64_t y = (mul_q62(fix_limbs(c), tb.dx_fix) + ((1ll << sh) >> 1)) >> sh;
     // near xi = 1 the lepton keeps gamma (1 - xi), a rounding of xi over 1 - xi: as before
     if (y < (1ll << 50)) return false;
-    xi = fix_to_double(fix_exp(-y, k, kFixExp), k - 62);
+    const int64_t e = fix_exp(-y, k, kFixExp);  // (its own statement: it sets k)
+    xi = fix_to_double(e, k - 62);
     return true;
 }
 static_assert(kGuideBins == 64, "the guide's bin is the top 6 bits of r");

@@ -1,0 +1,79 @@
+"""The FP64 inverse CDF of photon emission (csrc/physics.cuh), compiled for the host,
+against the same interpolation in extended precision."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import oracle
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+LD = np.longdouble
+EPS = LD(2) ** -53
+N_CHI, N_XI, LO, HI, XI_MIN = 48, 80, 1e-3, 1e3, 1e-12
+
+
+def ptr(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("sampling")
+    (d / "cuda_runtime.h").write_text('#include "device_shim.h"\n')
+    so = str(d / "sampling.so")
+    subprocess.run(["g++", "-O2", "-std=gnu++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", str(d), "-I", HERE,
+                    "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2110_00256_gb300", "csrc"),
+                    os.path.join(HERE, "sampling_shim.cpp"), "-o", so], check=True)
+    return ctypes.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def rows():
+    t = oracle.tables(qs_chi_min=LO, qs_chi_max=HI, qs_n_chi=N_CHI, qs_n_xi=N_XI, qs_xi_min=XI_MIN, bw_n_chi=8, bw_n_xi=8)
+    return np.ascontiguousarray(t.qs_lnP, dtype=np.float64).reshape(N_CHI, N_XI)
+
+
+def draws(lib, rows, chi, r):
+    """xi by the integers, which draws they took, by the general form and with FP64 logarithms throughout."""
+    n = r.size
+    out, ok = [np.zeros(n) for _ in range(3)], np.zeros(n, dtype=np.int32)
+    lib.host_qs(N_CHI, N_XI, ctypes.c_double(LO), ctypes.c_double(HI), ctypes.c_double(XI_MIN), ptr(rows),
+                ctypes.c_int64(n), ptr(chi), ptr(r), ptr(out[0]), ptr(ok), ptr(out[1]), ptr(out[2]))
+    return out[0], ok.astype(bool), out[1], out[2]
+
+
+def reference(rows, chi, r):
+    """xi in extended precision, and a bound of its relative error by roundings of the rows, of ln r and of the weight
+    between the rows (2^-53 of their magnitudes, the weight's by the logarithms in it), and of ln xi."""
+    lr = np.where(r > 0.5, np.log1p((r - 1.0).astype(LD)), np.log(r.astype(LD)))
+    l0, l1, lc = np.log(LD(LO)), np.log(LD(HI)), np.log(chi.astype(LD))
+    pos = np.clip((lc - l0) * (N_CHI - 1) / (l1 - l0), 0, N_CHI - 1)
+    k = np.minimum(pos.astype(int), N_CHI - 2)
+    a, b = rows[k].astype(LD), rows[k + 1].astype(LD)
+    row = a + (pos - k)[:, None] * (b - a)
+    m, i = np.clip((row <= lr[:, None]).sum(axis=1) - 1, 0, N_XI - 2), np.arange(r.size)
+    dp = row[i, m + 1] - row[i, m]
+    f = (lr - row[i, m]) / dp
+    dx = LD(-np.log(XI_MIN) / (N_XI - 1))
+    y = np.minimum((m + f - (N_XI - 1)) * dx, 0)
+    err_w = 4 * EPS * (np.abs(lc) + abs(l0)) * (N_CHI - 1) / (l1 - l0)
+    err_p = 3 * EPS * np.abs(row[i, m]) + err_w * np.maximum(np.abs(b - a)[i, m], np.abs(b - a)[i, m + 1]) + EPS * np.abs(lr)
+    return np.exp(y), err_p * (1 + np.abs(f)) / dp * dx + 4 * EPS * (1 + np.abs(y) + abs(np.log(LD(XI_MIN))))
+
+
+def test_photon_sampling_on_integers(lib, rows):
+    """A draw's xi on the integers is the interpolation's, whatever order a compiler evaluates arguments in."""
+    rng = np.random.default_rng(3)
+    n = 40_000
+    chi = np.exp(rng.uniform(np.log(LO), np.log(HI), n))
+    r = np.exp(rng.uniform(np.log(2.0 ** -20), 0.0, n))
+    r[::2] = rng.uniform(0.0, 0.95, r[::2].size)
+    xi, ok, general, _ = draws(lib, rows, chi, r)
+    assert ok.mean() > 0.8
+    ref, tol = reference(rows, chi, r)
+    assert np.all(np.abs(xi[ok] / ref[ok] - 1) <= tol[ok])
+    assert np.all(np.abs(general / ref - 1) <= tol)

@@ -294,7 +294,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1)
     __shared__ long long s_warp[THREADS / 32];
     __shared__ int s_abort;
 
-    stage_rates(rs, tab, dt, THREADS);
+    stage_rates(rs, tab, dt, cut_qs, cut_bw, THREADS);
     allow_next();
     wait_previous();
     if (threadIdx.x == 0) {

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
     __shared__ long long s_n[MAXSEG];
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
-    stage_rates(rs, a.tab, a.dt, blockDim.x);
+    stage_rates(rs, a.tab, a.dt, a.chi_cut[QED_PROC_QS], a.chi_cut[QED_PROC_BW], blockDim.x);
     allow_next();
     wait_previous();
     if (threadIdx.x == 0) {
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__((CW + 1) * 32, MINB)
     __shared__ long long s_n[MAXSEG];
     __shared__ int s_abort;
 
-    stage_rates(rs, a.tab, a.dt, blockDim.x);
+    stage_rates(rs, a.tab, a.dt, a.chi_cut[QED_PROC_QS], a.chi_cut[QED_PROC_BW], blockDim.x);
     allow_next();
     wait_previous();
     if (threadIdx.x == 0) {
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS)
     long long *s_end = s_dyn, *s_n = s_dyn + n_seg;
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
-    stage_rates(rs, tab, dt, THREADS);
+    stage_rates(rs, tab, dt, cut_qs, cut_bw, THREADS);
     allow_next();
     wait_previous();
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);

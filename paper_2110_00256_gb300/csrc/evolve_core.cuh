@@ -73,9 +73,11 @@ struct RateSmem<double> {
     int r[256];
     int off[2];  // per process: nonzero if a value or a step of its table does not fit the integers
     double coef_dt[2];  // per process: the rate's constant factor times dt
+    long long ln_cut[2];  // per process: its chi cut-off (fix_ln_cut)
 };
 
-__device__ __forceinline__ void stage_rates(RateSmem<float> &s, const TablesView<float> &tab, float, int threads)
+__device__ __forceinline__ void stage_rates(RateSmem<float> &s, const TablesView<float> &tab, float, float, float,
+                                            int threads)
 {
     for (int i = threadIdx.x; i < tab.qs_G.n; i += threads) s.qs[i] = tab.qs_G.ln_f[i];
     for (int i = threadIdx.x; i < tab.bw_T.n; i += threads) s.bw[i] = tab.bw_T.ln_f[i];
@@ -105,9 +107,13 @@ __device__ __forceinline__ int stage_fix(long long *out, const Table1D<double> &
 }
 
 // every thread of the CTA; the caller's next barrier publishes it
-__device__ __forceinline__ void stage_rates(RateSmem<double> &s, const TablesView<double> &tab, double dt, int threads)
+__device__ __forceinline__ void stage_rates(RateSmem<double> &s, const TablesView<double> &tab, double dt, double cut_qs,
+                                            double cut_bw, int threads)
 {
-    if (threadIdx.x < 2) s.off[threadIdx.x] = 0, s.coef_dt[threadIdx.x] = (threadIdx.x ? kAlpha : 2.0 / 3.0 * kAlpha) * dt;
+    if (threadIdx.x < 2) {
+        s.off[threadIdx.x] = 0, s.coef_dt[threadIdx.x] = (threadIdx.x ? kAlpha : 2.0 / 3.0 * kAlpha) * dt;
+        s.ln_cut[threadIdx.x] = fix_ln_cut(threadIdx.x ? cut_bw : cut_qs, kFixLogR, kFixLog);
+    }
     __syncthreads();
     if (stage_fix(s.qs, tab.qs_G, threads)) s.off[0] = 1;
     if (stage_fix(s.bw, tab.bw_T, threads)) s.off[1] = 1;
@@ -173,7 +179,7 @@ struct EvolvedFp64 {
 
 // The same in FP64 throughout, out of line: the particles that the integers of
 // fixed64.cuh leave to it (blocks of subnormal or huge values, infinities, NaN,
-// a force far below its terms, chi at a table's end or at the cut-off).
+// a force far below its terms, chi within rounding of a table's end or of the cut-off).
 static __device__ __noinline__ EvolvedFp64 evolve_one_fp64(int proc, const Table1D<double> &tb, double px, double py,
                                                            double pz, double ex, double ey, double ez, double bx,
                                                            double by, double bz, double dt, double cut, double tau)
@@ -203,8 +209,8 @@ __device__ __forceinline__ bool evolve_one(int proc, const RateSmem<double> &rs,
     bool fast = fix_particle(qs, px, py, pz, ex, ey, ez, bx, by, bz, tb.fix, qs ? rs.qs : rs.bw, rs.r, rs.ln, rs.ex, o);
     // (tau = 0 or NaN: a rate that the integers drop as below 1e-290 could decide)
     const long long tb_bits = __double_as_longlong(tau) & 0x7fffffffffffffffll;
-    fast = fast && rs.off[qs ? 0 : 1] == 0 && tb_bits != 0 && tb_bits <= 0x7ff0000000000000ll &&
-           __double_as_longlong(cut) <= 0;  // (no cut-off; compared as bits: no FP64 instruction)
+    const FixCut at = fix_cut(o.ln_chi, rs.ln_cut[qs ? 0 : 1]);
+    fast = fast && rs.off[qs ? 0 : 1] == 0 && tb_bits != 0 && tb_bits <= 0x7ff0000000000000ll && !at.near;
     if (!fast) {
         const auto mag = [](double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; };
         const long long inf = 0x7ff0000000000000ll;
@@ -219,7 +225,7 @@ __device__ __forceinline__ bool evolve_one(int proc, const RateSmem<double> &rs,
         return r.fire != 0;
     }
     // the only FP64 instruction: tau - (rate / coef) (coef dt)
-    tau = fma(-o.rate, rs.coef_dt[qs ? 0 : 1], tau);
+    tau = fma(at.below ? 0.0 : -o.rate, rs.coef_dt[qs ? 0 : 1], tau);
     const bool fire = __double_as_longlong(tau) < 0 && __double_as_longlong(tau) != (long long)0x8000000000000000ull;
     if (fire) chi_out = sqrt(scalbn((double)o.s, o.s_e));
     return fire;

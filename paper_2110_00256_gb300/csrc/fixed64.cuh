@@ -316,6 +316,33 @@ __device__ __forceinline__ int64_t fix_table(const FixAxis &ax, const long long 
     return a + mul_q62(f, fix_limbs(tab[i + 1] - a));
 }
 
+// A chi cut-off on the integers: ln cut in units of 2^-53 (a particle's ln chi on the
+// integers is within 333, 2^61.4 units); -2^62 where no particle is below it (no
+// cut-off, or below e^-499), 2^62 where every one is (above e^499, infinite).
+constexpr long long kFixFar = 1ll << 62;
+
+__device__ __forceinline__ int64_t fix_ln_cut(double cut, const int *tab_r, const long long *tab_ln)
+{
+    const int hi = __double2hiint(cut);
+    if (hi < (1023 - 720) << 20) return -kFixFar;  // (also negative)
+    if (hi >= (1023 + 720) << 20) return kFixFar;
+    const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(cut);
+    return 2 * fix_half_ln(m << 11, (hi >> 20) - 1023 - 63, tab_r, tab_ln);
+}
+
+// ln chi against a cut-off: below: no evolution; near: within rounding of it, for the FP64 form to decide.
+// (With every particle under a cut-off left to that form, 4e6 leptons took 705 us instead of 158,
+// photons 748 instead of 164.)
+struct FixCut {
+    bool below, near;
+};
+
+__device__ __forceinline__ FixCut fix_cut(int64_t ln_chi, int64_t ln_cut)
+{
+    const int64_t d = ln_chi - ln_cut;
+    return FixCut{d < 0, (uint64_t)(d + 1024) <= 2048ull};
+}
+
 struct FixOut {
     double rate;     // rate / coef: G(chi)/gamma, chi T(chi)/|p|
     int64_t ln_chi;  // 2^-53

@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     long long *s_end = s_dyn, *s_n = s_dyn + n_seg;
     constexpr int64_t tile = (int64_t)THREADS * VEC;
 
-    stage_rates(rs, tab, wt.dt, THREADS);
+    stage_rates(rs, tab, wt.dt, cut_qs, cut_bw, THREADS);
     allow_next();
     wait_previous();
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);

@@ -1,4 +1,5 @@
-// The FP64 sampling (csrc/physics.cuh) compiled for the host, for tests/test_sampling_host.py.
+// The FP64 sampling (csrc/physics.cuh) and chi cut-offs (csrc/fixed64.cuh) compiled for the
+// host, for tests/test_sampling_host.py and tests/test_cut_host.py.
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -79,5 +80,15 @@ extern "C" void host_qs(int n_chi, int n_xi, double lo, double hi, double xi_min
                            std::min((int)(r[i] * kGuideBins), kGuideBins - 1));
         const double dp = row_val(d0, d1, w, m), x0 = t.x0 + m * t.dx, x1 = m + 1 == n_xi - 1 ? 0.0 : t.x0 + (m + 1) * t.dx;
         tang[i] = dp > 0.0 ? exp_tang(std::min(x0 + (lr - row_val(r0, r1, w, m)) * (x1 - x0) / dp, 0.0)) : exp_tang(x0);
+    }
+}
+
+// ln cut in units of 2^-53, and ln chi values of those units against it (1 below, 2 near, 3 both)
+extern "C" void host_cut(double cut, int64_t n, const int64_t *ln_chi, int64_t *ln_cut, int *side)
+{
+    *ln_cut = fix_ln_cut(cut, kFixLogR, kFixLog);
+    for (int64_t i = 0; i < n; ++i) {
+        const FixCut c = fix_cut(ln_chi[i], *ln_cut);
+        side[i] = (c.below ? 1 : 0) + (c.near ? 2 : 0);
     }
 }

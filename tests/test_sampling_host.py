@@ -1,34 +1,21 @@
 """The FP64 inverse CDF of photon emission (csrc/physics.cuh), compiled for the host,
 against the same interpolation in extended precision."""
 import ctypes
-import os
-import subprocess
 
 import numpy as np
 import pytest
 
 import oracle
+from host_build import compile_shim, ptr
 
-HERE = os.path.dirname(os.path.abspath(__file__))
-ROOT = os.path.dirname(HERE)
 LD = np.longdouble
 EPS = LD(2) ** -53
 N_CHI, N_XI, LO, HI, XI_MIN = 48, 80, 1e-3, 1e3, 1e-12
 
 
-def ptr(a):
-    return a.ctypes.data_as(ctypes.c_void_p)
-
-
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
-    d = tmp_path_factory.mktemp("sampling")
-    (d / "cuda_runtime.h").write_text('#include "device_shim.h"\n')
-    so = str(d / "sampling.so")
-    subprocess.run(["g++", "-O2", "-std=gnu++17", "-ffp-contract=off", "-shared", "-fPIC", "-I", str(d), "-I", HERE,
-                    "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2110_00256_gb300", "csrc"),
-                    os.path.join(HERE, "sampling_shim.cpp"), "-o", so], check=True)
-    return ctypes.CDLL(so)
+    return compile_shim("sampling_shim.cpp", tmp_path_factory.mktemp("sampling"))
 
 
 @pytest.fixture(scope="module")

@@ -17,8 +17,12 @@ struct EventArgs {
     EventCommon<T> com;
 };
 
+// With the learned sampler (here and in bw_event_kernel) two CTAs of 128 registers per
+// SM: its layers wait on one another, and 16 warps hide that better than 8 with all
+// the registers they ask for (164).  4e6 emissions in FP32 437 us, one CTA 672; pairs
+// 506, one 790; FP64 530 and 725, one 808 and 1102.
 template <typename T, bool MLP>
-__global__ void __launch_bounds__(256, MLP ? 1 : 4) qs_event_kernel(const __grid_constant__ EventArgs<T> a)
+__global__ void __launch_bounds__(256, MLP ? 2 : 4) qs_event_kernel(const __grid_constant__ EventArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);
@@ -42,7 +46,7 @@ __global__ void __launch_bounds__(256, MLP ? 1 : 4) qs_event_kernel(const __grid
 // writes to 26 arrays, and more warps in flight scatter them (1e8 decays: 5.78 ms,
 // four 9.47; 2e6 with the ordering: 475 us, four 450)
 template <typename T, bool MLP>
-__global__ void __launch_bounds__(256, MLP ? 1 : (sizeof(T) == 8 ? 4 : 3)) bw_event_kernel(const __grid_constant__ EventArgs<T> a)
+__global__ void __launch_bounds__(256, MLP ? 2 : (sizeof(T) == 8 ? 4 : 3)) bw_event_kernel(const __grid_constant__ EventArgs<T> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     InferSmem &S = *reinterpret_cast<InferSmem *>(smem_raw);

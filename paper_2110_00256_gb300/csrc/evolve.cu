@@ -298,7 +298,7 @@ static qed_status launch_bulk(const EvolveArgs<float, MAXSEG> &a, int64_t capaci
 template <typename T, int VEC, int THREADS>
 __global__ void __launch_bounds__(THREADS, 768 / THREADS)
     evolve_seg_kernel(const EvolveSeg<T> *__restrict__ segs, int n_seg, const __grid_constant__ TablesView<T> tab, T dt, T cut_qs, T cut_bw,
-                      long long *stats, int dry)
+                      long long *stats, int dry, long long *live)
 {
     __shared__ RateSmem<T> rs;
     __shared__ long long s_warp[THREADS / 32];
@@ -309,7 +309,8 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS)
     stage_rates(rs, tab, dt, cut_qs, cut_bw, THREADS);
     allow_next();
     wait_previous();
-    const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);
+    if (keeps_removed(live, stats)) live[n_seg] = removed_photons(stats);
+    const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp, live);
     int bad = 0;
     for (long long t = blockIdx.x; t < total; t += gridDim.x) {
         const int lo = find_segment(s_end, n_seg, t);
@@ -318,13 +319,12 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS)
                                      sg.proc == QED_PROC_QS ? cut_qs : cut_bw, stats, dry, bad);
     }
     if (!dry) warp_count_err(stats ? stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
-    if (stats && !dry && blockIdx.x == 0 && threadIdx.x < 32) count_evolved(s_n, n_seg, stats);
 }
 
 template <typename T, int THREADS>
 static qed_status launch_seg_impl(const EvolveSeg<T> *segs, int n_seg, const TablesView<T> &tab, T dt, T cut_qs,
                                   T cut_bw, long long *stats, int dry, bool vec, int ctas_per_sm, cudaStream_t st,
-                                  bool early)
+                                  bool early, long long *live)
 {
     const size_t dyn = (size_t)n_seg * 2 * sizeof(long long);
     int grid = sm_count() * (ctas_per_sm > 0 ? ctas_per_sm : 768 / THREADS);
@@ -339,7 +339,7 @@ static qed_status launch_seg_impl(const EvolveSeg<T> *segs, int n_seg, const Tab
             attr = true;
         }
         QED_CUDA_TRY(launch_next(false, evolve_seg_kernel<T, V, THREADS>, grid, THREADS, dyn, st, segs, n_seg, tab, dt, cut_qs,
-                                 cut_bw, stats, dry));
+                                 cut_bw, stats, dry, live));
     } else {
         static bool attr = false;
         if (!attr) {
@@ -348,7 +348,7 @@ static qed_status launch_seg_impl(const EvolveSeg<T> *segs, int n_seg, const Tab
             attr = true;
         }
         QED_CUDA_TRY(launch_next(early, evolve_seg_kernel<T, 1, THREADS>, grid, THREADS, dyn, st, segs, n_seg, tab, dt, cut_qs,
-                                 cut_bw, stats, dry));
+                                 cut_bw, stats, dry, live));
     }
     QED_LAUNCH_CHECK();
     return QED_OK;
@@ -357,27 +357,28 @@ static qed_status launch_seg_impl(const EvolveSeg<T> *segs, int n_seg, const Tab
 template <typename T>
 qed_status launch_evolve_segments(const EvolveSeg<T> *d_segs, int n_seg, const TablesView<T> &tab, T dt, T cut_qs,
                                   T cut_bw, long long *stats, int dry, bool vec, int threads, int ctas_per_sm,
-                                  cudaStream_t st, bool early)
+                                  cudaStream_t st, bool early, long long *live)
 {
     if (n_seg <= 0) return QED_OK;
     switch (threads) {
     case 128:
         return launch_seg_impl<T, 128>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st,
-                                       early);
+                                       early, live);
     case 512:
         return launch_seg_impl<T, 512>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st,
-                                       early);
+                                       early, live);
     default:
         return launch_seg_impl<T, 256>(d_segs, n_seg, tab, dt, cut_qs, cut_bw, stats, dry, vec, ctas_per_sm, st,
-                                       early);
+                                       early, live);
     }
 }
 
 template qed_status launch_evolve_segments<float>(const EvolveSeg<float> *, int, const TablesView<float> &, float,
-                                                  float, float, long long *, int, bool, int, int, cudaStream_t, bool);
+                                                  float, float, long long *, int, bool, int, int, cudaStream_t, bool,
+                                                  long long *);
 template qed_status launch_evolve_segments<double>(const EvolveSeg<double> *, int, const TablesView<double> &,
                                                    double, double, double, long long *, int, bool, int, int,
-                                                   cudaStream_t, bool);
+                                                   cudaStream_t, bool, long long *);
 
 // clamp the firing counters to their capacity once the evolution is done
 __global__ void clamp_fire_counts(unsigned long long *c0, int64_t cap0, unsigned long long *c1, int64_t cap1,

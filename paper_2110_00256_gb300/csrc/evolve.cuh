@@ -59,11 +59,12 @@ bool fill_seg(EvolveSeg<T> &g, const qed_species *sp, int proc, const qed_fire_l
 
 // segments in device memory (the batched substep); threads in {128, 256, 512},
 // ctas_per_sm 0 = as many as the register budget allows; dry != 0 stores nothing;
-// cut_qs / cut_bw: chi thresholds of the two processes (rate zero below)
+// cut_qs / cut_bw: chi thresholds of the two processes (rate zero below); live: see
+// tile_prefix (NULL outside a step)
 template <typename T>
 qed_status launch_evolve_segments(const EvolveSeg<T> *d_segs, int n_seg, const TablesView<T> &tab, T dt, T cut_qs,
                                   T cut_bw, long long *stats, int dry, bool vec, int threads, int ctas_per_sm,
-                                  cudaStream_t st, bool early = false);
+                                  cudaStream_t st, bool early = false, long long *live = nullptr);
 
 qed_status check_fire(const qed_fire_list *f, const char *name);
 

@@ -331,13 +331,31 @@ __device__ __forceinline__ void load_scalar(const EvolveSeg<T> &sg, int64_t n, i
     }
 }
 
+// In a batched step, `live` (n_seg + 1 entries; else NULL) keeps the live counts as the
+// evolution reads them and, with stats, the photons removed by pair production that
+// are still in the arrays (read, but not evolved).  The step's events count the
+// evolved particles from them.  (A kernel that adds them up itself loses registers in
+// its loop: FP32 direct loads of 6e7 particles 541 us, so 512; with any code of it
+// after the loop 529.)
+__device__ __forceinline__ long long removed_photons(const long long *stats)
+{
+    return stats[QED_STAT_PAIRS] - stats[QED_STAT_COMPACTED];
+}
+
+__device__ __forceinline__ bool keeps_removed(const long long *live, const long long *stats)
+{
+    return live && stats && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0;  // (the last CTA has the fewest tiles)
+}
+
 // Segments in device memory (many patches): every CTA reads all segment
-// counts (clamped to capacity) into s_n, forms the inclusive prefix of their
-// tile counts in s_end by a block scan (thread k owns segments [k per,
-// (k+1) per)), and returns the total number of tiles.  Ends with a barrier.
+// counts (clamped to capacity) into s_n (and the first into `live`), forms the
+// inclusive prefix of their tile counts in s_end by a block scan (thread k owns
+// segments [k per, (k+1) per)), and returns the total number of tiles.  Ends with a
+// barrier.
 template <typename T, int THREADS>
 __device__ __forceinline__ long long tile_prefix(const EvolveSeg<T> *__restrict__ segs, int n_seg, int64_t tile,
-                                                 long long *s_end, long long *s_n, long long *s_warp)
+                                                 long long *s_end, long long *s_n, long long *s_warp,
+                                                 long long *live)
 {
     const int per = (n_seg + THREADS - 1) / THREADS;
     const int s0 = threadIdx.x * per, s1 = min(n_seg, s0 + per);
@@ -346,6 +364,7 @@ __device__ __forceinline__ long long tile_prefix(const EvolveSeg<T> *__restrict_
         long long n = *segs[s].count;
         n = n < 0 ? 0 : (n > segs[s].capacity ? segs[s].capacity : n);
         s_n[s] = n;
+        if (live && blockIdx.x == 0) live[s] = n;
         local += (n + tile - 1) / tile;
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -366,25 +385,6 @@ __device__ __forceinline__ long long tile_prefix(const EvolveSeg<T> *__restrict_
     }
     __syncthreads();
     return n_seg ? s_end[n_seg - 1] : 0;
-}
-
-// The batched step's particle count: one warp adds the live counts s_n of all
-// segments, as the evolution reads them, to QED_STAT_EVOLVED, less the photons
-// removed by pair production that are still in the arrays (QED_STAT_PAIRS -
-// QED_STAT_COMPACTED: they are read, but not evolved).  After a
-// kernel's loop, which it then costs no registers (before it, the cascade kernel
-// spilled and lost 5 %), and before the step's events.
-__device__ __forceinline__ void count_evolved(const long long *s_n, int n_seg, long long *stats)
-{
-    long long live = 0;
-    for (int i = threadIdx.x & 31; i < n_seg; i += 32) live += s_n[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) live += __shfl_xor_sync(0xffffffffu, live, o);
-    if ((threadIdx.x & 31) == 0) {
-        long long removed = stats[QED_STAT_PAIRS] - stats[QED_STAT_COMPACTED];
-        removed = removed < 0 ? 0 : (removed > live ? live : removed);
-        atomicAdd((unsigned long long *)(stats + QED_STAT_EVOLVED), (unsigned long long)(live - removed));
-    }
 }
 
 // the segment of tile t: the first s with s_end[s] > t

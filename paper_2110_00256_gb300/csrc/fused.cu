@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     push_evolve_kernel(const EvolveSeg<T> *__restrict__ segs, const PushSeg<T> *__restrict__ psegs, int n_seg,
                        const __grid_constant__ TablesView<T> tab, WaveT<T> wt, double t0, double dt_d,
                        const int64_t *d_step, int64_t step,
-                       T cut_qs, T cut_bw, long long *stats, int store_fields)
+                       T cut_qs, T cut_bw, long long *stats, int store_fields, long long *live)
 {
     __shared__ RateSmem<T> rs;
     __shared__ long long s_warp[THREADS / 32];
@@ -62,7 +62,10 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
     stage_rates(rs, tab, wt.dt, cut_qs, cut_bw, THREADS);
     allow_next();
     wait_previous();
-    const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp);
+    const bool keeps = keeps_removed(live, stats);
+    const long long removed = keeps ? removed_photons(stats) : 0;  // (its loads under way with those of the counts)
+    const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp, live);
+    if (keeps) live[n_seg] = removed;
     wt.t = (T)(t0 + (double)(d_step ? *d_step : step) * dt_d);
     const T dt = wt.dt;
     int bad = 0;
@@ -137,14 +140,13 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
         compact_fire<T, VEC>(sg, i0, fire, chi, cnt, stats);
     }
     warp_count_err(stats ? stats + QED_STAT_NONFINITE : nullptr, bad, QED_EW_NONFINITE);
-    if (stats && blockIdx.x == 0 && threadIdx.x < 32) count_evolved(s_n, n_seg, stats);
 }
 
 template <typename T, int VEC, bool YZ>
 static qed_status launch_fused_impl(const EvolveSeg<T> *segs, const PushSeg<T> *psegs, int n_seg,
                                     const TablesView<T> &tab, const WaveParams &w, double t0, double dt,
                                     const int64_t *d_step, int64_t step, T cut_qs, T cut_bw, long long *stats,
-                                    int store_fields, cudaStream_t st)
+                                    int store_fields, cudaStream_t st, long long *live)
 {
     constexpr int kThreads = 256;
     const size_t dyn = (size_t)n_seg * 2 * sizeof(long long);
@@ -160,20 +162,21 @@ static qed_status launch_fused_impl(const EvolveSeg<T> *segs, const PushSeg<T> *
         attr = true;
     }
     QED_CUDA_TRY(launch_next(false, push_evolve_kernel<T, VEC, kThreads, YZ>, sm_count() * per_sm, kThreads, dyn, st, segs, psegs,
-                             n_seg, tab, wave_in<T>(w, dt), t0, dt, d_step, step, cut_qs, cut_bw, stats, store_fields));
+                             n_seg, tab, wave_in<T>(w, dt), t0, dt, d_step, step, cut_qs, cut_bw, stats, store_fields, live));
     return QED_OK;
 }
 
 template <typename T>
 qed_status launch_push_evolve(const EvolveSeg<T> *d_segs, const void *d_push, int n_seg, const TablesView<T> &tab,
                               const WaveParams &w, double t0, double dt, const int64_t *d_step, int64_t step,
-                              T cut_qs, T cut_bw, long long *stats, int store_fields, bool vec, cudaStream_t st)
+                              T cut_qs, T cut_bw, long long *stats, int store_fields, bool vec, cudaStream_t st,
+                              long long *live)
 {
     if (n_seg <= 0) return QED_OK;
     const PushSeg<T> *p = (const PushSeg<T> *)d_push;
     const auto launch = [&](auto v, auto yz) {
         return launch_fused_impl<T, v.value, yz.value>(d_segs, p, n_seg, tab, w, t0, dt, d_step, step, cut_qs, cut_bw,
-                                                       stats, store_fields, st);
+                                                       stats, store_fields, st, live);
     };
     using One = std::integral_constant<int, 1>;
     using Two = std::integral_constant<int, 2>;
@@ -183,10 +186,10 @@ qed_status launch_push_evolve(const EvolveSeg<T> *d_segs, const void *d_push, in
 
 template qed_status launch_push_evolve<float>(const EvolveSeg<float> *, const void *, int, const TablesView<float> &,
                                               const WaveParams &, double, double, const int64_t *, int64_t, float,
-                                              float, long long *, int, bool, cudaStream_t);
+                                              float, long long *, int, bool, cudaStream_t, long long *);
 template qed_status launch_push_evolve<double>(const EvolveSeg<double> *, const void *, int,
                                                const TablesView<double> &, const WaveParams &, double, double,
                                                const int64_t *, int64_t, double, double, long long *, int, bool,
-                                               cudaStream_t);
+                                               cudaStream_t, long long *);
 
 }  // namespace qed

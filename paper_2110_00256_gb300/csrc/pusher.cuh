@@ -155,7 +155,8 @@ qed_status launch_push(const void *d_segs, int n_seg, const WaveParams &w, doubl
 template <typename T>
 qed_status launch_push_evolve(const EvolveSeg<T> *d_segs, const void *d_push, int n_seg, const TablesView<T> &tab,
                               const WaveParams &w, double t0, double dt, const int64_t *d_step, int64_t step,
-                              T cut_qs, T cut_bw, long long *stats, int store_fields, bool vec, cudaStream_t st);
+                              T cut_qs, T cut_bw, long long *stats, int store_fields, bool vec, cudaStream_t st,
+                              long long *live);
 
 qed_status check_wave(const qed_plane_wave *w);
 WaveParams wave_params(const qed_plane_wave *w);

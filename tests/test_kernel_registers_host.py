@@ -33,3 +33,11 @@ def test_event_kernels_with_the_learned_sampler_fit_twice(tmp_path):
     r = {k: v for k, v in resources("events.cu", tmp_path).items() if re.search(r"(qs|bw)_event_kernel<(float|double), true>", k)}
     assert len(r) == 4
     assert all(v[0] <= 128 for v in r.values()), r
+
+
+def test_direct_segment_evolution_reloads_no_more(tmp_path):
+    """FP32, four particles per thread at 80 registers: bound by its memory streams, and slower by 3 to 7 % with 64 bytes
+    of reloads per thread than with 44."""
+    r = {k: v for k, v in resources("evolve.cu", tmp_path).items() if re.search(r"evolve_seg_kernel<float, 4, (128|256)>", k)}
+    assert len(r) == 2
+    assert all(v[0] <= 80 and v[1] <= 44 for v in r.values()), r

@@ -742,7 +742,10 @@ extern "C" qed_status qed_tables_generate(const qed_table_params *params, qed_ta
     }();
     const int m = params->qs.n_xi > params->bw.n_xi ? params->qs.n_xi : params->bw.n_xi;
     const int dyn = (kPieces * kPieceRow + 3 * m) * (int)sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(table_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+    // (the largest row's size for every call: the attribute is the process's, and a smaller one set by
+    // another thread would refuse this launch)
+    constexpr int kMaxDyn = (kPieces * kPieceRow + 3 * QED_MAX_TABLE_N) * (int)sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(table_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDyn);
     if (e == cudaSuccess) {
         bessel_pieces_kernel<<<kPieces, 128, 0, st>>>(a.pieces);
         row_nodes_kernel<<<dim3((m + 3) / 4, 2), 128, 0, st>>>(a, gl);

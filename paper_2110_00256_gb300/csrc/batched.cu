@@ -589,6 +589,12 @@ static qed_status build_batch(const qed_patch *patches, int n, qed_batch *b, cud
     return QED_OK;
 }
 
+static qed_status record_event(void *event, cudaStream_t st)
+{
+    QED_CUDA_TRY(cudaEventRecord((cudaEvent_t)event, st));
+    return QED_OK;
+}
+
 // wave != NULL: the push in that wave is fused into the evolution (one pass
 // per particle), at time t0 + step * dt (step from opts->d_step when set)
 template <typename T>
@@ -630,22 +636,21 @@ static qed_status substep_batched_impl(const qed_tables *t, const qed_batch *b, 
                                       cut_bw, stats, 0, b->vec && !small, small ? 128 : threads, ctas, st, small,
                                       b->d_live);
     }
-    if (s) return s;
-    if (o && o->evolve_end) QED_CUDA_TRY(cudaEventRecord((cudaEvent_t)o->evolve_end, st));
+    if (s == QED_OK && o && o->evolve_end) s = record_event(o->evolve_end, st);
     const bool mlp = o && o->sampler == 1;
     const StepEnd end{b->d_clamp, b->d_count, n, o ? o->d_step : nullptr, b->d_live, stats};
-    if (mlp) {
+    if (s == QED_OK && mlp) {
         s = launch_events_batched<T, false>(b, event_common<T>(t, QED_PROC_BW, seed, step, o), StepEnd{}, true, st);
         if (s == QED_OK)
             s = launch_events_batched<T, true>(b, event_common<T>(t, QED_PROC_QS, seed, step, o), end, true, st);
-    } else {
+    } else if (s == QED_OK) {
         // the push fused into the evolution without stored fields computes every
         // particle's fields itself: the photons emitted get none
         EventCommon<T> cq = event_common<T>(t, QED_PROC_QS, seed, step, o);
         cq.copy_fields = (wave && !store_fields) ? 0 : 1;
         s = launch_events_batched_all<T>(b, cq, event_common<T>(t, QED_PROC_BW, seed, step, o), end, st);
     }
-    // (a step that was not ended leaves its firing counts behind)
+    // a step that was not ended leaves its firing counts behind, and the next one would take them for its own
     if (s) cudaMemsetAsync(b->d_count, 0, (3 * (size_t)n + 1) * sizeof(unsigned long long), st);
     return s;
 }

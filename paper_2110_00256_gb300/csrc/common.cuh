@@ -29,12 +29,16 @@ void clear_error();
         return (code);               \
     } while (0)
 
+// (the runtime keeps a failed call's error for the next cudaGetLastError: taken back,
+// so that the next launch check does not report it again)
 #define QED_CUDA_TRY(expr)                                                              \
     do {                                                                                \
         cudaError_t _e = (expr);                                                        \
-        if (_e != cudaSuccess)                                                          \
+        if (_e != cudaSuccess) {                                                        \
+            (void)cudaGetLastError();                                                   \
             QED_FAIL(QED_ERR_CUDA, "%s failed: %s (%s:%d)", #expr, cudaGetErrorString(_e), \
                      __FILE__, __LINE__);                                               \
+        }                                                                               \
     } while (0)
 
 #define QED_LAUNCH_CHECK()                                                               \

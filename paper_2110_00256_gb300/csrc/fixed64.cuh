@@ -249,28 +249,28 @@ __device__ __forceinline__ double fix_div(double a, double b)
 }
 
 // ln(n 2^e) = v 2^unit for n in [2^63, 2^64), |ln| < 62: the reduction of
-// fix_half_ln with the cubic term to 2^-58; within 2^-57 absolute, and 2^-53
-// relative (one rounding) above 1/8.  No FP64 instruction: one costs as much as
-// 76 issue slots, this function ~60.
+// fix_half_ln over intervals of 1/1024 (|u| < 2^-10.9, so that the cubic tail's 30
+// bits leave 2^-64): within 2^-62 absolute for arguments in [1/2, 2), where ln is
+// small, and 2^-57, less than a sixteenth of an ulp of FP64, beyond.  No FP64
+// instruction: one costs as much as 76 issue slots, this function ~60.
 __device__ __forceinline__ int64_t fix_ln_value(uint64_t n, int e, int &unit)
 {
-    const int j = (int)(n >> 55) & 255;
-    const uint32_t r = (uint32_t)__ldg(&kFixLogR[j]);
-    const int64_t u = (int64_t)((uwide((uint32_t)(n >> 32), r) << 17) + (uwide((uint32_t)n, r) >> 15));  // 2^-64
-    const int a = (int)(u >> 25);                  // 2^-39
-    const int b = (int)((uint32_t)u & 0x1ffffffu);  // 2^-64
-    const int64_t h2 = (wide(a, a) + (wide(a, b) >> 24)) >> 15;  // u^2/2, 2^-64
-    int t = 429496730 - (__mulhi(a, 357913941) >> 7);            // 1/3 - u/4 + u^2/5 - u^3/6, 2^-31
-    t = 536870912 - (__mulhi(a, t) >> 7);
-    t = 715827883 - (__mulhi(a, t) >> 7);
-    const int64_t c3 = wide((int)(h2 >> 15), (int)(wide(a, t) >> 29)) >> 25;  // u^3 t, 2^-64
-    const int64_t l = __ldg(&kFixLog[j]) + ((u - h2 + c3) >> 1);              // ln m, 2^-63
+    const int j = (int)(n >> 53) & 1023;
+    const uint32_t r = __ldg(&kFineLogR[j]);
+    const int64_t u = (int64_t)((uwide((uint32_t)(n >> 32), r) << 17) + ((uwide((uint32_t)n, r) + 16384) >> 15));  // 2^-64
+    const int a = (int)(u >> 24);                   // 2^-40
+    const int b = (int)((uint32_t)u & 0xffffffu);    // 2^-64
+    const int64_t h2 = (wide(a, a) + (wide(a, b) >> 23)) >> 17;  // u^2/2, 2^-64
+    int t = 536870912 - (__mulhi(a, 429496730) >> 8);            // 1/4 - u/5, 2^-31
+    t = 1431655765 - (__mulhi(a, t) >> 7);                       // 1/3 - u/4 + u^2/5, 2^-32
+    const int64_t c3 = wide((int)(h2 >> 11), (int)(wide(a, t) >> 29)) >> 31;  // u^3 t, 2^-64
+    const int64_t l = __ldg(&kFineLog[j]) + ((u - h2 + c3 + 1) >> 1);         // ln m, 2^-63
     const int k = 63 + e;
     // k ln 2 + ln m in 2^-57, or in 2^-63 where k is 0 or -1
     const bool fine = k == 0 || k == -1;
     const int64_t kl = (wide(k, (int)(kHalfLn2 >> 32)) << 27) + (wide(k, (int)((uint32_t)kHalfLn2 >> 1)) >> 4);
     unit = fine ? -63 : -57;
-    return fine ? (k ? l - 2 * kHalfLn2 : l) : kl + (l >> 6);
+    return fine ? (k ? l - kLn2 : l) : kl + ((l + 32) >> 6);
 }
 
 __device__ __forceinline__ double fix_ln(uint64_t n, int e)

@@ -40,6 +40,12 @@ def main():
     out.append("// r_j ~ 1/c_j, c_j = 1 + (j + 1/2)/256, 2^-16, and -ln r_j, 2^-63")
     out += table("kFixLogR", "int", r, 8, str)
     out += table("kFixLog", "long long", [q(-mp.log(mp.mpf(v) / 2 ** 16), 63) for v in r], 4, lambda v: hex(v) + "ll")
+    # the finer logarithm's: intervals of 1/1024
+    r = [q(1 / (1 + (mp.mpf(j) + mp.mpf(1) / 2) / 1024), 16) for j in range(1024)]
+    out.append("// the same for c_j = 1 + (j + 1/2)/1024; ln2, 2^-63")
+    out.append(f"constexpr long long kLn2 = {hex(q(ln2, 63))}ll;")
+    out += table("kFineLogR", "unsigned short", r, 12, str)
+    out += table("kFineLog", "long long", [q(-mp.log(mp.mpf(v) / 2 ** 16), 63) for v in r], 4, lambda v: hex(v) + "ll")
     print("\n".join(out))
 
 

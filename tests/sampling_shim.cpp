@@ -1,4 +1,4 @@
-// The FP64 sampling (csrc/physics.cuh) and chi cut-offs (csrc/fixed64.cuh) compiled for the
+// The FP64 sampling, the optical-depth draws (csrc/physics.cuh) and the chi cut-offs (csrc/fixed64.cuh) compiled for the
 // host, for tests/test_sampling_host.py and tests/test_cut_host.py.
 #include <algorithm>
 #include <cmath>
@@ -80,6 +80,18 @@ extern "C" void host_qs(int n_chi, int n_xi, double lo, double hi, double xi_min
                            std::min((int)(r[i] * kGuideBins), kGuideBins - 1));
         const double dp = row_val(d0, d1, w, m), x0 = t.x0 + m * t.dx, x1 = m + 1 == n_xi - 1 ? 0.0 : t.x0 + (m + 1) * t.dx;
         tang[i] = dp > 0.0 ? exp_tang(std::min(x0 + (lr - row_val(r0, r1, w, m)) * (x1 - x0) / dp, 0.0)) : exp_tang(x0);
+    }
+}
+
+// -ln U of the Philox words (lo, hi): the draw, and the table-driven FP64 logarithm
+extern "C" void host_draw(int64_t n, const uint32_t *lo, const uint32_t *hi, double *u, double *draw, double *tang)
+{
+    for (int64_t i = 0; i < n; ++i) {
+        int64_t v;
+        int unit;
+        u[i] = uniform53(lo[i], hi[i]);
+        draw[i] = neg_log_words(U4{lo[i], hi[i], 0, 0}, v, unit) ? fix_to_double(v, unit) : neg_log1p_series(u[i]);
+        tang[i] = u[i] > 1.0 - 0x1p-8 ? neg_log1p_series(u[i]) : -log_tang_core(u[i], 0);
     }
 }
 

@@ -64,3 +64,24 @@ def test_photon_sampling_on_integers(lib, rows):
     ref, tol = reference(rows, chi, r)
     assert np.all(np.abs(xi[ok] / ref[ok] - 1) <= tol[ok])
     assert np.all(np.abs(general / ref - 1) <= tol)
+
+
+def rms(x):
+    return float(np.sqrt(np.mean(np.asarray(x, dtype=np.float64) ** 2)))
+
+
+@pytest.mark.parametrize("lo,hi", [(2.0 ** -(k + 1), 2.0 ** -k) for k in range(16)] + [(1, 2), (2, 4), (4, 8), (8, 16), (16, 36)])
+def test_optical_depth_draws_are_no_further_off_than_in_fp64(lib, lo, hi):
+    """-ln U over its octaves, U with 53 random bits: rms and largest error no larger than with the table-driven FP64
+    logarithm (the series above U = 1 - 2^-8 is the same in both), and the largest at most 1.5 roundings (2^-53)."""
+    rng = np.random.default_rng(7)
+    n = 200_000
+    v = np.exp(-rng.uniform(lo, hi, n))
+    bits = (np.minimum((v * 2.0 ** 53).astype(np.uint64), np.uint64(2 ** 53 - 1)) << np.uint64(11)) | rng.integers(
+        0, 2048, n, dtype=np.uint64)
+    w0, w1 = (bits & np.uint64(0xffffffff)).astype(np.uint32), (bits >> np.uint64(32)).astype(np.uint32)
+    u, tau, tang = np.zeros(n), np.zeros(n), np.zeros(n)
+    lib.host_draw(ctypes.c_int64(n), ptr(w0), ptr(w1), ptr(u), ptr(tau), ptr(tang))
+    ref = np.where(u > 0.5, -np.log1p((u - 1.0).astype(LD)), -np.log(u.astype(LD)))
+    err, err64 = (np.abs(x / ref - 1).astype(np.float64) for x in (tau, tang))
+    assert rms(err) <= rms(err64) and err.max() <= err64.max() and err.max() <= 1.5 * 2.0 ** -53

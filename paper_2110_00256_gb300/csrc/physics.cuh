@@ -70,6 +70,14 @@ __device__ __forceinline__ double log_int(double x)
 // the tables' spacing) and Tang's exponential
 __device__ __forceinline__ float s_log(float x) { return logf(x); }
 __device__ __forceinline__ double s_log(double x) { return log_int(x); }
+// and of the draw r itself: near r = 1, where ln r is small and decides the hardest
+// photons' xi, by the series that the optical-depth resets take
+static __device__ __noinline__ double neg_log1p_series(double u);
+__device__ __forceinline__ float s_log_draw(float r) { return logf(r); }
+__device__ __forceinline__ double s_log_draw(double r)
+{
+    return __double_as_longlong(r) > __double_as_longlong(1.0 - 0x1p-8) ? -neg_log1p_series(r) : log_int(r);
+}
 __device__ __forceinline__ float s_exp(float x) { return expf(x); }
 __device__ __forceinline__ double s_exp(double x) { return exp_tang(x); }
 
@@ -334,7 +342,9 @@ __device__ __forceinline__ int search_row(const T *r0, const T *r1, T w, int M, 
 // They return false, for the general forms: chi outside [2^-86, 2^86], a table that
 // the units cannot hold, a draw off its row's ends or on a flat stretch, and small
 // draws -- BW r < 2^-9 (1 in 256), where FP64 holds more than the unit does, QS
-// r < 2^-20 -- and QS xi above e^(-1/8).
+// r < 2^-20 --, QS r above 1 - 2^-15, where ln P and ln r are small and FP64 holds more of
+// them (its error stays at 1e-15 with ln r by its series, the integers' is 1e-11 at 1 - 2^-30), and QS
+// xi above e^(-1/8).
 // ---------------------------------------------------------------------------
 struct UnitBW {  // a value in [0, 1], rounded down; anything else: ok = false
     static __device__ __forceinline__ int64_t of(double x, int, bool &ok)
@@ -420,7 +430,7 @@ __device__ __forceinline__ bool qs_sample_fixed(const Table2D<double> &tb, doubl
     const int hi = __double2hiint(r);
     bool ok = true;
     const int64_t v = UnitBW::of(r, 0, ok);
-    if (!ok || hi < 0x3eb00000 || !tb.dx_shift) return false;  // 2^-20 <= r <= 1
+    if (!ok || hi < 0x3eb00000 || hi >= 0x3fefffc0 || !tb.dx_shift) return false;  // 2^-20 <= r < 1 - 2^-15
     const uint64_t mr = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(r);
     int unit, m, k;
     int64_t f;
@@ -455,7 +465,7 @@ __device__ __forceinline__ T qs_sample_row(const Table2D<T> &tb, T chi, T r)
     size_t off;
     int row;
     locate_2d(tb, chi, r0, r1, w, off, row);
-    const T lr = s_log(r);
+    const T lr = s_log_draw(r);
     const int *g0 = tb.guide + (size_t)row * (kGuideBins + 1);
     int b = (int)(r * T(kGuideBins));
     b = b > kGuideBins - 1 ? kGuideBins - 1 : (b < 0 ? 0 : b);

@@ -70,6 +70,20 @@ def rms(x):
     return float(np.sqrt(np.mean(np.asarray(x, dtype=np.float64) ** 2)))
 
 
+@pytest.mark.parametrize("e", [*range(1, 20), 23, 27, 31, 35, 39, 43])
+def test_hard_photons_are_no_further_off_than_in_fp64(lib, rows, e):
+    """1 - r in [2^-(e+1), 2^-e]: the draw as the library makes it (integers, else the general form) has an rms error no
+    larger than the general form with FP64 logarithms; 2 % for what the two share, the table's arithmetic in FP64."""
+    rng = np.random.default_rng(100 + e)
+    n = 20_000
+    chi = np.exp(rng.uniform(np.log(LO), np.log(HI), n))
+    r = 1.0 - 2.0 ** -e * rng.uniform(0.5, 1.0, n)
+    xi, ok, general, tang = draws(lib, rows, chi, r)
+    ref, _ = reference(rows, chi, r)
+    now = np.where(ok, xi, general)
+    assert rms(now / ref - 1) <= 1.02 * rms(tang / ref - 1)
+
+
 @pytest.mark.parametrize("lo,hi", [(2.0 ** -(k + 1), 2.0 ** -k) for k in range(16)] + [(1, 2), (2, 4), (4, 8), (8, 16), (16, 36)])
 def test_optical_depth_draws_are_no_further_off_than_in_fp64(lib, lo, hi):
     """-ln U over its octaves, U with 53 random bits: rms and largest error no larger than with the table-driven FP64

@@ -363,9 +363,10 @@ __device__ __forceinline__ bool fix_particle(bool qs, double px, double py, doub
     int ep = imax(imax(mag_hi(px), mag_hi(py)), mag_hi(pz)) >> 20;
     const int me = imax(imax(mag_hi(ex), mag_hi(ey)), mag_hi(ez));
     const int mf = imax(imax(me, mag_hi(bx)), imax(mag_hi(by), mag_hi(bz))), ef = mf >> 20;
-    // blocks within 2^+-400 (no infinity, NaN or subnormal, and no overflow that FP64 would see)
-    bool ok = ax.ok && (unsigned)(ep - 623) <= 800u && (unsigned)(ef - 623) <= 800u;
     if (qs) ep = imax(ep, 1023);  // gamma^2 = 1 + p^2 on one scale
+    // blocks within 2^+-400 (no infinity, NaN or subnormal, and no overflow that FP64 would see; a lepton's
+    // momentum may be anything below 1, at rest too)
+    bool ok = ax.ok && (unsigned)(ep - 623) <= 800u && (unsigned)(ef - 623) <= 800u;
     const int tp = ep << 20 | 0xfffff, tf = ef << 20 | 0xfffff;
     const Fix x = fix_from(px, tp), y = fix_from(py, tp), z = fix_from(pz, tp);
     Acc a{wide(x.h, x.h) + wide(y.h, y.h) + wide(z.h, z.h), wide(x.h, x.l) + wide(y.h, y.l) + wide(z.h, z.l)};

@@ -66,3 +66,19 @@ def test_a_force_that_fp64_holds_is_left_to_it(lib):
     p[1:3] = r.normal(size=(2, N))
     p[7:] = 1e-6 * r.normal(size=(2, N))
     assert not run(lib, True, p)[3].any()
+
+
+@np.errstate(divide="ignore", invalid="ignore")
+def test_leptons_at_rest(lib):
+    """No momentum, or one far below 1 (subnormal too): chi = |E| and the rate as exact as the FP64 path's; taken where E is
+    of the fields' size (elsewhere FP64 holds gamma E better than a block scaled by B)."""
+    p = particles("gauss", N, 6)
+    p[:3] = 0.0
+    p[0, ::4] = 1e-310
+    p[1, 1::4] = -1e-200
+    p[:3, 2::4] = 1e-30
+    rate, _, chi, ok, (r_ref, c_ref, _), (r_64, c_64, _) = run(lib, True, p)
+    assert ok[np.abs(p[3:6]).max(0) >= np.abs(p[6:]).max(0) / 4].all() and ok.mean() > 0.9
+    assert np.all(np.abs(chi[ok] / c_ref[ok] - 1) <= 2.0 ** -51)
+    e, e64 = (np.abs(x[ok] / r_ref[ok] - 1).astype(np.float64) for x in (rate, r_64))
+    assert np.sqrt(np.mean(e ** 2)) <= np.sqrt(np.mean(e64 ** 2)) and e.max() <= e64.max()

@@ -319,7 +319,6 @@ __global__ void __launch_bounds__((CW + 1) * 32, 1)
 
     stage_rates(rs, tab, dt, cut_qs, cut_bw, THREADS);
     allow_next();
-    wait_previous();
     if (threadIdx.x == 0) {
         s_abort = 0;
         for (int k = 0; k < S; ++k) {

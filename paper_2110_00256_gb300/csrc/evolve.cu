@@ -159,7 +159,6 @@ __global__ void __launch_bounds__((CW + 1) * 32, MINB)
 
     stage_rates(rs, a.tab, a.dt, a.chi_cut[QED_PROC_QS], a.chi_cut[QED_PROC_BW], blockDim.x);
     allow_next();
-    wait_previous();
     if (threadIdx.x == 0) {
         long long acc = 0;
         for (int s = 0; s < a.n_seg; ++s) {

@@ -61,7 +61,6 @@ __global__ void __launch_bounds__(THREADS, sizeof(T) == 4 ? 4 : 2)
 
     stage_rates(rs, tab, wt.dt, cut_qs, cut_bw, THREADS);
     allow_next();
-    wait_previous();
     const bool keeps = keeps_removed(live, stats);
     const long long removed = keeps ? removed_photons(stats) : 0;  // (its loads under way with those of the counts)
     const long long total = tile_prefix<T, THREADS>(segs, n_seg, tile, s_end, s_n, s_warp, live);

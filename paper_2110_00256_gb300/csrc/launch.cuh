@@ -31,7 +31,8 @@ int resident_grid(int threads, size_t dyn, int64_t items)
 // (or exited), so that its launch and whatever it does before wait_previous()
 // overlap that kernel's tail.  wait_previous() returns when the kernel ahead has
 // ended and its writes are visible; a kernel launched this way calls it, in every
-// thread, before it touches anything that an earlier launch writes.  Used where
+// thread, before it touches anything that an earlier launch writes (one that is never
+// launched early -- the bulk copies, the fused push -- starts after it and has none).  Used where
 // the launches are most of a step (kSmallPerSm): the substep of 1e4 electrons
 // takes 13.6 us instead of 18.5; at 2e6 particles it changes nothing, and the bulk
 // pipeline loses 2 % to the waiting CTAs.

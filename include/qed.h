@@ -399,11 +399,11 @@ qed_status qed_batch_destroy(qed_batch *b);
 /* qed_substep for every patch of `b` (§3, §5), in two launches whatever the
  * number of patches: one persistent evolution launch over all 3 x n species
  * segments (tiles of every segment form one index space, so uneven patches
- * share the grid; FP32 with aligned arrays streams them through shared memory
- * by default; it adds the live counts to QED_STAT_EVOLVED); one event launch over
- * all firing lists (photon emission of the leptons and pair production of the
- * photons side by side; with the learned sampler, one launch per process),
- * which at its end clamps the counts and advances opts->d_step.  The firing
+ * share the grid; its form goes by the number of particles as qed_substep's); one
+ * event launch over all firing lists (photon emission of the leptons and pair
+ * production of the photons side by side; with the learned sampler, one launch per
+ * process), which adds the live counts that the evolution read to
+ * QED_STAT_EVOLVED and at its end clamps the counts and advances opts->d_step.  The firing
  * counts are kept in `b` during the step and written to the lists' d_count at
  * its end, so steps of one batch do not overlap.  Stream-ordered, allocates nothing,
  * graph-capturable.  Results per patch are those of qed_substep on that patch. */
@@ -564,7 +564,7 @@ qed_status qed_probe_fp64_fma(int64_t iters, int32_t ctas_per_sm, double *d_sink
 qed_status qed_probe_tanh(int64_t iters, int32_t ctas_per_sm, double *d_sink, double *tanh_per_s, float *ms_out,
                           void *stream);
 /* Not part of the method: the table-driven FP64 logarithm and exponential (Tang's
- * forms: of the rate lookups that the integers cannot hold, and of table
+ * forms: of arguments that the integer forms do not take, and of table
  * generation) beside the CUDA library's, for accuracy
  * checks.  d_out: 4 n device doubles, written as [log_tang(x) | exp_tang(x) |
  * log(x) | exp(x)] for the n device doubles d_x.  Stream-ordered; n <= 2^40. */

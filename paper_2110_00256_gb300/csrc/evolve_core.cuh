@@ -83,15 +83,6 @@ __device__ __forceinline__ void stage_rates(RateSmem<float> &s, const TablesView
     for (int i = threadIdx.x; i < tab.bw_T.n; i += threads) s.bw[i] = tab.bw_T.ln_f[i];
 }
 
-// x in units of 2^-53 (to nearest) from its bits, |x| < 700
-__device__ __forceinline__ long long fix_from_ln(double x)
-{
-    const int hi = __double2hiint(x), sh = 1032 - ((hi >> 20) & 0x7ff);  // the 53 bits << 11 have the unit 2^-63 at 2^9
-    uint64_t m = ((uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(x)) << 11;
-    m = sh > 60 ? 0 : ((m >> sh) + 1) >> 1;
-    return hi < 0 ? -(long long)m : (long long)m;
-}
-
 // the table on integers; nonzero where it does not fit: |ln f| < 700, steps below 500
 __device__ __forceinline__ int stage_fix(long long *out, const Table1D<double> &t, int threads)
 {
@@ -177,9 +168,11 @@ struct EvolvedFp64 {
     int fire, bad;
 };
 
-// The same in FP64 throughout, out of line: the particles that the integers of
-// fixed64.cuh leave to it (blocks of subnormal or huge values, infinities, NaN,
-// a force far below its terms, chi within rounding of a table's end or of the cut-off).
+// The same with chi and the interpolation in FP64, out of line: the particles that the
+// integers of fixed64.cuh leave to it (blocks of subnormal or huge values, infinities,
+// NaN, a force far below its terms, chi within rounding of a table's end or of the
+// cut-off).  They pay both forms: 4e6 leptons along a static B 526 us, photons 677 (in FP64
+// instructions throughout 705 and 838, and 603 and 730 without the integers ahead).
 static __device__ __noinline__ EvolvedFp64 evolve_one_fp64(int proc, const Table1D<double> &tb, double px, double py,
                                                            double pz, double ex, double ey, double ez, double bx,
                                                            double by, double bz, double dt, double cut, double tau)

@@ -144,6 +144,15 @@ __device__ __forceinline__ int64_t fix_exp(int64_t x, int &k, const long long *t
     return tj + ((wide(ft.h, fe.h) + ((wide(ft.h, fe.l) + wide(ft.l, fe.h)) >> 30)) >> 6);
 }
 
+// x in units of 2^-53 (to nearest) from its bits, |x| < 700
+__device__ __forceinline__ int64_t fix_from_ln(double x)
+{
+    const int hi = __double2hiint(x), sh = 1032 - ((hi >> 20) & 0x7ff);  // the 53 bits << 11 have the unit 2^-63 at 2^9
+    uint64_t m = ((uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(x)) << 11;
+    m = sh > 63 ? 0 : ((m >> sh) + 1) >> 1;
+    return hi < 0 ? -(int64_t)m : (int64_t)m;
+}
+
 // sq = sqrt(g2 2^60) for g2 in [2^58, 2^62 - 2^58], to 1, and its reciprocal:
 // 1/sqrt(g2 2^60) = inv 2^inv_e, inv in [2^62, 2^63], to 2^-59.  Newton steps on
 // the integers from the 22-bit reciprocal square root.

@@ -1,6 +1,6 @@
-// fp64_math.cuh -- table-driven FP64 exponential and logarithm: of the FP64 forms
-// behind the integer ones (fixed64.cuh: particles and draws that the integers
-// cannot hold) and of table generation.  GB300's FP64 pipe bounds those, so their
+// fp64_math.cuh -- table-driven FP64 exponential and logarithm: of table generation,
+// of the sampling's general form (the exponential), and of arguments outside the
+// integer forms' range (fixed64.cuh).  GB300's FP64 pipe bounds those, so their
 // speed is their FP64 instruction count.  Both take P. T. P. Tang's table-driven reductions (ACM TOMS 15 (1989)
 // 144 for the exponential, 16 (1990) 378 for the logarithm) with Taylor
 // polynomials of the reduced argument; the tables hold correctly rounded values

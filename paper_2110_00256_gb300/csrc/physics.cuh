@@ -15,16 +15,34 @@ __device__ __forceinline__ double d_exp(double x) { return exp(x); }
 __device__ __forceinline__ float d_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double d_sqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float d_fma(float a, float b, float c) { return fmaf(a, b, c); }
+// ln x on the integers (fixed64.cuh) for x in [2^-86, 2^86]; Tang's beyond
+__device__ __forceinline__ double log_int(double x)
+{
+    const int hi = __double2hiint(x);
+    if ((unsigned)(hi - (937 << 20)) >= (172u << 20)) return log_tang(x);  // (also zero, negative, NaN)
+    const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(x);
+    return fix_ln(m << 11, (hi >> 20) - 1023 - 63);
+}
+
+// e^x on the integers for |x| < 690 (one rounding of x to 2^-53, one of the result); Tang's beyond
+__device__ __forceinline__ double exp_int(double x)
+{
+    if ((__double2hiint(x) & 0x7fffffff) >= 0x40859000) return exp_tang(x);  // (also infinite, NaN)
+    int k;
+    const int64_t m = fix_exp(fix_from_ln(x), k, kFixExp);
+    return fix_to_double(m, k - 62);
+}
+
 // logarithm and exponential of the 1-D rate lookups: in FP32 the hardware's
 // approximate forms (__logf: absolute error ~2^-21 near 1; __expf: ~2 + 1.2 |x|
 // ulp), whose ~1e-6 relative effect on a rate is far below the tables'
-// interpolation error; in FP64 (the path behind the integer one of fixed64.cuh)
-// Tang's table-driven forms (fp64_math.cuh, within 2 ulp), which take fewer FP64
-// instructions than the library functions
+// interpolation error; in FP64 (the form behind the integer one of fixed64.cuh) the
+// integer logarithm and exponential, so that a particle that the integers gave up
+// costs no more than it did before there were any
 __device__ __forceinline__ float r_log(float x) { return __logf(x); }
-__device__ __forceinline__ double r_log(double x) { return log_tang(x); }
+__device__ __forceinline__ double r_log(double x) { return log_int(x); }
 __device__ __forceinline__ float r_exp(float x) { return __expf(x); }
-__device__ __forceinline__ double r_exp(double x) { return exp_tang(x); }
+__device__ __forceinline__ double r_exp(double x) { return exp_int(x); }
 __device__ __forceinline__ double d_fma(double a, double b, double c) { return fma(a, b, c); }
 // square root, reciprocal square root and quotient of the event kernels: FP32 as
 // they are; FP64 on the integers (fixed64.cuh) where the arguments are ordinary (an
@@ -55,18 +73,9 @@ __device__ __forceinline__ void e_norm(double p2, double &p, double &inv)
     }
 }
 
-// ln x on the integers (fixed64.cuh) for x in [2^-86, 2^86]; Tang's beyond
-__device__ __forceinline__ double log_int(double x)
-{
-    const int hi = __double2hiint(x);
-    if ((unsigned)(hi - (937 << 20)) >= (172u << 20)) return log_tang(x);  // (also zero, negative, NaN)
-    const uint64_t m = (uint64_t)((hi & 0x000fffff) | 0x00100000) << 32 | (uint32_t)__double2loint(x);
-    return fix_ln(m << 11, (hi >> 20) - 1023 - 63);
-}
-
 // logarithm and exponential of the 2-D inverse-CDF sampling: FP32 the library
 // forms; the general FP64 forms the integer logarithm (ln chi and ln r are
-// interpolation coordinates, where its 2^-57 absolute error near 1 is far below
+// interpolation coordinates, where its 2^-62 absolute error near 1 is far below
 // the tables' spacing) and Tang's exponential
 __device__ __forceinline__ float s_log(float x) { return logf(x); }
 __device__ __forceinline__ double s_log(double x) { return log_int(x); }

@@ -58,7 +58,7 @@ __device__ __forceinline__ void wave_fields(const WaveT<T> &w, T x, T &ex, T &ey
     bz = w.d * ey;
 }
 
-// the linearly polarised wave's fields that are not zero (without the sine)
+// the linearly polarised wave's fields that are not zero (the sine comes with the cosine and is not used)
 template <typename T>
 __device__ __forceinline__ void wave_fields_yz(const WaveT<T> &w, T x, T &ey, T &bz)
 {

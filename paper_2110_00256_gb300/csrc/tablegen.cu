@@ -13,8 +13,8 @@
 //   that variable (bessel_pieces_kernel) and the integrands evaluate the pieces'
 //   polynomials: 26 FMAs instead of ~25 steps of an exponential, a hyperbolic
 //   sine and divisions each.
-//   Outer integrals over xi: 16-point Gauss-Legendre on the table intervals
-//   where the integrand is smooth (gl_interval), at nodes that all rows share;
+//   Outer integrals over xi: Gauss-Legendre with 5, 8 or 16 points on the table
+//   intervals where the integrand is smooth (gl_points), at nodes that all rows share;
 //   tanh-sinh (double-exponential) quadrature (Takahasi & Mori 1974; Bailey,
 //   Jeyabalan & Li, Exp. Math. 14 (2005) 317) on the others, which absorbs the
 //   steep endpoint behaviour at xi -> 0 and 1.

@@ -36,10 +36,11 @@ qed_status check_params(const qed_table_params *p)
 // Rows of the FP32 2-D tables lie pitch32() apart: a draw's hot columns (where P is
 // large) are one or two of a row's 128-byte lines, and at a power-of-two distance
 // the rows' hot lines share a fraction of the cache's sets -- how large a one then
-// hangs on where the arrays happen to lie.  1e8 FP32 draws from 256x256 tables: ln P
-// 3.85e10 -> 5.35e10 per second (256 floats apart, as separate allocations: 4.06e10),
-// P 3.47e10 -> 3.9e10 to 4.2e10 with each process's arrays side by side (3.4e10 to
-// 3.6e10 scattered or with the guide between them; separate allocations 4.1e10 to 4.4e10).
+// hangs on where the arrays happen to lie.  5e7 FP32 draws from 256x256 tables, ten
+// tables of a process: ln P 941 us wherever they lie (256 floats apart, in separate
+// allocations: 931 to 1380, mean 1104).  P, whose hot columns spread over the row, still
+// hangs on the place: 1143 to 1553 us, mean 1298 (separate allocations: 1137 to 1676,
+// mean 1304); no pad from 0 to 160 floats and no gap up to 1 MB held for every place.
 static int pitch32(int n_xi) { return (n_xi + 31) / 32 * 32 + 32; }
 
 // Everything formed entry by entry from the FP64 tables, in one launch: the

@@ -104,3 +104,9 @@ extern "C" void host_cut(double cut, int64_t n, const int64_t *ln_chi, int64_t *
         side[i] = (c.below ? 1 : 0) + (c.near ? 2 : 0);
     }
 }
+
+// e^x and ln x of the rate lookups' FP64 form, and their table-driven forms
+extern "C" void host_logexp(int64_t n, const double *x, double *e, double *e64, double *l, double *l64)
+{
+    for (int64_t i = 0; i < n; ++i) e[i] = r_exp(x[i]), e64[i] = exp_tang(x[i]), l[i] = r_log(x[i]), l64[i] = log_tang(x[i]);
+}

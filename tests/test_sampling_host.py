@@ -99,3 +99,22 @@ def test_optical_depth_draws_are_no_further_off_than_in_fp64(lib, lo, hi):
     ref = np.where(u > 0.5, -np.log1p((u - 1.0).astype(LD)), -np.log(u.astype(LD)))
     err, err64 = (np.abs(x / ref - 1).astype(np.float64) for x in (tau, tang))
     assert rms(err) <= rms(err64) and err.max() <= err64.max() and err.max() <= 1.5 * 2.0 ** -53
+
+
+@np.errstate(all="ignore")
+def test_logarithm_and_exponential_of_the_rates_fp64_form(lib):
+    """On the integers within their range (e^x: x rounded to 2^-53 where that is coarser, the integers' 2^-58, one rounding;
+    ln x: 2^-57 and one rounding), the table-driven forms' values beyond it and for IEEE's special values."""
+    rng = np.random.default_rng(11)
+    x = np.concatenate([rng.uniform(-690, 690, 200_000), rng.uniform(-1, 1, 100_000), 10.0 ** rng.uniform(-25, 0, 50_000),
+                        2.0 ** rng.uniform(-1074, 1023, 50_000), -2.0 ** rng.uniform(-1074, 10, 50_000),
+                        [0.0, -0.0, np.inf, -np.inf, np.nan, 690.0, -690.0, np.nextafter(690, 0), -np.nextafter(690, 0), 5e-324, -1.0]])
+    e, e64, ln, l64 = (np.zeros(x.size) for _ in range(4))
+    lib.host_logexp(ctypes.c_int64(x.size), ptr(x), ptr(e), ptr(e64), ptr(ln), ptr(l64))
+    ins = np.abs(x) < 690
+    assert np.all(np.abs(e[ins] / np.exp(x[ins].astype(LD)) - 1) <= 2.0 ** -53 + 2.0 ** -54 + 2.0 ** -58)
+    assert np.array_equal(e[~ins], e64[~ins], equal_nan=True)
+    pos = (x >= 2.0 ** -86) & (x < 2.0 ** 86)
+    ref = np.log(x[pos].astype(LD))
+    assert np.all(np.abs(ln[pos] - ref) <= 2.0 ** -57 + 2.0 ** -53 * np.abs(ref))
+    assert np.array_equal(ln[~pos], l64[~pos], equal_nan=True)

@@ -283,6 +283,31 @@ __device__ __forceinline__ int64_t fix_ln_value(uint64_t n, int e, int &unit)
     return fine ? (k ? l - kLn2 : l) : kl + ((l + 32) >> 6);
 }
 
+// The same over the 256 intervals of fix_half_ln, within 2^-57 absolute at every argument:
+// of the FP32 path's optical depths, whose float pair holds 2^-48 (a pair's low word
+// is a rounding residual, and a last-bit change of the logarithm can move it by 2^-12
+// of itself a step later, so this form stays as it is).
+__device__ __forceinline__ int64_t fix_ln_48(uint64_t n, int e, int &unit)
+{
+    const int j = (int)(n >> 55) & 255;
+    const uint32_t r = (uint32_t)__ldg(&kFixLogR[j]);
+    const int64_t u = (int64_t)((uwide((uint32_t)(n >> 32), r) << 17) + (uwide((uint32_t)n, r) >> 15));  // 2^-64
+    const int a = (int)(u >> 25);                  // 2^-39
+    const int b = (int)((uint32_t)u & 0x1ffffffu);  // 2^-64
+    const int64_t h2 = (wide(a, a) + (wide(a, b) >> 24)) >> 15;  // u^2/2, 2^-64
+    int t = 429496730 - (__mulhi(a, 357913941) >> 7);            // 1/3 - u/4 + u^2/5 - u^3/6, 2^-31
+    t = 536870912 - (__mulhi(a, t) >> 7);
+    t = 715827883 - (__mulhi(a, t) >> 7);
+    const int64_t c3 = wide((int)(h2 >> 15), (int)(wide(a, t) >> 29)) >> 25;  // u^3 t, 2^-64
+    const int64_t l = __ldg(&kFixLog[j]) + ((u - h2 + c3) >> 1);              // ln m, 2^-63
+    const int k = 63 + e;
+    // k ln 2 + ln m in 2^-57, or in 2^-63 where k is 0 or -1
+    const bool fine = k == 0 || k == -1;
+    const int64_t kl = (wide(k, (int)(kHalfLn2 >> 32)) << 27) + (wide(k, (int)((uint32_t)kHalfLn2 >> 1)) >> 4);
+    unit = fine ? -63 : -57;
+    return fine ? (k ? l - 2 * kHalfLn2 : l) : kl + (l >> 6);
+}
+
 __device__ __forceinline__ double fix_ln(uint64_t n, int e)
 {
     int unit;

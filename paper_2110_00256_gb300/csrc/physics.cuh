@@ -625,6 +625,7 @@ static __device__ __noinline__ double neg_log1p_series(double u)
 
 // -ln U = v 2^unit for the 53-bit uniform U of the words (uniform53: M 2^-k, M from
 // the words' bits), without assembling U; false: U above 1 - 2^-8, by the series
+template <bool F64>
 __device__ __forceinline__ bool neg_log_words(const U4 &w, int64_t &v, int &unit)
 {
     const uint64_t d = (((uint64_t)w.y << 32) | w.x) >> 11;
@@ -633,7 +634,7 @@ __device__ __forceinline__ bool neg_log_words(const U4 &w, int64_t &v, int &unit
     const int lz = __clzll((long long)m), e = (big ? -53 : -54) - lz;
     const uint64_t n = m << lz;  // U = n 2^e
     if (e >= -64 && (e > -64 || (n >> 56) == 255)) return false;
-    v = -fix_ln_value(n, e, unit);
+    v = -(F64 ? fix_ln_value(n, e, unit) : fix_ln_48(n, e, unit));
     return true;
 }
 
@@ -643,7 +644,7 @@ __device__ __forceinline__ double tau_draw(uint64_t seed, uint64_t id, int64_t s
     const U4 w = draw(seed, id, step, purpose);
     int64_t v;
     int unit;
-    if (!neg_log_words(w, v, unit)) return neg_log1p_series(uniform53(w.x, w.y));
+    if (!neg_log_words<true>(w, v, unit)) return neg_log1p_series(uniform53(w.x, w.y));
     return fix_to_double(v, unit);
 }
 
@@ -676,7 +677,7 @@ __device__ __forceinline__ void store_draw(float *tau, float *tau_c, int64_t i, 
     int64_t v;
     int unit;
     float h, c;
-    if (neg_log_words(w, v, unit))
+    if (neg_log_words<false>(w, v, unit))
         split_fixed(v, unit, h, c);
     else
         split_f32_pair(neg_log1p_series(uniform53(w.x, w.y)), h, c);

@@ -90,7 +90,7 @@ extern "C" void host_draw(int64_t n, const uint32_t *lo, const uint32_t *hi, dou
         int64_t v;
         int unit;
         u[i] = uniform53(lo[i], hi[i]);
-        draw[i] = neg_log_words(U4{lo[i], hi[i], 0, 0}, v, unit) ? fix_to_double(v, unit) : neg_log1p_series(u[i]);
+        draw[i] = neg_log_words<true>(U4{lo[i], hi[i], 0, 0}, v, unit) ? fix_to_double(v, unit) : neg_log1p_series(u[i]);
         tang[i] = u[i] > 1.0 - 0x1p-8 ? neg_log1p_series(u[i]) : -log_tang_core(u[i], 0);
     }
 }
